@@ -118,6 +118,7 @@ int create_plan(clear_plan_t **out, const Shape &shape_in, bool host_only)
     }
     if (!host_only) {
         CLEAR_CUDA_TRY(cudaGetDevice(&p->device));
+        CLEAR_CUDA_TRY(cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, p->device));
         rc = upload(&p->d_half_width, p->sch.half_width);
         if (rc == CLEAR_OK) rc = upload(&p->d_items, p->sch.items);
         if (rc == CLEAR_OK) rc = upload(&p->d_tiles, p->sch.tiles);
@@ -263,6 +264,8 @@ int forward(const clear_plan *p, const void *q, const void *k, const void *v, vo
         rc = launch_tc(*p, q, k, v, out, scale, st);
     else if (p->kernel == CLEAR_KERNEL_TCGEN05_WS)
         rc = launch_ws(*p, q, k, v, out, scale, st);
+    else if (p->shape.mask_kind == CLEAR_MASK_DISC || p->shape.mask_kind == CLEAR_MASK_SQUARE)
+        rc = launch_f32(*p, q, k, v, out, scale, st);
     else
         rc = launch_simt(*p, q, k, v, out, scale, st);
     if (rc != CLEAR_OK) return rc;

@@ -3,7 +3,8 @@
 // through which the distillation losses of Sec. 3.3 (Eq. 4-6) reach the attention parameters.
 //
 // Two kernels, one warp per token, lanes split the head dimension, tokens walked as in the forward CUDA-core
-// kernel (the text tokens, then per grid row within reach the clipped run of columns):
+// kernel (the text tokens, then per grid row within reach the clipped run of columns).  Head sizes above 128 only: up to
+// there the tiled kernels of clear_f32_bwd.cu are 6 to 8 times faster, above their row sets do not fit shared memory.
 //   query kernel: sweep 1 over the query's keys: online softmax -> row maximum m, row sum l, the un-normalised
 //       output, hence delta = dO . O; the three row statistics are kept for the second kernel;
 //       sweep 2: p = exp(s - m) / l, dP = dO . v, dS = p (dP - delta), dQ += scale dS k;
@@ -211,15 +212,6 @@ int launch_bwd_typed(const clear_plan &p, const void *q, const void *k, const vo
 {
     const Shape &s = p.shape;
     const int64_t N = (int64_t)s.n_text + (int64_t)s.grid_h * s.grid_w;
-    // row statistics (m, 1 / l, delta) of every query: owned by the plan, allocated on its first backward call
-    // (calls of one plan are ordered on the device, so one buffer serves them all)
-    if (!p.d_bwd_stats) {
-        cudaError_t e = cudaMalloc((void **)&p.d_bwd_stats, (size_t)s.B * s.H * N * 3 * sizeof(float));
-        if (e != cudaSuccess) {
-            (void)cudaGetLastError();
-            return e == cudaErrorMemoryAllocation ? CLEAR_ERR_NO_MEMORY : CLEAR_ERR_CUDA;
-        }
-    }
     dim3 grid((unsigned)((N + kWarpsPerBlock - 1) / kWarpsPerBlock), (unsigned)(s.B * s.H));
     dim3 block(kWarpsPerBlock * 32);
     const int n_hw = (int)p.sch.half_width.size();
@@ -236,10 +228,6 @@ int launch_bwd_typed(const clear_plan &p, const void *q, const void *k, const vo
                                                                p.d_half_width, n_hw, scale);                            \
         break;
     switch (epl) {
-        CLEAR_BWD_CASE(1)
-        CLEAR_BWD_CASE(2)
-        CLEAR_BWD_CASE(3)
-        CLEAR_BWD_CASE(4)
         CLEAR_BWD_CASE(5)
         CLEAR_BWD_CASE(6)
         CLEAR_BWD_CASE(7)
@@ -254,9 +242,27 @@ int launch_bwd_typed(const clear_plan &p, const void *q, const void *k, const vo
 
 }  // namespace
 
+// Row statistics (m, 1 / l, delta) of every query: owned by the plan, allocated on its first backward call (calls of one
+// plan are ordered on the device, so one buffer serves them all).
+int ensure_bwd_stats(const clear_plan &p)
+{
+    if (p.d_bwd_stats) return CLEAR_OK;
+    const Shape &s = p.shape;
+    const int64_t N = (int64_t)s.n_text + (int64_t)s.grid_h * s.grid_w;
+    cudaError_t e = cudaMalloc((void **)&p.d_bwd_stats, (size_t)s.B * s.H * N * 3 * sizeof(float));
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? CLEAR_ERR_NO_MEMORY : CLEAR_ERR_CUDA;
+    }
+    return CLEAR_OK;
+}
+
 int launch_bwd(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
                void *dv, float scale, cudaStream_t stream)
 {
+    if (p.shape.head_dim <= 128) return launch_f32_bwd(p, q, k, v, d_out, dq, dk, dv, scale, stream);
+    const int rc = ensure_bwd_stats(p);
+    if (rc != CLEAR_OK) return rc;
     if (p.shape.dtype == CLEAR_F32) return launch_bwd_typed<float>(p, q, k, v, d_out, dq, dk, dv, scale, stream);
     return launch_bwd_typed<__nv_bfloat16>(p, q, k, v, d_out, dq, dk, dv, scale, stream);
 }

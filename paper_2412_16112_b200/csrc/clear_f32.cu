@@ -1,0 +1,271 @@
+// CLEAR attention forward on the CUDA cores, fp32 arithmetic throughout, as a tiled kernel: 64 queries against 64
+// keys at a time from shared memory (f32_tile.cuh).
+//
+// Serves fp32 tensors (where tensor-core input rounding would break a 1e-5 agreement), bf16 tensors of head sizes the
+// tensor-core kernels do not take, and non-positive scales, under the windows around the query (disc, square).
+//
+// What bounds it: the fp32 multiply-add units (2 x 64 x 64 x DP multiply-adds a step, DP = the head size rounded up
+// to 64, 128 or 256).  The keys are those of the union of the tile's windows and no others: rows are gathered run by
+// run, 64 at a time, so a step is only ever short at the end of the list.  An 8 x 8 patch is the split that wastes
+// least at the paper's radii with a 4 x 4 register tile: at r = 8 a patch walks 464 + n_text keys for windows of 193.
+// Two blocks share an SM (DP <= 128): one computes while the other waits for its rows.
+// A problem too small to give every SM a tile cuts the lists over a cluster of up to 8 blocks, which merge their
+// partial softmax through distributed shared memory in a fixed order: no workspace, no second launch.
+#include <cuda_bf16.h>
+#include <math_constants.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "clear_internal.hpp"
+#include "f32_tile.cuh"
+
+namespace clear {
+namespace {
+
+using namespace f32tile;
+namespace cg = cooperative_groups;
+
+struct F32Params {
+    Geometry g;
+    const void *q, *k, *v;
+    void *out;
+    int n_split;
+    float scale;
+};
+
+template <int DP> constexpr size_t forward_smem()
+{
+    return 3 * (size_t)kRows * kStride<DP> * sizeof(float) + 2 * sizeof(KeyTile) + 2 * kRows * sizeof(float) + 64 * sizeof(int);
+}
+
+template <typename T, int DP>
+__global__ void __launch_bounds__(kThreads, DP <= 128 ? 2 : 1)
+clear_f32_tile_kernel(const F32Params p)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    float *sQ = reinterpret_cast<float *>(smem), *sK = sQ + kRows * kStride<DP>, *sV = sK + kRows * kStride<DP>;
+    float *sP = sK;   // the weights take the place of the keys once the scores are in registers
+    KeyTile *keys = reinterpret_cast<KeyTile *>(sV + kRows * kStride<DP>);
+    float *sM = reinterpret_cast<float *>(keys + 2), *sL = sM + kRows;
+    int *red = reinterpret_cast<int *>(sL + kRows);
+
+    const int tid = threadIdx.x, ty = (tid >> 5) * 2 + ((tid >> 4) & 1), tx = tid & 15;
+    const int part = (int)(blockIdx.x % (unsigned)p.n_split);   // rank in the cluster
+    const TileRef tile = tile_of((int)(blockIdx.x / (unsigned)p.n_split), p.g);
+    const KeyRuns runs = runs_of(tile, p.g);
+    const long long base = (long long)tile.bh * runs.n_tokens * p.g.d;
+    const T *q = static_cast<const T *>(p.q) + base, *k = static_cast<const T *>(p.k) + base,
+            *v = static_cast<const T *>(p.v) + base;
+
+    // this block's share of the list: whole steps of 64 keys
+    const int n_steps_all = (list_length(runs, red) + kRows - 1) / kRows;
+    const int per = (n_steps_all + p.n_split - 1) / p.n_split;
+    const int step0 = min(part * per, n_steps_all), n_steps = min(per, n_steps_all - step0);
+    KeyCursor cur;
+    if (tid < kRows) {
+        cur.start(runs);
+        cur.advance(runs, step0 * kRows + tid);
+        int qy, qx;
+        keys[1].token[tid] = tile_token(tile, tid, p.g, qy, qx);
+    }
+    fill_key_tile(keys[0], cur, runs, n_steps > 0);
+    __syncthreads();
+    load_rows<T, DP>(sQ, q, keys[1].token, p.g.d);
+
+    int q_y[4], q_x[4];
+    long long q_tok[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q_tok[i] = tile_token(tile, ty + 16 * i, p.g, q_y[i], q_x[i]);
+
+    uint64_t o[4][DP / 64][2];
+    zero_acc<DP>(o);
+    float m[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        m[i] = -CUDART_INF_F;
+        l[i] = 0.f;
+    }
+
+    for (int s = 0; s < n_steps; ++s) {
+        const KeyTile &kt = keys[s & 1];
+        load_rows<T, DP>(sK, k, kt.token, p.g.d);
+        load_rows<T, DP>(sV, v, kt.token, p.g.d);
+        cp_async_wait<1>();   // Q and K are here
+        __syncthreads();
+        if (s + 1 < n_steps) fill_key_tile(keys[(s + 1) & 1], cur, runs, true);
+
+        float w[4][4];
+        tile_dot<DP>(sQ, sK, ty, tx, w);
+        __syncthreads();      // every warp is done with the keys: the weights may land on them
+
+        // online softmax; a row's 64 scores sit in 16 lanes of one warp
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float mx = -CUDART_INF_F;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = tx + 16 * j;
+                const bool on = kt.token[c] >= 0 && sees(runs, q_y[i], q_x[i], kt.ky[c], kt.kx[c]);
+                w[i][j] = on ? w[i][j] * p.scale : -CUDART_INF_F;
+                mx = fmaxf(mx, w[i][j]);
+            }
+            const float m_new = fmaxf(m[i], row_max16(mx));
+            const float m_ref = m_new == -CUDART_INF_F ? 0.f : m_new;
+            const float alpha = expf(m[i] - m_ref);   // m = -inf: 0
+            m[i] = m_new;
+            l[i] *= alpha;
+            const uint64_t a2 = ptx::pack2(alpha, alpha);
+#pragma unroll
+            for (int c = 0; c < DP / 64; ++c) {
+                o[i][c][0] = ptx::mul2(o[i][c][0], a2);
+                o[i][c][1] = ptx::mul2(o[i][c][1], a2);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float e = expf(w[i][j] - m_ref);
+                l[i] += e;
+                sP[(ty + 16 * i) * kPStride + tx + 16 * j] = e;
+            }
+        }
+        cp_async_wait<0>();
+        __syncthreads();      // V has landed for everybody, and the weights are written
+        tile_accumulate<DP>(sP, sV, ty, tx, o);
+        __syncthreads();      // before the next rows overwrite K, V
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) l[i] = row_sum16(l[i]);
+
+    T *out = static_cast<T *>(p.out) + base;
+    if (p.n_split == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            // a query sees itself or the text keys: l > 0 for every row that exists
+            const float inv = l[i] > 0.f ? 1.f / l[i] : 0.f;
+#pragma unroll
+            for (int c = 0; c < DP / 64; ++c) {
+                const int ch = 64 * c + 4 * tx;
+                if (q_tok[i] >= 0 && ch < p.g.d) store4(out + q_tok[i] * p.g.d + ch, acc_float4(o[i][c], inv));
+            }
+        }
+        return;
+    }
+
+    // merge over the cluster: every block leaves its un-normalised rows, maxima and sums in its own shared memory and
+    // finishes 64 / n_split rows from everybody's, in the order of the ranks
+    cg::cluster_group cluster = cg::this_cluster();
+    cp_async_wait<0>();
+    __syncthreads();
+    acc_to_rows<DP>(o, sV, ty, tx);
+    if (tx == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            sM[ty + 16 * i] = m[i];
+            sL[ty + 16 * i] = l[i];
+        }
+    }
+    cluster.sync();
+    const int rows = kRows / p.n_split;
+    for (int e = tid; e < rows * (DP / 4); e += kThreads) {
+        const int r = part * rows + e / (DP / 4), ch = e % (DP / 4) * 4;
+        int qy, qx;
+        const long long tok = tile_token(tile, r, p.g, qy, qx);
+        float mx = -CUDART_INF_F;
+        for (int c = 0; c < p.n_split; ++c) mx = fmaxf(mx, cluster.map_shared_rank(sM, c)[r]);
+        if (mx == -CUDART_INF_F) mx = 0.f;
+        float sum = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < p.n_split; ++c) {
+            const float f = expf(cluster.map_shared_rank(sM, c)[r] - mx);
+            sum = fmaf(f, cluster.map_shared_rank(sL, c)[r], sum);
+            const float4 x = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(sV, c) + r * kStride<DP> + ch);
+            acc.x = fmaf(f, x.x, acc.x);
+            acc.y = fmaf(f, x.y, acc.y);
+            acc.z = fmaf(f, x.z, acc.z);
+            acc.w = fmaf(f, x.w, acc.w);
+        }
+        const float inv = sum > 0.f ? 1.f / sum : 0.f;
+        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+        if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, acc);
+    }
+    cluster.sync();   // nobody leaves while its rows are being read
+}
+
+constexpr int blocks_per_sm(int d) { return d <= 128 ? 2 : 1; }
+
+template <typename T>
+int launch_typed(const F32Params &p, long long tiles, cudaStream_t stream)
+{
+    if (p.g.d <= 64) return launch_tiles(clear_f32_tile_kernel<T, 64>, p, tiles, p.n_split, forward_smem<64>(), stream);
+    if (p.g.d <= 128) return launch_tiles(clear_f32_tile_kernel<T, 128>, p, tiles, p.n_split, forward_smem<128>(), stream);
+    return launch_tiles(clear_f32_tile_kernel<T, 256>, p, tiles, p.n_split, forward_smem<256>(), stream);
+}
+
+}  // namespace
+
+namespace f32tile {
+
+Geometry geometry_of(const clear_plan &p)
+{
+    const Shape &s = p.shape;
+    Geometry g{};
+    g.half_width = p.d_half_width;
+    g.n_half_width = (int)p.sch.half_width.size();
+    g.grid_h = s.grid_h;
+    g.grid_w = s.grid_w;
+    g.n_text = s.n_text;
+    g.d = s.head_dim;
+    g.n_bh = s.B * s.H;
+    // 8 x 8 has the smallest union of windows; a grid narrower than that in one direction takes a longer patch, so
+    // that the tile's rows are not spent on cells off the grid
+    g.patch_w_log = 3;
+    while (g.patch_w_log > 0 && s.grid_w <= (1 << (g.patch_w_log - 1))) --g.patch_w_log;
+    while (g.patch_w_log < 6 && s.grid_h <= (kRows >> (g.patch_w_log + 1)) && s.grid_w > (1 << g.patch_w_log)) ++g.patch_w_log;
+    return g;
+}
+
+Extent extent_of(const clear_plan &p, const Geometry &g)
+{
+    const std::vector<int32_t> &hw = p.sch.half_width;
+    const long long T = g.n_text, N = g.n_tokens(), R = (long long)hw.size() - 1;
+    const long long n_txt = (T + kRows - 1) / kRows;
+    const long long n_img = (long long)((g.grid_h + g.patch_h() - 1) / g.patch_h()) * ((g.grid_w + g.patch_w() - 1) / g.patch_w());
+    // the list of an interior patch, as far as the grid has the columns and the tokens
+    long long keys = T;
+    for (long long dy = -R; dy < g.patch_h() + R && keys < N; ++dy) {
+        const long long dist = dy < 0 ? -dy : std::max(0ll, dy - (g.patch_h() - 1));
+        keys += std::min<long long>(g.grid_w, g.patch_w() + 2ll * hw[(size_t)dist]);
+    }
+    const long long img_steps = (std::min(keys, N) + kRows - 1) / kRows, txt_steps = (N + kRows - 1) / kRows;
+    return Extent{n_txt + n_img, n_txt > 0 ? std::max(img_steps, txt_steps) : img_steps, n_txt * txt_steps + n_img * img_steps};
+}
+
+// The fewest blocks with which the longest list is no longer than an even share of all steps over the resident
+// blocks, each with a step of its own: 1 where there are plenty of tiles; 8 for the tiny configuration (10 tiles of at
+// most 5 steps) and for a 1024px problem of two heads, whose text tiles walk 72 steps and its patches 15.
+int split_of(const Extent &e, int n_bh, int slots)
+{
+    int n = 1;
+    while (n < 8 && e.longest > n && (e.longest + n - 1) / n > std::max(1ll, e.steps * n_bh / slots)) n *= 2;
+    return n;
+}
+
+}  // namespace f32tile
+
+int launch_f32(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale, cudaStream_t stream)
+{
+    F32Params prm{};
+    prm.g = geometry_of(p);
+    prm.q = q;
+    prm.k = k;
+    prm.v = v;
+    prm.out = out;
+    prm.scale = scale;
+    const Extent e = extent_of(p, prm.g);
+    prm.n_split = split_of(e, prm.g.n_bh, p.n_sm * blocks_per_sm(prm.g.d));
+    const long long tiles = e.tiles * prm.g.n_bh;
+    if (p.shape.dtype == CLEAR_F32) return launch_typed<float>(prm, tiles, stream);
+    return launch_typed<__nv_bfloat16>(prm, tiles, stream);
+}
+
+}  // namespace clear

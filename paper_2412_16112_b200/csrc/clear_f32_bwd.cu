@@ -1,0 +1,342 @@
+// Backward pass of the CLEAR attention operator on the CUDA cores, fp32 arithmetic, as tiled kernels: 64 stationary
+// tokens against 64 streamed tokens at a time from shared memory (f32_tile.cuh).  Head sizes up to 128; the wider ones
+// do not leave room for four row sets and keep the kernels that take one warp per token (clear_bwd.cu).
+//
+//   query kernel: stationary Q_i, dO_i, streamed K_j, V_j.  Sweep 1: S = Q K^T and dP = dO V^T, an online softmax of S
+//       and with it delta = sum_j p dP / l (= dO . O); the three row statistics are left for the key kernel.  Sweep 2:
+//       p = exp(S - m) / l, dS = p (dP - delta) scale, dQ += dS K.
+//   key kernel: stationary K_j, V_j, streamed Q_i, dO_i with their statistics (the mask is symmetric, so the queries
+//       that see a key are the tokens that key's own query sees).  dV += P^T dO, dK += dS^T Q.
+// Bound by the fp32 multiply-add units: nine products of 64 x 64 x DP per pair of tiles.  The streamed rows go through
+// a ring of three buffers, so a row set travels while the two before it are worked on and a step has two barriers.
+// Every output element has one writer and a fixed order of summation (a list cut over a cluster is summed in the order
+// of the ranks): results repeat bit for bit.
+#include <cuda_bf16.h>
+#include <math_constants.h>
+
+#include "clear_internal.hpp"
+#include "f32_tile.cuh"
+
+namespace clear {
+namespace {
+
+using namespace f32tile;
+namespace cg = cooperative_groups;
+
+struct F32BwdParams {
+    Geometry g;
+    const void *q, *k, *v, *d_out;
+    void *out1, *out2;   // query kernel: dq, -; key kernel: dk, dv
+    float *stats;        // [bh][token][3]: m, 1 / l, delta
+    int n_split;
+    float scale;
+};
+
+template <int DP> struct BwdSmem {
+    float a1[kRows * kStride<DP>], a2[kRows * kStride<DP>];    // stationary rows
+    float ring[3][kRows * kStride<DP>];                        // streamed rows
+    float w[kRows * kPStride];                                 // weights of the accumulation
+    float row[3][kRows];                                       // query kernel: this block's m, l, delta
+    float col[3][3][kRows];                                    // key kernel: statistics of three streamed tiles
+    KeyTile keys[3];
+    int tokens[kRows];
+    int red[8];
+};
+
+// One streamed step after another: in step s the second row set (B2: V, or dO) of tile s is used first, then the first
+// (B1: K, or Q).  Positions 2 s and 2 s + 1 of a ring of three: B2 of the next tile lands where B1 of the tile before
+// was, B1 of the next tile where B2 of this one was.
+template <typename T, int DP> struct Stream {
+    BwdSmem<DP> &sm;
+    const KeyRuns &runs;
+    const T *b1, *b2;
+    const float *stats;   // of this (batch, head), or null
+    int d, first, n_steps, n_iters;   // first step of this block's share, its steps, steps of all sweeps
+    KeyCursor cur;
+
+    __device__ __forceinline__ float *slot(int pos) const { return sm.ring[pos % 3]; }
+    __device__ __forceinline__ float *b1_rows(int it) const { return slot(2 * it + 1); }
+    __device__ __forceinline__ float *b2_rows(int it) const { return slot(2 * it); }
+    // list of the tile of step `it`
+    __device__ __forceinline__ void fill(int it)
+    {
+        if (it >= n_iters) return;
+        if (threadIdx.x < kRows && it % n_steps == 0) {
+            cur.start(runs);
+            cur.advance(runs, first * kRows + (int)threadIdx.x);
+        }
+        fill_key_tile(sm.keys[it % 3], cur, runs, true);
+        if (stats && threadIdx.x < kRows) {
+            const int tok = sm.keys[it % 3].token[threadIdx.x];
+#pragma unroll
+            for (int u = 0; u < 3; ++u) sm.col[it % 3][u][threadIdx.x] = tok >= 0 ? __ldg(stats + 3ll * tok + u) : 0.f;
+        }
+    }
+    __device__ __forceinline__ void load_b2(int it)
+    {
+        if (it < n_iters)
+            load_rows<T, DP>(b2_rows(it), b2, sm.keys[it % 3].token, d);
+        else
+            cp_async_commit();
+    }
+    __device__ __forceinline__ void load_b1(int it)
+    {
+        if (it < n_iters)
+            load_rows<T, DP>(b1_rows(it), b1, sm.keys[it % 3].token, d);
+        else
+            cp_async_commit();
+    }
+};
+
+// Rows of an accumulator to global memory, summed over the cluster first when the list is cut.
+template <typename T, int DP>
+__device__ __forceinline__ void store_acc(const uint64_t (&acc)[4][DP / 64][2], float *scratch, T *out, const F32BwdParams &p,
+                                          const TileRef &tile, int part, int ty, int tx)
+{
+    if (p.n_split == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            int y, x;
+            const long long tok = tile_token(tile, ty + 16 * i, p.g, y, x);
+#pragma unroll
+            for (int c = 0; c < DP / 64; ++c) {
+                const int ch = 64 * c + 4 * tx;
+                if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, acc_float4(acc[i][c], 1.f));
+            }
+        }
+        return;
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    acc_to_rows<DP>(acc, scratch, ty, tx);
+    cluster.sync();
+    const int rows = kRows / p.n_split;
+    for (int e = threadIdx.x; e < rows * (DP / 4); e += kThreads) {
+        const int r = part * rows + e / (DP / 4), ch = e % (DP / 4) * 4;
+        int y, x;
+        const long long tok = tile_token(tile, r, p.g, y, x);
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < p.n_split; ++c) {
+            const float4 v = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(scratch, c) + r * kStride<DP> + ch);
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
+        }
+        if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, a);
+    }
+    cluster.sync();   // nobody leaves, or reuses the rows, while they are being read
+}
+
+template <typename T, int DP, bool KEY_ROLE>
+__global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kernel(const F32BwdParams p)
+{
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    BwdSmem<DP> &sm = *reinterpret_cast<BwdSmem<DP> *>(smem_raw);
+    const int tid = threadIdx.x, ty = (tid >> 5) * 2 + ((tid >> 4) & 1), tx = tid & 15;
+    const int part = (int)(blockIdx.x % (unsigned)p.n_split);
+    const TileRef tile = tile_of((int)(blockIdx.x / (unsigned)p.n_split), p.g);
+    const KeyRuns runs = runs_of(tile, p.g);
+    const long long base = (long long)tile.bh * runs.n_tokens * p.g.d;
+    const T *q = static_cast<const T *>(p.q) + base, *k = static_cast<const T *>(p.k) + base,
+            *v = static_cast<const T *>(p.v) + base, *go = static_cast<const T *>(p.d_out) + base;
+    float *stats = p.stats + (long long)tile.bh * runs.n_tokens * 3;
+
+    const int n_all = (list_length(runs, sm.red) + kRows - 1) / kRows, per = (n_all + p.n_split - 1) / p.n_split;
+    const int step0 = min(part * per, n_all), n_steps = min(per, n_all - step0);
+    Stream<T, DP> st{sm, runs, KEY_ROLE ? q : k, KEY_ROLE ? go : v, KEY_ROLE ? stats : nullptr, p.g.d, step0, n_steps,
+                     KEY_ROLE ? n_steps : 2 * n_steps};
+    if (tid < kRows) {
+        int y, x;
+        sm.tokens[tid] = tile_token(tile, tid, p.g, y, x);
+    }
+    st.fill(0);
+    st.fill(1);
+    __syncthreads();
+    load_rows<T, DP>(sm.a1, KEY_ROLE ? k : q, sm.tokens, p.g.d);
+    load_rows<T, DP>(sm.a2, KEY_ROLE ? v : go, sm.tokens, p.g.d);
+    st.load_b2(0);
+    st.load_b1(0);
+
+    int r_y[4], r_x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tile_token(tile, ty + 16 * i, p.g, r_y[i], r_x[i]);
+    uint64_t acc1[4][DP / 64][2], acc2[4][DP / 64][2];
+    zero_acc<DP>(acc1);
+    zero_acc<DP>(acc2);
+    float m[4], l[4], dl[4];   // query kernel: row maximum, row sum (then its inverse), delta
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        m[i] = -CUDART_INF_F;
+        l[i] = dl[i] = 0.f;
+    }
+
+    // the row statistics after sweep 1: over the row's 16 lanes, then over the cluster
+    auto close_sweep1 = [&]() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            l[i] = row_sum16(l[i]);
+            dl[i] = row_sum16(dl[i]);
+        }
+        if (p.n_split > 1) {
+            cg::cluster_group cluster = cg::this_cluster();
+            if (tx == 0)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    sm.row[0][ty + 16 * i] = m[i];
+                    sm.row[1][ty + 16 * i] = l[i];
+                    sm.row[2][ty + 16 * i] = dl[i];
+                }
+            cluster.sync();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = ty + 16 * i;
+                float mx = -CUDART_INF_F, sl = 0.f, sd = 0.f;
+                for (int c = 0; c < p.n_split; ++c) mx = fmaxf(mx, cluster.map_shared_rank(sm.row[0], c)[r]);
+                const float m_ref = mx == -CUDART_INF_F ? 0.f : mx;
+                for (int c = 0; c < p.n_split; ++c) {
+                    const float f = expf(cluster.map_shared_rank(sm.row[0], c)[r] - m_ref);
+                    sl = fmaf(f, cluster.map_shared_rank(sm.row[1], c)[r], sl);
+                    sd = fmaf(f, cluster.map_shared_rank(sm.row[2], c)[r], sd);
+                }
+                m[i] = mx;
+                l[i] = sl;
+                dl[i] = sd;
+            }
+            cluster.sync();
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            l[i] = l[i] > 0.f ? 1.f / l[i] : 0.f;   // l >= 1 for every row that exists (it sees itself or the text)
+            dl[i] *= l[i];
+            if (m[i] == -CUDART_INF_F) m[i] = 0.f;
+            const long long tok = sm.tokens[ty + 16 * i];
+            if (part == 0 && tx == 0 && tok >= 0) {
+                stats[tok * 3] = m[i];
+                stats[tok * 3 + 1] = l[i];
+                stats[tok * 3 + 2] = dl[i];
+            }
+        }
+    };
+    if (!KEY_ROLE && n_steps == 0) close_sweep1();   // a cluster's block without a share takes part in the merges
+
+    for (int it = 0; it < st.n_iters; ++it) {
+        const bool sweep1 = !KEY_ROLE && it < n_steps;
+        const KeyTile &kt = sm.keys[it % 3];
+        cp_async_wait<1>();   // the stationary rows and B2 of this step are here
+        __syncthreads();      // ... for everybody, and B1 of the step before is free
+        st.load_b2(it + 1);
+        float g[4][4], s[4][4];
+        tile_dot<DP>(sm.a2, st.b2_rows(it), ty, tx, g);
+        if (!KEY_ROLE) {
+            cp_async_wait<1>();
+            __syncthreads();  // B1 is here, B2 is free
+            st.load_b1(it + 1);
+            st.fill(it + 2);
+        } else {
+            cp_async_wait<1>();
+            __syncthreads();
+        }
+        tile_dot<DP>(sm.a1, st.b1_rows(it), ty, tx, s);
+
+        if (sweep1) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float mx = -CUDART_INF_F;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int c = tx + 16 * j;
+                    const bool on = kt.token[c] >= 0 && sees(runs, r_y[i], r_x[i], kt.ky[c], kt.kx[c]);
+                    s[i][j] = on ? s[i][j] * p.scale : -CUDART_INF_F;
+                    mx = fmaxf(mx, s[i][j]);
+                }
+                const float m_new = fmaxf(m[i], row_max16(mx)), m_ref = m_new == -CUDART_INF_F ? 0.f : m_new;
+                const float alpha = expf(m[i] - m_ref);   // m = -inf: 0
+                m[i] = m_new;
+                l[i] *= alpha;
+                dl[i] *= alpha;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float e = expf(s[i][j] - m_ref);
+                    l[i] += e;
+                    dl[i] = fmaf(e, g[i][j], dl[i]);
+                }
+            }
+            if (it + 1 == n_steps) close_sweep1();
+            continue;
+        }
+
+        // P and dS in place of S and dP
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = tx + 16 * j;
+                const bool on = kt.token[c] >= 0 && sees(runs, r_y[i], r_x[i], kt.ky[c], kt.kx[c]);
+                const float mm = KEY_ROLE ? sm.col[it % 3][0][c] : m[i], il = KEY_ROLE ? sm.col[it % 3][1][c] : l[i],
+                            de = KEY_ROLE ? sm.col[it % 3][2][c] : dl[i];
+                const float pr = on ? expf(s[i][j] * p.scale - mm) * il : 0.f;
+                s[i][j] = pr;
+                g[i][j] = pr * (g[i][j] - de) * p.scale;
+            }
+        if (KEY_ROLE) {
+            // dV += P^T dO; a row of weights is written and read by one warp
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sm.w[(ty + 16 * i) * kPStride + tx + 16 * j] = s[i][j];
+            __syncwarp();
+            tile_accumulate<DP>(sm.w, st.b2_rows(it), ty, tx, acc2);
+            __syncthreads();   // B2 is free
+            st.load_b1(it + 1);
+            st.fill(it + 2);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sm.w[(ty + 16 * i) * kPStride + tx + 16 * j] = g[i][j];
+        __syncwarp();
+        tile_accumulate<DP>(sm.w, st.b1_rows(it), ty, tx, acc1);   // dQ += dS K, or dK += dS^T Q
+        __syncwarp();
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    store_acc<T, DP>(acc1, sm.ring[0], static_cast<T *>(p.out1) + base, p, tile, part, ty, tx);
+    if (KEY_ROLE) store_acc<T, DP>(acc2, sm.ring[1], static_cast<T *>(p.out2) + base, p, tile, part, ty, tx);
+}
+
+template <typename T, int DP>
+int launch_dp(F32BwdParams p, void *dq, void *dk, void *dv, long long tiles, cudaStream_t stream)
+{
+    p.out1 = dq;
+    const int rc = launch_tiles(clear_f32_bwd_kernel<T, DP, false>, p, tiles, p.n_split, sizeof(BwdSmem<DP>), stream);
+    if (rc != CLEAR_OK) return rc;
+    p.out1 = dk;
+    p.out2 = dv;
+    return launch_tiles(clear_f32_bwd_kernel<T, DP, true>, p, tiles, p.n_split, sizeof(BwdSmem<DP>), stream);
+}
+
+}  // namespace
+
+int launch_f32_bwd(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
+                   void *dv, float scale, cudaStream_t stream)
+{
+    const int rc = ensure_bwd_stats(p);
+    if (rc != CLEAR_OK) return rc;
+    F32BwdParams prm{};
+    prm.g = geometry_of(p);
+    prm.q = q;
+    prm.k = k;
+    prm.v = v;
+    prm.d_out = d_out;
+    prm.stats = p.d_bwd_stats;
+    prm.scale = scale;
+    const Extent e = extent_of(p, prm.g);
+    prm.n_split = split_of(e, prm.g.n_bh, p.n_sm * (prm.g.d <= 64 ? 2 : 1));
+    const long long tiles = e.tiles * prm.g.n_bh;
+    if (p.shape.dtype == CLEAR_F32)
+        return prm.g.d <= 64 ? launch_dp<float, 64>(prm, dq, dk, dv, tiles, stream) : launch_dp<float, 128>(prm, dq, dk, dv, tiles, stream);
+    return prm.g.d <= 64 ? launch_dp<__nv_bfloat16, 64>(prm, dq, dk, dv, tiles, stream)
+                         : launch_dp<__nv_bfloat16, 128>(prm, dq, dk, dv, tiles, stream);
+}
+
+}  // namespace clear

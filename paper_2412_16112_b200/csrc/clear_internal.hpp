@@ -32,6 +32,7 @@ struct clear_plan {
     int kernel = CLEAR_KERNEL_SIMT;  // selected kernel (never AUTO)
     bool host_only = false;
     int device = -1;
+    int n_sm = 0;
 
     // device tables (owned)
     int32_t *d_half_width = nullptr;
@@ -95,11 +96,17 @@ void note_cuda_error(int err);
 
 int launch_simt(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale,
                 cudaStream_t stream);
+// The tiled form of the CUDA-core path, for the windows around the query (disc, square).
+int launch_f32(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale,
+               cudaStream_t stream);
 int launch_tc(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale,
               cudaStream_t stream);
 int launch_ws(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale,
               cudaStream_t stream);
 // Backward pass on the CUDA cores (fp32 arithmetic; tensors of the plan's dtype): a query kernel and a key kernel.
+int launch_f32_bwd(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
+                   void *dv, float scale, cudaStream_t stream);
+int ensure_bwd_stats(const clear_plan &p);
 int launch_bwd(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
                void *dv, float scale, cudaStream_t stream);
 // Row-band form: one (O, m, l) record per text row from a band-text plan's partial results, and the merge of the
