@@ -5,7 +5,8 @@
 // text row, the un-normalised result over ITS keys with the row's maximum and sum, and the merge over GPUs is
 // the merge of a split softmax: exact, and as cheap to exchange as the patch-wise average of Eq. 7, which is
 // here as the second mode of the same merge kernel.
-//   clear_text_export_kernel  partial results of the key splits of one GPU -> one (O, m, l) record per text row
+//   clear_tc_combine_kernel   (clear_tc.cu) partial results of the key splits of one GPU -> one record per text row: D values
+//                             of O (relative to m), then m (log2 units, scale included), then l
 //   clear_text_merge_kernel   records of all GPUs -> bf16 text rows (exact merge, or Eq. 7's average)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -17,34 +18,6 @@
 
 namespace clear {
 namespace {
-
-// One block per (text row, bh), one thread per channel.  Record layout: D values of O (relative to m), then m
-// (log2 units, scale included), then l.
-template <int D>
-__global__ void __launch_bounds__(D)
-clear_text_export_kernel(const float *__restrict__ partial_o, const float *__restrict__ partial_ml,
-                         float *__restrict__ records, int n_text, int n_splits, int n_slots)
-{
-    const int row = blockIdx.x, bh = blockIdx.y, e = threadIdx.x;
-    const int tq = row >> 7, rr = row & 127;
-    const int64_t slot0 = ((int64_t)bh * n_slots + (int64_t)tq * n_splits) * 128 + rr;
-    float m = -INFINITY;
-    for (int s = 0; s < n_splits; ++s) m = fmaxf(m, partial_ml[(slot0 + (int64_t)s * 128) * 2]);
-    float num = 0.f, den = 0.f;
-    for (int s = 0; s < n_splits; ++s) {
-        const int64_t rowi = slot0 + (int64_t)s * 128;
-        const float ms = partial_ml[rowi * 2];
-        const float w = ms == -INFINITY ? 0.f : exp2f(ms - m);
-        den = fmaf(w, partial_ml[rowi * 2 + 1], den);
-        num = fmaf(w, partial_o[rowi * D + e], num);
-    }
-    float *rec = records + ((int64_t)bh * n_text + row) * (D + 2);
-    rec[e] = num;
-    if (e == 0) {
-        rec[D] = m;
-        rec[D + 1] = den;
-    }
-}
 
 // records: [n_parts][BH][n_text][D + 2].  mode CLEAR_TEXT_MERGE_EXACT: sum_p w_p O_p / sum_p w_p l_p with
 // w_p = 2^(m_p - max m); CLEAR_TEXT_MERGE_AVERAGE (Eq. 7): (1 / n_parts) sum_p O_p / l_p.
@@ -80,22 +53,6 @@ clear_text_merge_kernel(const float *__restrict__ records, __nv_bfloat16 *__rest
 }
 
 }  // namespace
-
-int launch_text_export(const clear_plan &p, void *records, cudaStream_t stream)
-{
-    const Shape &s = p.shape;
-    if (p.sch.n_partial_slots <= 0 || s.n_text <= 0) return CLEAR_ERR_PLAN_MISMATCH;
-    dim3 grid((unsigned)s.n_text, (unsigned)(s.B * s.H));
-    if (s.head_dim == 128)
-        clear_text_export_kernel<128><<<grid, 128, 0, stream>>>(p.d_partial_o, p.d_partial_ml, static_cast<float *>(records),
-                                                                 s.n_text, p.sch.n_text_splits, p.sch.n_partial_slots);
-    else if (s.head_dim == 64)
-        clear_text_export_kernel<64><<<grid, 64, 0, stream>>>(p.d_partial_o, p.d_partial_ml, static_cast<float *>(records),
-                                                               s.n_text, p.sch.n_text_splits, p.sch.n_partial_slots);
-    else
-        return CLEAR_ERR_UNSUPPORTED;
-    return cudaGetLastError() == cudaSuccess ? CLEAR_OK : CLEAR_ERR_CUDA;
-}
 
 int launch_text_merge(const float *records, int n_parts, int n_bh, int n_text, int head_dim, int mode, void *out,
                       long long out_tokens, cudaStream_t stream)

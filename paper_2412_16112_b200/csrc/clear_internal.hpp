@@ -109,9 +109,7 @@ int launch_f32_bwd(const clear_plan &p, const void *q, const void *k, const void
 int ensure_bwd_stats(const clear_plan &p);
 int launch_bwd(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
                void *dv, float scale, cudaStream_t stream);
-// Row-band form: one (O, m, l) record per text row from a band-text plan's partial results, and the merge of the
-// records of all bands into bf16 text rows.
-int launch_text_export(const clear_plan &p, void *records, cudaStream_t stream);
+// Row-band form: the merge of the records of all bands into bf16 text rows.
 int launch_text_merge(const float *records, int n_parts, int n_bh, int n_text, int head_dim, int mode, void *out,
                       long long out_tokens, cudaStream_t stream);
 // Q/K preparation (RMS normalisation, rotary embedding, factor on Q): one elementwise pass, no plan.
@@ -122,7 +120,8 @@ int launch_qk_prep(const void *q_in, const void *k_in, void *q_out, void *k_out,
 // must have been built without text splits.
 int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
                   void *dv, float scale, cudaStream_t stream);
-// Merge of the split-KV partial results of the text-query rows (both tensor-core kernels).
+// Merge of the split-KV partial results of the text-query rows (both tensor-core kernels): bf16 rows of `out`, or, for
+// the text part of a band, one (O, m, l) record per text row.
 int launch_text_combine(const clear_plan &p, void *out, cudaStream_t stream);
 
 // Tensor map (a CUtensorMap, 128 bytes) of a bf16 tensor of `rank` dims, innermost first, with 128-byte swizzle

@@ -339,24 +339,20 @@ clear_tc_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
         if (alive) {
             ptx::tc_fence_after();
             if (item.partial_slot >= 0) {
-                // split text-query tile: un-normalised fp32 row, its maximum (log2 units) and its sum
-                const int64_t row = ((int64_t)bh * prm.n_partial_slots + item.partial_slot) * 128 + r;
-                float *dst = prm.partial_o + row * D;
+                // split text-query tile: un-normalised fp32 rows, channel by channel (32 rows of one channel are 128
+                // consecutive bytes), and per row its maximum (log2 units) and its sum
+                const int64_t slot_row = ((int64_t)bh * prm.n_partial_slots + item.partial_slot) * 128;
+                float *dst = prm.partial_o + slot_row * D + r;
 #pragma unroll
                 for (int w = 0; w < D / 32; ++w) {
                     uint32_t o[32];
                     ptx::tmem_ld32(tmem_O + lane_off + 32 * w, o);
                     ptx::tmem_wait_ld();
-                    if (q_valid) {
 #pragma unroll
-                        for (int j = 0; j < 32; j += 4)
-                            *reinterpret_cast<uint4 *>(dst + 32 * w + j) = make_uint4(o[j], o[j + 1], o[j + 2], o[j + 3]);
-                    }
+                    for (int j = 0; j < 32; ++j) dst[(32 * w + j) * 128] = __uint_as_float(o[j]);
                 }
-                if (q_valid) {
-                    prm.partial_ml[row * 2] = m_used * c;
-                    prm.partial_ml[row * 2 + 1] = l;
-                }
+                prm.partial_ml[(slot_row + r) * 2] = m_used * c;
+                prm.partial_ml[(slot_row + r) * 2 + 1] = l;
             } else {
                 const float inv = l > 0.f ? 1.f / l : 0.f;
                 uint8_t *o_gen = smem_gen;  // the Q buffer: every QK^T has retired
@@ -402,26 +398,64 @@ clear_tc_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
 }
 
 // Merge the split-KV partial results of the text-query rows: out = sum_s w_s O_s / sum_s w_s l_s,
-// w_s = 2^(m_s - max_s m_s).  One block per (text row, bh), one thread per channel.
-template <int D>
-__global__ void __launch_bounds__(D)
-clear_tc_combine_kernel(const float *__restrict__ partial_o, const float *__restrict__ partial_ml,
-                        __nv_bfloat16 *__restrict__ out, int n_text, int64_t n_tokens, int n_splits, int n_slots)
+// w_s = 2^(m_s - max_s m_s).  One block per 32 text rows and (batch, head).  The partial results lie channel by channel
+// (128 rows each), so a warp reads 32 rows of a channel as 128 consecutive bytes; the finished rows are turned round in
+// shared memory and written along their channels.  RECORDS: the merged row stays un-normalised, as D values followed
+// by its maximum and its sum (the record a band leaves for the merge over all bands).
+template <int D, bool RECORDS>
+__global__ void __launch_bounds__(256)
+clear_tc_combine_kernel(const float *__restrict__ partial_o, const float *__restrict__ partial_ml, void *__restrict__ out,
+                        int n_text, int64_t n_tokens, int n_splits, int n_slots)
 {
-    const int row = blockIdx.x, bh = blockIdx.y, e = threadIdx.x;
-    const int tq = row >> 7, rr = row & 127;
-    const int64_t slot0 = ((int64_t)bh * n_slots + (int64_t)tq * n_splits) * 128 + rr;
+    __shared__ float rows[32][D + 1];
+    const int row0 = blockIdx.x * 32, bh = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rr = (row0 & 127) + lane;
+    const int64_t slot0 = (int64_t)bh * n_slots + (int64_t)(row0 >> 7) * n_splits;
+    const bool on = row0 + lane < n_text;
     float m = -INFINITY;
-    for (int s = 0; s < n_splits; ++s) m = fmaxf(m, partial_ml[(slot0 + (int64_t)s * 128) * 2]);
-    float num = 0.f, den = 0.f;
-    for (int s = 0; s < n_splits; ++s) {
-        const int64_t rowi = slot0 + (int64_t)s * 128;
-        const float ms = partial_ml[rowi * 2];
-        const float w = ms == -INFINITY ? 0.f : exp2f(ms - m);
-        den = fmaf(w, partial_ml[rowi * 2 + 1], den);
-        num = fmaf(w, partial_o[rowi * D + e], num);
+    if (on)
+        for (int s = 0; s < n_splits; ++s) m = fmaxf(m, partial_ml[((slot0 + s) * 128 + rr) * 2]);
+    constexpr int kChannels = D / 8;  // per warp
+    float num[kChannels], den = 0.f;
+#pragma unroll
+    for (int e = 0; e < kChannels; ++e) num[e] = 0.f;
+    if (on) {
+        for (int s = 0; s < n_splits; ++s) {
+            const int64_t row = (slot0 + s) * 128 + rr;
+            const float ms = partial_ml[row * 2];
+            const float w = ms == -INFINITY ? 0.f : exp2f(ms - m);
+            den = fmaf(w, partial_ml[row * 2 + 1], den);
+            const float *src = partial_o + (slot0 + s) * 128 * D + rr;
+#pragma unroll
+            for (int e = 0; e < kChannels; ++e) num[e] = fmaf(w, src[(warp * kChannels + e) * 128], num[e]);
+        }
     }
-    out[((int64_t)bh * n_tokens + row) * D + e] = __float2bfloat16_rn(den > 0.f ? num / den : 0.f);
+    const float inv = RECORDS ? 1.f : den > 0.f ? 1.f / den : 0.f;
+#pragma unroll
+    for (int e = 0; e < kChannels; ++e) rows[lane][warp * kChannels + e] = num[e] * inv;
+    __syncthreads();
+    if constexpr (RECORDS) {
+        float *rec = static_cast<float *>(out) + ((int64_t)bh * n_text + row0) * (D + 2);
+        if (warp == 0 && on) {
+            rec[lane * (D + 2) + D] = m;
+            rec[lane * (D + 2) + D + 1] = den;
+        }
+        for (int i = threadIdx.x; i < 32 * D; i += 256) {
+            const int r = i / D, e = i % D;
+            if (row0 + r < n_text) rec[r * (D + 2) + e] = rows[r][e];
+        }
+    } else {
+        for (int i = threadIdx.x; i < 32 * (D / 8); i += 256) {
+            const int r = i / (D / 8), e = i % (D / 8) * 8;
+            if (row0 + r >= n_text) continue;
+            uint4 v;
+            v.x = ptx::pack_bf16(rows[r][e], rows[r][e + 1]);
+            v.y = ptx::pack_bf16(rows[r][e + 2], rows[r][e + 3]);
+            v.z = ptx::pack_bf16(rows[r][e + 4], rows[r][e + 5]);
+            v.w = ptx::pack_bf16(rows[r][e + 6], rows[r][e + 7]);
+            *reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(out) + ((int64_t)bh * n_tokens + row0 + r) * D + e) = v;
+        }
+    }
 }
 
 // ---- host side: tensor maps and launch ---------------------------------------------------------
@@ -479,18 +513,14 @@ int launch_text_combine(const clear_plan &p, void *out, cudaStream_t stream)
 {
     const Shape &s = p.shape;
     // the text part of a band leaves records for the merge over all bands instead of finished rows
-    if (s.part == CLEAR_PART_BAND_TEXT) return launch_text_export(p, out, stream);
-    if (p.sch.n_partial_slots <= 0) return CLEAR_OK;
+    const bool records = s.part == CLEAR_PART_BAND_TEXT;
+    if (p.sch.n_partial_slots <= 0) return records ? CLEAR_ERR_PLAN_MISMATCH : CLEAR_OK;
+    if (s.head_dim != 64 && s.head_dim != 128) return CLEAR_ERR_UNSUPPORTED;
     const int64_t N = (int64_t)s.n_text + (int64_t)s.grid_h * s.grid_w;
-    dim3 cgrid((unsigned)s.n_text, (unsigned)(s.B * s.H));
-    if (s.head_dim == 128)
-        clear_tc_combine_kernel<128><<<cgrid, 128, 0, stream>>>(p.d_partial_o, p.d_partial_ml, (__nv_bfloat16 *)out,
-                                                                s.n_text, N, p.sch.n_text_splits, p.sch.n_partial_slots);
-    else if (s.head_dim == 64)
-        clear_tc_combine_kernel<64><<<cgrid, 64, 0, stream>>>(p.d_partial_o, p.d_partial_ml, (__nv_bfloat16 *)out,
-                                                              s.n_text, N, p.sch.n_text_splits, p.sch.n_partial_slots);
-    else
-        return CLEAR_ERR_UNSUPPORTED;
+    const dim3 grid((unsigned)((s.n_text + 31) / 32), (unsigned)(s.B * s.H));
+    auto kernel = s.head_dim == 128 ? (records ? clear_tc_combine_kernel<128, true> : clear_tc_combine_kernel<128, false>)
+                                    : (records ? clear_tc_combine_kernel<64, true> : clear_tc_combine_kernel<64, false>);
+    kernel<<<grid, 256, 0, stream>>>(p.d_partial_o, p.d_partial_ml, out, s.n_text, N, p.sch.n_text_splits, p.sch.n_partial_slots);
     CLEAR_CUDA_TRY(cudaGetLastError());
     return CLEAR_OK;
 }

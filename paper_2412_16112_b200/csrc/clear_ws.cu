@@ -7,12 +7,11 @@
 //
 // Roles (384 threads):
 //   warp 0        : takes items from the queue and issues every TMA load (Q tiles, K/V ring);
-//   warp 1        : one thread issues every tcgen05.mma, alternating between the two query tiles:
-//                   S_t = Q_t K^T, O_t += P_t V; the softmax of one tile runs under the MMAs of the other;
+//   warps 1, 2    : issue every tcgen05.mma of query tile 0 / 1: S_t = Q_t K^T and O_t += P_t V;
 //   warps 4-7     : softmax and epilogue of query tile 0 (thread r owns query row r = tensor-memory
-//                   lane r): running maximum, P = exp2(.) on the keys Eq. 3 allows and 0 elsewhere, as
-//                   bf16 into tensor memory over S, row sum; at the end of an item O / l -> bf16 ->
-//                   global memory (or fp32 partial results of split text rows);
+//                   lane r): P = exp2(.) on the keys Eq. 3 allows and 0 elsewhere, as bf16 into tensor
+//                   memory over S, row sum; at the end of an item O / l -> bf16 -> global memory (or
+//                   fp32 partial results of split text rows);
 //   warps 8-11    : the same for query tile 1.
 // Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 columns each; P_t takes the first 64 columns of
 // S_t and is the tensor-memory operand of P_t V, so that P never crosses shared memory: with both MMA
@@ -24,9 +23,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <cstdio>
 #include <cstring>
-#include <type_traits>
 
 #include "clear_internal.hpp"
 #include "ptx.cuh"
@@ -35,30 +32,21 @@ namespace clear {
 namespace {
 
 constexpr int kWsThreads = 384;   // 4 control warps + 2 x 4 softmax warps
-constexpr int kRing = 5;
+constexpr uint32_t kRing = 5;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSpinLimit = 1u << 22;
 constexpr uint32_t kWaitHintNs = 20000;            // one sleep inside try_wait
-constexpr uint64_t kWaitLimitNs = 2000000000ull;   // a wait that lasts 2 s has failed
-constexpr float kRescaleThreshold = 8.f;  // log2 units: O is rescaled only when the row max grows by more
-constexpr float kMaxTileSum = 256.f;      // 2^kRescaleThreshold: a row sum of P up to this needs no look at the maximum
+constexpr uint32_t kWaitLimitUs = 2000000;         // a wait that lasts 2 s has failed
+constexpr float kRescaleThreshold = 8.f;  // log2 units: a reference is moved only when a row's maximum exceeds it by more
+constexpr float kBumpSum = 256.f;         // a row sum of P above this raises the row's reference for the next tile
+constexpr float kMaxTileSum = 0x1p64f;    // a row sum above this (or none at all, a NaN) has its tile taken again
 constexpr int kSchedDepth = 2;
-// arrivals that free a queue slot: the MMA thread and one lane of each of the 8 softmax warps
-constexpr uint32_t kSchedReaders = 9;
+// arrivals that free a queue slot: one lane of each of the 2 MMA warps and the 8 softmax warps
+constexpr uint32_t kSchedReaders = 10;
 // registers per thread of each role: 128 x 80 + 256 x 208 = 63488, within what the block is launched with
 // (384 threads x 168); raising a warp's budget only draws on registers other warps of the block gave back
 constexpr uint32_t kRegsControl = 80, kRegsSoftmax = 208;
 static_assert(128 * kRegsControl + 256 * kRegsSoftmax <= 384 * 168, "a raise beyond the block's registers would wait for ever");
-
-// Optional timeline of the softmax warps (compile with -DCLEAR_WS_TRACE): clocks per phase, summed over the
-// launch, printed by block 0.  Off in the product build.
-#ifdef CLEAR_WS_TRACE
-#define TRACE_DECL unsigned long long tr_acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0}; long long tr_t = clock64(); unsigned tr_steps = 0;
-#define TRACE_MARK(i) { const long long tr_n = clock64(); tr_acc[i] += (unsigned long long)(tr_n - tr_t); tr_t = tr_n; }
-#else
-#define TRACE_DECL
-#define TRACE_MARK(i)
-#endif
 
 struct WsParams {
     const clear_pair_item_t *items;
@@ -70,19 +58,28 @@ struct WsParams {
     long long n_tokens;
     int n_items, n_text_items, n_bh;
     float scale_log2;  // scale * log2(e)
-    float *partial_o;
-    float *partial_ml;
+    float *partial_o;  // split text rows, per (bh, slot): [D][128] un-normalised O, channel by channel
+    float *partial_ml; // and [128][2]: reference (log2 units) and row sum
     int n_partial_slots;
+    const __nv_bfloat16 *q, *k;
     __nv_bfloat16 *out;
     int *status;  // [0] status word of this launch, [1] queue head, [2] finished blocks, [3] status kept for the host
+};
+
+// Views of q, k, v (kMap*): patches of the image part, and runs of consecutive tokens.  Every view has five axes,
+// channel (64), column or token, row, channel half, (batch, head), so one copy instruction, with one of these maps and
+// its coordinates chosen at run time, brings any tile of 128 tokens and all its channels.
+enum { kMapQImg = 0, kMapQTxt = 1, kMapKImg = 2, kMapKLin = 3, kMapVImg = 4, kMapVLin = 5 };
+struct WsMaps {
+    CUtensorMap m[6];
 };
 
 struct Ctrl {
     uint64_t q_full[2], q_empty[2];
     uint64_t kv_full[kRing], kv_empty[kRing];
-    uint64_t s_full[2], p_ready[2], o_full[2], o_empty[2];
+    uint64_t sa_full[2], sb_full[2], sb_read[2], p_ready[2], o_full[2], o_empty[2];
     uint64_t sched_full[kSchedDepth], sched_empty[kSchedDepth];
-    uint64_t drain[1];
+    uint64_t turn[2], drain[2];
     int32_t sched_item[kSchedDepth];            // queue position, >= total: no more work
     int32_t sched_bh[kSchedDepth];
     clear_pair_item_t sched_rec[kSchedDepth];   // the item's record, read once from global memory
@@ -91,31 +88,31 @@ struct Ctrl {
     int skip;
 };
 
-// Bounded wait on an mbarrier phase.  Returns false once the block has given up.  The polling loop is
-// kept to two instructions per try, and roles that can afford it (SLEEP_NS > 0) sleep between tries:
-// a busily polling warp takes issue slots and instruction-cache lines from the softmax warps.
-template <uint32_t SLEEP_NS>
-__device__ __forceinline__ bool wait_bar_slow(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status, int code)
+// Bounded wait on an mbarrier phase.  Returns false once the block has given up.  The polling loop is a handful of
+// instructions in line (each wait is one more copy of it, and the kernel's code has to stay small enough for the
+// instruction caches); what happens every 128 tries -- the abort flag, the clock -- is one function.  Roles that can
+// afford it (SLEEP_NS > 0) sleep between tries: a polling warp takes issue slots from the softmax warps.
+__device__ __noinline__ uint32_t wait_tick(uint32_t t0, volatile int *abort_flag, int *status, int code)
 {
-    const uint64_t t0 = ptx::globaltimer_ns();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 128; ++i) {
-            if (ptx::mbar_try_wait_hint(bar, parity, kWaitHintNs)) return true;
-            if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
-        }
-        if (*abort_flag) return false;
-        if (ptx::globaltimer_ns() - t0 > kWaitLimitNs) break;
-    }
+    const uint32_t now = (uint32_t)(ptx::globaltimer_ns() >> 10) | 1u;  // about microseconds, never 0
+    if (t0 == 0) t0 = now;
+    if (*abort_flag) return 0;
+    if (now - t0 <= kWaitLimitUs) return t0;
     *abort_flag = 1;
     atomicCAS(status, 0, code);  // the first wait that expired names the cause
-    return false;
+    return 0;
 }
 template <uint32_t SLEEP_NS = 0>
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status, int code)
 {
     if (ptx::mbar_try_wait(bar, parity)) return true;
-    return wait_bar_slow<SLEEP_NS>(bar, parity, abort_flag, status, code);
+    uint32_t t0 = 0;
+#pragma unroll 1
+    for (uint32_t n = 1; !ptx::mbar_try_wait_hint(bar, parity, kWaitHintNs); ++n) {
+        if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
+        if ((n & 127u) == 0u && (t0 = wait_tick(t0, abort_flag, status, code)) == 0u) return false;
+    }
+    return true;
 }
 // One arrival for the whole warp, after every lane has got here (and its earlier writes with it).
 __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane)
@@ -124,8 +121,9 @@ __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane)
     if (lane == 0) ptx::mbar_arrive(bar);
 }
 // Drain: wait for a phase regardless of the abort flag (used before leaving with copies in flight).
-__device__ __forceinline__ void drain_bar(uint32_t bar, uint32_t parity)
+__device__ __noinline__ void drain_bar(uint32_t bar, uint32_t parity)
 {
+#pragma unroll 1
     for (uint32_t it = 0; it < kSpinLimit; ++it) {
         if (ptx::mbar_try_wait(bar, parity)) return;
         if (it > 64) __nanosleep(256);
@@ -173,18 +171,6 @@ __device__ __forceinline__ clear_pair_item_t load_item(const clear_pair_item_t *
     it.step_count = c.x; it.n_loads = c.y; it.partial_slot0 = c.z; it.partial_slot1 = c.w;
     return it;
 }
-// The part of a step record the softmax of one query tile of the pair needs on every step.
-struct SideStep {
-    int flags, n_valid;
-};
-__device__ __forceinline__ SideStep load_side_step(const clear_pair_step_t *p, int side)
-{
-    const int4 b = __ldg(reinterpret_cast<const int4 *>(p) + 1);
-    SideStep s;
-    s.flags = b.x;
-    s.n_valid = side ? b.z : b.y;
-    return s;
-}
 // Origin of the key patch of that tile (only clipped patches and plans without a mask table need it).
 __device__ __forceinline__ int2 load_side_origin(const clear_pair_step_t *p, int side)
 {
@@ -194,11 +180,224 @@ __device__ __forceinline__ int2 load_side_origin(const clear_pair_step_t *p, int
 static_assert(sizeof(clear_pair_step_t) == 32 && sizeof(clear_pair_item_t) == 48, "table records are read as int4");
 
 __device__ __forceinline__ bool step_uses(int flags, int side) { return (flags & (side ? CLEAR_STEP_USE1 : CLEAR_STEP_USE0)) != 0; }
-// A step's K tiles, and its V tiles, take one ring position per distinct key tile (tile 0's first):
-__device__ __forceinline__ int step_tile_index(int flags, int side)
+
+// ---- pieces of the softmax warps' work that are rare, or come once an item: functions of their own, so that their
+// registers do not crowd the exponentials of the common step (with them in line the compiler had too few left to overlap
+// with, and a pass over 128 scores took up to 1900 clocks instead of 1400) --------------------------------------------
+
+// A trip count the compiler cannot see: without it these loops are unrolled whatever the source says, and most of their time
+// goes into fetching instructions that run once.
+__device__ __forceinline__ int opaque(int n)
 {
-    if (side == 0 || (flags & CLEAR_STEP_SHARED)) return 0;
-    return (flags & CLEAR_STEP_USE0) ? 1 : 0;
+    asm volatile("" : "+r"(n));
+    return n;
+}
+
+// The row's O times alpha (O_t is at rest: P_t V of the step before is complete).
+template <int D>
+__device__ __noinline__ void rescale_rows(uint32_t tmem_o, float alpha)
+{
+#pragma unroll 1
+    for (int w = 0, n = opaque(D / 16); w < n; ++w) {
+        uint32_t o[16];
+        ptx::tmem_ld16(tmem_o + 16 * w, o);
+        ptx::tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
+        ptx::tmem_st16(tmem_o + 16 * w, o);
+    }
+}
+
+// P of 32 keys from their scores: 2^(S c - mc) on the allowed keys and 0 elsewhere, added to the row sum (two-wide fp32
+// FMA and ADD, four independent partial sums), as bf16 pairs (16 columns of tensor memory).
+template <bool kMasked>
+__device__ __forceinline__ void exp_chunk(const uint32_t (&sv)[32], uint32_t bits, uint64_t c2, uint64_t nmc2, uint64_t (&lsum)[2],
+                                          uint32_t (&pk)[16])
+{
+#pragma unroll
+    for (int j = 0; j < 32; j += 2) {
+        const uint64_t x2 = ptx::fma2(ptx::pack2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), c2, nmc2);
+        float x0, x1;
+        ptx::unpack2(x2, x0, x1);
+        if (kMasked) {
+            x0 = ((bits >> j) & 1u) ? x0 : -INFINITY;
+            x1 = ((bits >> (j + 1)) & 1u) ? x1 : -INFINITY;
+        }
+        const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
+        lsum[(j >> 1) & 1] = ptx::add2(lsum[(j >> 1) & 1], ptx::pack2(p0, p1));
+        pk[j >> 1] = ptx::pack_bf16(p0, p1);
+    }
+}
+__device__ __forceinline__ float sum4(const uint64_t (&lsum)[2])
+{
+    float a0, a1, a2, a3;
+    ptx::unpack2(lsum[0], a0, a1);
+    ptx::unpack2(lsum[1], a2, a3);
+    return (a0 + a1) + (a2 + a3);
+}
+
+struct RowState {
+    float ref, l, tile_sum;
+};
+// A step with a maximum pass: the maximum over the allowed keys, the row's reference, then P.  The scores are read from
+// tensor memory both times, 32 keys at a time (P of 32 keys takes 16 columns, so it never reaches scores still to be read).
+template <int D>
+__device__ __noinline__ RowState exact_step(uint32_t tmem_s, uint32_t tmem_o, uint4 mask, float c, float ref, float l, bool first)
+{
+    auto bits_of = [&](int w) { return w == 0 ? mask.x : w == 1 ? mask.y : w == 2 ? mask.z : mask.w; };
+    float mx = -INFINITY;
+#pragma unroll 1
+    for (int w = 0, n = opaque(4); w < n; ++w) {
+        uint32_t sv[32];
+        ptx::tmem_ld32(tmem_s + 32 * w, sv);
+        const uint32_t bits = bits_of(w);
+        ptx::tmem_wait_ld();
+        float mx2[2] = {mx, -INFINITY};
+#pragma unroll
+        for (int j = 0; j < 32; j += 2)
+            mx2[(j >> 1) & 1] = ptx::max3(mx2[(j >> 1) & 1], ((bits >> j) & 1u) ? __uint_as_float(sv[j]) : -INFINITY,
+                                          ((bits >> (j + 1)) & 1u) ? __uint_as_float(sv[j + 1]) : -INFINITY);
+        mx = fmaxf(mx2[0], mx2[1]);
+    }
+    const float m_new = fmaxf(ref, mx * c);
+    if (first) {
+        ref = m_new;
+    } else {
+        const bool need = m_new - ref > kRescaleThreshold;  // false for NaN (-inf minus -inf)
+        if (__any_sync(0xffffffffu, need)) {
+            const float alpha = need ? ptx::ex2(ref - m_new) : 1.f;
+            if (need) ref = m_new;
+            l *= alpha;
+            rescale_rows<D>(tmem_o, alpha);
+        }
+    }
+    const float mc = (ref == -INFINITY) ? 0.f : ref;
+    const uint64_t c2 = ptx::pack2(c, c), nmc2 = ptx::pack2(-mc, -mc);
+    uint64_t lsum[2] = {0ull, 0ull};
+#pragma unroll 1
+    for (int w = 0, n = opaque(4); w < n; ++w) {
+        uint32_t sv[32], pk[16];
+        ptx::tmem_ld32(tmem_s + 32 * w, sv);
+        ptx::tmem_wait_ld();
+        exp_chunk<true>(sv, bits_of(w), c2, nmc2, lsum, pk);
+        ptx::tmem_st16(tmem_s + 16 * w, pk);
+    }
+    return RowState{ref, l, sum4(lsum)};
+}
+
+// A step whose scores lie far above the row's reference: each row's scores once more, by its own thread from global memory
+// (those in tensor memory are gone), twice over -- for their maximum, and for P against it.  Slow, and as good as never run.
+template <int D>
+__device__ __noinline__ RowState rescue_step(const WsParams &prm, uint32_t tmem_p, uint32_t tmem_o, uint4 mask, float c, float ref, float l,
+                                             long long row0, long long q_tok, int2 org, bool linear)
+{
+    ptx::tmem_wait_st();
+    auto allowed = [&](int key) { return (((key < 32 ? mask.x : key < 64 ? mask.y : key < 96 ? mask.z : mask.w) >> (key & 31)) & 1u) != 0u; };
+    auto score = [&](int key) {
+        const int ky = org.y + (key >> 4), kx = org.x + (key & 15);
+        const bool on = linear ? org.x + key < prm.n_tokens : ky >= 0 && ky < prm.grid_h && kx >= 0 && kx < prm.grid_w;
+        const long long tok = linear ? org.x + key : prm.n_text + (long long)ky * prm.grid_w + kx;
+        float dot = 0.f;
+        if (on && q_tok >= 0) {
+            const __nv_bfloat16 *q_row = prm.q + (row0 + q_tok) * D, *k_row = prm.k + (row0 + tok) * D;
+#pragma unroll 1
+            for (int e = 0; e < D; ++e) dot = fmaf(__bfloat162float(q_row[e]), __bfloat162float(k_row[e]), dot);
+        }
+        return dot;
+    };
+    float mx = -INFINITY;
+#pragma unroll 1
+    for (int key = 0; key < 128; ++key)
+        if (allowed(key)) mx = fmaxf(mx, score(key));
+    const float m_new = fmaxf(ref, mx * c);
+    const bool need = m_new - ref > kRescaleThreshold;
+    const float alpha = need ? ptx::ex2(ref - m_new) : 1.f;
+    if (need) ref = m_new;
+    l *= alpha;
+    __syncwarp();
+    rescale_rows<D>(tmem_o, alpha);
+    const float mc = (ref == -INFINITY) ? 0.f : ref;
+    float sum = 0.f;
+#pragma unroll 1
+    for (int w = 0; w < 4; ++w) {
+        uint32_t pk[16];
+#pragma unroll 1
+        for (int j = 0; j < 16; ++j) {
+            float p[2];
+#pragma unroll 1
+            for (int u = 0; u < 2; ++u) {
+                const int key = 32 * w + 2 * j + u;
+                const float x = allowed(key) ? ptx::ex2(fmaf(score(key), c, -mc)) : 0.f;
+                sum += x;
+                if (u == 0) p[0] = x;
+                else p[1] = x;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (i == j) pk[i] = ptx::pack_bf16(p[0], p[1]);
+        }
+        __syncwarp();
+        ptx::tmem_st16(tmem_p + 16 * w, pk);
+    }
+    return RowState{ref, l, sum};
+}
+
+// End of an item for one query tile: O / l, or the partial results of split text rows, to global memory.  `first_x`: first
+// token (text) or grid column, `first_y`: grid row of the tile; n_rows: rows of a text tile, -1 for a patch.  Tells the
+// MMA warp (o_empty) as soon as O has been read.
+template <int D>
+__device__ __noinline__ void store_tile(const WsParams &prm, uint32_t tmem_o, uint32_t b_o_empty, int first_x, int first_y, int n_rows,
+                                        int slot, int bh, float ref, float l)
+{
+    const int lane = threadIdx.x & 31, q4 = (threadIdx.x >> 5) & 3, r = q4 * 32 + lane;
+    tmem_o += (uint32_t)(q4 * 32) << 16;
+    if (slot >= 0) {
+        // split text-query tile: un-normalised fp32 rows, channel by channel (a warp writes 32 rows of one channel as
+        // 128 consecutive bytes), and per row its reference (log2 units) and its sum
+        const long long slot_row = ((long long)bh * prm.n_partial_slots + slot) * 128;
+        float *dst = prm.partial_o + slot_row * D + r;
+#pragma unroll 1
+        for (int w = 0, n = opaque(D / 16); w < n; ++w) {
+            uint32_t o[16];
+            ptx::tmem_ld16(tmem_o + 16 * w, o);
+            ptx::tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) dst[(16 * w + j) * 128] = __uint_as_float(o[j]);
+        }
+        ptx::tc_fence_before();
+        warp_arrive(b_o_empty, lane);
+        prm.partial_ml[(slot_row + r) * 2] = ref;
+        prm.partial_ml[(slot_row + r) * 2 + 1] = l;
+        return;
+    }
+    // O / l as bf16, 16 channels (32 bytes, a memory sector) of the thread's row at a time.  Once an item, so cold: a short loop
+    // rather than a fast one.  (Unrolled, and with the rows exchanged between threads for wider runs, the same took 4200
+    // clocks, most of them for fetching its instructions.)
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    const int y = first_y + (r >> 4), x = first_x + (r & 15);
+    const bool on = n_rows >= 0 ? r < n_rows : (y < prm.grid_h && x < prm.grid_w);
+    const long long token = n_rows >= 0 ? (long long)first_x + r : prm.n_text + (long long)y * prm.grid_w + x;
+    __nv_bfloat16 *dst = prm.out + ((long long)bh * prm.n_tokens + token) * D;
+    const bool wide = (reinterpret_cast<uintptr_t>(prm.out) & 31u) == 0u;  // tensors are 16-byte aligned at least
+#pragma unroll 1
+    for (int w = 0, n = opaque(D / 16); w < n; ++w) {
+        uint32_t o[16];
+        ptx::tmem_ld16(tmem_o + 16 * w, o);
+        ptx::tmem_wait_ld();
+        uint32_t u[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) u[j] = ptx::pack_bf16(__uint_as_float(o[2 * j]) * inv, __uint_as_float(o[2 * j + 1]) * inv);
+        if (on) {
+            if (wide) {
+                ptx::stg_u256(dst + 16 * w, u);
+            } else {
+                *reinterpret_cast<uint4 *>(dst + 16 * w) = make_uint4(u[0], u[1], u[2], u[3]);
+                *reinterpret_cast<uint4 *>(dst + 16 * w + 8) = make_uint4(u[4], u[5], u[6], u[7]);
+            }
+        }
+    }
+    ptx::tc_fence_before();
+    warp_arrive(b_o_empty, lane);
 }
 
 // The last block of a launch to leave: the work queue goes back to zero, and a status some block raised
@@ -213,15 +412,12 @@ __device__ __forceinline__ void close_launch(int *status)
 
 template <int D>
 __global__ void __launch_bounds__(kWsThreads, 1)
-clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_constant__ CUtensorMap tm_k_img,
-                const __grid_constant__ CUtensorMap tm_v_img, const __grid_constant__ CUtensorMap tm_q_txt,
-                const __grid_constant__ CUtensorMap tm_k_lin, const __grid_constant__ CUtensorMap tm_v_lin,
-                const WsParams prm)
+clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsParams prm)
 {
     constexpr int kHalves = D / 64;                 // 64-channel (128-byte) column blocks of a tile
     constexpr uint32_t kHalfBytes = 128 * 128;      // 128 rows x 128 B
     constexpr uint32_t kTileBytes = kHalves * kHalfBytes;
-    constexpr uint32_t kIdescQK = ptx::idesc_bf16(128, false);
+    constexpr uint32_t kIdescQK = ptx::idesc_bf16(64, false);
     constexpr uint32_t kIdescPV = ptx::idesc_bf16(D, true);
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -260,20 +456,23 @@ clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
         for (int i = 0; i < 2; ++i) {
             ptx::mbar_init(ptx::smem_u32(&ctrl->q_full[i]), 1);
             ptx::mbar_init(ptx::smem_u32(&ctrl->q_empty[i]), 1);
-            ptx::mbar_init(ptx::smem_u32(&ctrl->s_full[i]), 1);
-            ptx::mbar_init(ptx::smem_u32(&ctrl->p_ready[i]), 4);  // one arrival per softmax warp of the tile
+            ptx::mbar_init(ptx::smem_u32(&ctrl->sa_full[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&ctrl->sb_full[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&ctrl->sb_read[i]), 4);  // one arrival per softmax warp of the tile
+            ptx::mbar_init(ptx::smem_u32(&ctrl->p_ready[i]), 4);
             ptx::mbar_init(ptx::smem_u32(&ctrl->o_full[i]), 1);
             ptx::mbar_init(ptx::smem_u32(&ctrl->o_empty[i]), 4);
+            ptx::mbar_init(ptx::smem_u32(&ctrl->turn[i]), 1);
         }
-        for (int i = 0; i < kRing; ++i) {
+        for (uint32_t i = 0; i < kRing; ++i) {
             ptx::mbar_init(ptx::smem_u32(&ctrl->kv_full[i]), 1);
-            ptx::mbar_init(ptx::smem_u32(&ctrl->kv_empty[i]), 1);
+            ptx::mbar_init(ptx::smem_u32(&ctrl->kv_empty[i]), 2);  // one arrival per MMA warp
         }
         for (int i = 0; i < kSchedDepth; ++i) {
             ptx::mbar_init(ptx::smem_u32(&ctrl->sched_full[i]), 1);
             ptx::mbar_init(ptx::smem_u32(&ctrl->sched_empty[i]), kSchedReaders);
         }
-        ptx::mbar_init(ptx::smem_u32(&ctrl->drain[0]), 1);
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(ptx::smem_u32(&ctrl->drain[i]), 1);
         ptx::fence_mbar_init();
     }
     if (warp == 1) {
@@ -290,7 +489,10 @@ clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
         if (warp == 0 && lane == 0) {
             // ================= loader: work queue + every TMA load ====================================
             uint32_t n_loads = 0;    // K/V stages filled so far by this block
+            uint32_t stage = 0, stage_par = 0;  // the stage the next one goes to, parity of its fill
+            const uint32_t b_full0 = ptx::smem_u32(&ctrl->kv_full[0]), b_empty0 = ptx::smem_u32(&ctrl->kv_empty[0]);
             uint32_t n_q[2] = {0, 0};
+#pragma unroll 1
             for (uint32_t k = 0;; ++k) {
                 const uint32_t slot = k % kSchedDepth, use = k / kSchedDepth;
                 if (!wait_bar<200>(ptx::smem_u32(&ctrl->sched_empty[slot]), (use & 1u) ^ 1u, abort_flag, prm.status, 1)) break;
@@ -307,54 +509,50 @@ clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
                 ptx::mbar_arrive(ptx::smem_u32(&ctrl->sched_full[slot]));
                 if (g >= total_items) break;
                 bool ok = true;
+#pragma unroll 1
                 for (int t = 0; t < item.n_sides && ok; ++t) {
                     const uint32_t bar = ptx::smem_u32(&ctrl->q_full[t]);
                     ok = wait_bar<200>(ptx::smem_u32(&ctrl->q_empty[t]), (n_q[t] & 1u) ^ 1u, abort_flag, prm.status, 2);
                     if (!ok) break;
                     ptx::mbar_expect_tx(bar, kTileBytes);
-#pragma unroll
-                    for (int h = 0; h < kHalves; ++h) {
-                        const uint32_t dst = sQ + t * kTileBytes + h * kHalfBytes;
-                        if (item.kind == 1)
-                            ptx::tma_load_3d(dst, &tm_q_txt, bar, h * 64, item.qx + t * 128, ref.bh);
-                        else
-                            ptx::tma_load_4d(dst, &tm_q_img, bar, h * 64, item.qx, t ? item.qy1 : item.qy0, ref.bh);
-                    }
+                    const bool txt = item.kind == 1;
+                    ptx::tma_load_5d(sQ + t * kTileBytes, &maps.m[txt ? kMapQTxt : kMapQImg], bar, 0,
+                                     txt ? item.qx + t * 128 : item.qx, txt ? 0 : t ? item.qy1 : item.qy0, 0, ref.bh);
                     ++n_q[t];
                 }
-                // K/V stages in the plan's staging order: for every step its K tiles, then its V tiles
-                auto stage_tiles = [&](const clear_pair_step_t &st, int kv) {
-                    const bool has_a = (st.flags & CLEAR_STEP_USE0) != 0;
-                    const bool has_b = (st.flags & CLEAR_STEP_USE1) && !(st.flags & CLEAR_STEP_SHARED);
-                    const bool linear = (st.flags & CLEAR_STEP_LINEAR) != 0;
-#pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        if (!ok || (t == 0 ? !has_a : !has_b)) continue;
-                        const uint32_t stage = n_loads % kRing, fill = n_loads / kRing;
-                        ok = wait_bar<100>(ptx::smem_u32(&ctrl->kv_empty[stage]), (fill & 1u) ^ 1u, abort_flag, prm.status, 3);
-                        if (!ok) continue;
-                        const uint32_t bar = ptx::smem_u32(&ctrl->kv_full[stage]);
-                        const uint32_t dst = sRing + stage * kTileBytes;
-                        const int x = t ? st.x1 : st.x0, y = t ? st.y1 : st.y0;
-                        ptx::mbar_expect_tx(bar, kTileBytes);
-#pragma unroll
-                        for (int h = 0; h < kHalves; ++h) {
-                            if (linear)
-                                ptx::tma_load_3d(dst + h * kHalfBytes, kv ? &tm_v_lin : &tm_k_lin, bar, h * 64, x, ref.bh);
-                            else
-                                ptx::tma_load_4d(dst + h * kHalfBytes, kv ? &tm_v_img : &tm_k_img, bar, h * 64, x, y, ref.bh);
-                        }
-                        ++n_loads;
-                    }
-                };
+                // staging order = reading order: the K tiles of a step come before the V tiles of the step before it
                 const clear_pair_step_t *steps = prm.steps + item.step_begin;
-                clear_pair_step_t st = load_step(steps);
-                for (int s = 0; s < item.step_count && ok; ++s) {
+                clear_pair_step_t st = load_step(steps), st_prev = st;
+                st_prev.flags = 0;
+#pragma unroll 1
+                for (int s = 0; s <= item.step_count && ok; ++s) {
                     // records are fetched ahead of their use, so their latency is off the critical path
                     clear_pair_step_t st_next = st;
                     if (s + 1 < item.step_count) st_next = load_step(steps + s + 1);
-                    stage_tiles(st, 0);
-                    stage_tiles(st, 1);
+                    else st_next.flags = 0;
+#pragma unroll 1
+                    for (int i = 0; i < 4 && ok; ++i) {
+                        // tile 0's, and tile 1's when it is another one
+                        const int t = i & 1;
+                        const bool k = i < 2;
+                        const int flags = k ? st.flags : st_prev.flags;
+                        if (!(t ? (flags & (CLEAR_STEP_USE1 | CLEAR_STEP_SHARED)) == CLEAR_STEP_USE1 : (flags & CLEAR_STEP_USE0) != 0)) continue;
+                        ok = wait_bar<100>(b_empty0 + 8 * stage, stage_par ^ 1u, abort_flag, prm.status, 3);
+                        if (!ok) break;
+                        const bool linear = (flags & CLEAR_STEP_LINEAR) != 0;
+                        const int x = k ? (t ? st.x1 : st.x0) : (t ? st_prev.x1 : st_prev.x0);
+                        const int y = k ? (t ? st.y1 : st.y0) : (t ? st_prev.y1 : st_prev.y0);
+                        const uint32_t bar = b_full0 + 8 * stage;
+                        ptx::mbar_expect_tx(bar, kTileBytes);
+                        ptx::tma_load_5d(sRing + stage * kTileBytes, &maps.m[(k ? kMapKImg : kMapVImg) + (linear ? 1 : 0)], bar, 0, x,
+                                         linear ? 0 : y, 0, ref.bh);
+                        ++n_loads;
+                        if (++stage == kRing) {
+                            stage = 0;
+                            stage_par ^= 1u;
+                        }
+                    }
+                    st_prev = st;
                     st = st_next;
                 }
                 if (!ok) break;
@@ -363,174 +561,203 @@ clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
                 // leave no copy in flight: whatever was issued must land before the block exits
                 for (int t = 0; t < 2; ++t)
                     if (n_q[t] > 0) drain_bar(ptx::smem_u32(&ctrl->q_full[t]), (n_q[t] - 1) & 1u);
-                for (uint32_t j = 0; j < (uint32_t)kRing && j < n_loads; ++j) {
+                for (uint32_t j = 0; j < kRing && j < n_loads; ++j) {
                     const uint32_t idx = n_loads - 1 - j;
                     drain_bar(ptx::smem_u32(&ctrl->kv_full[idx % kRing]), (idx / kRing) & 1u);
                 }
             }
-        } else if (warp == 1) {
-            // ================= MMA issuer: S_t = Q_t K^T, O_t += P_t V for both query tiles ============
-            // One thread issues for both tiles in a fixed order -- at every step, for t = 0, 1:
-            // P_t V of tile t's previous step (as soon as its softmax warps have put P_t into tensor
-            // memory), then S_t = Q_t K^T of this step, which overwrites P_t only after P_t V has read it
-            // (same issue order, same pipe).  The tensor core runs the groups in that order, so S_0 is
-            // ready half a step before S_1, the two softmax phases settle half a step apart, and each
-            // tile's exponentials run under the other tile's MMAs.
-            // The whole warp walks the loop in step and one elected lane issues: with warp-uniform control
-            // flow and values the descriptor arithmetic stays on the uniform datapath, and an MMA costs few
-            // enough issue slots to keep the tensor core fed while the softmax warps of the same scheduler
-            // are in their exponential phase (a lone thread in a divergent branch could not: 96 clocks per
-            // MMA against 64 of execution).
+        } else if (warp == 1 || warp == 2) {
+            // ================= MMA issue: S_t = Q_t K^T, O_t += P_t V, one warp per query tile t ==============
+            // S_t of a step comes in two halves of 64 keys.  The softmax warps take the second half first; P_t of the whole
+            // step lies over the first half, so the second half is free as soon as its scores are in registers, and the
+            // next step's is computed there while the exponentials of this one run.  What is left on the critical path of
+            // a tile is P_t V and then the first half of the next Q_t K^T, over P_t (same thread, same pipe: P_t V has read
+            // it by then), and meanwhile the softmax warps work on the second half.  (An MMA of 64 keys takes 48 clocks
+            // where one of 128 takes 64: the tensor core works 25 % more, and waits far less.)
+            // The two warps take turns with P_t V and the first halves, step by step.  Left to themselves the tiles fall
+            // into lockstep, both in their exponentials and then both waiting for MMAs; with the groups issued in turn,
+            // tile 1's scores follow tile 0's by a group and each tile's exponentials run under the other's MMAs.  (With the
+            // turn passed on earlier, behind P_t V, they are back in lockstep; passed on behind the second half, later, the
+            // pipe idles at every hand-over, 400 clocks of barrier latency: 2048px 534 and 673 us against 525.)
+            // The tensor core holds about two MMAs ahead of the one it works on, some 150 clocks, and every barrier or
+            // shuffle instruction of these warps spends 100 to 200 in the queue it shares with the exponentials of two
+            // softmax warps: hence a warp per tile, the waits of one in the shadow of the other's MMAs (one warp for both
+            // tiles: 560 us; a third one for the second halves: their MMAs get in the way of the critical ones, 552).
+            // A whole warp walks the loop in step and one elected lane issues: with warp-uniform control flow an MMA
+            // costs few enough issue slots to keep the tensor core fed while the softmax warps of the same scheduler
+            // are in their exponential phase (a lone thread in a divergent branch could not: 96 clocks per MMA
+            // against 64 of execution).
+            const int t = warp - 1;
+            const int use_bit = t ? CLEAR_STEP_USE1 : CLEAR_STEP_USE0;
             constexpr uint32_t kDescHiK = ptx::smem_desc_hi_sw128(1024);  // 8-row groups are 1024 bytes apart
             auto uni = [](int v) { return __shfl_sync(0xffffffffu, v, 0); };  // tells the compiler v is warp-uniform
-            uint32_t ring_base = 0;  // K/V stages filled by the items before this one
-            uint32_t n_it[2] = {0, 0};   // items in which the query tile existed
-            uint32_t n_pv[2] = {0, 0};   // steps whose P V has been issued
+            const uint32_t tmem_S = tmem + t * 128, tmem_O = tmem + 256 + t * 128;
+            const uint32_t b_full0 = ptx::smem_u32(&ctrl->kv_full[0]), b_empty0 = ptx::smem_u32(&ctrl->kv_empty[0]);
+            const uint32_t b_p = ptx::smem_u32(&ctrl->p_ready[t]), b_read = ptx::smem_u32(&ctrl->sb_read[t]);
+            const uint32_t b_turn = ptx::smem_u32(&ctrl->turn[t]), b_other = ptx::smem_u32(&ctrl->turn[t ^ 1]);
+            const uint32_t v_lo0 = ptx::smem_desc_lo(sRing, kHalfBytes), k_lo0 = ptx::smem_desc_lo(sRing, 16);
+            const uint32_t q_lo = ptx::smem_desc_lo(sQ + t * kTileBytes, 16);
+            uint32_t n_it = 0;                           // items in which the query tile existed
+            uint32_t p_par = 0, sb_par = 1;              // parities of the next P_t and of the next reading of the second half
+            uint32_t turn_par = t ? 0u : 1u;             // tile 0 has the first turn
+            uint32_t ring_stage = 0, ring_par = 0;       // next fill of the ring, in staging order
             bool ok = true;
-            TRACE_DECL
-            // Every staged tile is read by this warp: it waits once for the fill of a ring position and
-            // frees the stage with an MMA commit behind the last MMA that reads it (a key tile both query
-            // tiles share is read by tile 0 first and freed behind tile 1's MMA).
-            auto kv_wait = [&](uint32_t pos) {
-                if (ok)
-                    ok = __all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->kv_full[pos % kRing]), (pos / kRing) & 1u, abort_flag, prm.status, 4));
+            // A wait whose outcome the lanes agree on later, once per group of MMAs (ok_all).
+            auto wait_lane = [&](uint32_t bar, uint32_t parity, int code) {
+                if (ok) ok = wait_bar(bar, parity, abort_flag, prm.status, code);
             };
+            auto ok_all = [&]() { return ok = __all_sync(0xffffffffu, ok); };
+            // Both warps pass every fill of the ring in staging order and arrive once for it, after they have seen it: with
+            // an MMA commit behind the MMAs that read the tile, or at once if they have no use for it.  So no phase can be
+            // freed, and no warp lapped, before both have passed.
+            auto take = [&]() -> uint32_t {
+                const uint32_t st = ring_stage;
+                wait_lane(b_full0 + 8 * st, ring_par, 4);
+                const bool wrap = st == kRing - 1;
+                ring_stage = wrap ? 0u : st + 1u;
+                ring_par ^= wrap ? 1u : 0u;
+                return st;
+            };
+            auto pass = [&]() {
+                const uint32_t st = take();
+                __syncwarp();  // every lane has seen the fill
+                if (lane == 0) ptx::mbar_arrive(b_empty0 + 8 * st);
+            };
+            // The K tiles, or the V tiles, of a step: this warp's one is returned, the other one (if any) passed.
+            auto take_own = [&](int f) -> uint32_t {
+                uint32_t own = 0;
+                if (f & CLEAR_STEP_USE0) {
+                    if (t == 0 || (f & CLEAR_STEP_SHARED)) own = take();
+                    else pass();
+                }
+                if ((f & (CLEAR_STEP_USE1 | CLEAR_STEP_SHARED)) == CLEAR_STEP_USE1) {
+                    if (t == 1) own = take();
+                    else pass();
+                }
+                return own;
+            };
+            // S of 64 keys: 64 columns from D / 16 MMAs; the second half's keys are 64 rows, 8192 bytes, into the K tile.
+            // Both operands K-major: 16 contraction channels are 32 bytes along a 128-byte row, the next 64 channels are
+            // the tile's second half.
+            auto issue_qk = [&](uint32_t k_st, uint32_t half) {
+                const uint32_t k_lo = k_lo0 + k_st * (kTileBytes >> 4) + half * (8192 >> 4);
+                ptx::mma_ss_c<false>(tmem_S + 64 * half, ptx::make_desc(q_lo, kDescHiK), ptx::make_desc(k_lo, kDescHiK), kIdescQK);
+#pragma unroll
+                for (int kk = 1; kk < D / 16; ++kk) {
+                    const uint32_t off16 = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
+                    ptx::mma_ss_c<true>(tmem_S + 64 * half, ptx::make_desc(q_lo + off16, kDescHiK), ptx::make_desc(k_lo + off16, kDescHiK), kIdescQK);
+                }
+            };
+            // The second half of S_t for the step whose K tile is in stage k_st, as soon as the one before has been read.
+            auto issue_second_half = [&](uint32_t k_st) {
+                wait_lane(b_read, sb_par, 12);
+                sb_par ^= 1u;
+                if (!ok_all()) return;
+                ptx::tc_fence_after();
+                if (ptx::elect_one()) {
+                    issue_qk(k_st, 1);
+                    ptx::tc_commit(ptx::smem_u32(&ctrl->sb_full[t]));
+                }
+                __syncwarp();
+            };
+#pragma unroll 1
             for (uint32_t k = 0; ok; ++k) {
                 const uint32_t slot = k % kSchedDepth, use = k / kSchedDepth;
-                if (!__all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->sched_full[slot]), use & 1u, abort_flag, prm.status, 5))) break;
+                wait_lane(ptx::smem_u32(&ctrl->sched_full[slot]), use & 1u, 5);
+                if (!ok_all()) break;
                 const int g = uni(ctrl->sched_item[slot]);
                 const int n_sides = uni(ctrl->sched_rec[slot].n_sides);
                 const int step_begin = uni(ctrl->sched_rec[slot].step_begin);
                 const int n = uni(ctrl->sched_rec[slot].step_count);
-                const int n_loads = uni(ctrl->sched_rec[slot].n_loads);
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&ctrl->sched_empty[slot]));
                 if (g >= total_items) break;
-                const clear_pair_step_t *steps = prm.steps + step_begin;
-                for (int t = 0; t < n_sides && ok; ++t)
-                    ok = __all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->q_full[t]), n_it[t] & 1u, abort_flag, prm.status, 6));
-                if (!ok) break;
-
-                // One group of MMAs for query tile t: O_t += P_t V of its previous step (if one is pending:
-                // pv), then S_t = Q_t K^T of this step (if it takes part: qk).  Everything that does not
-                // need P_t -- the fills of the V and K stages, the descriptors -- comes before the wait for
-                // P_t, so that between the arrival of P_t and the MMAs lie as few instructions as possible:
-                // this warp shares its scheduler with two softmax warps in their exponential phase.
-                //   P_t V : P_t (bf16 pairs) in the first 64 columns of S_t, 16 keys = 8 columns; V MN-major,
-                //           16 keys are 16 rows of 128 bytes = 2048 bytes;
-                //   Q K^T : both operands K-major: 16 contraction channels are 32 bytes along a 128-byte row,
-                //           the next 64 channels are the tile's second half.
-                auto issue_group = [&](int t, bool pv, int pv_flags, int pv_base, bool first_pv, bool qk, int qk_flags,
-                                       int qk_base, bool last) {
-                    const bool pv_shared = (pv_flags & CLEAR_STEP_SHARED) != 0, qk_shared = (qk_flags & CLEAR_STEP_SHARED) != 0;
-                    const uint32_t pos_v = ring_base + ((uint32_t)pv_base >> 16) + (uint32_t)step_tile_index(pv_flags, t);
-                    const uint32_t pos_k = ring_base + ((uint32_t)qk_base & 0xffffu) + (uint32_t)step_tile_index(qk_flags, t);
-                    TRACE_MARK(0)
-                    if (pv && !(pv_shared && t == 1)) kv_wait(pos_v);
-                    if (qk && !(qk_shared && t == 1)) kv_wait(pos_k);
+                const int *step_flags = &prm.steps[step_begin].flags;
+                constexpr int kStepInts = sizeof(clear_pair_step_t) / sizeof(int);
+                // the flags of 32 steps at a time, one step per lane; the 32 after them are fetched meanwhile
+                auto fetch_flags = [&](int s0) { return s0 + lane < n ? ptx::ldg_u32(step_flags + (s0 + lane) * kStepInts) : 0u; };
+                uint32_t lane_flags = fetch_flags(0), lane_flags_next = fetch_flags(32);
+                int pend = 0;            // flags of the step before (0: none)
+                int flags = (int)__shfl_sync(0xffffffffu, lane_flags, 0);
+                uint32_t acc = 0;        // O_t holds something of this item
+                const bool exists = t < n_sides;
+                if (exists) wait_lane(ptx::smem_u32(&ctrl->q_full[t]), n_it & 1u, 6);
+#pragma unroll 1
+                for (int s = 0; s <= n && ok; ++s) {
+                    // one step past the end: the last P_t V
+                    const bool last = s == n;
+                    if (((s + 1) & 31) == 0) {
+                        lane_flags = lane_flags_next;
+                        lane_flags_next = fetch_flags(s + 33);
+                    }
+                    const int flags_next = (int)__shfl_sync(0xffffffffu, lane_flags, (s + 1) & 31);  // 0 past the end
+                    const bool pv = (pend & use_bit) != 0, qk = (flags & use_bit) != 0;
+                    const uint32_t k_st = take_own(flags);
+                    if (qk) issue_second_half(k_st);
+                    const uint32_t v_st = take_own(pend);
                     // the epilogue must have read the previous item's O_t out of tensor memory
-                    if (ok && pv && first_pv)
-                        ok = __all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->o_empty[t]), (n_it[t] & 1u) ^ 1u, abort_flag, prm.status, 8));
-                    TRACE_MARK(1)  // wait for K, V
-                    const uint32_t tmem_S = tmem + t * 128, tmem_O = tmem + 256 + t * 128;
-                    const uint32_t v_lo = ptx::smem_desc_lo(sRing + (pos_v % kRing) * kTileBytes, kHalfBytes);
-                    const uint32_t q_lo = ptx::smem_desc_lo(sQ + t * kTileBytes, 16);
-                    const uint32_t k_lo = ptx::smem_desc_lo(sRing + (pos_k % kRing) * kTileBytes, 16);
-                    const uint32_t b_vfree = ptx::smem_u32(&ctrl->kv_empty[pos_v % kRing]);
-                    const uint32_t b_kfree = ptx::smem_u32(&ctrl->kv_empty[pos_k % kRing]);
-                    const bool free_v = !pv_shared || t == 1, free_k = !qk_shared || t == 1;
-                    if (ok && pv) ok = __all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->p_ready[t]), n_pv[t] & 1u, abort_flag, prm.status, 7));
-                    if (!ok) return;
-                    TRACE_MARK(4)  // wait for P
+                    if (pv && !acc) wait_lane(ptx::smem_u32(&ctrl->o_empty[t]), (n_it & 1u) ^ 1u, 8);
+                    wait_lane(b_turn, turn_par, 11);
+                    turn_par ^= 1u;
+                    if (pv) {
+                        wait_lane(b_p, p_par, 7);
+                        p_par ^= 1u;
+                    }
+                    if (!ok_all()) break;
                     ptx::tc_fence_after();
                     if (ptx::elect_one()) {
                         if (pv) {
-                            ptx::mma_ts(tmem_O, tmem_S, ptx::make_desc(v_lo, kDescHiK), kIdescPV, first_pv ? 0u : 1u);
+                            // P_t (bf16 pairs) in the first 64 columns of S_t, 16 keys = 8 columns; V MN-major, 16 keys are 16
+                            // rows of 128 bytes = 2048 bytes
+                            const uint32_t v_lo = v_lo0 + v_st * (kTileBytes >> 4);
+                            ptx::mma_ts(tmem_O, tmem_S, ptx::make_desc(v_lo, kDescHiK), kIdescPV, acc);
 #pragma unroll
                             for (int kk = 1; kk < 8; ++kk)
                                 ptx::mma_ts_c<true>(tmem_O, tmem_S + kk * 8, ptx::make_desc(v_lo + kk * (2048 >> 4), kDescHiK), kIdescPV);
-                            if (free_v) ptx::tc_commit(b_vfree);
                         }
                         if (qk) {
-                            ptx::mma_ss_c<false>(tmem_S, ptx::make_desc(q_lo, kDescHiK), ptx::make_desc(k_lo, kDescHiK), kIdescQK);
-#pragma unroll
-                            for (int kk = 1; kk < D / 16; ++kk) {
-                                const uint32_t off16 = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
-                                ptx::mma_ss_c<true>(tmem_S, ptx::make_desc(q_lo + off16, kDescHiK),
-                                                    ptx::make_desc(k_lo + off16, kDescHiK), kIdescQK);
-                            }
-                            ptx::tc_commit(ptx::smem_u32(&ctrl->s_full[t]));
-                            if (free_k) ptx::tc_commit(b_kfree);
+                            issue_qk(k_st, 0);
+                            ptx::tc_commit(ptx::smem_u32(&ctrl->sa_full[t]));
                         }
-                        // the item's last group of the tile: its output is complete once these MMAs are
-                        if (last) ptx::tc_commit(ptx::smem_u32(&ctrl->o_full[t]));
+                        ptx::mbar_arrive(b_other);  // the other tile's turn
+                        if (qk) ptx::tc_commit(b_empty0 + 8 * k_st);
+                        if (pv) ptx::tc_commit(b_empty0 + 8 * v_st);
+                        // behind the item's last Q K^T the next Q_t may land; behind its last P V the output is complete
+                        if (s == n - 1 && exists) ptx::tc_commit(ptx::smem_u32(&ctrl->q_empty[t]));
+                        if (last && exists) ptx::tc_commit(ptx::smem_u32(&ctrl->o_full[t]));
                     }
                     __syncwarp();
-                    if (pv) ++n_pv[t];
-                    TRACE_MARK(5)  // issue
-                };
-
-                int pend_flags[2] = {0, 0}, pend_base[2] = {0, 0};  // the step whose P_t V is still to be issued
-                bool pending[2] = {false, false};
-                bool first_pv[2] = {true, true};
-                int4 rec = __ldg(reinterpret_cast<const int4 *>(steps) + 1);  // flags, n_valid0, n_valid1, load_base
-                for (int s = 0; s < n && ok; ++s) {
-                    const int flags = uni(rec.x), load_base = uni(rec.w);
-                    if (s + 1 < n) rec = __ldg(reinterpret_cast<const int4 *>(steps + s + 1) + 1);  // one step ahead
-#pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        if (t >= n_sides || !ok) continue;
-                        const bool qk = step_uses(flags, t);
-                        if (!pending[t] && !qk) continue;
-                        issue_group(t, pending[t], pend_flags[t], pend_base[t], first_pv[t], qk, flags, load_base, false);
-                        if (pending[t]) first_pv[t] = false;
-                        pending[t] = qk;
-                        pend_flags[t] = flags;
-                        pend_base[t] = load_base;
-                    }
+                    if (pv) acc = 1u;
+                    pend = flags;
+                    flags = flags_next;
                 }
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    if (t >= n_sides || !ok) continue;
-                    // every Q_t K^T of the item has been issued: the next item's Q tile may land
-                    if (ptx::elect_one()) ptx::tc_commit(ptx::smem_u32(&ctrl->q_empty[t]));
-                    __syncwarp();
-                    issue_group(t, pending[t], pend_flags[t], pend_base[t], first_pv[t], false, 0, 0, true);
-                    ++n_it[t];
-                }
-                ring_base += (uint32_t)n_loads;
+                if (exists) ++n_it;
             }
-#ifdef CLEAR_WS_TRACE
-            TRACE_MARK(0)
-            if (blockIdx.x == 0 && lane == 0)
-                printf("mma thread: other %llu waitK %llu issueQK %llu waitV %llu waitP %llu issuePV %llu\n", tr_acc[0], tr_acc[1],
-                       tr_acc[2], tr_acc[3], tr_acc[4], tr_acc[5]);
-#endif
             if (*abort_flag) {
                 // MMAs that were issued must retire before tensor memory is given back
                 if (lane == 0) {
-                    ptx::tc_commit(ptx::smem_u32(&ctrl->drain[0]));
-                    drain_bar(ptx::smem_u32(&ctrl->drain[0]), 0);
+                    ptx::tc_commit(ptx::smem_u32(&ctrl->drain[t]));
+                    drain_bar(ptx::smem_u32(&ctrl->drain[t]), 0);
                 }
             }
         }
         __syncwarp();
     } else {
         // ================= softmax warps: thread r owns query row r (tensor-memory lane r) of its tile =====
-        // Per step: S_t into registers, row maximum, P = exp2(.) under the Eq. 3 mask as bf16 into tensor
-        // memory over S_t, row sum; at the end of an item O_t / l -> bf16 -> global memory (or fp32 partial
+        // Per step: S_t into registers, half by half, P = exp2(.) under the Eq. 3 mask as bf16 into tensor memory over
+        // the first half of S_t, row sum; at the end of an item O_t / l -> bf16 -> global memory (or fp32 partial
         // results of split text rows).
         ptx::setmaxnreg_inc<kRegsSoftmax>();
-        TRACE_DECL
         const int t = (warp - 4) >> 2;  // query tile of the pair
         const int q4 = warp & 3;        // tensor-memory lane quadrant
         const int r = q4 * 32 + lane;   // query row of the tile
         const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
         const uint32_t tmem_S = tmem + t * 128, tmem_O = tmem + 256 + t * 128;
         const float c = prm.scale_log2;
-        const uint32_t b_s = ptx::smem_u32(&ctrl->s_full[t]), b_pready = ptx::smem_u32(&ctrl->p_ready[t]);
+        const uint32_t b_sa = ptx::smem_u32(&ctrl->sa_full[t]), b_sb = ptx::smem_u32(&ctrl->sb_full[t]), b_pready = ptx::smem_u32(&ctrl->p_ready[t]);
         uint32_t n_s = 0, n_items_seen = 0;
         bool alive = true;
+#pragma unroll 1
         for (uint32_t k = 0; alive; ++k) {
             const uint32_t slot = k % kSchedDepth, use = k / kSchedDepth;
             if (!__all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->sched_full[slot]), use & 1u, abort_flag, prm.status, 9)))
@@ -548,28 +775,44 @@ clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
             // grid position of this row's query (image tiles), and whether the row exists
             const int q_y = (t ? item.qy1 : item.qy0) + (r >> 4), q_x = item.qx + (r & 15);
             const bool q_valid = is_text ? r < (t ? item.n_rows1 : item.n_rows0) : (q_y < prm.grid_h && q_x < prm.grid_w);
-            float m_used = -INFINITY, l = 0.f;
+            float ref = -INFINITY, l = 0.f;  // reference of the row's exponents (log2 units) and row sum
+            int bump = 0;                    // powers of two the reference is to be raised by before the next tile
             bool first = true;
 
-            // Step records are fetched two steps ahead and this row's precomputed mask words one step ahead,
-            // so that neither latency is on the critical path.
+            // The flags and the key count (or mask entry) of 32 steps at a time, one step per lane, the 32 after them
+            // fetched meanwhile; taken out of the lanes two steps ahead, and this row's precomputed mask words fetched one
+            // step ahead.  No latency is on the critical path, and the loads stay where they are written (left to the
+            // compiler, they sank to their use).
             const int kMaskedBit = t ? CLEAR_STEP_MASKED1 : CLEAR_STEP_MASKED0;
-            auto load_mask_row = [&](const SideStep &q) -> uint4 {
-                if (step_uses(q.flags, t) && (q.flags & kMaskedBit) && !(q.flags & CLEAR_STEP_LINEAR) && q.n_valid >= 0)
-                    return __ldg(reinterpret_cast<const uint4 *>(prm.mask_table) + ((size_t)q.n_valid * 128 + r));
+            const int *rec = &steps->flags;
+            constexpr int kStepInts = sizeof(clear_pair_step_t) / sizeof(int);
+            struct Rec {
+                int flags, n_valid;
+            };
+            auto fetch_steps = [&](int s0) -> Rec {
+                const bool on = s0 + lane < step_count;
+                return Rec{on ? (int)ptx::ldg_u32(rec + (s0 + lane) * kStepInts) : 0, on ? (int)ptx::ldg_u32(rec + (s0 + lane) * kStepInts + 1 + t) : 0};
+            };
+            auto load_mask_row = [&](const Rec &x) -> uint4 {
+                if (step_uses(x.flags, t) && (x.flags & kMaskedBit) && !(x.flags & CLEAR_STEP_LINEAR) && x.n_valid >= 0)
+                    return ptx::ldg_u128(reinterpret_cast<const uint4 *>(prm.mask_table) + ((size_t)x.n_valid * 128 + r));
                 return make_uint4(0u, 0u, 0u, 0u);
             };
-            SideStep st_next = load_side_step(steps, t);
-            SideStep st_next2 = st_next;
-            if (step_count > 1) st_next2 = load_side_step(steps + 1, t);
-            uint4 mrow_next = load_mask_row(st_next);
-            TRACE_MARK(8)  // between items
+            Rec lanes = fetch_steps(0), lanes_next = fetch_steps(32);
+            auto from_lane = [&](int s) { return Rec{__shfl_sync(0xffffffffu, lanes.flags, s & 31), __shfl_sync(0xffffffffu, lanes.n_valid, s & 31)}; };
+            Rec st, st1 = from_lane(0), st2 = from_lane(1);
+            uint4 mrow, mrow1 = load_mask_row(st1);
+#pragma unroll 1
             for (int s = 0; s < step_count; ++s) {
-                const SideStep st = st_next;
-                const uint4 mrow = mrow_next;
-                st_next = st_next2;  // fetched a step ago: the mask row's address does not wait for it
-                if (s + 2 < step_count) st_next2 = load_side_step(steps + s + 2, t);
-                if (s + 1 < step_count) mrow_next = load_mask_row(st_next);
+                st = st1;
+                mrow = mrow1;
+                st1 = st2;
+                mrow1 = load_mask_row(st1);
+                if (((s + 2) & 31) == 0) {
+                    lanes = lanes_next;
+                    lanes_next = fetch_steps(s + 34);
+                }
+                st2 = from_lane(s + 2);   // 0 past the end
                 if (!step_uses(st.flags, t)) continue;
                 const bool masked = (st.flags & kMaskedBit) != 0;
                 // ---- mask bits of this row for the tile (bit j of word w = key 32 w + j allowed) --------
@@ -624,198 +867,113 @@ clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
                     }
                 }
 
-                TRACE_MARK(0)  // step prologue: records, mask words
-                // warp-uniform outcome: the tcgen05.ld / st below need the whole warp.  Once S_t of this step
-                // is complete, so is P_t V of the step before (same thread, same pipe, issued earlier).
-                if (!__all_sync(0xffffffffu, wait_bar(b_s, n_s & 1u, abort_flag, prm.status, 10))) {
+                // P = 2^(S c - ref) with a reference per row that need not be the running maximum: P, the row sum and O
+                // are floating-point numbers of full precision at any scale, so the reference only has to keep them
+                // within range.  It is the maximum of the row's first tile; when a tile's row sum exceeds 2^8 the
+                // reference is raised before the next tile, by a whole power of two and without a look at the maximum.
+                // No maximum pass, then, on any tile but the first, and the scores die as their P is formed.  A row sum
+                // beyond 2^64 means scores 64 powers of two above everything seen before; the warp then computes its
+                // scores again, from global memory, before anybody has used P.
+                const bool raise = __any_sync(0xffffffffu, bump != 0);
+                float alpha = 1.f;
+                if (raise) {
+                    alpha = ptx::ex2(-(float)bump);
+                    ref += (float)bump;
+                    l *= alpha;
+                    bump = 0;
+                }
+                const bool exact = __any_sync(0xffffffffu, first || (ref == -INFINITY && q_valid));
+                float tile_sum = 0.f;
+                // warp-uniform outcome of the waits: the tcgen05.ld / st below need the whole warp.  Once the first half of
+                // S_t is complete, so is P_t V of the step before (same thread, same pipe, issued earlier).
+                if (!__all_sync(0xffffffffu, wait_bar(b_sb, n_s & 1u, abort_flag, prm.status, 10))) {
                     alive = false;
                     break;
                 }
-                ++n_s;
-                TRACE_MARK(1)  // wait for S
                 ptx::tc_fence_after();
-                uint32_t sv[4][32];
-#pragma unroll
-                for (int w = 0; w < 4; ++w) ptx::tmem_ld32(tmem_S + lane_off + 32 * w, sv[w]);
-                ptx::tmem_wait_ld();
-                TRACE_MARK(2)  // S into registers
-
-                // ---- P = exp2(S * c - m * c) on the allowed keys, 0 elsewhere; row sum; bf16 pairs into
-                // tensor memory, 32 keys (16 columns) at a time (two-wide fp32 FMA and ADD; four independent
-                // partial sums)
-                float tile_sum = 0.f;
-                auto exp_pass = [&](auto masked_c, float mc) {
-                    constexpr bool kMasked = decltype(masked_c)::value;
+                if (__builtin_expect(!exact, 1)) {
+                    const float mc = (ref == -INFINITY) ? 0.f : ref;
                     const uint64_t c2 = ptx::pack2(c, c), nmc2 = ptx::pack2(-mc, -mc);
                     uint64_t lsum[2] = {0ull, 0ull};
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        uint32_t pk[16];
-#pragma unroll
-                        for (int j = 0; j < 32; j += 2) {
-                            const uint64_t x2 =
-                                ptx::fma2(ptx::pack2(__uint_as_float(sv[w][j]), __uint_as_float(sv[w][j + 1])), c2, nmc2);
-                            float x0, x1;
-                            ptx::unpack2(x2, x0, x1);
-                            if (kMasked) {
-                                x0 = ((mw[w] >> j) & 1u) ? x0 : -INFINITY;
-                                x1 = ((mw[w] >> (j + 1)) & 1u) ? x1 : -INFINITY;
-                            }
-                            const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
-                            lsum[(j >> 1) & 1] = ptx::add2(lsum[(j >> 1) & 1], ptx::pack2(p0, p1));
-                            pk[j >> 1] = ptx::pack_bf16(p0, p1);
-                        }
-                        ptx::tmem_st16(tmem_S + lane_off + 16 * w, pk);
+                    uint32_t sv[2][32], pk[2][16];
+                    ptx::tmem_ld32(tmem_S + lane_off + 64, sv[0]);
+                    ptx::tmem_ld32(tmem_S + lane_off + 96, sv[1]);
+                    ptx::tmem_wait_ld();
+                    ptx::tc_fence_before();
+                    warp_arrive(ptx::smem_u32(&ctrl->sb_read[t]), lane);
+                    if (masked) {
+                        exp_chunk<true>(sv[0], mw[2], c2, nmc2, lsum, pk[0]);
+                        exp_chunk<true>(sv[1], mw[3], c2, nmc2, lsum, pk[1]);
+                    } else {
+                        exp_chunk<false>(sv[0], 0u, c2, nmc2, lsum, pk[0]);
+                        exp_chunk<false>(sv[1], 0u, c2, nmc2, lsum, pk[1]);
                     }
-                    float a0, a1, a2, a3;
-                    ptx::unpack2(lsum[0], a0, a1);
-                    ptx::unpack2(lsum[1], a2, a3);
-                    tile_sum = (a0 + a1) + (a2 + a3);
-                };
-                // The running maximum m of a row moves only when a tile's maximum over the allowed keys
-                // exceeds it by more than the threshold, i.e. when some P of the tile would exceed
-                // 2^threshold.  So P is formed against the maximum as it stands, and only when a row's sum
-                // over the tile exceeds 2^threshold (no single P can otherwise), or the row has no maximum
-                // yet, is the tile's maximum taken, m moved by the rule above, O rescaled and P formed again:
-                // the same results as with a maximum pass on every tile, which costs a third of the
-                // exponentials' time and is needed on the first tile of a row and hardly ever after.
-                bool use_mask = masked;
-                bool exact = __any_sync(0xffffffffu, first || (m_used == -INFINITY && q_valid));
-#pragma unroll 1
-                for (;;) {
-                    if (exact) {
-                        // maximum over the allowed keys (the scores Eq. 3 forbids become -inf in place)
-                        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                        if (use_mask) {
-#pragma unroll
-                            for (int w = 0; w < 4; ++w)
-#pragma unroll
-                                for (int j = 0; j < 32; j += 2) {
-                                    const float v0 = ((mw[w] >> j) & 1u) ? __uint_as_float(sv[w][j]) : -INFINITY;
-                                    const float v1 = ((mw[w] >> (j + 1)) & 1u) ? __uint_as_float(sv[w][j + 1]) : -INFINITY;
-                                    sv[w][j] = __float_as_uint(v0);
-                                    sv[w][j + 1] = __float_as_uint(v1);
-                                    mx4[(j >> 1) & 3] = ptx::max3(mx4[(j >> 1) & 3], v0, v1);
-                                }
-                            use_mask = false;
-                        } else {
-#pragma unroll
-                            for (int w = 0; w < 4; ++w)
-#pragma unroll
-                                for (int j = 0; j < 32; j += 2)
-                                    mx4[(j >> 1) & 3] = ptx::max3(mx4[(j >> 1) & 3], __uint_as_float(sv[w][j]), __uint_as_float(sv[w][j + 1]));
-                        }
-                        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-                        const float m_new = fmaxf(m_used, mx);
-                        if (first) {
-                            m_used = m_new;
-                        } else {
-                            const bool need = (m_new - m_used) * c > kRescaleThreshold;  // false for NaN (-inf minus -inf)
-                            if (__any_sync(0xffffffffu, need)) {
-                                float alpha = 1.f;
-                                if (need) {
-                                    alpha = ptx::ex2((m_used - m_new) * c);
-                                    m_used = m_new;
-                                    l *= alpha;
-                                }
-#pragma unroll 1
-                                for (int w = 0; w < D / 16; ++w) {
-                                    uint32_t o[16];
-                                    ptx::tmem_ld16(tmem_O + lane_off + 16 * w, o);
-                                    ptx::tmem_wait_ld();
-#pragma unroll
-                                    for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
-                                    ptx::tmem_st16(tmem_O + lane_off + 16 * w, o);
-                                }
-                            }
-                        }
+                    if (!__all_sync(0xffffffffu, wait_bar(b_sa, n_s & 1u, abort_flag, prm.status, 13))) {
+                        alive = false;
+                        break;
                     }
-                    const float mc = (m_used == -INFINITY) ? 0.f : m_used * c;
-                    if (use_mask)
-                        exp_pass(std::true_type{}, mc);
-                    else
-                        exp_pass(std::false_type{}, mc);
-                    if (exact) break;
-                    exact = __any_sync(0xffffffffu, !(tile_sum <= kMaxTileSum));  // also for a NaN
-                    if (!exact) break;
+                    ptx::tc_fence_after();
+                    ptx::tmem_ld32(tmem_S + lane_off, sv[0]);
+                    ptx::tmem_ld32(tmem_S + lane_off + 32, sv[1]);
+                    ptx::tmem_wait_ld();
+                    ptx::tmem_st16(tmem_S + lane_off + 32, pk[0]);
+                    ptx::tmem_st16(tmem_S + lane_off + 48, pk[1]);
+                    if (masked) {
+                        exp_chunk<true>(sv[0], mw[0], c2, nmc2, lsum, pk[0]);
+                        ptx::tmem_st16(tmem_S + lane_off, pk[0]);
+                        exp_chunk<true>(sv[1], mw[1], c2, nmc2, lsum, pk[1]);
+                        ptx::tmem_st16(tmem_S + lane_off + 16, pk[1]);
+                    } else {
+                        exp_chunk<false>(sv[0], 0u, c2, nmc2, lsum, pk[0]);
+                        ptx::tmem_st16(tmem_S + lane_off, pk[0]);
+                        exp_chunk<false>(sv[1], 0u, c2, nmc2, lsum, pk[1]);
+                        ptx::tmem_st16(tmem_S + lane_off + 16, pk[1]);
+                    }
+                    tile_sum = sum4(lsum);
+                    if (raise) rescale_rows<D>(tmem_O + lane_off, alpha);
+                    if (__builtin_expect(__any_sync(0xffffffffu, !(tile_sum <= kMaxTileSum)), 0)) {
+                        const int2 org = load_side_origin(steps + s, t);
+                        const long long q_tok = is_text ? (long long)item.qx + t * 128 + r : prm.n_text + (long long)q_y * prm.grid_w + q_x;
+                        const RowState rs = rescue_step<D>(prm, tmem_S + lane_off, tmem_O + lane_off, make_uint4(mw[0], mw[1], mw[2], mw[3]), c, ref,
+                                                           l, (long long)bh * prm.n_tokens, q_valid ? q_tok : -1, org,
+                                                           (st.flags & CLEAR_STEP_LINEAR) != 0);
+                        ref = rs.ref;
+                        l = rs.l;
+                        tile_sum = rs.tile_sum;
+                    }
+                } else {
+                    if (!__all_sync(0xffffffffu, wait_bar(b_sa, n_s & 1u, abort_flag, prm.status, 13))) {
+                        alive = false;
+                        break;
+                    }
+                    ptx::tc_fence_after();
+                    if (raise) rescale_rows<D>(tmem_O + lane_off, alpha);
+                    const RowState rs = exact_step<D>(tmem_S + lane_off, tmem_O + lane_off, make_uint4(mw[0], mw[1], mw[2], mw[3]), c, ref, l, first);
+                    ref = rs.ref;
+                    l = rs.l;
+                    tile_sum = rs.tile_sum;
+                    ptx::tc_fence_before();
+                    warp_arrive(ptx::smem_u32(&ctrl->sb_read[t]), lane);
                 }
+                ++n_s;
                 first = false;
                 l += tile_sum;
-                TRACE_MARK(5)  // exponentials
+                if (tile_sum > kBumpSum) bump = (int)((__float_as_uint(tile_sum) >> 23) & 0xffu) - 127;
                 // P_t (and a rescaled O_t) must be in tensor memory before the MMA thread is told
                 ptx::tmem_wait_st();
                 ptx::tc_fence_before();
                 warp_arrive(b_pready, lane);
-                TRACE_MARK(6)  // arrival
-#ifdef CLEAR_WS_TRACE
-                ++tr_steps;
-#endif
             }
             if (!alive) break;
-            TRACE_MARK(0)
 
             // ---- epilogue: the last P_t V has retired once o_full completes; O_t / l -> global memory -----
             if (!__all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->o_full[t]), n_items_seen & 1u, abort_flag, prm.status, 14)))
                 break;
             ++n_items_seen;
             ptx::tc_fence_after();
-            const int slot_p = t ? item.partial_slot1 : item.partial_slot0;
-            if (slot_p >= 0) {
-                // split text-query tile: un-normalised fp32 row, its maximum (log2 units) and its sum
-                const long long row = ((long long)bh * prm.n_partial_slots + slot_p) * 128 + r;
-                float *dst = prm.partial_o + row * D;
-#pragma unroll
-                for (int w = 0; w < D / 32; ++w) {
-                    uint32_t o[32];
-                    ptx::tmem_ld32(tmem_O + lane_off + 32 * w, o);
-                    ptx::tmem_wait_ld();
-                    if (w == D / 32 - 1) {
-                        ptx::tc_fence_before();
-                        warp_arrive(ptx::smem_u32(&ctrl->o_empty[t]), lane);
-                    }
-                    if (q_valid) {
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4)
-                            *reinterpret_cast<uint4 *>(dst + 32 * w + j) = make_uint4(o[j], o[j + 1], o[j + 2], o[j + 3]);
-                    }
-                }
-                if (q_valid) {
-                    prm.partial_ml[row * 2] = m_used * c;
-                    prm.partial_ml[row * 2 + 1] = l;
-                }
-            } else {
-                const float inv = l > 0.f ? 1.f / l : 0.f;
-                const long long token = is_text ? (long long)(item.qx + t * 128 + r) : prm.n_text + (long long)q_y * prm.grid_w + q_x;
-                __nv_bfloat16 *dst = prm.out + ((long long)bh * prm.n_tokens + token) * D;
-#pragma unroll
-                for (int w = 0; w < D / 32; ++w) {
-                    uint32_t o[32];
-                    ptx::tmem_ld32(tmem_O + lane_off + 32 * w, o);
-                    ptx::tmem_wait_ld();
-                    if (w == D / 32 - 1) {
-                        ptx::tc_fence_before();
-                        warp_arrive(ptx::smem_u32(&ctrl->o_empty[t]), lane);
-                    }
-                    if (q_valid) {
-#pragma unroll
-                        for (int cc = 0; cc < 4; ++cc) {
-                            uint4 val;
-                            val.x = ptx::pack_bf16(__uint_as_float(o[8 * cc + 0]) * inv, __uint_as_float(o[8 * cc + 1]) * inv);
-                            val.y = ptx::pack_bf16(__uint_as_float(o[8 * cc + 2]) * inv, __uint_as_float(o[8 * cc + 3]) * inv);
-                            val.z = ptx::pack_bf16(__uint_as_float(o[8 * cc + 4]) * inv, __uint_as_float(o[8 * cc + 5]) * inv);
-                            val.w = ptx::pack_bf16(__uint_as_float(o[8 * cc + 6]) * inv, __uint_as_float(o[8 * cc + 7]) * inv);
-                            *reinterpret_cast<uint4 *>(dst + 32 * w + 8 * cc) = val;
-                        }
-                    }
-                }
-            }
-            TRACE_MARK(7)  // epilogue
+            store_tile<D>(prm, tmem_O, ptx::smem_u32(&ctrl->o_empty[t]), item.qx + (is_text ? t * 128 : 0), t ? item.qy1 : item.qy0,
+                          is_text ? (t ? item.n_rows1 : item.n_rows0) : -1, t ? item.partial_slot1 : item.partial_slot0, bh, ref, l);
         }
-#ifdef CLEAR_WS_TRACE
-        if (blockIdx.x == 0 && lane == 0)
-            printf("tile %d warp %d steps %u: prologue %llu waitS %llu ldS %llu max %llu rescale %llu exp %llu arrive %llu epilogue %llu between items %llu\n",
-                   t, q4, tr_steps, tr_acc[0], tr_acc[1], tr_acc[2], tr_acc[3], tr_acc[4], tr_acc[5], tr_acc[6], tr_acc[7], tr_acc[8]);
-#endif
     }
 
     ptx::tc_fence_before();
@@ -832,31 +990,27 @@ clear_ws_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
 }
 
 // ---- host side: tensor maps and launch ---------------------------------------------------------
-// Maps 0..2: image part of q, k, v as [BH][grid_h][grid_w][d]; 3: text prefix of q as [BH][n_text][d];
-// 4, 5: k, v as the token sequence [BH][N][d].
+// Image part of a tensor as [BH][half][grid_h][grid_w][64], runs of tokens as [BH][half][1][tokens][64]; the text
+// prefix of q ends at n_text (rows past it read as zero), the token sequence of k, v at N.
 int build_maps(const clear_plan &p, const void *q, const void *k, const void *v)
 {
     const Shape &s = p.shape;
-    const uint64_t d = (uint64_t)s.head_dim, gw = (uint64_t)s.grid_w, gh = (uint64_t)s.grid_h, T = (uint64_t)s.n_text;
-    const uint64_t N = T + gw * gh, BH = (uint64_t)s.B * s.H;
-    const uint64_t row_b = d * 2;
+    const uint64_t gw = (uint64_t)s.grid_w, gh = (uint64_t)s.grid_h, T = (uint64_t)s.n_text;
+    const uint64_t N = T + gw * gh, BH = (uint64_t)s.B * s.H, halves = (uint64_t)s.head_dim / 64;
+    const uint64_t row_b = (uint64_t)s.head_dim * 2;
     CUtensorMap *tm = reinterpret_cast<CUtensorMap *>(p.tm_storage);
     const void *ptrs[3] = {q, k, v};
-    const uint64_t dims4[4] = {d, gw, gh, BH};
-    const uint64_t str4[3] = {row_b, gw * row_b, N * row_b};
-    const uint32_t box4[4] = {64, (uint32_t)kTileW, (uint32_t)kTileH, 1};
+    const uint64_t dims_img[5] = {64, gw, gh, halves, BH}, str_img[4] = {row_b, gw * row_b, 128, N * row_b};
+    const uint32_t box_img[5] = {64, (uint32_t)kTileW, (uint32_t)kTileH, (uint32_t)halves, 1};
+    const uint64_t str_lin[4] = {row_b, N * row_b, 128, N * row_b};
+    const uint32_t box_lin[5] = {64, (uint32_t)kTileTokens, 1, (uint32_t)halves, 1};
     for (int t = 0; t < 3; ++t) {
-        const char *base = static_cast<const char *>(ptrs[t]) + T * row_b;
-        if (!encode_bf16_map(&tm[t], base, 4, dims4, str4, box4)) return CLEAR_ERR_CUDA;
+        const uint64_t dims_lin[5] = {64, t == 0 ? std::max<uint64_t>(T, 1) : N, 1, halves, BH};
+        if (!encode_bf16_map(&tm[2 * t], static_cast<const char *>(ptrs[t]) + T * row_b, 5, dims_img, str_img, box_img) ||
+            !encode_bf16_map(&tm[2 * t + 1], ptrs[t], 5, dims_lin, str_lin, box_lin))
+            return CLEAR_ERR_CUDA;
+        p.tm_ptrs[t] = ptrs[t];
     }
-    const uint64_t dims3[3] = {d, N, BH};
-    const uint64_t dims3t[3] = {d, T > 0 ? T : 1, BH};
-    const uint64_t str3[2] = {row_b, N * row_b};
-    const uint32_t box3[3] = {64, (uint32_t)kTileTokens, 1};
-    if (!encode_bf16_map(&tm[3], q, 3, dims3t, str3, box3)) return CLEAR_ERR_CUDA;
-    if (!encode_bf16_map(&tm[4], k, 3, dims3, str3, box3)) return CLEAR_ERR_CUDA;
-    if (!encode_bf16_map(&tm[5], v, 3, dims3, str3, box3)) return CLEAR_ERR_CUDA;
-    for (int t = 0; t < 3; ++t) p.tm_ptrs[t] = ptrs[t];
     p.tm_ptrs[3] = nullptr;
     p.tm_valid = true;
     return CLEAR_OK;
@@ -871,7 +1025,7 @@ DeviceInfo g_dev[64];
 std::mutex g_dev_mutex;
 
 template <int D>
-int launch_variant(const clear_plan &p, const CUtensorMap *tm, const WsParams &prm, cudaStream_t stream)
+int launch_variant(const clear_plan &p, const WsMaps &maps, const WsParams &prm, cudaStream_t stream)
 {
     constexpr size_t kSmem = (size_t)(2 + kRing) * (D / 64) * 16384 + sizeof(Ctrl);
     static_assert(kSmem <= 232448, "shared memory of one block");
@@ -892,7 +1046,7 @@ int launch_variant(const clear_plan &p, const CUtensorMap *tm, const WsParams &p
     }
     const long long total = (long long)prm.n_items * prm.n_bh;
     const unsigned grid = (unsigned)std::min<long long>(n_sm, total);
-    clear_ws_kernel<D><<<grid, kWsThreads, kSmem, stream>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], prm);
+    clear_ws_kernel<D><<<grid, kWsThreads, kSmem, stream>>>(maps, prm);
     CLEAR_CUDA_TRY(cudaGetLastError());
     return launch_text_combine(p, prm.out, stream);
 }
@@ -905,7 +1059,7 @@ int launch_ws(const clear_plan &p, const void *q, const void *k, const void *v, 
     if (!(scale > 0.f)) return CLEAR_ERR_UNSUPPORTED;
     const long long total = (long long)p.sch.pair_items.size() * p.shape.B * p.shape.H;
     if (total <= 0 || total >= (1ll << 30)) return CLEAR_ERR_UNSUPPORTED;
-    CUtensorMap tm[6];
+    WsMaps maps;
     {
         std::lock_guard<std::mutex> lock(p.tm_mutex);
         if (!(p.tm_valid && p.tm_ptrs[0] == q && p.tm_ptrs[1] == k && p.tm_ptrs[2] == v)) {
@@ -915,7 +1069,7 @@ int launch_ws(const clear_plan &p, const void *q, const void *k, const void *v, 
                 return rc;
             }
         }
-        std::memcpy(tm, p.tm_storage, sizeof(tm));
+        std::memcpy(&maps, p.tm_storage, sizeof(maps));
     }
     WsParams prm;
     prm.items = p.d_pair_items;
@@ -934,10 +1088,12 @@ int launch_ws(const clear_plan &p, const void *q, const void *k, const void *v, 
     prm.partial_o = p.d_partial_o;
     prm.partial_ml = p.d_partial_ml;
     prm.n_partial_slots = p.sch.n_partial_slots;
+    prm.q = static_cast<const __nv_bfloat16 *>(q);
+    prm.k = static_cast<const __nv_bfloat16 *>(k);
     prm.out = static_cast<__nv_bfloat16 *>(out);
     prm.status = p.d_status;
-    if (p.shape.head_dim == 128) return launch_variant<128>(p, tm, prm, stream);
-    if (p.shape.head_dim == 64) return launch_variant<64>(p, tm, prm, stream);
+    if (p.shape.head_dim == 128) return launch_variant<128>(p, maps, prm, stream);
+    if (p.shape.head_dim == 64) return launch_variant<64>(p, maps, prm, stream);
     return CLEAR_ERR_UNSUPPORTED;
 }
 

@@ -638,3 +638,15 @@ def test_window_grid_and_strided_masks_match_their_oracle(dtype, kind, a, b, gh,
         err = np.abs(out.cpu().to(torch.float64).numpy() - want)
         assert err.max() <= 1e-5, float(err.max())
     plan.destroy()
+
+
+@pytest.mark.parametrize("gh,gw,T,r,d", [(24, 40, 130, 8.0, 128), (19, 23, 0, 4.0, 64), (40, 24, 128, 6.0, 128)])
+def test_ws_kernel_scores_far_above_a_rows_reference(gh, gw, T, r, d):
+    """A few keys 60 times longer than the rest: scores hundreds of powers of two above a row's reference, in a tile
+    that is not its first, so that the tile is taken again from global memory."""
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, seed=3)
+    g = torch.Generator(device="cpu").manual_seed(1)
+    k[:, :, torch.randint(T, T + gh * gw, (40,), generator=g)] *= 60
+    scale = 4 / math.sqrt(d)
+    want = oracle.attn(q, k, v, gh, gw, T, r, scale)
+    assert_close_bf16(run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS), want, "far scores")
