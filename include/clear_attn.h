@@ -81,7 +81,7 @@ typedef struct clear_plan_info {
 
 /* One key/value tile of 128 keys that a work item visits. */
 typedef struct clear_kv_tile {
-    int32_t x;       /* image patch: grid column of its first key (may be negative or reach past  */
+    int32_t x;       /* image patch: grid column of its first key (its last ones may lie past     */
     int32_t y;       /*   the grid: such keys are masked); linear tile: x = first token, y = 0    */
     int32_t flags;   /* CLEAR_TILE_* bits                                                         */
     int32_t n_valid; /* linear tile: keys [0, n_valid) of the tile exist / are allowed            */
@@ -123,10 +123,11 @@ typedef struct clear_pair_step {
     int32_t flags;      /* CLEAR_STEP_* bits                                                        */
     int32_t n_valid0;   /* linear tiles: keys [0, n_valid) of the tile exist / are allowed; 2-D patches: */
     int32_t n_valid1;   /*   index of the tile pair's entry in the mask table, or -1 if it has none      */
-    int32_t load_base;  /* where this step's tiles sit in the item's staging order, which runs, for every
-                           step in turn, its K tiles and then its V tiles.  Low 16 bits: position of the
-                           step's first K tile; high 16 bits: position of its first V tile (a step with two
-                           distinct key tiles takes two consecutive positions each time, tile 0's first). */
+    int32_t load_base;  /* where this step's tiles sit among the tiles the item stages, counted for every step in
+                           turn, its K tiles and then its V tiles.  Low 16 bits: position of the step's first K
+                           tile; high 16 bits: position of its first V tile (a step with two distinct key tiles
+                           takes two consecutive positions each time, tile 0's first).  An item whose positions
+                           outgrow 16 bits is not built. */
 } clear_pair_step_t;
 
 /* One unit of work of the TCGEN05_WS kernel: two 128-query tiles walking one step list. */
@@ -353,9 +354,9 @@ int clear_plan_pair_tables(const clear_plan_t *plan, const clear_pair_item_t **i
                            const clear_pair_step_t **steps, int32_t *n_steps);
 
 /* Mask table of a TCGEN05_WS plan: Eq. 3 evaluated once per relative position of a key patch to a query
- * patch (the mask depends only on that offset).  Entry e is 128 rows (queries of the patch, row-major)
- * of four 32-bit words; bit j of word w tells whether key 32 w + j of the patch (row-major) lies within
- * the radius of that query.  Grid clipping is not part of it (CLEAR_STEP_CLIP*).  Errors: INVALID_ARG. */
+ * patch and number of the key patch's rows and columns on the grid (the mask depends on nothing else).  Entry e is
+ * 128 rows (queries of the patch, row-major) of four 32-bit words; bit j of word w tells whether key 32 w + j of the
+ * patch (row-major) exists and lies within the radius of that query.  Errors: INVALID_ARG. */
 int clear_plan_mask_table(const clear_plan_t *plan, const uint32_t **words, int32_t *n_entries);
 
 /* Forward pass with an explicit plan.  Tensor dtype is the plan's.  Calls on one plan share its

@@ -3,6 +3,7 @@
 #include "clear_plan.hpp"
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <climits>
 #include <cstdlib>
@@ -139,13 +140,75 @@ static bool window_allows(const Schedule &sch, int64_t dy, int64_t dx)
     return dy < (int64_t)sch.half_width.size() && dx <= sch.half_width[(size_t)dy];
 }
 
+// ---- key patches of an item ------------------------------------------------------------------------
+// Key patches need not lie on the lattice of the query patches: any 8 x 16 box of the grid can be staged.  So each axis
+// of an item gets the lattice offset with which its queries' windows take the fewest patches (the query patches' own
+// lattice where it is as good, which keeps the number of distinct masks small).  With a reach of 7 a 16-wide query patch
+// needs 30 columns: two patches instead of three; with a reach of 12 an 8-high one needs 32 rows: four instead of five.
+// `lo`, `hi` (n of them): the cells the item's query tiles reach on this axis; the first patch never starts off the grid.
+static int lattice_offset(const int *lo, const int *hi, int n, int step)
+{
+    int best = 0, best_count = 0;
+    for (int off = 0; off < step; ++off) {
+        int count = 0;
+        bool inside = true;
+        for (int i = 0; i < n; ++i) {
+            const int a = (lo[i] - off + step) / step, b = (hi[i] - off + step) / step;  // + step: never negative
+            count += b - a + 1;
+            inside = inside && (a - 1) * step + off >= 0;
+        }
+        if (off == 0 || (inside && count < best_count)) {
+            best = off;
+            best_count = count;
+        }
+    }
+    return best;
+}
+
+struct PatchTile {
+    int x, y;
+    bool masked;
+    bool clipped;  // part of the patch lies outside the grid
+};
+struct Reach {
+    int x_lo, x_hi, y_lo, y_hi;  // cells of the grid within reach of a query patch
+};
+static Reach reach_of(const Shape &s, const Schedule &sch, int qx, int qy)
+{
+    const int R = (int)sch.half_width.size() - 1, W = sch.half_width[0];
+    return Reach{std::max(0, qx - W), (int)std::min<int64_t>(s.grid_w - 1, (int64_t)qx + kTileW - 1 + W), std::max(0, qy - R),
+                 (int)std::min<int64_t>(s.grid_h - 1, (int64_t)qy + kTileH - 1 + R)};
+}
+
+// Key patches (on the lattice offset by off_x, off_y) that hold at least one key allowed to some query of the patch
+// at (qx, qy), each with the flag "some pair of the tile is not allowed".
+static std::vector<PatchTile> patches_of(const Shape &s, const Schedule &sch, int qx, int qy, int off_x, int off_y)
+{
+    const int gh = s.grid_h, gw = s.grid_w;
+    const int qx1 = std::min(qx + kTileW - 1, gw - 1), qy1 = std::min(qy + kTileH - 1, gh - 1);
+    const Reach reach = reach_of(s, sch, qx, qy);
+    std::vector<PatchTile> out;
+    for (int by = reach.y_lo - (reach.y_lo - off_y + kTileH) % kTileH; by <= reach.y_hi; by += kTileH) {
+        for (int bx = reach.x_lo - (reach.x_lo - off_x + kTileW) % kTileW; bx <= reach.x_hi; bx += kTileW) {
+            const int kx1 = std::min(bx + kTileW - 1, gw - 1), ky1 = std::min(by + kTileH - 1, gh - 1);
+            // smallest and largest coordinate differences between the two (clipped) patches
+            const int64_t gx = std::max({0, bx - qx1, qx - kx1});
+            const int64_t gy = std::max({0, by - qy1, qy - ky1});
+            if (!window_allows(sch, gy, gx)) continue;
+            const int64_t fx = std::max(kx1 - qx, qx1 - bx);
+            const int64_t fy = std::max(ky1 - qy, qy1 - by);
+            const bool whole = (bx + kTileW <= gw) && (by + kTileH <= gh);
+            out.push_back(PatchTile{bx, by, !(whole && window_allows(sch, fy, fx)), !whole});
+        }
+    }
+    return out;
+}
+
 void build_tile_schedule(const Shape &s, Schedule &sch)
 {
     build_geometry(s, sch);
     const int gh = s.grid_h, gw = s.grid_w, T = s.n_text;
     const int64_t N = (int64_t)gh * gw + T;
-    const int R = (int)sch.half_width.size() - 1;  // rows a window reaches up and down
-
     sch.items.clear();
     sch.tiles.clear();
 
@@ -185,7 +248,6 @@ void build_tile_schedule(const Shape &s, Schedule &sch)
 
     // ---- image-query patches: text tiles, then the key patches that meet the dilated patch -----
     const int ntx = (gw + kTileW - 1) / kTileW, nty = (gh + kTileH - 1) / kTileH;
-    const int reach_x = sch.half_width[0] / kTileW + 1, reach_y = R / kTileH + 1;
     for (int ty = 0; ty < nty; ++ty) {
         for (int tx = 0; tx < ntx; ++tx) {
             clear_work_item_t it{};
@@ -203,24 +265,15 @@ void build_tile_schedule(const Shape &s, Schedule &sch)
                 kt.flags = CLEAR_TILE_LINEAR | (kt.n_valid < kTileTokens ? CLEAR_TILE_MASKED : 0);
                 sch.tiles.push_back(kt);
             }
-            for (int j = std::max(0, ty - reach_y); j <= std::min(nty - 1, ty + reach_y); ++j) {
-                for (int i = std::max(0, tx - reach_x); i <= std::min(ntx - 1, tx + reach_x); ++i) {
-                    const int bx = i * kTileW, by = j * kTileH;
-                    const int kx1 = std::min(bx + kTileW - 1, gw - 1), ky1 = std::min(by + kTileH - 1, gh - 1);
-                    // smallest and largest coordinate differences between the two (clipped) patches
-                    const int64_t gx = std::max({0, bx - qx1, it.qx - kx1});
-                    const int64_t gy = std::max({0, by - qy1, it.qy - ky1});
-                    if (!window_allows(sch, gy, gx)) continue;
-                    const int64_t fx = std::max(kx1 - it.qx, qx1 - bx);
-                    const int64_t fy = std::max(ky1 - it.qy, qy1 - by);
-                    const bool whole = (bx + kTileW <= gw) && (by + kTileH <= gh);
-                    clear_kv_tile_t kt{};
-                    kt.x = bx;
-                    kt.y = by;
-                    kt.n_valid = kTileTokens;
-                    kt.flags = (whole && window_allows(sch, fy, fx)) ? 0 : CLEAR_TILE_MASKED;
-                    sch.tiles.push_back(kt);
-                }
+            const Reach reach = reach_of(s, sch, it.qx, it.qy);
+            const int off_x = lattice_offset(&reach.x_lo, &reach.x_hi, 1, kTileW), off_y = lattice_offset(&reach.y_lo, &reach.y_hi, 1, kTileH);
+            for (const PatchTile &pt : patches_of(s, sch, it.qx, it.qy, off_x, off_y)) {
+                clear_kv_tile_t kt{};
+                kt.x = pt.x;
+                kt.y = pt.y;
+                kt.n_valid = kTileTokens;
+                kt.flags = pt.masked ? CLEAR_TILE_MASKED : 0;
+                sch.tiles.push_back(kt);
             }
             it.tile_count = (int32_t)sch.tiles.size() - it.tile_begin;
             it.partial_slot = -1;
@@ -242,42 +295,6 @@ void build_tile_schedule(const Shape &s, Schedule &sch)
 }
 
 // ---- pair schedule of the warp-specialised kernel ------------------------------------------------
-namespace {
-
-struct PatchTile {
-    int x, y;
-    bool masked;
-    bool clipped;  // part of the patch lies outside the grid
-};
-
-// Key patches (on the 8 x 16 lattice) that hold at least one key allowed to some query of the patch
-// at (qx, qy), each with the flag "some pair of the tile is not allowed".
-std::vector<PatchTile> patches_of(const Shape &s, const Schedule &sch, int R, int qx, int qy)
-{
-    const int gh = s.grid_h, gw = s.grid_w;
-    const int ntx = (gw + kTileW - 1) / kTileW, nty = (gh + kTileH - 1) / kTileH;
-    const int tx = qx / kTileW, ty = qy / kTileH;
-    const int reach_x = sch.half_width[0] / kTileW + 1, reach_y = R / kTileH + 1;
-    const int qx1 = std::min(qx + kTileW - 1, gw - 1), qy1 = std::min(qy + kTileH - 1, gh - 1);
-    std::vector<PatchTile> out;
-    for (int j = std::max(0, ty - reach_y); j <= std::min(nty - 1, ty + reach_y); ++j) {
-        for (int i = std::max(0, tx - reach_x); i <= std::min(ntx - 1, tx + reach_x); ++i) {
-            const int bx = i * kTileW, by = j * kTileH;
-            const int kx1 = std::min(bx + kTileW - 1, gw - 1), ky1 = std::min(by + kTileH - 1, gh - 1);
-            const int64_t gx = std::max({0, bx - qx1, qx - kx1});
-            const int64_t gy = std::max({0, by - qy1, qy - ky1});
-            if (!window_allows(sch, gy, gx)) continue;
-            const int64_t fx = std::max(kx1 - qx, qx1 - bx);
-            const int64_t fy = std::max(ky1 - qy, qy1 - by);
-            const bool whole = (bx + kTileW <= gw) && (by + kTileH <= gh);
-            out.push_back(PatchTile{bx, by, !(whole && window_allows(sch, fy, fx)), !whole});
-        }
-    }
-    return out;
-}
-
-}  // namespace
-
 void build_pair_schedule(const Shape &s, Schedule &sch)
 {
     build_geometry(s, sch);
@@ -306,25 +323,28 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
     sch.mask_table.clear();
     sch.pair_overflow = false;
 
-    // Eq. 3 for a key patch at offset (dy, dx) from a query patch, once per distinct offset
+    // Eq. 3 for a key patch at offset (dy, dx) from a query patch of which rows x cols keys are on the grid, once per
+    // distinct case
     // (CLEAR_MAX_MASK_ENTRIES lowers the cap of the table; with 0 every masked patch takes the kernel's
     // table-free path, which is otherwise reached only by very large radii)
     int max_entries = kMaxMaskEntries;
     if (const char *e = std::getenv("CLEAR_MAX_MASK_ENTRIES")) max_entries = std::max(0, std::min(kMaxMaskEntries, std::atoi(e)));
-    std::map<std::pair<int, int>, int> mask_ids;
-    auto mask_entry = [&](int dy, int dx) -> int {
-        auto it = mask_ids.find({dy, dx});
+    std::map<std::array<int, 4>, int> mask_ids;
+    auto mask_entry = [&](const PatchTile &pt, int qy0, int qx0) -> int {
+        const int dy = pt.y - qy0, dx = pt.x - qx0, rows = std::min(kTileH, gh - pt.y), cols = std::min(kTileW, gw - pt.x);
+        const std::array<int, 4> key{dy, dx, rows, cols};
+        auto it = mask_ids.find(key);
         if (it != mask_ids.end()) return it->second;
         if ((int)mask_ids.size() >= max_entries) return -1;
         const int id = (int)mask_ids.size();
-        mask_ids[{dy, dx}] = id;
+        mask_ids[key] = id;
         sch.mask_table.resize((size_t)(id + 1) * kTileTokens * 4, 0u);
         uint32_t *e = sch.mask_table.data() + (size_t)id * kTileTokens * 4;
         for (int r = 0; r < kTileTokens; ++r) {
             const int qy = r / kTileW, qx = r % kTileW;
             for (int j = 0; j < kTileTokens; ++j) {
                 const int64_t ddy = dy + j / kTileW - qy, ddx = dx + j % kTileW - qx;
-                if (window_allows(sch, ddy, ddx)) e[r * 4 + (j >> 5)] |= 1u << (j & 31);
+                if (j / kTileW < rows && j % kTileW < cols && window_allows(sch, ddy, ddx)) e[r * 4 + (j >> 5)] |= 1u << (j & 31);
             }
         }
         return id;
@@ -436,8 +456,11 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
             // text keys: tokens past n_text in the last tile are image keys, not allowed through it
             for (int t0 = 0; t0 < T; t0 += kTileTokens) linear_step(t0, std::min(kTileTokens, T - t0), it.n_sides);
 
-            std::vector<PatchTile> a = patches_of(s, sch, R, it.qx, it.qy0), b;
-            if (it.n_sides == 2) b = patches_of(s, sch, R, it.qx, it.qy1);
+            const Reach r0 = reach_of(s, sch, it.qx, it.qy0), r1 = reach_of(s, sch, it.qx, it.n_sides == 2 ? it.qy1 : it.qy0);
+            const int y_lo[2] = {r0.y_lo, r1.y_lo}, y_hi[2] = {r0.y_hi, r1.y_hi};
+            const int off_x = lattice_offset(&r0.x_lo, &r0.x_hi, 1, kTileW), off_y = lattice_offset(y_lo, y_hi, it.n_sides, kTileH);
+            std::vector<PatchTile> a = patches_of(s, sch, it.qx, it.qy0, off_x, off_y), b;
+            if (it.n_sides == 2) b = patches_of(s, sch, it.qx, it.qy1, off_x, off_y);
             auto find = [](const std::vector<PatchTile> &v, const PatchTile &t) -> const PatchTile * {
                 for (const PatchTile &u : v)
                     if (u.x == t.x && u.y == t.y) return &u;
@@ -454,9 +477,10 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
             }
             for (const PatchTile &t : b)
                 if (!find(a, t)) only_b.push_back(t);
-            // key patches only one tile needs are taken two at a time, one per tile, so that both
-            // tiles stay busy; what is left over runs one-sided
-            for (size_t i = 0; i < std::max(only_a.size(), only_b.size()); ++i) {
+            // Key patches only one tile needs are taken two at a time, one per tile, so that both tiles stay busy; what
+            // is left over runs one-sided.  Such a step stages twice the tiles of a shared one, so these steps are
+            // spread evenly between the shared ones: in a row, they would outrun the copies behind the staging ring.
+            auto own_step = [&](size_t i) {
                 clear_pair_step_t st{};
                 st.n_valid0 = st.n_valid1 = kTileTokens;
                 if (i < only_a.size()) {
@@ -464,29 +488,35 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
                     st.y0 = only_a[i].y;
                     st.flags |= CLEAR_STEP_USE0 | (only_a[i].masked ? CLEAR_STEP_MASKED0 : 0) |
                                 (only_a[i].clipped ? CLEAR_STEP_CLIP0 : 0);
-                    st.n_valid0 = only_a[i].masked ? mask_entry(st.y0 - it.qy0, st.x0 - it.qx) : -1;
+                    st.n_valid0 = only_a[i].masked ? mask_entry(only_a[i], it.qy0, it.qx) : -1;
                 }
                 if (i < only_b.size()) {
                     st.x1 = only_b[i].x;
                     st.y1 = only_b[i].y;
                     st.flags |= CLEAR_STEP_USE1 | (only_b[i].masked ? CLEAR_STEP_MASKED1 : 0) |
                                 (only_b[i].clipped ? CLEAR_STEP_CLIP1 : 0);
-                    st.n_valid1 = only_b[i].masked ? mask_entry(st.y1 - it.qy1, st.x1 - it.qx) : -1;
+                    st.n_valid1 = only_b[i].masked ? mask_entry(only_b[i], it.qy1, it.qx) : -1;
                 }
                 sch.pair_steps.push_back(st);
-            }
-            for (const auto &ab : both) {
+            };
+            auto shared_step = [&](const std::pair<PatchTile, PatchTile> &ab) {
                 clear_pair_step_t st{};
-                st.n_valid0 = st.n_valid1 = kTileTokens;
                 st.x0 = st.x1 = ab.first.x;
                 st.y0 = st.y1 = ab.first.y;
                 st.flags = CLEAR_STEP_USE0 | CLEAR_STEP_USE1 | CLEAR_STEP_SHARED |
                            (ab.first.masked ? CLEAR_STEP_MASKED0 : 0) | (ab.second.masked ? CLEAR_STEP_MASKED1 : 0) |
                            (ab.first.clipped ? (CLEAR_STEP_CLIP0 | CLEAR_STEP_CLIP1) : 0);
-                st.n_valid0 = ab.first.masked ? mask_entry(st.y0 - it.qy0, st.x0 - it.qx) : -1;
-                st.n_valid1 = ab.second.masked ? mask_entry(st.y1 - it.qy1, st.x1 - it.qx) : -1;
+                st.n_valid0 = ab.first.masked ? mask_entry(ab.first, it.qy0, it.qx) : -1;
+                st.n_valid1 = ab.second.masked ? mask_entry(ab.second, it.qy1, it.qx) : -1;
                 sch.pair_steps.push_back(st);
+            };
+            const size_t n_own = std::max(only_a.size(), only_b.size());
+            size_t own = 0;
+            for (size_t i = 0; i < both.size(); ++i) {
+                for (; own < n_own && (own + 1) * both.size() <= i * (n_own + 1); ++own) own_step(own);
+                shared_step(both[i]);
             }
+            for (; own < n_own; ++own) own_step(own);
             finish_item(it);
             // a list too long for the step records' 16-bit ring positions: this kernel cannot run the
             // shape, and the remaining lists (gigabytes at such radii) are not worth building

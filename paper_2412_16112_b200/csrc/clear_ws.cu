@@ -52,7 +52,7 @@ struct WsParams {
     const clear_pair_item_t *items;
     const clear_pair_step_t *steps;
     const int32_t *half_width;
-    const uint32_t *mask_table;  // [entry][128 query rows][4 words]: Eq. 3 per relative patch offset
+    const uint32_t *mask_table;  // [entry][128 query rows][4 words]: Eq. 3 per relative patch offset and border case
     int n_half_width;
     int grid_h, grid_w, n_text;
     long long n_tokens;
@@ -171,7 +171,7 @@ __device__ __forceinline__ clear_pair_item_t load_item(const clear_pair_item_t *
     it.step_count = c.x; it.n_loads = c.y; it.partial_slot0 = c.z; it.partial_slot1 = c.w;
     return it;
 }
-// Origin of the key patch of that tile (only clipped patches and plans without a mask table need it).
+// Origin of the key patch of that tile (only plans without a mask table and recomputed tiles need it).
 __device__ __forceinline__ int2 load_side_origin(const clear_pair_step_t *p, int side)
 {
     const int4 a = __ldg(reinterpret_cast<const int4 *>(p));
@@ -825,23 +825,11 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                             mw[w] = nv == 32 ? 0xffffffffu : ((1u << nv) - 1u);
                         }
                     } else if (st.n_valid >= 0) {
-                        // Eq. 3 from the table; keys of the patch that lie off the grid do not exist
+                        // Eq. 3 from the table, the grid's border included
                         mw[0] = mrow.x;
                         mw[1] = mrow.y;
                         mw[2] = mrow.z;
                         mw[3] = mrow.w;
-                        if (st.flags & (t ? CLEAR_STEP_CLIP1 : CLEAR_STEP_CLIP0)) {
-                            const int2 org = load_side_origin(steps + s, t);
-                            const int lo = max(0, -org.x), hi = min(15, prm.grid_w - 1 - org.x);
-                            const uint32_t cols = lo <= hi ? (((1u << (hi - lo + 1)) - 1u) << lo) : 0u;
-#pragma unroll
-                            for (int w = 0; w < 4; ++w) {
-                                const int ky0 = org.y + 2 * w, ky1 = ky0 + 1;
-                                const uint32_t ok0 = (ky0 >= 0 && ky0 < prm.grid_h) ? cols : 0u;
-                                const uint32_t ok1 = (ky1 >= 0 && ky1 < prm.grid_h) ? cols : 0u;
-                                mw[w] &= ok0 | (ok1 << 16);
-                            }
-                        }
                     } else {
                         // no table entry (very large radius): Eq. 3 row by row from the half widths
                         const int2 org = load_side_origin(steps + s, t);

@@ -650,3 +650,12 @@ def test_ws_kernel_scores_far_above_a_rows_reference(gh, gw, T, r, d):
     scale = 4 / math.sqrt(d)
     want = oracle.attn(q, k, v, gh, gw, T, r, scale)
     assert_close_bf16(run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS), want, "far scores")
+
+
+@pytest.mark.parametrize("kernel", TC_KERNELS, ids=TC_IDS)
+@pytest.mark.parametrize("gh,gw,T,r,d", [(45, 70, 17, 12.5, 64), (40, 67, 3, 4.5, 128), (31, 33, 0, 7.5, 64)])
+def test_tc_kernels_with_key_patches_off_the_query_lattice(gh, gw, T, r, d, kernel):
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, seed=gh * 100 + gw)
+    scale = 1 / math.sqrt(d)
+    want = oracle.attn(q, k, v, gh, gw, T, r, scale)
+    assert_close_bf16(run_plan(q, k, v, gh, gw, T, r, scale, kernel), want, "shifted key patches")

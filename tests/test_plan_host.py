@@ -477,3 +477,18 @@ def test_comparison_mask_plans_reject_bad_arguments():
     # the tensor-core kernels' tables do not carry these masks
     with pytest.raises(clear.ClearError):
         clear.Plan(1, 1, 8, 8, 2, 128, 4, kernel=clear.KERNEL_TCGEN05_WS, host_only=True, mask_kind=clear.MASK_WINDOWS)
+
+
+@pytest.mark.parametrize("gh,gw,T,r,interior", [
+    (48, 64, 0, 8.0, 6),      # reach 7: 30 columns in two patches, 22 rows in three
+    (45, 70, 17, 12.5, 12),   # reach 12: 32 rows in four; ragged grid
+    (40, 67, 3, 4.5, 4),      # reach 4: 16 rows in two, 24 columns in two
+    (48, 64, 0, 16.0, 15),    # reach 15: the query patches' own lattice is as good
+])
+def test_key_patches_take_the_lattice_offset_with_the_fewest(gh, gw, T, r, interior):
+    test_tile_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r)
+    test_pair_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r)
+    p = clear.Plan(1, 1, gh, gw, T, 128, r, kernel=clear.KERNEL_TCGEN05, host_only=True)
+    items, _, _ = p.tables()
+    longest = max(it.tile_count for it in items if it.kind == 0)
+    assert longest - math.ceil(T / 128) == interior
