@@ -370,7 +370,7 @@ int clear_attn_fwd_planned(const clear_plan_t *plan, const void *q, const void *
 /* Forward pass on HOST tensors (same layout and dtype as the plan's): copies q, k, v to staging
  * buffers the plan owns (allocated on first use), runs the kernels, copies `out` back, and returns
  * after synchronising `stream`.  A problem of more than one chunk (a chunk = whole (b, h) slices of
- * at least 96 MiB per tensor, at most 16 chunks; the environment variable CLEAR_HOST_CHUNK_BYTES,
+ * at least 4 MiB per tensor, at most 16 chunks; the environment variable CLEAR_HOST_CHUNK_BYTES,
  * read at the plan's first call, changes the size) runs as a three-stage pipeline: the copies in,
  * the kernels (on `stream`, with a plan per chunk size that this plan owns) and the copies out each
  * work on a different chunk, on two extra streams the plan creates, so both PCIe directions and
