@@ -104,7 +104,14 @@ int create_plan(clear_plan_t **out, const Shape &shape_in, bool host_only)
                 p->sch = Schedule();
             }
         }
-        if (kernel == CLEAR_KERNEL_TCGEN05)
+        if (s.backward) {
+            build_backward_schedule(s, p->sch);
+            if (p->sch.pair_overflow) {  // lists too long for the forward kernel: the CUDA-core backward pass
+                kernel = CLEAR_KERNEL_SIMT;
+                p->sch = Schedule();
+            }
+        }
+        if (kernel == CLEAR_KERNEL_TCGEN05 && !s.backward)
             build_tile_schedule(s, p->sch);
         else if (kernel == CLEAR_KERNEL_SIMT)
             build_geometry(s, p->sch);
@@ -359,7 +366,7 @@ static int backward(const void *q, const void *k, const void *v, const void *d_o
                     void *stream, bool tensor_cores = false)
 {
     Shape s{B, H, grid_h, grid_w, n_text, head_dim, radius, dtype, tensor_cores ? CLEAR_KERNEL_TCGEN05 : CLEAR_KERNEL_SIMT};
-    s.no_text_split = tensor_cores ? 1 : 0;
+    s.backward = tensor_cores ? 1 : 0;
     int rc = validate_shape(s);
     if (rc != CLEAR_OK) return rc;
     if (!std::isfinite(scale)) return CLEAR_ERR_INVALID_ARG;
@@ -371,7 +378,7 @@ static int backward(const void *q, const void *k, const void *v, const void *d_o
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         std::lock_guard<std::mutex> lock(plan->launch_mutex);
         if (plan->has_last && plan->last_stream != st) CLEAR_CUDA_TRY(cudaStreamWaitEvent(st, plan->ev_last, 0));
-        const int rc2 = tensor_cores ? launch_bwd_tc(*plan, q, k, v, d_out, dq, dk, dv, scale, st)
+        const int rc2 = plan->kernel != CLEAR_KERNEL_SIMT ? launch_bwd_tc(*plan, q, k, v, d_out, dq, dk, dv, scale, st)
                                      : launch_bwd(*plan, q, k, v, d_out, dq, dk, dv, scale, st);
         if (rc2 != CLEAR_OK) return rc2;
         CLEAR_CUDA_TRY(cudaEventRecord(plan->ev_last, st));

@@ -204,7 +204,47 @@ static std::vector<PatchTile> patches_of(const Shape &s, const Schedule &sch, in
     return out;
 }
 
-void build_tile_schedule(const Shape &s, Schedule &sch)
+// Eq. 3 for a key patch at offset (dy, dx) from a query patch of which rows x cols keys are on the grid, once per
+// distinct case (CLEAR_MAX_MASK_ENTRIES lowers the cap of the table; with 0 every masked patch takes the kernels'
+// table-free path, which is otherwise reached only by very large radii).
+class MaskTable {
+public:
+    MaskTable(const Shape &s, Schedule &sch) : s_(s), sch_(sch)
+    {
+        sch.mask_table.clear();
+        if (const char *e = std::getenv("CLEAR_MAX_MASK_ENTRIES")) max_entries_ = std::max(0, std::min(kMaxMaskEntries, std::atoi(e)));
+    }
+    // Index of the entry, -1 when the table is full.
+    int entry(const PatchTile &pt, int qy0, int qx0)
+    {
+        const int dy = pt.y - qy0, dx = pt.x - qx0, rows = std::min(kTileH, s_.grid_h - pt.y), cols = std::min(kTileW, s_.grid_w - pt.x);
+        const std::array<int, 4> key{dy, dx, rows, cols};
+        auto it = ids_.find(key);
+        if (it != ids_.end()) return it->second;
+        if ((int)ids_.size() >= max_entries_) return -1;
+        const int id = (int)ids_.size();
+        ids_[key] = id;
+        sch_.mask_table.resize((size_t)(id + 1) * kTileTokens * 4, 0u);
+        uint32_t *e = sch_.mask_table.data() + (size_t)id * kTileTokens * 4;
+        for (int r = 0; r < kTileTokens; ++r) {
+            const int qy = r / kTileW, qx = r % kTileW;
+            for (int j = 0; j < kTileTokens; ++j) {
+                const int64_t ddy = dy + j / kTileW - qy, ddx = dx + j % kTileW - qx;
+                if (j / kTileW < rows && j % kTileW < cols && window_allows(sch_, ddy, ddx)) e[r * 4 + (j >> 5)] |= 1u << (j & 31);
+            }
+        }
+        return id;
+    }
+
+private:
+    const Shape &s_;
+    Schedule &sch_;
+    int max_entries_ = kMaxMaskEntries;
+    std::map<std::array<int, 4>, int> ids_;
+};
+
+// With a mask table, the masked image tiles name their entry in n_valid (the tile kernel evaluates Eq. 3 itself).
+static void build_tiles(const Shape &s, Schedule &sch, MaskTable *masks)
 {
     build_geometry(s, sch);
     const int gh = s.grid_h, gw = s.grid_w, T = s.n_text;
@@ -216,7 +256,7 @@ void build_tile_schedule(const Shape &s, Schedule &sch)
     const int n_lin = (int)((N + kTileTokens - 1) / kTileTokens);
     sch.n_text_tiles = (T + kTileTokens - 1) / kTileTokens;
     int chunk = n_lin, n_splits = 1;
-    if (sch.n_text_tiles > 0 && !s.no_text_split) {
+    if (sch.n_text_tiles > 0 && !s.backward) {
         n_splits = (n_lin + kSplitTargetTiles - 1) / kSplitTargetTiles;
         chunk = (n_lin + n_splits - 1) / n_splits;
         n_splits = (n_lin + chunk - 1) / chunk;
@@ -271,7 +311,7 @@ void build_tile_schedule(const Shape &s, Schedule &sch)
                 clear_kv_tile_t kt{};
                 kt.x = pt.x;
                 kt.y = pt.y;
-                kt.n_valid = kTileTokens;
+                kt.n_valid = masks && pt.masked ? masks->entry(pt, it.qy, it.qx) : kTileTokens;
                 kt.flags = pt.masked ? CLEAR_TILE_MASKED : 0;
                 sch.tiles.push_back(kt);
             }
@@ -295,7 +335,7 @@ void build_tile_schedule(const Shape &s, Schedule &sch)
 }
 
 // ---- pair schedule of the warp-specialised kernel ------------------------------------------------
-void build_pair_schedule(const Shape &s, Schedule &sch)
+static void build_pairs(const Shape &s, Schedule &sch, MaskTable &masks)
 {
     build_geometry(s, sch);
     const int gh = s.grid_h, gw = s.grid_w, T = s.n_text;
@@ -320,35 +360,7 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
 
     sch.pair_items.clear();
     sch.pair_steps.clear();
-    sch.mask_table.clear();
     sch.pair_overflow = false;
-
-    // Eq. 3 for a key patch at offset (dy, dx) from a query patch of which rows x cols keys are on the grid, once per
-    // distinct case
-    // (CLEAR_MAX_MASK_ENTRIES lowers the cap of the table; with 0 every masked patch takes the kernel's
-    // table-free path, which is otherwise reached only by very large radii)
-    int max_entries = kMaxMaskEntries;
-    if (const char *e = std::getenv("CLEAR_MAX_MASK_ENTRIES")) max_entries = std::max(0, std::min(kMaxMaskEntries, std::atoi(e)));
-    std::map<std::array<int, 4>, int> mask_ids;
-    auto mask_entry = [&](const PatchTile &pt, int qy0, int qx0) -> int {
-        const int dy = pt.y - qy0, dx = pt.x - qx0, rows = std::min(kTileH, gh - pt.y), cols = std::min(kTileW, gw - pt.x);
-        const std::array<int, 4> key{dy, dx, rows, cols};
-        auto it = mask_ids.find(key);
-        if (it != mask_ids.end()) return it->second;
-        if ((int)mask_ids.size() >= max_entries) return -1;
-        const int id = (int)mask_ids.size();
-        mask_ids[key] = id;
-        sch.mask_table.resize((size_t)(id + 1) * kTileTokens * 4, 0u);
-        uint32_t *e = sch.mask_table.data() + (size_t)id * kTileTokens * 4;
-        for (int r = 0; r < kTileTokens; ++r) {
-            const int qy = r / kTileW, qx = r % kTileW;
-            for (int j = 0; j < kTileTokens; ++j) {
-                const int64_t ddy = dy + j / kTileW - qy, ddx = dx + j % kTileW - qx;
-                if (j / kTileW < rows && j % kTileW < cols && window_allows(sch, ddy, ddx)) e[r * 4 + (j >> 5)] |= 1u << (j & 31);
-            }
-        }
-        return id;
-    };
 
     auto finish_item = [&](clear_pair_item_t &it) {
         // staging order: for every step its K tiles, then its V tiles (the order the MMAs read them in)
@@ -488,14 +500,14 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
                     st.y0 = only_a[i].y;
                     st.flags |= CLEAR_STEP_USE0 | (only_a[i].masked ? CLEAR_STEP_MASKED0 : 0) |
                                 (only_a[i].clipped ? CLEAR_STEP_CLIP0 : 0);
-                    st.n_valid0 = only_a[i].masked ? mask_entry(only_a[i], it.qy0, it.qx) : -1;
+                    st.n_valid0 = only_a[i].masked ? masks.entry(only_a[i], it.qy0, it.qx) : -1;
                 }
                 if (i < only_b.size()) {
                     st.x1 = only_b[i].x;
                     st.y1 = only_b[i].y;
                     st.flags |= CLEAR_STEP_USE1 | (only_b[i].masked ? CLEAR_STEP_MASKED1 : 0) |
                                 (only_b[i].clipped ? CLEAR_STEP_CLIP1 : 0);
-                    st.n_valid1 = only_b[i].masked ? mask_entry(only_b[i], it.qy1, it.qx) : -1;
+                    st.n_valid1 = only_b[i].masked ? masks.entry(only_b[i], it.qy1, it.qx) : -1;
                 }
                 sch.pair_steps.push_back(st);
             };
@@ -506,8 +518,8 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
                 st.flags = CLEAR_STEP_USE0 | CLEAR_STEP_USE1 | CLEAR_STEP_SHARED |
                            (ab.first.masked ? CLEAR_STEP_MASKED0 : 0) | (ab.second.masked ? CLEAR_STEP_MASKED1 : 0) |
                            (ab.first.clipped ? (CLEAR_STEP_CLIP0 | CLEAR_STEP_CLIP1) : 0);
-                st.n_valid0 = ab.first.masked ? mask_entry(ab.first, it.qy0, it.qx) : -1;
-                st.n_valid1 = ab.second.masked ? mask_entry(ab.second, it.qy1, it.qx) : -1;
+                st.n_valid0 = ab.first.masked ? masks.entry(ab.first, it.qy0, it.qx) : -1;
+                st.n_valid1 = ab.second.masked ? masks.entry(ab.second, it.qy1, it.qx) : -1;
                 sch.pair_steps.push_back(st);
             };
             const size_t n_own = std::max(only_a.size(), only_b.size());
@@ -539,6 +551,26 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
             sch.executed_pairs += (int64_t)uses * kTileTokens * kTileTokens;
         }
     }
+}
+
+void build_tile_schedule(const Shape &s, Schedule &sch) { build_tiles(s, sch, nullptr); }
+
+void build_pair_schedule(const Shape &s, Schedule &sch)
+{
+    MaskTable masks(s, sch);
+    build_pairs(s, sch, masks);
+}
+
+void build_backward_schedule(const Shape &s, Schedule &sch)
+{
+    MaskTable masks(s, sch);
+    build_pairs(s, sch, masks);
+    if (sch.pair_overflow) return;
+    // text splits, and the workspace they need, are the pair schedule's
+    const int n_text_splits = sch.n_text_splits, n_partial_slots = sch.n_partial_slots;
+    build_tiles(s, sch, &masks);
+    sch.n_text_splits = n_text_splits;
+    sch.n_partial_slots = n_partial_slots;
 }
 
 }  // namespace clear
