@@ -211,36 +211,33 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 }
             }
         } else if (warp == 1) {
-            // ================= every MMA: the whole warp walks the loop, one elected lane issues ====================
-            bool ok = true;
-            auto wait_lane = [&](uint32_t bar, uint32_t parity, int code) {
-                if (ok) ok = bwd_wait(bar, parity, abort_flag, prm.status, code);
-            };
-            auto ok_all = [&]() { return ok = __all_sync(0xffffffffu, ok); };
-            wait_lane(b_a, 0, 2);
-            const uint32_t a_lo0 = ptx::smem_desc_lo(sA, 16), bk_lo0 = ptx::smem_desc_lo(sB, 16), bm_lo0 = ptx::smem_desc_lo(sB, kHalfBytes);
-            constexpr uint32_t kTile16 = kTileBytes >> 4;
-            // stages of the streamed pair that the products use next, and of the one the accumulations use
-            uint32_t t_st[2] = {0, 0}, t_par = 0, next = 0, acc_st[2] = {0, 0};
-            // T1, T2 of a half: D / 16 MMAs of 16 channels each; the second half's tokens are 64 rows, 8192 bytes, further
-            auto issue_t = [&](int half) {
-                if (half == 0) {
+            // ================= every MMA, all from one lane ==========================================================
+            // The pipe takes about two MMAs ahead, so what this lane does between an accumulation and the next products
+            // is time that the pipe stands idle, and beside 16 busy row warps every instruction of it is slow. So nothing
+            // stands there: the loop goes by tiles with both halves written out, one lane walks it without votes, and the
+            // waits sit behind products that are still running.
+            if (ptx::elect_one()) {
+                bool ok = bwd_wait(b_a, 0, abort_flag, prm.status, 2);
+                const uint32_t a_lo0 = ptx::smem_desc_lo(sA, 16), bk_lo0 = ptx::smem_desc_lo(sB, 16), bm_lo0 = ptx::smem_desc_lo(sB, kHalfBytes);
+                constexpr uint32_t kTile16 = kTileBytes >> 4;
+                uint32_t next = 0, next_par = 0;
+                // the next pair of streamed tiles: their offsets in the ring, in descriptor units
+                auto wait_pair = [&](uint32_t (&st)[2]) {
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        wait_lane(b_full0 + 8 * next, t_par, 3);
-                        t_st[j] = next;
+                        st[j] = next;
+                        ok = ok && bwd_wait(b_full0 + 8 * next, next_par, abort_flag, prm.status, 3);
                         if (++next == kBwdStages) {
                             next = 0;
-                            t_par ^= 1u;
+                            next_par ^= 1u;
                         }
                     }
-                }
-                if (!ok_all()) return;
-                ptx::tc_fence_after();
-                if (ptx::elect_one()) {
+                };
+                // T1, T2 of a half: D / 16 MMAs of 16 channels each; the second half's tokens are 64 rows, 8192 bytes, further
+                auto issue_t = [&](const uint32_t (&st)[2], int half) {
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        const uint32_t d = tmem + half * 128 + j * 64, a = a_lo0 + j * kTile16, b = bk_lo0 + t_st[j] * kTile16 + half * (8192 >> 4);
+                        const uint32_t d = tmem + half * 128 + j * 64, a = a_lo0 + j * kTile16, b = bk_lo0 + st[j] * kTile16 + half * (8192 >> 4);
                         ptx::mma_ss_c<false>(d, ptx::make_desc(a, kDescHi), ptx::make_desc(b, kDescHi), kIdescT);
 #pragma unroll
                         for (int kk = 1; kk < D / 16; ++kk) {
@@ -249,49 +246,56 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                         }
                     }
                     ptx::tc_commit(ptx::smem_u32(&ctrl->t_full[half]));
-                }
-                __syncwarp();
-            };
-            issue_t(0);
-            ok_all();
-#pragma unroll 1
-            for (int h = 0; h < 2 * n_tiles && ok; ++h) {
-                const int half = h & 1;
-                if (half == 0) {
-                    acc_st[0] = t_st[0];
-                    acc_st[1] = t_st[1];
-                }
-                if (h + 1 < 2 * n_tiles) issue_t(half ^ 1);
-                // the rows have read T1, T2 of this half and put P / dS over them
-                wait_lane(ptx::smem_u32(&ctrl->p_ready[half]), (uint32_t)(h >> 1) & 1u, 4);
-                if (!ok_all()) break;
-                ptx::tc_fence_after();
-                if (ptx::elect_one()) {
-                    // 4 MMAs over 16 streamed tokens each (16 rows of 128 bytes = 2048 bytes), B read MN-major; the bf16
-                    // columns of the two row groups start at the groups' own fp32 columns
+                };
+                // 4 MMAs over 16 streamed tokens each (16 rows of 128 bytes = 2048 bytes), B read MN-major; the bf16 columns
+                // of the two row groups start at the groups' own fp32 columns
+                auto issue_acc = [&](const uint32_t (&st)[2], int half, uint32_t before) {
                     const uint32_t p1 = tmem + half * 128, p2 = p1 + 64;
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
-                        const uint32_t acc = (h > 0 || kk > 0) ? 1u : 0u, col = (kk >> 1) * 32 + (kk & 1) * 8, off = half * (8192 >> 4) + kk * (2048 >> 4);
+                        const uint32_t acc = kk > 0 ? 1u : before, col = (kk >> 1) * 32 + (kk & 1) * 8, off = half * (8192 >> 4) + kk * (2048 >> 4);
                         if (KEY_ROLE) {
-                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + acc_st[1] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dV += P^T dO
-                            ptx::mma_ts(tmem_A2, p2 + col, ptx::make_desc(bm_lo0 + acc_st[0] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dK += dS^T Q
+                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + st[1] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dV += P^T dO
+                            ptx::mma_ts(tmem_A2, p2 + col, ptx::make_desc(bm_lo0 + st[0] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dK += dS^T Q
                         } else {
-                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + acc_st[0] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dQ += dS K
+                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + st[0] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dQ += dS K
                         }
                     }
-                    if (half == 1) {
-                        ptx::tc_commit(b_empty0 + 8 * acc_st[0]);
-                        ptx::tc_commit(b_empty0 + 8 * acc_st[1]);
-                    }
-                    if (h == 2 * n_tiles - 1) ptx::tc_commit(b_acc);
+                };
+                const uint32_t b_p0 = ptx::smem_u32(&ctrl->p_ready[0]), b_p1 = ptx::smem_u32(&ctrl->p_ready[1]);
+                uint32_t st[2], st_next[2] = {0, 0};
+                wait_pair(st);
+                if (ok) {
+                    ptx::tc_fence_after();
+                    issue_t(st, 0);
                 }
-                __syncwarp();
-            }
-            if (*abort_flag && lane == 0) {
-                // MMAs that were issued must retire before tensor memory is given back
-                ptx::tc_commit(ptx::smem_u32(&ctrl->drain));
-                bwd_drain(ptx::smem_u32(&ctrl->drain), 0);
+#pragma unroll 1
+                for (int i = 0; i < n_tiles && ok; ++i) {
+                    const uint32_t par = (uint32_t)i & 1u;
+                    issue_t(st, 1);
+                    const bool more = i + 1 < n_tiles;
+                    if (more) wait_pair(st_next);
+                    // the rows have read T1, T2 of a half and put P / dS over them
+                    ok = ok && bwd_wait(b_p0, par, abort_flag, prm.status, 4);
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    issue_acc(st, 0, i > 0 ? 1u : 0u);
+                    if (more) issue_t(st_next, 0);
+                    ok = bwd_wait(b_p1, par, abort_flag, prm.status, 4);
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    issue_acc(st, 1, 1u);
+                    ptx::tc_commit(b_empty0 + 8 * st[0]);
+                    ptx::tc_commit(b_empty0 + 8 * st[1]);
+                    if (!more) ptx::tc_commit(b_acc);
+                    st[0] = st_next[0];
+                    st[1] = st_next[1];
+                }
+                if (*abort_flag) {
+                    // MMAs that were issued must retire before tensor memory is given back
+                    ptx::tc_commit(ptx::smem_u32(&ctrl->drain));
+                    bwd_drain(ptx::smem_u32(&ctrl->drain), 0);
+                }
             }
         } else if (warp == 2 && KEY_ROLE) {
             // ================= statistics of the streamed tiles' columns, ahead of the row warps =====================
