@@ -35,7 +35,10 @@ namespace {
 constexpr int kRowWarps = 16;
 constexpr int kBwdThreads = 128 + 32 * kRowWarps;
 constexpr uint32_t kBwdTmemCols = 512;   // two buffers of T1 | T2 (64 columns each), ACC1, ACC2 (128 each)
-constexpr uint32_t kBwdStages = 5;       // ring of streamed tiles, one of the pair a stage
+// Ring of streamed tokens: a stage holds a half (64 tokens) of both tensors of the pair and is given back after the half's
+// accumulation.  With a tile of one tensor a stage (the same 160 KB) the next pair's second tile could only be asked for
+// when the tile before had been used up, and came about 800 clocks late on every tile.
+constexpr uint32_t kBwdStages = 5;
 constexpr uint32_t kColStages = 2;       // key role: statistics of streamed tiles
 constexpr uint32_t kBwdSpinLimit = 1u << 22;
 constexpr uint32_t kBwdWaitUs = 2000000;
@@ -54,9 +57,9 @@ struct BwdParams {
     __nv_bfloat16 *out1, *out2;  // query role: dq, -; key role: dv, dk
     int *status;
 };
-// Views of a tensor for whole tiles: patches of the image part, runs of tokens, runs of text tokens.
+// Views of a tensor: whole tiles (patches of the image part, runs of text tokens) and half ones (patches, runs of tokens).
 struct BwdViews {
-    CUtensorMap img, lin, txt;
+    CUtensorMap img, txt, half_img, half_lin;
 };
 struct BwdMaps {
     BwdViews a[2], b[2];  // stationary and streamed tensors
@@ -105,13 +108,14 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
 {
     constexpr int kHalves = D / 64;                 // 64-channel (128-byte) column blocks of a tile
     constexpr uint32_t kHalfBytes = 128 * 128;      // 128 rows x 128 B
-    constexpr uint32_t kTileBytes = kHalves * kHalfBytes;
+    constexpr uint32_t kTileBytes = kHalves * kHalfBytes;   // also a stage: two tensors, 64 rows
+    constexpr uint32_t kSubBytes = kTileBytes / 2, kSubHalfBytes = kHalfBytes / 2;
     constexpr uint32_t kIdescT = ptx::idesc_bf16(64, false);    // [128 rows] x [64 columns], both operands K-major
     constexpr uint32_t kIdescAcc = ptx::idesc_bf16(D, true);    // [128 rows] x [D channels], B read MN-major
     constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const uint32_t sA = ptx::smem_u32(smem_raw), sB = sA + 2 * kTileBytes;  // two stationary tiles, ring of streamed ones
+    const uint32_t sA = ptx::smem_u32(smem_raw), sB = sA + 2 * kTileBytes;  // two stationary tiles, ring of streamed halves
     BwdCtrl *ctrl = reinterpret_cast<BwdCtrl *>(smem_raw + (2 + kBwdStages) * kTileBytes);
     volatile int *abort_flag = &ctrl->abort_flag;
     const uint32_t b_a = ptx::smem_u32(&ctrl->a_full), b_full0 = ptx::smem_u32(&ctrl->b_full[0]),
@@ -188,12 +192,16 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 const clear_kv_tile_t t_next = tiles[min(i + 1, n_tiles - 1)];
                 const bool linear = (t.flags & CLEAR_TILE_LINEAR) != 0;
 #pragma unroll 1
-                for (int j = 0; j < 2 && ok; ++j) {
+                for (int h = 0; h < 2; ++h) {
                     ok = bwd_wait(b_empty0 + 8 * stage, par ^ 1u, abort_flag, prm.status, 1);
                     if (!ok) break;
                     const uint32_t bar = b_full0 + 8 * stage;
                     ptx::mbar_expect_tx(bar, kTileBytes);
-                    ptx::tma_load_5d(sB + stage * kTileBytes, linear ? &maps.b[j].lin : &maps.b[j].img, bar, 0, t.x, linear ? 0 : t.y, 0, bh);
+                    // (a half that lies past the last row or token reads as zero)
+#pragma unroll 1
+                    for (int j = 0; j < 2; ++j)
+                        ptx::tma_load_5d(sB + stage * kTileBytes + j * kSubBytes, linear ? &maps.b[j].half_lin : &maps.b[j].half_img, bar, 0,
+                                         linear ? t.x + 64 * h : t.x, linear ? 0 : t.y + 4 * h, 0, bh);
                     ++n_loads;
                     if (++stage == kBwdStages) {
                         stage = 0;
@@ -218,78 +226,77 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             // waits sit behind products that are still running.
             if (ptx::elect_one()) {
                 bool ok = bwd_wait(b_a, 0, abort_flag, prm.status, 2);
-                const uint32_t a_lo0 = ptx::smem_desc_lo(sA, 16), bk_lo0 = ptx::smem_desc_lo(sB, 16), bm_lo0 = ptx::smem_desc_lo(sB, kHalfBytes);
-                constexpr uint32_t kTile16 = kTileBytes >> 4;
+                const uint32_t a_lo0 = ptx::smem_desc_lo(sA, 16), bk_lo0 = ptx::smem_desc_lo(sB, 16), bm_lo0 = ptx::smem_desc_lo(sB, kSubHalfBytes);
+                constexpr uint32_t kTile16 = kTileBytes >> 4, kSub16 = kSubBytes >> 4;
                 uint32_t next = 0, next_par = 0;
-                // the next pair of streamed tiles: their offsets in the ring, in descriptor units
-                auto wait_pair = [&](uint32_t (&st)[2]) {
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        st[j] = next;
-                        ok = ok && bwd_wait(b_full0 + 8 * next, next_par, abort_flag, prm.status, 3);
-                        if (++next == kBwdStages) {
-                            next = 0;
-                            next_par ^= 1u;
-                        }
+                // the next half of the streamed pair: its stage
+                auto wait_half = [&]() -> uint32_t {
+                    const uint32_t st = next;
+                    ok = ok && bwd_wait(b_full0 + 8 * next, next_par, abort_flag, prm.status, 3);
+                    if (++next == kBwdStages) {
+                        next = 0;
+                        next_par ^= 1u;
                     }
+                    return st;
                 };
-                // T1, T2 of a half: D / 16 MMAs of 16 channels each; the second half's tokens are 64 rows, 8192 bytes, further
-                auto issue_t = [&](const uint32_t (&st)[2], int half) {
+                // T1, T2 of a half: D / 16 MMAs of 16 channels each
+                auto issue_t = [&](uint32_t st, int half) {
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        const uint32_t d = tmem + half * 128 + j * 64, a = a_lo0 + j * kTile16, b = bk_lo0 + st[j] * kTile16 + half * (8192 >> 4);
+                        const uint32_t d = tmem + half * 128 + j * 64, a = a_lo0 + j * kTile16, b = bk_lo0 + st * kTile16 + j * kSub16;
                         ptx::mma_ss_c<false>(d, ptx::make_desc(a, kDescHi), ptx::make_desc(b, kDescHi), kIdescT);
 #pragma unroll
                         for (int kk = 1; kk < D / 16; ++kk) {
-                            const uint32_t off16 = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
-                            ptx::mma_ss_c<true>(d, ptx::make_desc(a + off16, kDescHi), ptx::make_desc(b + off16, kDescHi), kIdescT);
+                            const uint32_t a16 = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4, b16 = ((kk >> 2) * kSubHalfBytes + (kk & 3) * 32) >> 4;
+                            ptx::mma_ss_c<true>(d, ptx::make_desc(a + a16, kDescHi), ptx::make_desc(b + b16, kDescHi), kIdescT);
                         }
                     }
                     ptx::tc_commit(ptx::smem_u32(&ctrl->t_full[half]));
                 };
                 // 4 MMAs over 16 streamed tokens each (16 rows of 128 bytes = 2048 bytes), B read MN-major; the bf16 columns
                 // of the two row groups start at the groups' own fp32 columns
-                auto issue_acc = [&](const uint32_t (&st)[2], int half, uint32_t before) {
+                auto issue_acc = [&](uint32_t st, int half, uint32_t before) {
                     const uint32_t p1 = tmem + half * 128, p2 = p1 + 64;
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
-                        const uint32_t acc = kk > 0 ? 1u : before, col = (kk >> 1) * 32 + (kk & 1) * 8, off = half * (8192 >> 4) + kk * (2048 >> 4);
+                        const uint32_t acc = kk > 0 ? 1u : before, col = (kk >> 1) * 32 + (kk & 1) * 8, off = st * kTile16 + kk * (2048 >> 4);
                         if (KEY_ROLE) {
-                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + st[1] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dV += P^T dO
-                            ptx::mma_ts(tmem_A2, p2 + col, ptx::make_desc(bm_lo0 + st[0] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dK += dS^T Q
+                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + kSub16 + off, kDescHi), kIdescAcc, acc);  // dV += P^T dO
+                            ptx::mma_ts(tmem_A2, p2 + col, ptx::make_desc(bm_lo0 + off, kDescHi), kIdescAcc, acc);  // dK += dS^T Q
                         } else {
-                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + st[0] * kTile16 + off, kDescHi), kIdescAcc, acc);  // dQ += dS K
+                            ptx::mma_ts(tmem_A1, p1 + col, ptx::make_desc(bm_lo0 + off, kDescHi), kIdescAcc, acc);  // dQ += dS K
                         }
                     }
+                    ptx::tc_commit(b_empty0 + 8 * st);
                 };
                 const uint32_t b_p0 = ptx::smem_u32(&ctrl->p_ready[0]), b_p1 = ptx::smem_u32(&ctrl->p_ready[1]);
-                uint32_t st[2], st_next[2] = {0, 0};
-                wait_pair(st);
+                uint32_t st0 = wait_half(), st1 = 0;
                 if (ok) {
                     ptx::tc_fence_after();
-                    issue_t(st, 0);
+                    issue_t(st0, 0);
+                    st1 = wait_half();
                 }
 #pragma unroll 1
                 for (int i = 0; i < n_tiles && ok; ++i) {
                     const uint32_t par = (uint32_t)i & 1u;
-                    issue_t(st, 1);
                     const bool more = i + 1 < n_tiles;
-                    if (more) wait_pair(st_next);
+                    ptx::tc_fence_after();
+                    issue_t(st1, 1);
+                    const uint32_t st2 = more ? wait_half() : 0u;
                     // the rows have read T1, T2 of a half and put P / dS over them
                     ok = ok && bwd_wait(b_p0, par, abort_flag, prm.status, 4);
                     if (!ok) break;
                     ptx::tc_fence_after();
-                    issue_acc(st, 0, i > 0 ? 1u : 0u);
-                    if (more) issue_t(st_next, 0);
-                    ok = bwd_wait(b_p1, par, abort_flag, prm.status, 4);
+                    issue_acc(st0, 0, i > 0 ? 1u : 0u);
+                    if (more) issue_t(st2, 0);
+                    const uint32_t st3 = more ? wait_half() : 0u;
+                    ok = ok && bwd_wait(b_p1, par, abort_flag, prm.status, 4);
                     if (!ok) break;
                     ptx::tc_fence_after();
-                    issue_acc(st, 1, 1u);
-                    ptx::tc_commit(b_empty0 + 8 * st[0]);
-                    ptx::tc_commit(b_empty0 + 8 * st[1]);
+                    issue_acc(st1, 1, 1u);
                     if (!more) ptx::tc_commit(b_acc);
-                    st[0] = st_next[0];
-                    st[1] = st_next[1];
+                    st0 = st2;
+                    st1 = st3;
                 }
                 if (*abort_flag) {
                     // MMAs that were issued must retire before tensor memory is given back
@@ -503,20 +510,23 @@ int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void 
     const int rc = launch_ws_stats(p, q, k, v, d_out, p.d_bwd_stats, scale, stream);
     if (rc != CLEAR_OK) return rc;
 
-    // Per tensor three views of [BH][half][rows][cols][64]: the image part in 8 x 16 patches, runs of 128 tokens of the
-    // sequence, and of its text prefix (rows past the text read as zero).
+    // Per tensor four views of [BH][half][rows][cols][64]: the image part in patches of 8 x 16 and of 4 x 16, runs of 128
+    // tokens of the text prefix (rows past the text read as zero) and of 64 tokens of the whole sequence.
     const uint64_t row_b = (uint64_t)s.head_dim * 2;
     const uint64_t dims_img[5] = {64, gw, gh, halves, BH}, str_img[4] = {row_b, gw * row_b, 128, N * row_b};
     const uint32_t box_img[5] = {64, (uint32_t)kTileW, (uint32_t)kTileH, (uint32_t)halves, 1};
     const uint64_t dims_lin[5] = {64, N, 1, halves, BH}, dims_txt[5] = {64, T > 0 ? T : 1, 1, halves, BH};
     const uint64_t str_lin[4] = {row_b, N * row_b, 128, N * row_b};
-    const uint32_t box_lin[5] = {64, (uint32_t)kTileTokens, 1, (uint32_t)halves, 1};
+    const uint32_t box_txt[5] = {64, (uint32_t)kTileTokens, 1, (uint32_t)halves, 1};
+    const uint32_t box_himg[5] = {64, (uint32_t)kTileW, (uint32_t)kTileH / 2, (uint32_t)halves, 1};
+    const uint32_t box_hlin[5] = {64, (uint32_t)kTileTokens / 2, 1, (uint32_t)halves, 1};
     BwdViews views[4];
     const void *tensors[4] = {q, k, v, d_out};
     for (int t = 0; t < 4; ++t)
         if (!encode_bf16_map(&views[t].img, static_cast<const char *>(tensors[t]) + T * row_b, 5, dims_img, str_img, box_img) ||
-            !encode_bf16_map(&views[t].lin, tensors[t], 5, dims_lin, str_lin, box_lin) ||
-            !encode_bf16_map(&views[t].txt, tensors[t], 5, dims_txt, str_lin, box_lin))
+            !encode_bf16_map(&views[t].txt, tensors[t], 5, dims_txt, str_lin, box_txt) ||
+            !encode_bf16_map(&views[t].half_img, static_cast<const char *>(tensors[t]) + T * row_b, 5, dims_img, str_img, box_himg) ||
+            !encode_bf16_map(&views[t].half_lin, tensors[t], 5, dims_lin, str_lin, box_hlin))
             return CLEAR_ERR_CUDA;
 
     BwdParams prm{};
