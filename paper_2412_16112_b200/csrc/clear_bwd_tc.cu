@@ -38,7 +38,7 @@ constexpr uint32_t kBwdTmemCols = 512;   // two buffers of T1 | T2 (64 columns e
 // Ring of streamed tokens: a stage holds a half (64 tokens) of both tensors of the pair and is given back after the half's
 // accumulation.  With a tile of one tensor a stage (the same 160 KB) the next pair's second tile could only be asked for
 // when the tile before had been used up, and came about 800 clocks late on every tile.
-constexpr uint32_t kBwdStages = 5;
+constexpr uint32_t kKeyStages = 5, kQueryStages = 7;   // (the query role keeps its stationary tiles in tensor memory)
 constexpr uint32_t kColStages = 2;       // key role: statistics of streamed tiles
 constexpr uint32_t kBwdSpinLimit = 1u << 22;
 constexpr uint32_t kBwdWaitUs = 2000000;
@@ -54,20 +54,23 @@ struct BwdParams {
     long long n_tokens;
     float scale, scale_log2;   // scale, scale * log2(e)
     const float2 *stats;       // [bh][token]: m', delta
-    __nv_bfloat16 *out1, *out2;  // query role: dq, -; key role: dv, dk
     int *status;
 };
 // Views of a tensor: whole tiles (patches of the image part, runs of text tokens) and half ones (patches, runs of tokens).
 struct BwdViews {
     CUtensorMap img, txt, half_img, half_lin;
 };
+struct BwdOut {
+    CUtensorMap img, txt;
+};
 struct BwdMaps {
     BwdViews a[2], b[2];  // stationary and streamed tensors
+    BwdOut o[2];          // query role: dq, -; key role: dv, dk
 };
 
 struct BwdCtrl {
-    uint64_t a_full, b_full[kBwdStages], b_empty[kBwdStages], t_full[2], p_ready[2], acc_done, col_full[kColStages],
-        col_empty[kColStages], drain;
+    uint64_t a_full, b_full[kQueryStages], b_empty[kQueryStages], t_full[2], p_ready[2], acc_done, col_full[kColStages],
+        col_empty[kColStages], a_moved, out_ready, drain;
     alignas(16) float2 col[kColStages][128];   // key role: statistics of the streamed tile's 128 columns
     uint32_t tmem_base;
     int abort_flag, skip;
@@ -113,13 +116,16 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
     constexpr uint32_t kIdescT = ptx::idesc_bf16(64, false);    // [128 rows] x [64 columns], both operands K-major
     constexpr uint32_t kIdescAcc = ptx::idesc_bf16(D, true);    // [128 rows] x [D channels], B read MN-major
     constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
+    constexpr uint32_t kStages = KEY_ROLE ? kKeyStages : kQueryStages, kFixed = KEY_ROLE ? 2 : 0;
+    constexpr uint32_t kAStage = KEY_ROLE ? 0 : kStages - 2;   // where the stationary tiles land; the query role's ring gets the place back
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const uint32_t sA = ptx::smem_u32(smem_raw), sB = sA + 2 * kTileBytes;  // two stationary tiles, ring of streamed halves
-    BwdCtrl *ctrl = reinterpret_cast<BwdCtrl *>(smem_raw + (2 + kBwdStages) * kTileBytes);
+    const uint32_t s0 = ptx::smem_u32(smem_raw), sA = s0 + kAStage * kTileBytes, sB = s0 + kFixed * kTileBytes;
+    BwdCtrl *ctrl = reinterpret_cast<BwdCtrl *>(smem_raw + (kFixed + kStages) * kTileBytes);
     volatile int *abort_flag = &ctrl->abort_flag;
     const uint32_t b_a = ptx::smem_u32(&ctrl->a_full), b_full0 = ptx::smem_u32(&ctrl->b_full[0]),
-                   b_empty0 = ptx::smem_u32(&ctrl->b_empty[0]), b_acc = ptx::smem_u32(&ctrl->acc_done);
+                   b_empty0 = ptx::smem_u32(&ctrl->b_empty[0]), b_acc = ptx::smem_u32(&ctrl->acc_done),
+                   b_moved = ptx::smem_u32(&ctrl->a_moved);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int bh, item_id;
@@ -136,23 +142,34 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
     const int n_tiles = item.tile_count;
     const bool is_text = item.kind == 1;
 
+    // row of the stationary tile that a thread of the row warps works on
+    const int r = (warp & 3) * 32 + lane;
+    const int q_y = item.qy + (r >> 4), q_x = item.qx + (r & 15);
+    const bool row_valid = is_text ? r < item.n_rows : q_y < prm.grid_h && q_x < prm.grid_w;
+    const long long row_token = is_text ? (long long)item.qx + r : (long long)prm.n_text + (long long)q_y * prm.grid_w + q_x;
+    // one streamed half into a stage (a half that lies past the last row or token reads as zero)
+    auto load_half = [&](const clear_kv_tile_t &t, int h, uint32_t stage) {
+        const bool linear = (t.flags & CLEAR_TILE_LINEAR) != 0;
+        const uint32_t bar = b_full0 + 8 * stage;
+        ptx::mbar_expect_tx(bar, kTileBytes);
+#pragma unroll 1
+        for (int j = 0; j < 2; ++j)
+            ptx::tma_load_5d(sB + stage * kTileBytes + j * kSubBytes, linear ? &maps.b[j].half_lin : &maps.b[j].half_img, bar, 0,
+                             linear ? t.x + 64 * h : t.x, linear ? 0 : t.y + 4 * h, 0, bh);
+    };
     // once any CTA of this plan has given up, the rest of the grid leaves at once; a window that is not 1024-byte
     // aligned (never expected) cannot hold swizzled tiles
     if (tid == 0) {
         int skip = *reinterpret_cast<volatile int *>(prm.status);
-        if ((sA & 1023u) != 0u) {
+        if ((s0 & 1023u) != 0u) {
             atomicCAS(prm.status, 0, 100);
             skip = 1;
         }
         ctrl->skip = skip;
-    }
-    __syncthreads();
-    if (ctrl->skip != 0) return;
-
-    if (tid == 0) {
         ctrl->abort_flag = 0;
         ptx::mbar_init(b_a, 1);
-        for (uint32_t i = 0; i < kBwdStages; ++i) {
+        ptx::mbar_init(b_moved, kRowWarps);
+        for (uint32_t i = 0; i < kStages; ++i) {
             ptx::mbar_init(b_full0 + 8 * i, 1);
             ptx::mbar_init(b_empty0 + 8 * i, 1);
         }
@@ -165,8 +182,19 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             ptx::mbar_init(ptx::smem_u32(&ctrl->col_empty[i]), kRowWarps);
         }
         ptx::mbar_init(b_acc, 1);
+        ptx::mbar_init(ptx::smem_u32(&ctrl->out_ready), kRowWarps);
         ptx::mbar_init(ptx::smem_u32(&ctrl->drain), 1);
         ptx::fence_mbar_init();
+        if (skip == 0) {
+            // the first copies leave before the block has met: one CTA fills an SM, so nothing else covers their way
+            ptx::mbar_expect_tx(b_a, 2 * kTileBytes);
+#pragma unroll 1
+            for (int i = 0; i < 2; ++i)
+                ptx::tma_load_5d(sA + i * kTileBytes, is_text ? &maps.a[i].txt : &maps.a[i].img, b_a, 0, item.qx, is_text ? 0 : item.qy, 0, bh);
+            const clear_kv_tile_t t = tiles[0];
+            load_half(t, 0, 0);
+            load_half(t, 1, 1);
+        }
     }
     if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_u32(&ctrl->tmem_base), kBwdTmemCols);
@@ -175,35 +203,29 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem = ctrl->tmem_base, tmem_A1 = tmem + 256, tmem_A2 = tmem + 384;
+    const uint32_t tmem = ctrl->tmem_base, tmem_A1 = tmem + 256, tmem_A2 = tmem + 384;  // query role: q | dO in A2's place
+    if (ctrl->skip != 0) {
+        if (warp == 1) ptx::tmem_dealloc(tmem, kBwdTmemCols);
+        return;
+    }
 
     if (warp < 4) {
         if (warp == 0 && lane == 0) {
             // ================= loader ===========================================================================
-            ptx::mbar_expect_tx(b_a, 2 * kTileBytes);
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i)
-                ptx::tma_load_5d(sA + i * kTileBytes, is_text ? &maps.a[i].txt : &maps.a[i].img, b_a, 0, item.qx, is_text ? 0 : item.qy, 0, bh);
-            uint32_t n_loads = 0, stage = 0, par = 0;
+            uint32_t n_loads = 2, stage = 2, par = 0;
             bool ok = true;
-            clear_kv_tile_t t = tiles[0];
+            clear_kv_tile_t t = tiles[min(1, n_tiles - 1)];
 #pragma unroll 1
-            for (int i = 0; i < n_tiles && ok; ++i) {
+            for (int i = 1; i < n_tiles && ok; ++i) {
                 const clear_kv_tile_t t_next = tiles[min(i + 1, n_tiles - 1)];
-                const bool linear = (t.flags & CLEAR_TILE_LINEAR) != 0;
 #pragma unroll 1
                 for (int h = 0; h < 2; ++h) {
-                    ok = bwd_wait(b_empty0 + 8 * stage, par ^ 1u, abort_flag, prm.status, 1);
+                    if (!KEY_ROLE && n_loads == kAStage) ok = bwd_wait(b_moved, 0, abort_flag, prm.status, 9);
+                    ok = ok && bwd_wait(b_empty0 + 8 * stage, par ^ 1u, abort_flag, prm.status, 1);
                     if (!ok) break;
-                    const uint32_t bar = b_full0 + 8 * stage;
-                    ptx::mbar_expect_tx(bar, kTileBytes);
-                    // (a half that lies past the last row or token reads as zero)
-#pragma unroll 1
-                    for (int j = 0; j < 2; ++j)
-                        ptx::tma_load_5d(sB + stage * kTileBytes + j * kSubBytes, linear ? &maps.b[j].half_lin : &maps.b[j].half_img, bar, 0,
-                                         linear ? t.x + 64 * h : t.x, linear ? 0 : t.y + 4 * h, 0, bh);
+                    load_half(t, h, stage);
                     ++n_loads;
-                    if (++stage == kBwdStages) {
+                    if (++stage == kStages) {
                         stage = 0;
                         par ^= 1u;
                     }
@@ -213,9 +235,9 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             if (*abort_flag) {
                 // leave no copy in flight: whatever was issued must land before the block exits
                 bwd_drain(b_a, 0);
-                for (uint32_t j = 0; j < kBwdStages && j < n_loads; ++j) {
+                for (uint32_t j = 0; j < kStages && j < n_loads; ++j) {
                     const uint32_t idx = n_loads - 1 - j;
-                    bwd_drain(b_full0 + 8 * (idx % kBwdStages), (idx / kBwdStages) & 1u);
+                    bwd_drain(b_full0 + 8 * (idx % kStages), (idx / kStages) & 1u);
                 }
             }
         } else if (warp == 1) {
@@ -225,7 +247,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             // stands there: the loop goes by tiles with both halves written out, one lane walks it without votes, and the
             // waits sit behind products that are still running.
             if (ptx::elect_one()) {
-                bool ok = bwd_wait(b_a, 0, abort_flag, prm.status, 2);
+                bool ok = bwd_wait(KEY_ROLE ? b_a : b_moved, 0, abort_flag, prm.status, 2);
                 const uint32_t a_lo0 = ptx::smem_desc_lo(sA, 16), bk_lo0 = ptx::smem_desc_lo(sB, 16), bm_lo0 = ptx::smem_desc_lo(sB, kSubHalfBytes);
                 constexpr uint32_t kTile16 = kTileBytes >> 4, kSub16 = kSubBytes >> 4;
                 uint32_t next = 0, next_par = 0;
@@ -233,7 +255,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 auto wait_half = [&]() -> uint32_t {
                     const uint32_t st = next;
                     ok = ok && bwd_wait(b_full0 + 8 * next, next_par, abort_flag, prm.status, 3);
-                    if (++next == kBwdStages) {
+                    if (++next == kStages) {
                         next = 0;
                         next_par ^= 1u;
                     }
@@ -244,6 +266,14 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const uint32_t d = tmem + half * 128 + j * 64, a = a_lo0 + j * kTile16, b = bk_lo0 + st * kTile16 + j * kSub16;
+                        if (!KEY_ROLE) {
+                            const uint32_t a_tmem = tmem_A2 + j * (D / 2);
+                            ptx::mma_ts_c<false>(d, a_tmem, ptx::make_desc(b, kDescHi), kIdescT);
+#pragma unroll
+                            for (int kk = 1; kk < D / 16; ++kk)
+                                ptx::mma_ts_c<true>(d, a_tmem + 8 * kk, ptx::make_desc(b + (((kk >> 2) * kSubHalfBytes + (kk & 3) * 32) >> 4), kDescHi), kIdescT);
+                            continue;
+                        }
                         ptx::mma_ss_c<false>(d, ptx::make_desc(a, kDescHi), ptx::make_desc(b, kDescHi), kIdescT);
 #pragma unroll
                         for (int kk = 1; kk < D / 16; ++kk) {
@@ -335,13 +365,35 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
         // ================= row warps: warp (g, quadrant); group g takes the halves h = g & 1 and of them the columns
         // [32 (g >> 1), +32); thread = row of the stationary tile =================
         const int g = (warp - 4) >> 2, half = g & 1, hc = g >> 1;
-        const int r = (warp & 3) * 32 + lane;    // row of the tile
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tmem_T1 = tmem + half * 128 + 32 * hc + lane_off, tmem_T2 = tmem_T1 + 64;
         const float c = prm.scale_log2;
-        const int q_y = item.qy + (r >> 4), q_x = item.qx + (r & 15);
-        const bool row_valid = is_text ? r < item.n_rows : q_y < prm.grid_h && q_x < prm.grid_w;
-        const long long row_token = is_text ? (long long)item.qx + r : (long long)prm.n_text + (long long)q_y * prm.grid_w + q_x;
+        bool alive = true;
+        if (!KEY_ROLE) {
+            // The stationary rows go on to tensor memory, where an MMA of 64 columns takes 32 clocks instead of the 48 that
+            // both operands need out of shared memory: group g moves 64 channels of q (g < 2) or of dO.  (Loaded straight
+            // from global memory, a row a thread, they took 8000 clocks.)
+            alive = __all_sync(0xffffffffu, bwd_wait(b_a, 0, abort_flag, prm.status, 10));
+            if (alive) {
+                if ((g & 1) * 64 < D) {
+                    uint32_t w[32];
+                    const uint8_t *src = smem_raw + (kAStage + (g >> 1)) * kTileBytes + (g & 1) * kHalfBytes + r * 128;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const uint4 v = *reinterpret_cast<const uint4 *>(src + ((j ^ (r & 7)) << 4));
+                        w[4 * j] = v.x;
+                        w[4 * j + 1] = v.y;
+                        w[4 * j + 2] = v.z;
+                        w[4 * j + 3] = v.w;
+                    }
+                    ptx::tmem_st32(tmem_A2 + lane_off + (g >> 1) * (D / 2) + (g & 1) * 32, w);
+                    ptx::tmem_wait_st();
+                }
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(b_moved);
+            }
+        }
         float2 row_stat = make_float2(0.f, 0.f);
         if (!KEY_ROLE && row_valid) row_stat = prm.stats[(long long)bh * prm.n_tokens + row_token];
         // mask bits of this row for its 32 columns of a tile (bit j = column allowed; the mask is symmetric, so the row's
@@ -367,13 +419,12 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             return bits;
         };
         const uint32_t b_t = ptx::smem_u32(&ctrl->t_full[half]), b_p = ptx::smem_u32(&ctrl->p_ready[half]);
-        bool alive = true;
         // tile records two ahead, mask words one ahead
         clear_kv_tile_t t_next = tiles[min(1, n_tiles - 1)];
         uint32_t mw_next = mask_word(tiles[0]);
         uint32_t col_st = 0, col_par = 0;
 #pragma unroll 1
-        for (int i = 0; i < n_tiles; ++i) {
+        for (int i = 0; i < n_tiles && alive; ++i) {
             const uint32_t mw = mw_next;
             mw_next = mask_word(t_next);
             t_next = tiles[min(i + 2, n_tiles - 1)];
@@ -428,32 +479,48 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             }
         }
 
-        // ---- epilogue: after the last accumulation every group stores a quarter of the channels of its rows ----
+        // ---- epilogue: after the last accumulation every group brings a quarter of the channels of its rows into shared
+        // memory, which nothing reads any more, and a TMA store takes the tile from there (rows outside the tensor are
+        // left out by its bounds).  Stored by the threads themselves, a row each, the key role's two tensors took
+        // 3900 clocks. ----
         if (alive) alive = __all_sync(0xffffffffu, bwd_wait(b_acc, 0, abort_flag, prm.status, 8));
         if (alive) {
             ptx::tc_fence_after();
-            auto store_rows = [&](uint32_t tmem_acc, __nv_bfloat16 *base, float factor) {
-                __nv_bfloat16 *dst = base + ((long long)bh * prm.n_tokens + row_token) * D + g * (D / 4);
-                const bool wide = (reinterpret_cast<uintptr_t>(base) & 31u) == 0u;  // tensors are 16-byte aligned at least
-#pragma unroll 1
-                for (int w = 0; w < D / 64; ++w) {
-                    uint32_t o[16], u[8];
-                    ptx::tmem_ld16(tmem_acc + lane_off + g * (D / 4) + 16 * w, o);
-                    ptx::tmem_wait_ld();
+            auto stage_rows = [&](uint32_t tmem_acc, uint32_t tile, float factor) {
+                uint8_t *dst = smem_raw + tile * kTileBytes + (D == 128 ? (g >> 1) * kHalfBytes : 0) + r * 128;
+                constexpr int kChunks = D / 32;   // 16-byte chunks of a group
+                const int first = g * kChunks & 7;
+                uint32_t o[4 * kChunks * 2];
+                if constexpr (D == 128)
+                    ptx::tmem_ld32(tmem_acc + lane_off + g * (D / 4), o);
+                else
+                    ptx::tmem_ld16(tmem_acc + lane_off + g * (D / 4), o);
+                ptx::tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) u[j] = ptx::pack_bf16(__uint_as_float(o[2 * j]) * factor, __uint_as_float(o[2 * j + 1]) * factor);
-                    if (row_valid) {
-                        if (wide) {
-                            ptx::stg_u256(dst + 16 * w, u);
-                        } else {
-                            *reinterpret_cast<uint4 *>(dst + 16 * w) = make_uint4(u[0], u[1], u[2], u[3]);
-                            *reinterpret_cast<uint4 *>(dst + 16 * w + 8) = make_uint4(u[4], u[5], u[6], u[7]);
-                        }
-                    }
+                for (int j = 0; j < kChunks; ++j) {
+                    uint32_t u[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        u[k] = ptx::pack_bf16(__uint_as_float(o[8 * j + 2 * k]) * factor, __uint_as_float(o[8 * j + 2 * k + 1]) * factor);
+                    *reinterpret_cast<uint4 *>(dst + (((first + j) ^ (r & 7)) << 4)) = make_uint4(u[0], u[1], u[2], u[3]);
                 }
             };
-            store_rows(tmem_A1, prm.out1, KEY_ROLE ? 1.f : prm.scale);    // dV, or dQ
-            if (KEY_ROLE) store_rows(tmem_A2, prm.out2, prm.scale);       // dK
+            stage_rows(tmem_A1, 0, KEY_ROLE ? 1.f : prm.scale);    // dV, or dQ
+            if (KEY_ROLE) stage_rows(tmem_A2, 1, prm.scale);       // dK
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                ptx::mbar_arrive(ptx::smem_u32(&ctrl->out_ready));
+                if (warp == 4 && bwd_wait(ptx::smem_u32(&ctrl->out_ready), 0, abort_flag, prm.status, 11)) {
+                    ptx::fence_proxy_async_smem();
+#pragma unroll 1
+                    for (int i = 0; i < (KEY_ROLE ? 2 : 1); ++i)
+                        ptx::tma_store_5d(is_text ? &maps.o[i].txt : &maps.o[i].img, s0 + i * kTileBytes, 0, item.qx, is_text ? 0 : item.qy, 0, bh);
+                    ptx::bulk_commit_group();
+                    ptx::bulk_wait_group0();
+                }
+            }
+            __syncwarp();
         }
     }
 
@@ -466,22 +533,19 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
 }
 
 template <int D>
-int launch_roles(const BwdViews &q, const BwdViews &k, const BwdViews &v, const BwdViews &g, BwdParams prm, void *dq, void *dk,
-                 void *dv, cudaStream_t stream)
+int launch_roles(const BwdViews &q, const BwdViews &k, const BwdViews &v, const BwdViews &g, const BwdOut &dq,
+                 const BwdOut &dk, const BwdOut &dv, const BwdParams &prm, cudaStream_t stream)
 {
-    constexpr size_t kSmem = (2 + kBwdStages) * (D / 64) * 16384 + sizeof(BwdCtrl);
-    static_assert(kSmem <= 232448, "shared memory of one block");
+    constexpr size_t kSmem = 7 * (D / 64) * 16384 + sizeof(BwdCtrl);
+    static_assert(kKeyStages + 2 == 7 && kQueryStages == 7 && kSmem <= 232448, "both roles take seven tiles of shared memory");
     auto kernel_q = clear_bwd_tc_kernel<D, false>;
     auto kernel_k = clear_bwd_tc_kernel<D, true>;
     CLEAR_CUDA_TRY(cudaFuncSetAttribute(kernel_q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
     CLEAR_CUDA_TRY(cudaFuncSetAttribute(kernel_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
     const unsigned grid = (unsigned)prm.n_items * (unsigned)prm.n_bh;
-    prm.out1 = static_cast<__nv_bfloat16 *>(dq);
-    kernel_q<<<grid, kBwdThreads, kSmem, stream>>>(BwdMaps{{q, g}, {k, v}}, prm);
+    kernel_q<<<grid, kBwdThreads, kSmem, stream>>>(BwdMaps{{q, g}, {k, v}, {dq, dq}}, prm);
     CLEAR_CUDA_TRY(cudaGetLastError());
-    prm.out1 = static_cast<__nv_bfloat16 *>(dv);
-    prm.out2 = static_cast<__nv_bfloat16 *>(dk);
-    kernel_k<<<grid, kBwdThreads, kSmem, stream>>>(BwdMaps{{k, v}, {q, g}}, prm);
+    kernel_k<<<grid, kBwdThreads, kSmem, stream>>>(BwdMaps{{k, v}, {q, g}, {dv, dk}}, prm);
     CLEAR_CUDA_TRY(cudaGetLastError());
     return CLEAR_OK;
 }
@@ -528,6 +592,12 @@ int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void 
             !encode_bf16_map(&views[t].half_img, static_cast<const char *>(tensors[t]) + T * row_b, 5, dims_img, str_img, box_himg) ||
             !encode_bf16_map(&views[t].half_lin, tensors[t], 5, dims_lin, str_lin, box_hlin))
             return CLEAR_ERR_CUDA;
+    BwdOut outs[3];
+    void *grads[3] = {dq, dk, dv};
+    for (int t = 0; t < 3; ++t)
+        if (!encode_bf16_map(&outs[t].img, static_cast<char *>(grads[t]) + T * row_b, 5, dims_img, str_img, box_img) ||
+            !encode_bf16_map(&outs[t].txt, grads[t], 5, dims_txt, str_lin, box_txt))
+            return CLEAR_ERR_CUDA;
 
     BwdParams prm{};
     prm.items = p.d_items;
@@ -548,8 +618,8 @@ int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void 
     prm.scale_log2 = scale * 1.4426950408889634f;
     prm.stats = reinterpret_cast<const float2 *>(p.d_bwd_stats);
     prm.status = p.d_status;
-    if (s.head_dim == 128) return launch_roles<128>(views[0], views[1], views[2], views[3], prm, dq, dk, dv, stream);
-    return launch_roles<64>(views[0], views[1], views[2], views[3], prm, dq, dk, dv, stream);
+    if (s.head_dim == 128) return launch_roles<128>(views[0], views[1], views[2], views[3], outs[0], outs[1], outs[2], prm, stream);
+    return launch_roles<64>(views[0], views[1], views[2], views[3], outs[0], outs[1], outs[2], prm, stream);
 }
 
 }  // namespace clear
