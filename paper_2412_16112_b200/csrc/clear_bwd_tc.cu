@@ -71,7 +71,7 @@ struct BwdMaps {
 struct BwdCtrl {
     uint64_t a_full, b_full[kQueryStages], b_empty[kQueryStages], t_full[2], p_ready[2], acc_done, col_full[kColStages],
         col_empty[kColStages], a_moved, out_ready, drain;
-    alignas(16) float2 col[kColStages][128];   // key role: statistics of the streamed tile's 128 columns
+    alignas(16) float4 col[kColStages][64];   // key role: -m', -m', -delta, -delta of two columns of the streamed tile
     uint32_t tmem_base;
     int abort_flag, skip;
 };
@@ -355,7 +355,11 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 ok = __all_sync(0xffffffffu, bwd_wait(ptx::smem_u32(&ctrl->col_empty[st]), (use & 1u) ^ 1u, abort_flag, prm.status, 5));
                 if (!ok) break;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) ctrl->col[st][32 * j + lane] = v[j];
+                for (int j = 0; j < 4; ++j) {
+                    float *dst = reinterpret_cast<float *>(&ctrl->col[st][16 * j + (lane >> 1)]) + (lane & 1);
+                    dst[0] = -v[j].x;
+                    dst[2] = -v[j].y;
+                }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&ctrl->col_full[st]));
             }
@@ -419,6 +423,8 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             return bits;
         };
         const uint32_t b_t = ptx::smem_u32(&ctrl->t_full[half]), b_p = ptx::smem_u32(&ctrl->p_ready[half]);
+        const uint64_t c2 = ptx::pack2(c, c), row_nm = ptx::pack2(-row_stat.x, -row_stat.x),
+                       row_nd = ptx::pack2(-row_stat.y, -row_stat.y);
         // tile records two ahead, mask words one ahead
         clear_kv_tile_t t_next = tiles[min(1, n_tiles - 1)];
         uint32_t mw_next = mask_word(tiles[0]);
@@ -429,42 +435,61 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             mw_next = mask_word(t_next);
             t_next = tiles[min(i + 2, n_tiles - 1)];
             // warp-uniform outcome: the tcgen05.ld / st below need the whole warp
-            bool got = bwd_wait(b_t, (uint32_t)i & 1u, abort_flag, prm.status, 6);
-            if (KEY_ROLE) got = got && bwd_wait(ptx::smem_u32(&ctrl->col_full[col_st]), col_par, abort_flag, prm.status, 7);
+            bool got = true;
+            if (KEY_ROLE) got = bwd_wait(ptx::smem_u32(&ctrl->col_full[col_st]), col_par, abort_flag, prm.status, 7);
+            // kPass columns at a time.  The key role's statistics come out of shared memory, which the MMAs keep busy: 16
+            // columns' worth are asked for together, the first ones before T is there, and with 32 columns at once there
+            // would be no registers to hold them.
+            constexpr int kPass = KEY_ROLE ? 16 : 32;
+            uint64_t nm[KEY_ROLE ? kPass / 2 : 1], nd[KEY_ROLE ? kPass / 2 : 1];
+            if (!KEY_ROLE) {
+                nm[0] = row_nm;
+                nd[0] = row_nd;
+            }
+            const uint32_t cols = ptx::smem_u32(&ctrl->col[col_st][32 * half + 16 * hc]);
+            auto load_cols = [&](int pass) {
+                if constexpr (KEY_ROLE) {
+#pragma unroll
+                    for (int j = 0; j < kPass / 2; ++j) ptx::lds_pairs(cols + (pass * kPass / 2 + j) * 16, nm[j], nd[j]);
+                }
+            };
+            if (got) load_cols(0);
+            got = got && bwd_wait(b_t, (uint32_t)i & 1u, abort_flag, prm.status, 6);
             if (!__all_sync(0xffffffffu, got)) {
                 alive = false;
                 break;
             }
             ptx::tc_fence_after();
-            uint32_t s[32], gg[32];
-            ptx::tmem_ld32(tmem_T1, s);
-            ptx::tmem_ld32(tmem_T2, gg);
-            ptx::tmem_wait_ld();
-            uint32_t pk[16], dk[16];
-            const float4 *cols = reinterpret_cast<const float4 *>(&ctrl->col[col_st][64 * half + 32 * hc]);
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-                float m0 = row_stat.x, d0 = row_stat.y, m1 = m0, d1 = d0;
-                if (KEY_ROLE) {
-                    const float4 v = cols[j >> 1];
-                    m0 = v.x;
-                    d0 = v.y;
-                    m1 = v.z;
-                    d1 = v.w;
+            for (int pass = 0; pass < 32 / kPass; ++pass) {
+                uint32_t s[kPass], gg[kPass], pk[kPass / 2], dk[kPass / 2];
+                if (pass > 0) load_cols(pass);
+                if constexpr (KEY_ROLE) {
+                    ptx::tmem_ld16(tmem_T1 + pass * kPass, s);
+                    ptx::tmem_ld16(tmem_T2 + pass * kPass, gg);
+                } else {
+                    ptx::tmem_ld32(tmem_T1, s);
+                    ptx::tmem_ld32(tmem_T2, gg);
                 }
-                float x0 = fmaf(__uint_as_float(s[j]), c, -m0), x1 = fmaf(__uint_as_float(s[j + 1]), c, -m1);
-                x0 = ((mw >> j) & 1u) ? x0 : -INFINITY;
-                x1 = ((mw >> (j + 1)) & 1u) ? x1 : -INFINITY;
-                const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
-                if (KEY_ROLE) pk[j >> 1] = ptx::pack_bf16(p0, p1);
-                dk[j >> 1] = ptx::pack_bf16(p0 * (__uint_as_float(gg[j]) - d0), p1 * (__uint_as_float(gg[j + 1]) - d1));
-            }
-            // a thread's bf16 columns sit at the start of its own fp32 columns, all of which it has in registers by now
-            if (KEY_ROLE) {
-                ptx::tmem_st16(tmem_T1, pk);
-                ptx::tmem_st16(tmem_T2, dk);
-            } else {
-                ptx::tmem_st16(tmem_T1, dk);
+                ptx::tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < kPass; j += 2) {
+                    const int jc = KEY_ROLE ? j >> 1 : 0, bit = pass * kPass + j;
+                    float x0, x1, p0, p1, d0, d1;
+                    ptx::unpack2(ptx::fma2(ptx::pack2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])), c2, nm[jc]), x0, x1);
+                    p0 = ptx::ex2(((mw >> bit) & 1u) ? x0 : -INFINITY);
+                    p1 = ptx::ex2(((mw >> (bit + 1)) & 1u) ? x1 : -INFINITY);
+                    ptx::unpack2(ptx::mul2(ptx::pack2(p0, p1), ptx::add2(ptx::pack2(__uint_as_float(gg[j]), __uint_as_float(gg[j + 1])), nd[jc])), d0, d1);
+                    if (KEY_ROLE) pk[j >> 1] = ptx::pack_bf16(p0, p1);
+                    dk[j >> 1] = ptx::pack_bf16(d0, d1);
+                }
+                // a thread's bf16 columns sit at the start of its own fp32 columns, in cells that it has read by now
+                if constexpr (KEY_ROLE) {
+                    ptx::tmem_st8(tmem_T1 + pass * (kPass / 2), pk);
+                    ptx::tmem_st8(tmem_T2 + pass * (kPass / 2), dk);
+                } else {
+                    ptx::tmem_st16(tmem_T1, dk);
+                }
             }
             ptx::tmem_wait_st();
             ptx::tc_fence_before();
