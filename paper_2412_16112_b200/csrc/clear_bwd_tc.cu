@@ -128,6 +128,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                    b_moved = ptx::smem_u32(&ctrl->a_moved);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (!KEY_ROLE) ptx::grid_launch_dependents();
     int bh, item_id;
     if ((int)blockIdx.x < prm.n_first * prm.n_bh) {
         item_id = (int)blockIdx.x / prm.n_bh;
@@ -206,6 +207,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
     const uint32_t tmem = ctrl->tmem_base, tmem_A1 = tmem + 256, tmem_A2 = tmem + 384;  // query role: q | dO in A2's place
     if (ctrl->skip != 0) {
         if (warp == 1) ptx::tmem_dealloc(tmem, kBwdTmemCols);
+        if (KEY_ROLE) ptx::grid_wait();
         return;
     }
 
@@ -542,7 +544,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                     for (int i = 0; i < (KEY_ROLE ? 2 : 1); ++i)
                         ptx::tma_store_5d(is_text ? &maps.o[i].txt : &maps.o[i].img, s0 + i * kTileBytes, 0, item.qx, is_text ? 0 : item.qy, 0, bh);
                     ptx::bulk_commit_group();
-                    ptx::bulk_wait_group0();
+                    ptx::bulk_wait_group0_read();   // the block may leave once its shared memory has been read
                 }
             }
             __syncwarp();
@@ -555,6 +557,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, kBwdTmemCols);
     }
+    if (KEY_ROLE) ptx::grid_wait();
 }
 
 template <int D>
@@ -570,7 +573,19 @@ int launch_roles(const BwdViews &q, const BwdViews &k, const BwdViews &v, const 
     const unsigned grid = (unsigned)prm.n_items * (unsigned)prm.n_bh;
     kernel_q<<<grid, kBwdThreads, kSmem, stream>>>(BwdMaps{{q, g}, {k, v}, {dq, dq}}, prm);
     CLEAR_CUDA_TRY(cudaGetLastError());
-    kernel_k<<<grid, kBwdThreads, kSmem, stream>>>(BwdMaps{{k, v}, {q, g}, {dv, dk}}, prm);
+    // The roles share nothing but their inputs, so the key role's blocks may take the SMs that the query role's last blocks
+    // leave free (each of them ends only when the query role has).
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kBwdThreads);
+    cfg.dynamicSmemBytes = kSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    CLEAR_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel_k, BwdMaps{{k, v}, {q, g}, {dv, dk}}, prm));
     CLEAR_CUDA_TRY(cudaGetLastError());
     return CLEAR_OK;
 }

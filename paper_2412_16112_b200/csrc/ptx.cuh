@@ -106,6 +106,10 @@ __device__ __forceinline__ void fence_proxy_async_smem()
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_group0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_group0_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// Programmatic launches: let the next grid of the stream start; wait for the grid before to have ended.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- TMA tiled loads / stores ----------------------------------------------------------------
 // Innermost coordinate c0 must keep c0 * element_size a multiple of 16 bytes.
