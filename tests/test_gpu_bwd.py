@@ -169,6 +169,38 @@ def test_tensor_core_backward_at_workload_sizes(name, heads):
     clear.clear_cache_clear()
 
 
+@pytest.mark.parametrize("gh,gw,T,r,d,cap", [
+    (4, 16, 0, 2.0, 64, None),       # one key patch, whose second half lies past the last row
+    (8, 16, 40, 3.0, 128, None),     # two: the ring never reaches the stages that hold the stationary tiles
+    (24, 16, 64, 30.0, 128, None),   # four: one half more than the ring of the query role has stages
+    (21, 33, 129, 9.0, 128, "0"),    # no mask table: every masked patch from the half widths
+    (21, 33, 129, 9.0, 64, "2"),     # a table that runs out
+])
+def test_tensor_core_backward_edges(gh, gw, T, r, d, cap, monkeypatch):
+    """Ring lengths, halves outside the grid and table-free masks; the outputs start 16 but not 32 bytes off an aligned
+    buffer and nothing outside them may change (bound as above)."""
+    if cap is not None:
+        monkeypatch.setenv("CLEAR_MAX_MASK_ENTRIES", cap)
+    clear.clear_cache_clear()
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, dtype="bf16", seed=gh + gw + d)
+    g = torch.Generator(device="cpu").manual_seed(gh * gw)
+    d_out = torch.randn(q.shape, generator=g, dtype=torch.float32).to(torch.bfloat16)
+    scale = 1 / math.sqrt(d)
+    want = oracle_bwd.attn_bwd(q, k, v, d_out, gh, gw, T, r, scale)
+    dev = torch.device("cuda:0")
+    n, pad = q.numel(), 8
+    bufs = [torch.full((n + 2 * pad,), 7.0, dtype=torch.bfloat16, device=dev) for _ in range(3)]
+    outs = [b[pad:pad + n].view(q.shape) for b in bufs]
+    clear.clear_attn_bwd_bf16_tc(*(t.to(dev) for t in (q, k, v, d_out)), *outs, gh, gw, T, r, scale)
+    torch.cuda.synchronize()
+    clear.clear_cache_check()
+    for name, buf, got, ref in zip(("dq", "dk", "dv"), bufs, outs, want):
+        err = np.abs(got.cpu().double().numpy() - ref)
+        assert err.max() <= _tc_bound(ref), f"{name}: max {err.max():.3e}"
+        assert (buf[:pad] == 7.0).all() and (buf[pad + n:] == 7.0).all(), f"{name}: guard band"
+    clear.clear_cache_clear()
+
+
 def test_tensor_core_backward_argument_errors():
     dev = torch.device("cuda:0")
     x = torch.zeros(1, 1, 272, 64, device=dev, dtype=torch.bfloat16)
