@@ -84,7 +84,8 @@ typedef struct clear_kv_tile {
     int32_t x;       /* image patch: grid column of its first key (its last ones may lie past     */
     int32_t y;       /*   the grid: such keys are masked); linear tile: x = first token, y = 0    */
     int32_t flags;   /* CLEAR_TILE_* bits                                                         */
-    int32_t n_valid; /* linear tile: keys [0, n_valid) of the tile exist / are allowed            */
+    int32_t n_valid; /* linear tile: keys [0, n_valid) of the tile exist / are allowed; patch of a */
+                     /*   backward schedule: its entry in the mask table, or -1 if it has none   */
 } clear_kv_tile_t;
 
 enum {
@@ -171,10 +172,10 @@ int clear_attn_fwd_f32(const void *q, const void *k, const void *v, void *out, i
  *     dS_ij = p_ij (d_out_i . v_j - sum_j' p_ij' d_out_i . v_j'),
  *     dq_i = scale sum_j dS_ij k_j,   dk_j = scale sum_i dS_ij q_i,   dv_j = sum_i p_ij d_out_i.
  * All seven tensors are device pointers, [B, H, N, head_dim] contiguous fp32, 16-byte aligned; q, k, v,
- * d_out are read, dq, dk, dv fully written.  Two CUDA-core kernels: one warp per query (row statistics, dq), then
- * one warp per key (dk, dv; the mask is symmetric, so the queries that see a key are the tokens that key's own
- * query sees): every output element has one writer and a fixed order of summation, so results repeat bit for
- * bit.  The first call for a shape allocates 12 bytes per token and (b, h) for the row statistics; calls for one
+ * d_out are read, dq, dk, dv fully written.  Two CUDA-core kernels: one by queries (row statistics, dq), then one by
+ * keys (dk, dv; the mask is symmetric, so the queries that see a key are the tokens that key's own query sees), on
+ * tiles of 64 tokens up to 128 channels and a warp per token above: every output element has one writer and a fixed
+ * order of summation, so results repeat bit for bit.  The first call for a shape allocates 12 bytes per token and (b, h) for the row statistics; calls for one
  * shape are ordered on the device like those of clear_attn_fwd.  Nothing but `stream` is synchronised.  Meant for
  * small problems (four dot products per allowed pair on the CUDA cores).
  * Errors: INVALID_ARG, MISALIGNED, UNSUPPORTED (head_dim > 256), CUDA. */
@@ -219,12 +220,13 @@ int clear_qk_norm_rope(const void *q_in, const void *k_in, void *q_out, void *k_
 float clear_log_scale_factor(long long n_tokens, long long n_train_tokens);
 
 /* The backward pass for bf16 tensors on the tensor cores (head_dim 64 or 128, scale > 0): same arguments and
- * results as clear_attn_bwd_bf16, computed with tcgen05 MMAs over the forward pass's tile schedule -- a launch in
- * which every 128-query tile meets its key tiles (row statistics and delta = dO . O in a first sweep, dQ in a second)
- * and a launch in which every 128-key tile meets the query tiles that see it (dK, dV; Eq. 3's mask is symmetric, so
+ * results as clear_attn_bwd_bf16, computed with tcgen05 MMAs over the forward pass's tile schedule -- a launch of
+ * the forward kernel that keeps row statistics and dO . O instead of O, a launch in which every 128-query tile meets its
+ * key tiles (dQ) and a launch in which every 128-key tile meets the query tiles that see it (dK, dV; Eq. 3's mask is symmetric, so
  * these are the same lists).  P and dS enter the MMAs rounded to bf16, as P does in the forward pass: gradients
  * agree with the exact ones to about 1e-2 of the largest gradient of the tensor.  One writer per element: results
- * repeat bit for bit.  The first call for a shape allocates its schedule tables and 16 bytes per token and (b, h).
+ * repeat bit for bit.  The first call for a shape allocates its schedule tables, 8 bytes per token and (b, h), and
+ * where long text rows are split the forward pass's workspace.
  * Errors: INVALID_ARG, MISALIGNED, UNSUPPORTED (other head sizes, scale <= 0), CUDA; a kernel whose bounded wait
  * expired is found by clear_cache_check. */
 int clear_attn_bwd_bf16_tc(const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,

@@ -2,8 +2,8 @@
 // upstream gradient dO of  O = softmax(scale Q K^T + log M) V  (Eq. 1 under the mask of Eq. 3), the step
 // through which the distillation losses of Sec. 3.3 (Eq. 4-6) reach the attention parameters.
 //
-// Two kernels, one warp per token, lanes split the head dimension, tokens walked as in the forward CUDA-core
-// kernel (the text tokens, then per grid row within reach the clipped run of columns).  Head sizes above 128 only: up to
+// Two kernels, one warp per token, lanes split the head dimension, tokens walked as clear_simt.cu
+// does (the text tokens, then per grid row within reach the clipped run of columns).  Head sizes above 128 only: up to
 // there the tiled kernels of clear_f32_bwd.cu are 6 to 8 times faster, above their row sets do not fit shared memory.
 //   query kernel: sweep 1 over the query's keys: online softmax -> row maximum m, row sum l, the un-normalised
 //       output, hence delta = dO . O; the three row statistics are kept for the second kernel;

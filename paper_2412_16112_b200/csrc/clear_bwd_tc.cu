@@ -15,9 +15,15 @@
 // each), so the products of the next half run while the elementwise step of this one does; the accumulations of a half
 // go behind them on the same pipe.  The order on the pipe is T(0), T(1), ACC(0), T(2), ACC(1), ...: a half's products
 // overwrite P / dS of the half two before it only after its accumulations have read them.
-// What bounds it: the MMAs.  64 columns cost 48 clocks per 16 channels instead of 32 (the stationary operand is read anew),
-// so a tile takes 1536 clocks of products and 512 or 1024 of accumulations: 2048 in the query role, 2560 in the key role.
-// The elementwise step (16 warps, 32 columns a thread) takes about 700 a half.
+// What bounds it: the MMAs, and at short lists the start and end of a block, which nothing covers (one block fills an SM:
+// all 512 tensor-memory columns and 227 KB).  With both operands in shared memory, 64 columns cost 48 clocks per 16
+// channels instead of 32, so the key role's tile takes 1536 clocks of products and 1024 of accumulations; measured 2900 a
+// tile.  The query role has 128 tensor-memory columns to spare and keeps its stationary operands there: 1024 + 512,
+// measured 2000.  The elementwise step (16 warps, 32 columns a thread) takes 700 (query) or 830 (key role) a half.
+// Around the list go 4500 clocks from the block's start to its first products and 3000 behind its last ones.
+// 1024 px, radius 8, 24 heads of 128: 384 us a call; with one lane's votes and waits between the MMAs, a tile of one tensor
+// a ring stage, statistics read one by one and rows stored by threads it was 487, before that (P and dS of whole tiles,
+// statistics in a sweep of the query role) 873.
 //   warp 0: TMA loads; warp 1: every MMA; warp 2 (key role): statistics of the streamed tiles; warps 4..19: rows.
 // Every output element has one writer and a fixed order of summation.  Every wait is bounded: on expiry the CTA raises the
 // plan's status word and leaves.

@@ -1,12 +1,8 @@
-// CLEAR attention forward on the CUDA cores: one warp per query, fp32 arithmetic throughout.
-//
-// This is the exact-order path: it serves fp32 tensors (where tensor-core input rounding would
-// break a 1e-5 agreement), head sizes the tensor-core kernel does not take, and non-positive
-// scales.  Each warp walks the keys its query may see under Eq. 3 -- the text tokens, then for
-// every grid row within reach the run of columns [x - m(dy), x + m(dy)] clipped to the grid --
-// and keeps an online softmax (Eq. 1) over blocks of 8 keys.  Lanes split the head dimension.
-// The two comparison masks of the appendix that are no window around the query run here too: the
-// shifted window grid (a rectangle of keys per query) and the strided mask (every r-th row and column).
+// CLEAR attention forward on the CUDA cores for the two comparison masks of the appendix that are no window around the
+// query: the shifted window grid (a rectangle of keys per query) and the strided mask (every r-th row and column).  One
+// warp per query, fp32 arithmetic throughout, any tensor type.  Each warp walks the text tokens and then the grid rows of
+// its query's keys and keeps an online softmax (Eq. 1) over blocks of 8 keys; lanes split the head dimension.  (The disc
+// and the square run on the tiles of clear_f32.cu, which a mask without neighbourhoods does not fill.)
 #include <cuda_bf16.h>
 
 #include "clear_internal.hpp"
@@ -25,8 +21,7 @@ __device__ __forceinline__ void from_f32(__nv_bfloat16 *p, float x) { *p = __flo
 template <typename T, int EPL>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 clear_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, T *__restrict__ out,
-                  int grid_h, int grid_w, int n_text, int d, const int32_t *__restrict__ half_width, int n_half_width,
-                  int mask_kind, int mask_size, int mask_param, float scale)
+                  int grid_h, int grid_w, int n_text, int d, int mask_kind, int mask_size, int mask_param, float scale)
 {
     const int lane = threadIdx.x & 31;
     const int64_t N = (int64_t)n_text + (int64_t)grid_h * grid_w;
@@ -105,7 +100,7 @@ clear_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__r
                 const int64_t row0 = (int64_t)n_text + (int64_t)yy * grid_w;
                 run(row0 + x_lo, row0 + x_hi, 1);
             }
-        } else if (mask_kind == CLEAR_MASK_STRIDED) {
+        } else {
             // rows congruent to y + (l div r), columns congruent to x + (l mod r), modulo the stride r
             const int r = mask_size;
             const int y0 = (y + (mask_param / r) % r) % r, x0 = (x + mask_param % r) % r;
@@ -113,20 +108,10 @@ clear_simt_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__r
                 const int64_t row0 = (int64_t)n_text + (int64_t)yy * grid_w;
                 run(row0 + x0, row0 + grid_w, r);
             }
-        } else {
-            const int R = n_half_width - 1;
-            for (int dy = -R; dy <= R; ++dy) {
-                const int yy = y + dy;
-                if (yy < 0 || yy >= grid_h) continue;
-                const int hw = half_width[dy < 0 ? -dy : dy];
-                const int lo = max(x - hw, 0), hi = min(x + hw, grid_w - 1);
-                const int64_t row0 = (int64_t)n_text + (int64_t)yy * grid_w;
-                run(row0 + lo, row0 + hi + 1, 1);
-            }
         }
     }
 
-    // l > 0: an image query sees itself under the disc, the square and the windows, and the text keys always;
+    // l > 0: an image query sees itself under the windows, and the text keys always;
     // under the strided mask with no text a query may see nothing: its output is 0
     const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
@@ -144,13 +129,12 @@ int launch_typed(const clear_plan &p, const void *q, const void *k, const void *
     const int64_t N = (int64_t)s.n_text + (int64_t)s.grid_h * s.grid_w;
     dim3 grid((unsigned)((N + kWarpsPerBlock - 1) / kWarpsPerBlock), (unsigned)(s.B * s.H));
     dim3 block(kWarpsPerBlock * 32);
-    const int n_hw = (int)p.sch.half_width.size();
     const int epl = (s.head_dim + 31) / 32;
 #define CLEAR_SIMT_CASE(E)                                                                                      \
     case E:                                                                                                     \
         clear_simt_kernel<T, E><<<grid, block, 0, stream>>>((const T *)q, (const T *)k, (const T *)v, (T *)out, \
                                                             s.grid_h, s.grid_w, s.n_text, s.head_dim,           \
-                                                            p.d_half_width, n_hw, s.mask_kind, (int)s.radius,   \
+                                                            s.mask_kind, (int)s.radius,                         \
                                                             s.mask_param, scale);                               \
         break;
     switch (epl) {

@@ -46,18 +46,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
-// Whether the phase has completed, without waiting (try_wait may suspend the thread for a while).
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
 // try_wait with a suspend-time hint: the thread may sleep in hardware until the phase completes or
 // about `ns` nanoseconds have passed, instead of coming back at once to poll again.
 __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity, uint32_t ns)
@@ -151,10 +139,6 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap *tm, uint32_t src
     asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];"
                  ::"l"(tm), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
                  : "memory");
-}
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *tm)
-{
-    asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
 
 // ---- tensor memory ---------------------------------------------------------------------------
@@ -259,32 +243,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
-}
-// 16 lanes x 32 columns: thread t of the warp gets, for the eight-column group i, columns 8 i + 2 (t % 4) and the next
-// one of lane t / 4 in r[4 i], r[4 i + 1] and of lane t / 4 + 8 in r[4 i + 2], r[4 i + 3].
-__device__ __forceinline__ void tmem_ld_quads(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-// 4 x 4 transpose within each group of four threads: u[g] of thread ql becomes u[ql] of thread g.
-__device__ __forceinline__ void transpose_quad(uint32_t (&u)[4], int ql)
-{
-#pragma unroll
-    for (int b = 1; b <= 2; b *= 2)
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            if (g & b) continue;
-            const bool hi = (ql & b) != 0;
-            const uint32_t got = __shfl_xor_sync(0xffffffffu, hi ? u[g] : u[g | b], b);
-            if (hi) u[g] = got;
-            else u[g | b] = got;
-        }
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16])
 {
