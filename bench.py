@@ -366,7 +366,7 @@ def run_ours(args, w):
         alu_peak = 148 * 128 * 2 * float(peaks.get("sm_max_mhz", 1965.0)) * 1e6 / 1e12
         roofline = {"bound": "alu", "achieved": per_gpu_tflops, "peak": alu_peak, "unit": "TFLOP/s",
                     "frac": per_gpu_tflops / alu_peak, "traffic": traffic, "peak_kind": "148 SMs x 128 fp32 FMA lanes",
-                    "kernel": "clear_simt_kernel"}
+                    "kernel": "clear_f32_tile_kernel"}
 
     # ---- the Q/K preparation that precedes the attention call in the model (outside `value`) -------------
     qk_prep = None
