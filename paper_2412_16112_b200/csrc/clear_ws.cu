@@ -596,7 +596,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                     drain_bar(ptx::smem_u32(&ctrl->kv_full[idx % kRing]), (idx / kRing) & 1u);
                 }
             }
-        } else if (warp == 1 || warp == 2) {
+        } else if ((warp == 1 || warp == 2) && ptx::elect_one()) {
             // ================= MMA issue: S_t = Q_t K^T, O_t += P_t V, one warp per query tile t ==============
             // S_t of a step comes in two halves of 64 keys.  The softmax warps take the second half first; P_t of the whole
             // step lies over the first half, so the second half is free as soon as its scores are in registers, and the
@@ -613,14 +613,12 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             // shuffle instruction of these warps spends 100 to 200 in the queue it shares with the exponentials of two
             // softmax warps: hence a warp per tile, the waits of one in the shadow of the other's MMAs (one warp for both
             // tiles: 560 us; a third one for the second halves: their MMAs get in the way of the critical ones, 552).
-            // A whole warp walks the loop in step and one elected lane issues: with warp-uniform control flow an MMA
-            // costs few enough issue slots to keep the tensor core fed while the softmax warps of the same scheduler
-            // are in their exponential phase (a lone thread in a divergent branch could not: 96 clocks per MMA
-            // against 64 of execution).
+            // One elected lane walks the whole loop.  With the warp walking in step and a lane elected for each group, a vote
+            // and two warp barriers stood between a wait's end and the first MMA (1024px: 106 us against 98.5, 2048px: 517
+            // against 499, 8K: 8.40 ms against 8.24).
             const int t = warp - 1;
             const int use_bit = t ? CLEAR_STEP_USE1 : CLEAR_STEP_USE0;
             constexpr uint32_t kDescHiK = ptx::smem_desc_hi_sw128(1024);  // 8-row groups are 1024 bytes apart
-            auto uni = [](int v) { return __shfl_sync(0xffffffffu, v, 0); };  // tells the compiler v is warp-uniform
             const uint32_t tmem_S = tmem + t * 128, tmem_O = tmem + 256 + t * 128;
             const uint32_t b_full0 = ptx::smem_u32(&ctrl->kv_full[0]), b_empty0 = ptx::smem_u32(&ctrl->kv_empty[0]);
             const uint32_t b_p = ptx::smem_u32(&ctrl->p_ready[t]), b_read = ptx::smem_u32(&ctrl->sb_read[t]);
@@ -632,11 +630,10 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             uint32_t turn_par = t ? 0u : 1u;             // tile 0 has the first turn
             uint32_t ring_stage = 0, ring_par = 0;       // next fill of the ring, in staging order
             bool ok = true;
-            // A wait whose outcome the lanes agree on later, once per group of MMAs (ok_all).
+            // A wait whose outcome is looked at once per group of MMAs.
             auto wait_lane = [&](uint32_t bar, uint32_t parity, int code) {
                 if (ok) ok = wait_bar(bar, parity, abort_flag, prm.status, code);
             };
-            auto ok_all = [&]() { return ok = __all_sync(0xffffffffu, ok); };
             // Both warps pass every fill of the ring in staging order and arrive once for it, after they have seen it: with
             // an MMA commit behind the MMAs that read the tile, or at once if they have no use for it.  So no phase can be
             // freed, and no warp lapped, before both have passed.
@@ -650,8 +647,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             };
             auto pass = [&]() {
                 const uint32_t st = take();
-                __syncwarp();  // every lane has seen the fill
-                if (lane == 0) ptx::mbar_arrive(b_empty0 + 8 * st);
+                if (ok) ptx::mbar_arrive(b_empty0 + 8 * st);
             };
             // The K tiles, or the V tiles, of a step: this warp's one is returned, the other one (if any) passed.
             auto take_own = [&](int f) -> uint32_t {
@@ -682,33 +678,28 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             auto issue_second_half = [&](uint32_t k_st) {
                 wait_lane(b_read, sb_par, 12);
                 sb_par ^= 1u;
-                if (!ok_all()) return;
+                if (!ok) return;
                 ptx::tc_fence_after();
-                if (ptx::elect_one()) {
-                    issue_qk(k_st, 1);
-                    ptx::tc_commit(ptx::smem_u32(&ctrl->sb_full[t]));
-                }
-                __syncwarp();
+                issue_qk(k_st, 1);
+                ptx::tc_commit(ptx::smem_u32(&ctrl->sb_full[t]));
             };
 #pragma unroll 1
             for (uint32_t k = 0; ok; ++k) {
                 const uint32_t slot = k % kSchedDepth, use = k / kSchedDepth;
                 wait_lane(ptx::smem_u32(&ctrl->sched_full[slot]), use & 1u, 5);
-                if (!ok_all()) break;
-                const int g = uni(ctrl->sched_item[slot]);
-                const int n_sides = uni(ctrl->sched_rec[slot].n_sides);
-                const int step_begin = uni(ctrl->sched_rec[slot].step_begin);
-                const int n = uni(ctrl->sched_rec[slot].step_count);
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&ctrl->sched_empty[slot]));
+                if (!ok) break;
+                const int g = ctrl->sched_item[slot];
+                const int n_sides = ctrl->sched_rec[slot].n_sides;
+                const int step_begin = ctrl->sched_rec[slot].step_begin;
+                const int n = ctrl->sched_rec[slot].step_count;
+                ptx::mbar_arrive(ptx::smem_u32(&ctrl->sched_empty[slot]));
                 if (g >= total_items) break;
                 const int *step_flags = &prm.steps[step_begin].flags;
                 constexpr int kStepInts = sizeof(clear_pair_step_t) / sizeof(int);
-                // the flags of 32 steps at a time, one step per lane; the 32 after them are fetched meanwhile
-                auto fetch_flags = [&](int s0) { return s0 + lane < n ? ptx::ldg_u32(step_flags + (s0 + lane) * kStepInts) : 0u; };
-                uint32_t lane_flags = fetch_flags(0), lane_flags_next = fetch_flags(32);
+                // the flags of the next two steps are on their way
+                auto fetch_flags = [&](int s) { return s < n ? (int)ptx::ldg_u32(step_flags + s * kStepInts) : 0; };
                 int pend = 0;            // flags of the step before (0: none)
-                int flags = (int)__shfl_sync(0xffffffffu, lane_flags, 0);
+                int flags = fetch_flags(0), flags_next = fetch_flags(1);
                 uint32_t acc = 0;        // O_t holds something of this item
                 const bool exists = t < n_sides;
                 if (exists) wait_lane(ptx::smem_u32(&ctrl->q_full[t]), n_it & 1u, 6);
@@ -716,59 +707,57 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                 for (int s = 0; s <= n && ok; ++s) {
                     // one step past the end: the last P_t V
                     const bool last = s == n;
-                    if (((s + 1) & 31) == 0) {
-                        lane_flags = lane_flags_next;
-                        lane_flags_next = fetch_flags(s + 33);
-                    }
-                    const int flags_next = (int)__shfl_sync(0xffffffffu, lane_flags, (s + 1) & 31);  // 0 past the end
+                    const int flags_after = fetch_flags(s + 2);  // 0 past the end
                     const bool pv = (pend & use_bit) != 0, qk = (flags & use_bit) != 0;
                     const uint32_t k_st = take_own(flags);
                     if (qk) issue_second_half(k_st);
                     const uint32_t v_st = take_own(pend);
                     // the epilogue must have read the previous item's O_t out of tensor memory
                     if (pv && !acc) wait_lane(ptx::smem_u32(&ctrl->o_empty[t]), (n_it & 1u) ^ 1u, 8);
+                    // Which wait comes first was decided by the clock: P's at 64 channels (67 x 120: 231 us, the turn first
+                    // 236), the turn at 128 (2048px: 506 us, P first 511; 1024px: no difference).
+                    auto wait_p = [&]() {
+                        if (pv) {
+                            wait_lane(b_p, p_par, 7);
+                            p_par ^= 1u;
+                        }
+                    };
+                    if constexpr (D == 64) wait_p();
                     wait_lane(b_turn, turn_par, 11);
                     turn_par ^= 1u;
-                    if (pv) {
-                        wait_lane(b_p, p_par, 7);
-                        p_par ^= 1u;
-                    }
-                    if (!ok_all()) break;
+                    if constexpr (D != 64) wait_p();
+                    if (!ok) break;
                     ptx::tc_fence_after();
-                    if (ptx::elect_one()) {
-                        if (pv) {
-                            // P_t (bf16 pairs) in the first 64 columns of S_t, 16 keys = 8 columns; V MN-major, 16 keys are 16
-                            // rows of 128 bytes = 2048 bytes
-                            const uint32_t v_lo = v_lo0 + v_st * (kTileBytes >> 4);
-                            ptx::mma_ts(tmem_O, tmem_S, ptx::make_desc(v_lo, kDescHiK), kIdescPV, acc);
+                    if (pv) {
+                        // P_t (bf16 pairs) in the first 64 columns of S_t, 16 keys = 8 columns; V MN-major, 16 keys are 16
+                        // rows of 128 bytes = 2048 bytes
+                        const uint32_t v_lo = v_lo0 + v_st * (kTileBytes >> 4);
+                        ptx::mma_ts(tmem_O, tmem_S, ptx::make_desc(v_lo, kDescHiK), kIdescPV, acc);
 #pragma unroll
-                            for (int kk = 1; kk < 8; ++kk)
-                                ptx::mma_ts_c<true>(tmem_O, tmem_S + kk * 8, ptx::make_desc(v_lo + kk * (2048 >> 4), kDescHiK), kIdescPV);
-                        }
-                        if (qk) {
-                            issue_qk(k_st, 0);
-                            ptx::tc_commit(ptx::smem_u32(&ctrl->sa_full[t]));
-                        }
-                        ptx::mbar_arrive(b_other);  // the other tile's turn
-                        if (qk) ptx::tc_commit(b_empty0 + 8 * k_st);
-                        if (pv) ptx::tc_commit(b_empty0 + 8 * v_st);
-                        // behind the item's last Q K^T the next Q_t may land; behind its last P V the output is complete
-                        if (s == n - 1 && exists) ptx::tc_commit(ptx::smem_u32(&ctrl->q_empty[t]));
-                        if (last && exists) ptx::tc_commit(ptx::smem_u32(&ctrl->o_full[t]));
+                        for (int kk = 1; kk < 8; ++kk)
+                            ptx::mma_ts_c<true>(tmem_O, tmem_S + kk * 8, ptx::make_desc(v_lo + kk * (2048 >> 4), kDescHiK), kIdescPV);
                     }
-                    __syncwarp();
+                    if (qk) {
+                        issue_qk(k_st, 0);
+                        ptx::tc_commit(ptx::smem_u32(&ctrl->sa_full[t]));
+                    }
+                    ptx::mbar_arrive(b_other);  // the other tile's turn
+                    if (qk) ptx::tc_commit(b_empty0 + 8 * k_st);
+                    if (pv) ptx::tc_commit(b_empty0 + 8 * v_st);
+                    // behind the item's last Q K^T the next Q_t may land; behind its last P V the output is complete
+                    if (s == n - 1 && exists) ptx::tc_commit(ptx::smem_u32(&ctrl->q_empty[t]));
+                    if (last && exists) ptx::tc_commit(ptx::smem_u32(&ctrl->o_full[t]));
                     if (pv) acc = 1u;
                     pend = flags;
                     flags = flags_next;
+                    flags_next = flags_after;
                 }
                 if (exists) ++n_it;
             }
             if (*abort_flag) {
                 // MMAs that were issued must retire before tensor memory is given back
-                if (lane == 0) {
-                    ptx::tc_commit(ptx::smem_u32(&ctrl->drain[t]));
-                    drain_bar(ptx::smem_u32(&ctrl->drain[t]), 0);
-                }
+                ptx::tc_commit(ptx::smem_u32(&ctrl->drain[t]));
+                drain_bar(ptx::smem_u32(&ctrl->drain[t]), 0);
             }
         }
         __syncwarp();
