@@ -220,13 +220,14 @@ int clear_qk_norm_rope(const void *q_in, const void *k_in, void *q_out, void *k_
 float clear_log_scale_factor(long long n_tokens, long long n_train_tokens);
 
 /* The backward pass for bf16 tensors on the tensor cores (head_dim 64 or 128, scale > 0): same arguments and
- * results as clear_attn_bwd_bf16, computed with tcgen05 MMAs over the forward pass's tile schedule -- a launch of
- * the forward kernel that keeps row statistics and dO . O instead of O, a launch in which every 128-query tile meets its
- * key tiles (dQ) and a launch in which every 128-key tile meets the query tiles that see it (dK, dV; Eq. 3's mask is symmetric, so
- * these are the same lists).  P and dS enter the MMAs rounded to bf16, as P does in the forward pass: gradients
- * agree with the exact ones to about 1e-2 of the largest gradient of the tensor.  One writer per element: results
- * repeat bit for bit.  The first call for a shape allocates its schedule tables, 8 bytes per token and (b, h), and
- * where long text rows are split the forward pass's workspace.
+ * results as clear_attn_bwd_bf16, computed with tcgen05 MMAs over the forward pass's tile schedule -- a launch in
+ * which every 128-query tile meets its key tiles (row statistics and delta = sum_j p_ij d_out_i . v_j in a first sweep, dQ in
+ * a second; with few heads the first sweep is a launch of its own) and a launch in which every 128-key tile meets the query
+ * tiles that see it (dK, dV; Eq. 3's mask is symmetric, so these are the same lists).  P and dS enter the MMAs rounded to
+ * bf16, as P does in the forward pass; statistics and delta are fp32 sums of the unrounded P.  Gradients agree with the exact
+ * ones to about 1e-2 of the largest gradient of the tensor.  One writer per element: results repeat bit for bit.  The
+ * first call for a shape allocates its schedule tables, 8 bytes per token and (b, h), and with few heads 16 KB per text tile
+ * and (b, h).
  * Errors: INVALID_ARG, MISALIGNED, UNSUPPORTED (other head sizes, scale <= 0), CUDA; a kernel whose bounded wait
  * expired is found by clear_cache_check. */
 int clear_attn_bwd_bf16_tc(const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,

@@ -45,6 +45,7 @@ int free_device_parts(clear_plan *p)
     };
     rel(p->d_half_width);
     rel(p->d_items);
+    rel(p->d_stat_items);
     rel(p->d_tiles);
     rel(p->d_pair_items);
     rel(p->d_pair_steps);
@@ -63,6 +64,7 @@ int free_device_parts(clear_plan *p)
     }
     p->d_half_width = nullptr;
     p->d_items = nullptr;
+    p->d_stat_items = nullptr;
     p->d_tiles = nullptr;
     p->d_pair_items = nullptr;
     p->d_pair_steps = nullptr;
@@ -104,14 +106,9 @@ int create_plan(clear_plan_t **out, const Shape &shape_in, bool host_only)
                 p->sch = Schedule();
             }
         }
-        if (s.backward) {
+        if (s.backward)
             build_backward_schedule(s, p->sch);
-            if (p->sch.pair_overflow) {  // lists too long for the forward kernel: the CUDA-core backward pass
-                kernel = CLEAR_KERNEL_SIMT;
-                p->sch = Schedule();
-            }
-        }
-        if (kernel == CLEAR_KERNEL_TCGEN05 && !s.backward)
+        else if (kernel == CLEAR_KERNEL_TCGEN05)
             build_tile_schedule(s, p->sch);
         else if (kernel == CLEAR_KERNEL_SIMT)
             build_geometry(s, p->sch);
@@ -128,6 +125,7 @@ int create_plan(clear_plan_t **out, const Shape &shape_in, bool host_only)
         CLEAR_CUDA_TRY(cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, p->device));
         rc = upload(&p->d_half_width, p->sch.half_width);
         if (rc == CLEAR_OK) rc = upload(&p->d_items, p->sch.items);
+        if (rc == CLEAR_OK) rc = upload(&p->d_stat_items, p->sch.stat_items);
         if (rc == CLEAR_OK) rc = upload(&p->d_tiles, p->sch.tiles);
         if (rc == CLEAR_OK) rc = upload(&p->d_pair_items, p->sch.pair_items);
         if (rc == CLEAR_OK) rc = upload(&p->d_pair_steps, p->sch.pair_steps);
@@ -378,7 +376,7 @@ static int backward(const void *q, const void *k, const void *v, const void *d_o
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         std::lock_guard<std::mutex> lock(plan->launch_mutex);
         if (plan->has_last && plan->last_stream != st) CLEAR_CUDA_TRY(cudaStreamWaitEvent(st, plan->ev_last, 0));
-        const int rc2 = plan->kernel != CLEAR_KERNEL_SIMT ? launch_bwd_tc(*plan, q, k, v, d_out, dq, dk, dv, scale, st)
+        const int rc2 = tensor_cores ? launch_bwd_tc(*plan, q, k, v, d_out, dq, dk, dv, scale, st)
                                      : launch_bwd(*plan, q, k, v, d_out, dq, dk, dv, scale, st);
         if (rc2 != CLEAR_OK) return rc2;
         CLEAR_CUDA_TRY(cudaEventRecord(plan->ev_last, st));
@@ -686,6 +684,8 @@ int clear_plan_check(clear_plan_t *plan, void *stream)
         g_last_device_status = status;
         // a block that gave up may have left the work queue of the persistent kernel mid-way
         CLEAR_CUDA_TRY(cudaMemsetAsync(plan->d_status, 0, kStatusWords * sizeof(int), cs));
+        // ... and the tensor-core backward pass its counts of finished parts
+        if (plan->d_bwd_stats) CLEAR_CUDA_TRY(cudaMemsetAsync(plan->d_bwd_stats, 0, plan->bwd_stats_bytes, cs));
         CLEAR_CUDA_TRY(cudaStreamSynchronize(cs));
         return CLEAR_ERR_DEVICE_TIMEOUT;
     }

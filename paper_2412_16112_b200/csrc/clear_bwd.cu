@@ -249,7 +249,8 @@ int ensure_bwd_stats(const clear_plan &p)
     if (p.d_bwd_stats) return CLEAR_OK;
     const Shape &s = p.shape;
     const int64_t N = (int64_t)s.n_text + (int64_t)s.grid_h * s.grid_w;
-    cudaError_t e = cudaMalloc((void **)&p.d_bwd_stats, (size_t)s.B * s.H * N * 3 * sizeof(float));
+    p.bwd_stats_bytes = (size_t)s.B * s.H * N * 3 * sizeof(float);
+    cudaError_t e = cudaMalloc((void **)&p.d_bwd_stats, p.bwd_stats_bytes);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? CLEAR_ERR_NO_MEMORY : CLEAR_ERR_CUDA;

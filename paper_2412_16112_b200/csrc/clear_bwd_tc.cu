@@ -2,15 +2,23 @@
 // dV for an upstream gradient dO of  O = softmax(scale Q K^T + log M) V  (Eq. 1 under the mask of Eq. 3), the step
 // through which the distillation losses of Sec. 3.3 (Eq. 4-6) reach the attention parameters.
 //
-// The row statistics come from the forward kernel (clear_ws.cu): per query m' = maximum + log2(row sum), in log2 units with
-// the scale included, so that P = 2^(c S - m') is normalised, and delta = dO . O.  Then one kernel, two roles; a CTA runs
-// one work item of the forward tile schedule: a STATIONARY tile of 128 tokens (an 8 x 16 patch of the grid, or 128 text
-// tokens) against the list of 128-token tiles the schedule gives it.  Eq. 3's mask is symmetric, so the list of key tiles a
-// query tile sees is also the list of query tiles that see it as keys.
-//   query role  stationary Q_i, dO_i; streamed K_j, V_j.  S = Q K^T, dP = dO V^T; dS = P (dP - delta) as bf16 over S;
-//               dQ += dS K (dS the tensor-memory operand, K read MN-major from the same shared-memory tile).
+// One kernel, three roles, launched one after the other; a CTA runs one work item of the forward tile schedule: a STATIONARY
+// tile of 128 tokens (an 8 x 16 patch of the grid, or 128 text tokens) against the list of 128-token tiles the schedule gives
+// it.  Eq. 3's mask is symmetric, so the list of key tiles a query tile sees is also the list of query tiles that see it as
+// keys.
+//   statistics  stationary Q_i, dO_i; streamed K_j, V_j.  S = Q K^T, dP = dO V^T; per query m' = maximum + log2(row sum), in
+//               log2 units with the scale included, so that P = 2^(c S - m') is normalised, and delta = sum_j P dP, in fp32
+//               from the unrounded P.  (dO . O from the forward kernel comes with the rounding of its P to bf16: where the dP
+//               of a row have a common part, which dP - delta takes away, dQ and dK came out up to six times worse.)
+//   query role  the same tiles: dS = P (dP - delta) as bf16 over S; dQ += dS K (dS the tensor-memory operand, K read MN-major
+//               from the same shared-memory tile).
 //   key role    stationary K_j, V_j; streamed Q_i, dO_i with the statistics of the queries i.  S^T = K Q^T,
 //               dP^T = V dO^T; P^T and dS^T as bf16 over them; dV += P^T dO, dK += dS^T Q.
+// The statistics are a first sweep of the query role over its list, unless a text tile, which sees every token, has more than
+// an even share of all tiles over the SMs (few heads): then they are a launch of their own, in which the lists of the text
+// tiles are cut over up to kStatParts CTAs, the last of which merges, and the other two roles run side by side behind it.
+// 24 heads: 1024 px, radius 8 424 us a call in sweeps (433 in launches), 2048 px, radius 16 2288 (2332); two heads at
+// 128 x 128, radius 8: 470 in sweeps, 266 in launches.
 // A streamed tile is taken in two halves of 64 tokens, each with a buffer of its own in tensor memory (T1 | T2, 64 columns
 // each), so the products of the next half run while the elementwise step of this one does; the accumulations of a half
 // go behind them on the same pipe.  The order on the pipe is T(0), T(1), ACC(0), T(2), ACC(1), ...: a half's products
@@ -21,9 +29,8 @@
 // tile.  The query role has 128 tensor-memory columns to spare and keeps its stationary operands there: 1024 + 512,
 // measured 2000.  The elementwise step (16 warps, 32 columns a thread) takes 700 (query) or 830 (key role) a half.
 // Around the list go 4500 clocks from the block's start to its first products and 3000 behind its last ones.
-// 1024 px, radius 8, 24 heads of 128: 384 us a call; with one lane's votes and waits between the MMAs, a tile of one tensor
-// a ring stage, statistics read one by one and rows stored by threads it was 487, before that (P and dS of whole tiles,
-// statistics in a sweep of the query role) 873.
+// A step of the statistics sweep takes 2200 clocks a tile (1024 of products, 1024 of exponentials).
+// 1024 px, radius 8, 24 heads of 128: 424 us a call; with P and dS of whole tiles in turn with the MMAs it was 873.
 //   warp 0: TMA loads; warp 1: every MMA; warp 2 (key role): statistics of the streamed tiles; warps 4..19: rows.
 // Every output element has one writer and a fixed order of summation.  Every wait is bounded: on expiry the CTA raises the
 // plan's status word and leaves.
@@ -59,7 +66,12 @@ struct BwdParams {
     int n_items, n_first, n_bh;  // the first n_first items (the longest) of every head come before all others
     long long n_tokens;
     float scale, scale_log2;   // scale, scale * log2(e)
-    const float2 *stats;       // [bh][token]: m', delta
+    float2 *stats;             // [bh][token]: m', delta
+    // statistics of text tiles whose lists are cut: [bh][tile][part][128] maximum, row sum, sum of p dP; finished parts [bh][tile]
+    float4 *parts;
+    int *part_count;
+    int n_parts, n_part_slots;
+    int key_waits;             // key role: the launch before it leaves the statistics
     int *status;
 };
 // Views of a tensor: whole tiles (patches of the image part, runs of text tokens) and half ones (patches, runs of tokens).
@@ -79,7 +91,8 @@ struct BwdCtrl {
         col_empty[kColStages], a_moved, out_ready, drain;
     alignas(16) float4 col[kColStages][64];   // key role: -m', -m', -delta, -delta of two columns of the streamed tile
     uint32_t tmem_base;
-    int abort_flag, skip;
+    int abort_flag, merge;
+    int skip;   // 1: leave at once; 2: leave, with the first copies under way
 };
 
 __device__ __noinline__ uint32_t bwd_tick(uint32_t t0, volatile int *abort_flag, int *status, int code)
@@ -111,10 +124,32 @@ __device__ __noinline__ void bwd_drain(uint32_t bar, uint32_t parity)
     }
 }
 
-template <int D, bool KEY_ROLE>
+enum Role { kStats, kQuery, kStatsQuery, kKey };   // kStatsQuery: both sweeps in one CTA
+// Running statistics of a row: maximum (log2 units), row sum and sum of p dP relative to it.
+struct RowStat {
+    float m, l, d;
+    __device__ __forceinline__ void start()
+    {
+        m = -INFINITY;
+        l = d = 0.f;
+    }
+    __device__ __forceinline__ void add(float m2, float l2, float d2)
+    {
+        const float m_new = fmaxf(m, m2), m_ref = m_new == -INFINITY ? 0.f : m_new;
+        const float a = ptx::ex2(m - m_ref), b = ptx::ex2(m2 - m_ref);   // -inf: 0
+        l = fmaf(b, l2, a * l);
+        d = fmaf(b, d2, a * d);
+        m = m_new;
+    }
+    // l >= 1 for every row that exists: it sees itself or the text (a NaN stays one)
+    __device__ __forceinline__ float2 result() const { return l == 0.f ? make_float2(0.f, 0.f) : make_float2(m + log2f(l), d / l); }
+};
+
+template <int D, Role ROLE>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant__ BwdParams prm)
 {
+    constexpr bool KEY_ROLE = ROLE == kKey, STATS = ROLE == kStats || ROLE == kStatsQuery, GRAD = ROLE != kStats;
     constexpr int kHalves = D / 64;                 // 64-channel (128-byte) column blocks of a tile
     constexpr uint32_t kHalfBytes = 128 * 128;      // 128 rows x 128 B
     constexpr uint32_t kTileBytes = kHalves * kHalfBytes;   // also a stage: two tensors, 64 rows
@@ -134,7 +169,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                    b_moved = ptx::smem_u32(&ctrl->a_moved);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (!KEY_ROLE) ptx::grid_launch_dependents();
+    if (STATS) ptx::grid_launch_dependents();
     int bh, item_id;
     if ((int)blockIdx.x < prm.n_first * prm.n_bh) {
         item_id = (int)blockIdx.x / prm.n_bh;
@@ -146,7 +181,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
     }
     const clear_work_item_t item = prm.items[item_id];
     const clear_kv_tile_t *tiles = prm.tiles + item.tile_begin;
-    const int n_tiles = item.tile_count;
+    const int n_tiles = item.tile_count, n_iters = ROLE == kStatsQuery ? 2 * n_tiles : n_tiles;   // steps of all sweeps
     const bool is_text = item.kind == 1;
 
     // row of the stationary tile that a thread of the row warps works on
@@ -167,7 +202,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
     // once any CTA of this plan has given up, the rest of the grid leaves at once; a window that is not 1024-byte
     // aligned (never expected) cannot hold swizzled tiles
     if (tid == 0) {
-        int skip = *reinterpret_cast<volatile int *>(prm.status);
+        int skip = *reinterpret_cast<volatile int *>(prm.status) != 0 ? 1 : 0;
         if ((s0 & 1023u) != 0u) {
             atomicCAS(prm.status, 0, 100);
             skip = 1;
@@ -203,6 +238,13 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             load_half(t, 1, 1);
         }
     }
+    if (ROLE == kQuery) {
+        // Up to here beside the last CTAs of the statistics launch.  The key role may follow from here on: once every CTA of
+        // this role has come this far, the statistics of all rows are there.
+        ptx::grid_wait();
+        ptx::grid_launch_dependents();
+        if (tid == 0 && ctrl->skip == 0 && *reinterpret_cast<volatile int *>(prm.status) != 0) ctrl->skip = 2;
+    }
     if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_u32(&ctrl->tmem_base), kBwdTmemCols);
         ptx::tmem_relinquish();
@@ -211,21 +253,27 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = ctrl->tmem_base, tmem_A1 = tmem + 256, tmem_A2 = tmem + 384;  // query role: q | dO in A2's place
-    if (ctrl->skip != 0) {
+    uint32_t n_loads = 2;   // halves that the loader has asked for
+    const int skip = ctrl->skip;
+    if (skip == 1) {
         if (warp == 1) ptx::tmem_dealloc(tmem, kBwdTmemCols);
         if (KEY_ROLE) ptx::grid_wait();
         return;
     }
 
-    if (warp < 4) {
+    if (skip == 2) {
+        // the statistics launch gave up: only the copies under way are left to wait for
+    } else if (warp < 4) {
         if (warp == 0 && lane == 0) {
             // ================= loader ===========================================================================
-            uint32_t n_loads = 2, stage = 2, par = 0;
+            uint32_t stage = 2, par = 0;
             bool ok = true;
-            clear_kv_tile_t t = tiles[min(1, n_tiles - 1)];
+            int next = n_tiles > 1 ? 1 : 0;   // the list is walked once a sweep
+            clear_kv_tile_t t = tiles[next];
 #pragma unroll 1
-            for (int i = 1; i < n_tiles && ok; ++i) {
-                const clear_kv_tile_t t_next = tiles[min(i + 1, n_tiles - 1)];
+            for (int it = 1; it < n_iters && ok; ++it) {
+                if (++next >= n_tiles) next = 0;
+                const clear_kv_tile_t t_next = tiles[next];
 #pragma unroll 1
                 for (int h = 0; h < 2; ++h) {
                     if (!KEY_ROLE && n_loads == kAStage) ok = bwd_wait(b_moved, 0, abort_flag, prm.status, 9);
@@ -239,14 +287,6 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                     }
                 }
                 t = t_next;
-            }
-            if (*abort_flag) {
-                // leave no copy in flight: whatever was issued must land before the block exits
-                bwd_drain(b_a, 0);
-                for (uint32_t j = 0; j < kStages && j < n_loads; ++j) {
-                    const uint32_t idx = n_loads - 1 - j;
-                    bwd_drain(b_full0 + 8 * (idx % kStages), (idx / kStages) & 1u);
-                }
             }
         } else if (warp == 1) {
             // ================= every MMA, all from one lane ==========================================================
@@ -270,7 +310,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                     return st;
                 };
                 // T1, T2 of a half: D / 16 MMAs of 16 channels each
-                auto issue_t = [&](uint32_t st, int half) {
+                auto issue_t = [&](uint32_t st, int half, bool grad) {
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const uint32_t d = tmem + half * 128 + j * 64, a = a_lo0 + j * kTile16, b = bk_lo0 + st * kTile16 + j * kSub16;
@@ -290,7 +330,9 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                         }
                     }
                     ptx::tc_commit(ptx::smem_u32(&ctrl->t_full[half]));
+                    if (!grad) ptx::tc_commit(b_empty0 + 8 * st);   // nothing else reads the half
                 };
+                auto is_grad = [&](int it) { return GRAD && (ROLE != kStatsQuery || it >= n_tiles); };
                 // 4 MMAs over 16 streamed tokens each (16 rows of 128 bytes = 2048 bytes), B read MN-major; the bf16 columns
                 // of the two row groups start at the groups' own fp32 columns
                 auto issue_acc = [&](uint32_t st, int half, uint32_t before) {
@@ -311,28 +353,28 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 uint32_t st0 = wait_half(), st1 = 0;
                 if (ok) {
                     ptx::tc_fence_after();
-                    issue_t(st0, 0);
+                    issue_t(st0, 0, is_grad(0));
                     st1 = wait_half();
                 }
 #pragma unroll 1
-                for (int i = 0; i < n_tiles && ok; ++i) {
-                    const uint32_t par = (uint32_t)i & 1u;
-                    const bool more = i + 1 < n_tiles;
+                for (int it = 0; it < n_iters && ok; ++it) {
+                    const uint32_t par = (uint32_t)it & 1u;
+                    const bool more = it + 1 < n_iters, grad = is_grad(it);
                     ptx::tc_fence_after();
-                    issue_t(st1, 1);
+                    issue_t(st1, 1, grad);
                     const uint32_t st2 = more ? wait_half() : 0u;
-                    // the rows have read T1, T2 of a half and put P / dS over them
+                    // the rows have read T1, T2 of a half and put P / dS over them (statistics: only read them)
                     ok = ok && bwd_wait(b_p0, par, abort_flag, prm.status, 4);
                     if (!ok) break;
                     ptx::tc_fence_after();
-                    issue_acc(st0, 0, i > 0 ? 1u : 0u);
-                    if (more) issue_t(st2, 0);
+                    if (grad) issue_acc(st0, 0, it > n_iters - n_tiles ? 1u : 0u);
+                    if (more) issue_t(st2, 0, is_grad(it + 1));
                     const uint32_t st3 = more ? wait_half() : 0u;
                     ok = ok && bwd_wait(b_p1, par, abort_flag, prm.status, 4);
                     if (!ok) break;
                     ptx::tc_fence_after();
-                    issue_acc(st1, 1, 1u);
-                    if (!more) ptx::tc_commit(b_acc);
+                    if (grad) issue_acc(st1, 1, 1u);
+                    if (GRAD && !more) ptx::tc_commit(b_acc);
                     st0 = st2;
                     st1 = st3;
                 }
@@ -347,6 +389,13 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             // (a column that does not exist is masked; its address stays inside the buffer, which is padded by one tile)
             const float2 *stats = prm.stats + (long long)bh * prm.n_tokens;
             bool ok = true;
+            if (prm.key_waits) {
+                // the query role leaves the statistics, and may still be at work; the rest of this CTA has started beside
+                // its last ones.  If it has given up there are none, and the CTA leaves without a result.
+                ptx::grid_wait();
+                ok = *reinterpret_cast<volatile int *>(prm.status) == 0;
+                if (!ok) *abort_flag = 1;
+            }
 #pragma unroll 1
             for (int i = 0; i < n_tiles && ok; ++i) {
                 const uint32_t st = (uint32_t)i % kColStages, use = (uint32_t)i / kColStages;
@@ -358,7 +407,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                     const long long tok = (t.flags & CLEAR_TILE_LINEAR)
                                               ? (long long)t.x + c
                                               : prm.n_text + (long long)min(t.y + (c >> 4), prm.grid_h - 1) * prm.grid_w + t.x + (c & 15);
-                    v[j] = __ldg(stats + tok);
+                    v[j] = __ldcg(stats + tok);
                 }
                 ok = __all_sync(0xffffffffu, bwd_wait(ptx::smem_u32(&ctrl->col_empty[st]), (use & 1u) ^ 1u, abort_flag, prm.status, 5));
                 if (!ok) break;
@@ -406,8 +455,6 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 if (lane == 0) ptx::mbar_arrive(b_moved);
             }
         }
-        float2 row_stat = make_float2(0.f, 0.f);
-        if (!KEY_ROLE && row_valid) row_stat = prm.stats[(long long)bh * prm.n_tokens + row_token];
         // mask bits of this row for its 32 columns of a tile (bit j = column allowed; the mask is symmetric, so the row's
         // token plays the query whichever role the kernel runs in)
         auto mask_word = [&](const clear_kv_tile_t &t) -> uint32_t {
@@ -431,17 +478,121 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             return bits;
         };
         const uint32_t b_t = ptx::smem_u32(&ctrl->t_full[half]), b_p = ptx::smem_u32(&ctrl->p_ready[half]);
-        const uint64_t c2 = ptx::pack2(c, c), row_nm = ptx::pack2(-row_stat.x, -row_stat.x),
-                       row_nd = ptx::pack2(-row_stat.y, -row_stat.y);
+        const uint64_t c2 = ptx::pack2(c, c);
         // tile records two ahead, mask words one ahead
         clear_kv_tile_t t_next = tiles[min(1, n_tiles - 1)];
         uint32_t mw_next = mask_word(tiles[0]);
-        uint32_t col_st = 0, col_par = 0;
-#pragma unroll 1
-        for (int i = 0; i < n_tiles && alive; ++i) {
+        auto next_mask = [&](int i) -> uint32_t {
             const uint32_t mw = mw_next;
             mw_next = mask_word(t_next);
             t_next = tiles[min(i + 2, n_tiles - 1)];
+            return mw;
+        };
+        float2 row_stat = make_float2(0.f, 0.f);
+        if constexpr (STATS) {
+            // ---- online softmax over the thread's own columns: maximum (log2 units), row sum, sum of p dP ----
+            float m = -INFINITY, l = 0.f, dl = 0.f;
+#pragma unroll 1
+            for (int i = 0; i < n_tiles && alive; ++i) {
+                const uint32_t mw = next_mask(i);
+                if (!__all_sync(0xffffffffu, bwd_wait(b_t, (uint32_t)i & 1u, abort_flag, prm.status, 12))) {
+                    alive = false;
+                    break;
+                }
+                ptx::tc_fence_after();
+                uint32_t s[32], gg[32];
+                ptx::tmem_ld32(tmem_T1, s);
+                ptx::tmem_ld32(tmem_T2, gg);
+                ptx::tmem_wait_ld();
+                // nothing is written back: the next products may land as soon as these have been read
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(b_p);
+                if (__any_sync(0xffffffffu, mw != 0xffffffffu)) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (!((mw >> j) & 1u)) s[j] = 0xff800000u;   // -inf
+                }
+                float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+                for (int j = 0; j < 32; j += 2) {
+                    mx[(j >> 1) & 1] = ptx::max3(mx[(j >> 1) & 1], __uint_as_float(s[j]), __uint_as_float(s[j + 1]));
+                }
+                const float m_new = fmaxf(m, fmaxf(mx[0], mx[1]) * c), m_ref = m_new == -INFINITY ? 0.f : m_new;
+                const float alpha = ptx::ex2(m - m_ref);   // m = -inf: 0
+                m = m_new;
+                const uint64_t nm2 = ptx::pack2(-m_ref, -m_ref);
+                uint64_t l2 = ptx::pack2(l * alpha, 0.f), d2 = ptx::pack2(dl * alpha, 0.f);
+#pragma unroll
+                for (int j = 0; j < 32; j += 2) {
+                    float x0, x1;
+                    ptx::unpack2(ptx::fma2(ptx::pack2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])), c2, nm2), x0, x1);
+                    const uint64_t p2 = ptx::pack2(ptx::ex2(x0), ptx::ex2(x1));
+                    l2 = ptx::add2(l2, p2);
+                    d2 = ptx::fma2(p2, ptx::pack2(__uint_as_float(gg[j]), __uint_as_float(gg[j + 1])), d2);
+                }
+                float a, b;
+                ptx::unpack2(l2, a, b);
+                l = a + b;
+                ptx::unpack2(d2, a, b);
+                dl = a + b;
+            }
+            t_next = tiles[min(1, n_tiles - 1)];
+            mw_next = mask_word(tiles[0]);
+            // the four threads of a row meet in tensor memory, in columns that the accumulation takes over afterwards (its
+            // first MMA waits for rows that have passed the second barrier)
+            ptx::tmem_st4(tmem_A1 + lane_off + 4 * g, __float_as_uint(m), __float_as_uint(l), __float_as_uint(dl), 0u);
+            ptx::tmem_wait_st();
+            ptx::tc_fence_before();
+            ptx::named_barrier(1, 32 * kRowWarps);
+            ptx::tc_fence_after();
+            uint32_t part[16];
+            ptx::tmem_ld16(tmem_A1 + lane_off, part);
+            ptx::tmem_wait_ld();
+            if constexpr (GRAD) {
+                ptx::tc_fence_before();
+                ptx::named_barrier(1, 32 * kRowWarps);
+                ptx::tc_fence_after();
+            }
+            RowStat st;
+            st.start();
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                st.add(__uint_as_float(part[4 * u]), __uint_as_float(part[4 * u + 1]), __uint_as_float(part[4 * u + 2]));
+            if (g == 0) {
+                if (item.partial_slot < 0) {
+                    if (row_valid && alive) prm.stats[(long long)bh * prm.n_tokens + row_token] = st.result();
+                } else {
+                    // a part of a text tile's list: whichever CTA leaves the last part merges them, in their order
+                    const int tile0 = item.partial_slot / prm.n_parts * prm.n_parts;
+                    float4 *parts = prm.parts + ((long long)bh * prm.n_part_slots + tile0) * 128 + r;
+                    __stcg(parts + (item.partial_slot - tile0) * 128, make_float4(st.m, st.l, st.d, 0.f));
+                    __threadfence();
+                    ptx::named_barrier(2, 128);   // (every warp of the group comes here, also one that has given up)
+                    int *count = prm.part_count + bh * (prm.n_part_slots / prm.n_parts) + tile0 / prm.n_parts;
+                    if (r == 0) ctrl->merge = *abort_flag == 0 && atomicAdd(count, 1) == prm.n_parts - 1 ? 1 : 0;
+                    ptx::named_barrier(2, 128);
+                    if (ctrl->merge != 0) {
+                        __threadfence();
+                        st.start();
+                        for (int u = 0; u < prm.n_parts; ++u) {
+                            const float4 x = __ldcg(parts + u * 128);
+                            st.add(x.x, x.y, x.z);
+                        }
+                        if (row_valid) prm.stats[(long long)bh * prm.n_tokens + row_token] = st.result();
+                        if (r == 0) *count = 0;   // for the next call
+                    }
+                }
+            }
+            row_stat = st.result();
+        }
+        if (ROLE == kQuery && row_valid) row_stat = __ldcg(prm.stats + (long long)bh * prm.n_tokens + row_token);
+        const uint64_t row_nm = ptx::pack2(-row_stat.x, -row_stat.x), row_nd = ptx::pack2(-row_stat.y, -row_stat.y);
+        const uint32_t it0 = ROLE == kStatsQuery ? (uint32_t)n_tiles : 0u;   // steps of the sweep before
+        uint32_t col_st = 0, col_par = 0;
+#pragma unroll 1
+        for (int i = 0; i < n_tiles && alive && GRAD; ++i) {
+            const uint32_t mw = next_mask(i);
             // warp-uniform outcome: the tcgen05.ld / st below need the whole warp
             bool got = true;
             if (KEY_ROLE) got = bwd_wait(ptx::smem_u32(&ctrl->col_full[col_st]), col_par, abort_flag, prm.status, 7);
@@ -462,7 +613,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 }
             };
             if (got) load_cols(0);
-            got = got && bwd_wait(b_t, (uint32_t)i & 1u, abort_flag, prm.status, 6);
+            got = got && bwd_wait(b_t, (it0 + (uint32_t)i) & 1u, abort_flag, prm.status, 6);
             if (!__all_sync(0xffffffffu, got)) {
                 alive = false;
                 break;
@@ -512,6 +663,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             }
         }
 
+        if constexpr (GRAD) {
         // ---- epilogue: after the last accumulation every group brings a quarter of the channels of its rows into shared
         // memory, which nothing reads any more, and a TMA store takes the tile from there (rows outside the tensor are
         // left out by its bounds).  Stored by the threads themselves, a row each, the key role's two tensors took
@@ -555,6 +707,7 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             }
             __syncwarp();
         }
+        }
     }
 
     ptx::tc_fence_before();
@@ -563,37 +716,66 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, kBwdTmemCols);
     }
-    if (KEY_ROLE) ptx::grid_wait();
+    if (tid == 0 && (skip == 2 || *abort_flag)) {
+        // leave no copy in flight: whatever was issued must land before the block exits (looked at only now: the block may
+        // give up after the loader has issued its last copy)
+        bwd_drain(b_a, 0);
+        for (uint32_t j = 0; j < kStages && j < n_loads; ++j) {
+            const uint32_t idx = n_loads - 1 - j;
+            bwd_drain(b_full0 + 8 * (idx % kStages), (idx / kStages) & 1u);
+        }
+    }
+    if (KEY_ROLE) ptx::grid_wait();   // the call is over when both roles are
 }
 
 template <int D>
 int launch_roles(const BwdViews &q, const BwdViews &k, const BwdViews &v, const BwdViews &g, const BwdOut &dq,
-                 const BwdOut &dk, const BwdOut &dv, const BwdParams &prm, cudaStream_t stream)
+                 const BwdOut &dk, const BwdOut &dv, const BwdParams &stat_prm, const BwdParams &prm, cudaStream_t stream)
 {
     constexpr size_t kSmem = 7 * (D / 64) * 16384 + sizeof(BwdCtrl);
-    static_assert(kKeyStages + 2 == 7 && kQueryStages == 7 && kSmem <= 232448, "both roles take seven tiles of shared memory");
-    auto kernel_q = clear_bwd_tc_kernel<D, false>;
-    auto kernel_k = clear_bwd_tc_kernel<D, true>;
-    CLEAR_CUDA_TRY(cudaFuncSetAttribute(kernel_q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
-    CLEAR_CUDA_TRY(cudaFuncSetAttribute(kernel_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
-    const unsigned grid = (unsigned)prm.n_items * (unsigned)prm.n_bh;
-    kernel_q<<<grid, kBwdThreads, kSmem, stream>>>(BwdMaps{{q, g}, {k, v}, {dq, dq}}, prm);
-    CLEAR_CUDA_TRY(cudaGetLastError());
-    // The roles share nothing but their inputs, so the key role's blocks may take the SMs that the query role's last blocks
-    // leave free (each of them ends only when the query role has).
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kBwdThreads);
-    cfg.dynamicSmemBytes = kSmem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    CLEAR_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel_k, BwdMaps{{k, v}, {q, g}, {dv, dk}}, prm));
-    CLEAR_CUDA_TRY(cudaGetLastError());
-    return CLEAR_OK;
+    static_assert(kKeyStages + 2 == 7 && kQueryStages == 7 && kSmem <= 232448, "all roles take seven tiles of shared memory");
+    // Each launch may start on the SMs that the one before leaves free (programmatic launches); what it waits for stands in
+    // the kernel.
+    auto run = [&](auto kernel, const BwdMaps &maps, const BwdParams &p, bool follows) -> int {
+        CLEAR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)p.n_items * (unsigned)p.n_bh);
+        cfg.blockDim = dim3(kBwdThreads);
+        cfg.dynamicSmemBytes = kSmem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = follows ? 1 : 0;
+        CLEAR_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, maps, p));
+        return CLEAR_OK;
+    };
+    int rc = CLEAR_OK;
+    if (prm.n_parts == 1) {
+        rc = run(clear_bwd_tc_kernel<D, kStatsQuery>, BwdMaps{{q, g}, {k, v}, {dq, dq}}, prm, false);
+    } else {
+        rc = run(clear_bwd_tc_kernel<D, kStats>, BwdMaps{{q, g}, {k, v}, {dq, dq}}, stat_prm, false);
+        if (rc == CLEAR_OK) rc = run(clear_bwd_tc_kernel<D, kQuery>, BwdMaps{{q, g}, {k, v}, {dq, dq}}, prm, true);
+    }
+    if (rc == CLEAR_OK) rc = run(clear_bwd_tc_kernel<D, kKey>, BwdMaps{{k, v}, {q, g}, {dv, dk}}, prm, true);
+    return rc;
+}
+
+// The text tiles, which see every token, lead the list unless the grid is tiny: that many items of every head come first.
+int count_first(const std::vector<clear_work_item_t> &items)
+{
+    size_t n = 0;
+    while (n < items.size() && items[n].kind == 1) ++n;
+    return n < items.size() ? (int)n : 0;
+}
+
+// Statistics of every row, and one tile of padding (those of columns past the end are read, and masked), to 256 bytes.
+size_t row_stats_bytes(const clear_plan &p)
+{
+    const Shape &s = p.shape;
+    const size_t rows = (size_t)s.B * s.H * ((size_t)s.n_text + (size_t)s.grid_h * s.grid_w) + kTileTokens;
+    return (rows * sizeof(float2) + 255) / 256 * 256;
 }
 
 }  // namespace
@@ -606,19 +788,19 @@ int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void 
     if (s.head_dim != 64 && s.head_dim != 128) return CLEAR_ERR_UNSUPPORTED;
     const uint64_t gw = (uint64_t)s.grid_w, gh = (uint64_t)s.grid_h, T = (uint64_t)s.n_text;
     const uint64_t N = T + gw * gh, BH = (uint64_t)s.B * s.H, halves = (uint64_t)s.head_dim / 64;
-    if (p.sch.items.size() * BH > (uint64_t)INT32_MAX) return CLEAR_ERR_UNSUPPORTED;
+    if (p.sch.stat_items.size() * BH > (uint64_t)INT32_MAX) return CLEAR_ERR_UNSUPPORTED;   // (no fewer than p.sch.items)
     if (!p.d_bwd_stats) {
-        // one tile of padding: the statistics of columns past the end are read (and masked), never used
-        const size_t bytes = ((size_t)BH * N + kTileTokens) * sizeof(float2);
+        // behind them the partial statistics of cut text tiles and the counts of their finished parts
+        const size_t slots = (size_t)BH * p.sch.n_stat_slots;
+        const size_t bytes = row_stats_bytes(p) + slots * (kTileTokens * sizeof(float4) + sizeof(int));
         cudaError_t e = cudaMalloc((void **)&p.d_bwd_stats, bytes);
         if (e == cudaSuccess) e = cudaMemsetAsync(p.d_bwd_stats, 0, bytes, stream);
         if (e != cudaSuccess) {
             (void)cudaGetLastError();
             return e == cudaErrorMemoryAllocation ? CLEAR_ERR_NO_MEMORY : CLEAR_ERR_CUDA;
         }
+        p.bwd_stats_bytes = bytes;
     }
-    const int rc = launch_ws_stats(p, q, k, v, d_out, p.d_bwd_stats, scale, stream);
-    if (rc != CLEAR_OK) return rc;
 
     // Per tensor four views of [BH][half][rows][cols][64]: the image part in patches of 8 x 16 and of 4 x 16, runs of 128
     // tokens of the text prefix (rows past the text read as zero) and of 64 tokens of the whole sequence.
@@ -646,6 +828,11 @@ int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void 
             return CLEAR_ERR_CUDA;
 
     BwdParams prm{};
+    prm.parts = reinterpret_cast<float4 *>(reinterpret_cast<char *>(p.d_bwd_stats) + row_stats_bytes(p));
+    prm.part_count = reinterpret_cast<int *>(prm.parts + (size_t)BH * p.sch.n_stat_slots * kTileTokens);
+    prm.n_parts = p.sch.n_stat_parts;
+    prm.n_part_slots = p.sch.n_stat_slots;
+    prm.key_waits = p.sch.n_stat_parts == 1;
     prm.items = p.d_items;
     prm.tiles = p.d_tiles;
     prm.mask_table = p.d_mask_table;
@@ -655,17 +842,19 @@ int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void 
     prm.grid_w = s.grid_w;
     prm.n_text = s.n_text;
     prm.n_items = (int)p.sch.items.size();
-    // items are sorted by length; the text tiles, which see every token, lead the list unless the grid is tiny
-    while (prm.n_first < prm.n_items && p.sch.items[(size_t)prm.n_first].kind == 1) ++prm.n_first;
-    if (prm.n_first == prm.n_items) prm.n_first = 0;
+    prm.n_first = count_first(p.sch.items);
     prm.n_bh = (int)BH;
     prm.n_tokens = (long long)N;
     prm.scale = scale;
     prm.scale_log2 = scale * 1.4426950408889634f;
-    prm.stats = reinterpret_cast<const float2 *>(p.d_bwd_stats);
+    prm.stats = reinterpret_cast<float2 *>(p.d_bwd_stats);
     prm.status = p.d_status;
-    if (s.head_dim == 128) return launch_roles<128>(views[0], views[1], views[2], views[3], outs[0], outs[1], outs[2], prm, stream);
-    return launch_roles<64>(views[0], views[1], views[2], views[3], outs[0], outs[1], outs[2], prm, stream);
+    BwdParams stat_prm = prm;
+    stat_prm.items = p.d_stat_items;
+    stat_prm.n_items = (int)p.sch.stat_items.size();
+    stat_prm.n_first = count_first(p.sch.stat_items);
+    if (s.head_dim == 128) return launch_roles<128>(views[0], views[1], views[2], views[3], outs[0], outs[1], outs[2], stat_prm, prm, stream);
+    return launch_roles<64>(views[0], views[1], views[2], views[3], outs[0], outs[1], outs[2], stat_prm, prm, stream);
 }
 
 }  // namespace clear

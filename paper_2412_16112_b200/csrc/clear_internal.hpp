@@ -37,6 +37,7 @@ struct clear_plan {
     // device tables (owned)
     int32_t *d_half_width = nullptr;
     clear_work_item_t *d_items = nullptr;
+    clear_work_item_t *d_stat_items = nullptr;
     clear_kv_tile_t *d_tiles = nullptr;
     clear_pair_item_t *d_pair_items = nullptr;
     clear_pair_step_t *d_pair_steps = nullptr;
@@ -63,6 +64,7 @@ struct clear_plan {
     float *d_partial_ml = nullptr;
     // backward pass: statistics per query row, allocated on the plan's first backward call
     mutable float *d_bwd_stats = nullptr;
+    mutable size_t bwd_stats_bytes = 0;
     int64_t workspace_bytes = 0;
 
     // staging buffers of the host-tensor entry point (owned, allocated on first use)
@@ -116,18 +118,13 @@ int launch_text_merge(const float *records, int n_parts, int n_bh, int n_text, i
 int launch_qk_prep(const void *q_in, const void *k_in, void *q_out, void *k_out, const float *gain_q, const float *gain_k,
                    int n_bh, int grid_h, int grid_w, int n_text, int head_dim, int dtype, const int axes_dim[3],
                    double theta, double ntk_factor, float eps, float q_factor, cudaStream_t stream);
-// Backward pass on the tensor cores (bf16): the forward kernel for the row statistics, then a query-role and a key-role
-// launch over the plan's tile schedule (a plan made with Shape::backward).
+// Backward pass on the tensor cores (bf16): a query-role and a key-role launch over the plan's tile schedule (a plan made
+// with Shape::backward).
 int launch_bwd_tc(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
                   void *dv, float scale, cudaStream_t stream);
 // Merge of the split-KV partial results of the text-query rows (both tensor-core kernels): bf16 rows of `out`, or, for
 // the text part of a band, one (O, m, l) record per text row.
 int launch_text_combine(const clear_plan &p, void *out, cudaStream_t stream);
-// The warp-specialised forward kernel as the backward pass needs it: per row its reference + log2(row sum) and dO . O
-// (float2 [BH][N]) instead of the output; and the merge of split text rows into the same.
-int launch_ws_stats(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *stats, float scale,
-                    cudaStream_t stream);
-int launch_text_stats(const clear_plan &p, const void *d_out, void *stats, cudaStream_t stream);
 
 // Tensor map (a CUtensorMap, 128 bytes) of a bf16 tensor of `rank` dims, innermost first, with 128-byte swizzle
 // and out-of-bounds elements read as zero; strides in bytes for dims 1..rank-1.  False if the driver refuses.

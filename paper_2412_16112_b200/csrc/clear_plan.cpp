@@ -564,13 +564,35 @@ void build_pair_schedule(const Shape &s, Schedule &sch)
 void build_backward_schedule(const Shape &s, Schedule &sch)
 {
     MaskTable masks(s, sch);
-    build_pairs(s, sch, masks);
-    if (sch.pair_overflow) return;
-    // text splits, and the workspace they need, are the pair schedule's
-    const int n_text_splits = sch.n_text_splits, n_partial_slots = sch.n_partial_slots;
     build_tiles(s, sch, &masks);
-    sch.n_text_splits = n_text_splits;
-    sch.n_partial_slots = n_partial_slots;
+    // The lists of the text tiles, which are the longest, cut as far as an even share of all tiles over the SMs asks for it
+    // (one part: the statistics need no launch of their own).
+    int64_t all = 0;
+    int longest = 0;
+    for (const clear_work_item_t &it : sch.items) {
+        all += it.tile_count;
+        if (it.kind == 1) longest = it.tile_count;
+    }
+    const int64_t share = std::max<int64_t>(kStatPartTiles, all * s.B * s.H / kSms);
+    int parts = (int)std::min<int64_t>(kStatParts, (longest + share - 1) / share);
+    const int chunk = parts > 1 ? (longest + parts - 1) / parts : longest;
+    parts = parts > 1 ? (longest + chunk - 1) / chunk : 1;
+    sch.n_stat_parts = parts;
+    sch.n_stat_slots = parts > 1 ? sch.n_text_tiles * parts : 0;
+    sch.stat_items.clear();
+    for (const clear_work_item_t &it : sch.items) {
+        if (it.kind != 1 || parts == 1) {
+            sch.stat_items.push_back(it);
+            continue;
+        }
+        for (int p = 0; p < parts; ++p) {
+            clear_work_item_t part = it;
+            part.tile_begin += p * chunk;
+            part.tile_count = std::min(chunk, it.tile_count - p * chunk);
+            part.partial_slot = it.qx / kTileTokens * parts + p;
+            sch.stat_items.push_back(part);
+        }
+    }
 }
 
 }  // namespace clear

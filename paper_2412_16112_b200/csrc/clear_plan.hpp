@@ -14,6 +14,9 @@ constexpr int kTileTokens = 128;
 constexpr int kSplitTargetTiles = 64;  // key tiles per split of a text-query tile
 constexpr int kMaxMaskEntries = 512;   // relative patch offsets with a precomputed mask (2 KB each)
 
+constexpr int kStatParts = 8, kStatPartTiles = 16;   // backward statistics: most parts of a text tile's list, fewest tiles of one
+constexpr int kSms = 148;              // of the one device this library is built for
+
 struct Shape {
     int B = 0, H = 0, grid_h = 0, grid_w = 0, n_text = 0, head_dim = 0;
     float radius = 0.f;
@@ -26,8 +29,7 @@ struct Shape {
     int part = 0;
     int q_row_begin = 0, q_row_end = 0;  // rows of the band inside the grid (band parts only)
     int text_keys = 1;                   // CLEAR_PART_BAND_TEXT: are the text tokens among the keys
-    int backward = 0;                    // both schedules: the tile schedule with one item per text tile over all its keys, whose
-                                         // masked image tiles name mask-table entries, and the pair schedule
+    int backward = 0;                    // the tile schedule as the tensor-core backward pass needs it
     bool operator==(const Shape &o) const
     {
         return B == o.B && H == o.H && grid_h == o.grid_h && grid_w == o.grid_w && n_text == o.n_text &&
@@ -42,6 +44,8 @@ struct Schedule {
     std::vector<int32_t> half_width;     // half_width[dy] = max |dx| allowed at row offset dy (the window, whatever its kind)
     std::vector<clear_work_item_t> items;
     std::vector<clear_kv_tile_t> tiles;
+    std::vector<clear_work_item_t> stat_items;   // backward pass: `items` with the lists of text tiles cut into n_stat_parts parts
+    int n_stat_parts = 1, n_stat_slots = 0;      // parts of all text tiles of one (b, h); 0: no list is cut
     std::vector<clear_pair_item_t> pair_items;   // TCGEN05_WS: text items first, then image items
     std::vector<clear_pair_step_t> pair_steps;
     int n_text_pair_items = 0;
@@ -70,7 +74,7 @@ void build_tile_schedule(const Shape &s, Schedule &sch);
 // Pair items and step lists of the warp-specialised tensor-core kernel (calls build_geometry first).
 void build_pair_schedule(const Shape &s, Schedule &sch);
 
-// Both for the backward pass (pair_overflow: the pair schedule was given up, and nothing else is built).
+// The tile schedule of the backward pass: one item per text tile over all its keys; masked image tiles name mask-table entries.
 void build_backward_schedule(const Shape &s, Schedule &sch);
 
 }  // namespace clear

@@ -401,13 +401,11 @@ clear_tc_kernel(const __grid_constant__ CUtensorMap tm_q_img, const __grid_const
 // w_s = 2^(m_s - max_s m_s).  One block per 32 text rows and (batch, head).  The partial results lie channel by channel
 // (128 rows each), so a warp reads 32 rows of a channel as 128 consecutive bytes; the finished rows are turned round in
 // shared memory and written along their channels.  kRecords: the merged row stays un-normalised, as D values followed
-// by its maximum and its sum (the record a band leaves for the merge over all bands).  kStats: instead of the row, what the
-// backward pass needs of it (out: [bh][token], maximum + log2(sum) and dO . O).
-enum CombineMode { kRows, kRecords, kStats };
-template <int D, CombineMode MODE>
+// by its maximum and its sum (the record a band leaves for the merge over all bands).
+template <int D, bool kRecords>
 __global__ void __launch_bounds__(256)
-clear_tc_combine_kernel(const float *__restrict__ partial_o, const float *__restrict__ partial_ml, void *__restrict__ out,
-                        const __nv_bfloat16 *__restrict__ d_out, int n_text, int64_t n_tokens, int n_splits, int n_slots)
+clear_tc_combine_kernel(const float *__restrict__ partial_o, const float *__restrict__ partial_ml, void *__restrict__ out, int n_text,
+                        int64_t n_tokens, int n_splits, int n_slots)
 {
     __shared__ float rows[32][D + 1];
     const int row0 = blockIdx.x * 32, bh = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -432,11 +430,11 @@ clear_tc_combine_kernel(const float *__restrict__ partial_o, const float *__rest
             for (int e = 0; e < kChannels; ++e) num[e] = fmaf(w, src[(warp * kChannels + e) * 128], num[e]);
         }
     }
-    const float inv = MODE == kRecords ? 1.f : den > 0.f ? 1.f / den : 0.f;
+    const float inv = kRecords ? 1.f : den > 0.f ? 1.f / den : 0.f;
 #pragma unroll
     for (int e = 0; e < kChannels; ++e) rows[lane][warp * kChannels + e] = num[e] * inv;
     __syncthreads();
-    if constexpr (MODE == kRecords) {
+    if constexpr (kRecords) {
         float *rec = static_cast<float *>(out) + ((int64_t)bh * n_text + row0) * (D + 2);
         if (warp == 0 && on) {
             rec[lane * (D + 2) + D] = m;
@@ -445,18 +443,6 @@ clear_tc_combine_kernel(const float *__restrict__ partial_o, const float *__rest
         for (int i = threadIdx.x; i < 32 * D; i += 256) {
             const int r = i / D, e = i % D;
             if (row0 + r < n_text) rec[r * (D + 2) + e] = rows[r][e];
-        }
-    } else if constexpr (MODE == kStats) {
-        __shared__ float lse[32];
-        if (warp == 0) lse[lane] = m + log2f(den);
-        __syncthreads();
-        for (int r = warp; r < 32 && row0 + r < n_text; r += 8) {
-            float dot = 0.f;
-            for (int e = lane; e < D; e += 32)
-                dot = fmaf(rows[r][e], __bfloat162float(d_out[((int64_t)bh * n_tokens + row0 + r) * D + e]), dot);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-            if (lane == 0) static_cast<float2 *>(out)[(int64_t)bh * n_tokens + row0 + r] = make_float2(lse[r], dot);
         }
     } else {
         for (int i = threadIdx.x; i < 32 * (D / 8); i += 256) {
@@ -523,33 +509,20 @@ int launch_variant(const clear_plan &p, const CUtensorMap *tm, const TcParams &p
 
 }  // namespace
 
-static int launch_combine(const clear_plan &p, CombineMode mode, void *out, const void *d_out, cudaStream_t stream)
+int launch_text_combine(const clear_plan &p, void *out, cudaStream_t stream)
 {
     const Shape &s = p.shape;
+    // the text part of a band leaves records for the merge over all bands instead of finished rows
+    const bool records = s.part == CLEAR_PART_BAND_TEXT;
+    if (p.sch.n_partial_slots <= 0) return records ? CLEAR_ERR_PLAN_MISMATCH : CLEAR_OK;
     if (s.head_dim != 64 && s.head_dim != 128) return CLEAR_ERR_UNSUPPORTED;
     const int64_t N = (int64_t)s.n_text + (int64_t)s.grid_h * s.grid_w;
     const dim3 grid((unsigned)((s.n_text + 31) / 32), (unsigned)(s.B * s.H));
-    auto pick = [&](auto rows, auto records, auto stats) { return mode == kRows ? rows : mode == kRecords ? records : stats; };
-    auto kernel = s.head_dim == 128
-                      ? pick(clear_tc_combine_kernel<128, kRows>, clear_tc_combine_kernel<128, kRecords>, clear_tc_combine_kernel<128, kStats>)
-                      : pick(clear_tc_combine_kernel<64, kRows>, clear_tc_combine_kernel<64, kRecords>, clear_tc_combine_kernel<64, kStats>);
-    kernel<<<grid, 256, 0, stream>>>(p.d_partial_o, p.d_partial_ml, out, static_cast<const __nv_bfloat16 *>(d_out), s.n_text, N,
-                                     p.sch.n_text_splits, p.sch.n_partial_slots);
+    auto kernel = s.head_dim == 128 ? (records ? clear_tc_combine_kernel<128, true> : clear_tc_combine_kernel<128, false>)
+                                    : (records ? clear_tc_combine_kernel<64, true> : clear_tc_combine_kernel<64, false>);
+    kernel<<<grid, 256, 0, stream>>>(p.d_partial_o, p.d_partial_ml, out, s.n_text, N, p.sch.n_text_splits, p.sch.n_partial_slots);
     CLEAR_CUDA_TRY(cudaGetLastError());
     return CLEAR_OK;
-}
-
-int launch_text_combine(const clear_plan &p, void *out, cudaStream_t stream)
-{
-    // the text part of a band leaves records for the merge over all bands instead of finished rows
-    const bool records = p.shape.part == CLEAR_PART_BAND_TEXT;
-    if (p.sch.n_partial_slots <= 0) return records ? CLEAR_ERR_PLAN_MISMATCH : CLEAR_OK;
-    return launch_combine(p, records ? kRecords : kRows, out, nullptr, stream);
-}
-
-int launch_text_stats(const clear_plan &p, const void *d_out, void *stats, cudaStream_t stream)
-{
-    return p.sch.n_partial_slots > 0 ? launch_combine(p, kStats, stats, d_out, stream) : CLEAR_OK;
 }
 
 int launch_tc(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale,

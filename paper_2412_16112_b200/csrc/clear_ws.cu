@@ -63,10 +63,6 @@ struct WsParams {
     int n_partial_slots;
     const __nv_bfloat16 *q, *k;
     __nv_bfloat16 *out;
-    // backward pass: the launch leaves statistics of the rows instead of `out` ([bh][token]: reference + log2(row sum),
-    // dO . O); null otherwise
-    const __nv_bfloat16 *d_out;
-    float2 *stats;
     int *status;  // [0] status word of this launch, [1] queue head, [2] finished blocks, [3] status kept for the host
 };
 
@@ -382,32 +378,6 @@ __device__ __noinline__ void store_tile(const WsParams &prm, uint32_t tmem_o, ui
     const bool on = n_rows >= 0 ? r < n_rows : (y < prm.grid_h && x < prm.grid_w);
     const long long token = n_rows >= 0 ? (long long)first_x + r : prm.n_text + (long long)y * prm.grid_w + x;
     __nv_bfloat16 *dst = prm.out + ((long long)bh * prm.n_tokens + token) * D;
-    if (prm.stats != nullptr) {
-        const __nv_bfloat16 *g = prm.d_out + ((long long)bh * prm.n_tokens + token) * D;
-        float dot = 0.f;
-#pragma unroll 1
-        for (int w = 0, n = opaque(D / 16); w < n; ++w) {
-            uint4 gv[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
-            if (on) {
-                gv[0] = __ldg(reinterpret_cast<const uint4 *>(g + 16 * w));
-                gv[1] = __ldg(reinterpret_cast<const uint4 *>(g + 16 * w) + 1);
-            }
-            uint32_t o[16];
-            ptx::tmem_ld16(tmem_o + 16 * w, o);
-            ptx::tmem_wait_ld();
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint4 &v = gv[j >> 2];
-                const uint32_t u = (j & 3) == 0 ? v.x : (j & 3) == 1 ? v.y : (j & 3) == 2 ? v.z : v.w;
-                dot = fmaf(__uint_as_float(o[2 * j]), __uint_as_float(u << 16), dot);
-                dot = fmaf(__uint_as_float(o[2 * j + 1]), __uint_as_float(u & 0xffff0000u), dot);
-            }
-        }
-        ptx::tc_fence_before();
-        warp_arrive(b_o_empty, lane);
-        if (on) prm.stats[(long long)bh * prm.n_tokens + token] = make_float2(ref + log2f(l), dot * inv);
-        return;
-    }
     const bool wide = (reinterpret_cast<uintptr_t>(prm.out) & 31u) == 0u;  // tensors are 16-byte aligned at least
 #pragma unroll 1
     for (int w = 0, n = opaque(D / 16); w < n; ++w) {
@@ -1055,12 +1025,12 @@ int launch_variant(const clear_plan &p, const WsMaps &maps, const WsParams &prm,
     const unsigned grid = (unsigned)std::min<long long>(n_sm, total);
     clear_ws_kernel<D><<<grid, kWsThreads, kSmem, stream>>>(maps, prm);
     CLEAR_CUDA_TRY(cudaGetLastError());
-    if (prm.stats != nullptr) return launch_text_stats(p, prm.d_out, prm.stats, stream);
     return launch_text_combine(p, prm.out, stream);
 }
 
-int launch(const clear_plan &p, const void *q, const void *k, const void *v, void *out, const void *d_out, void *stats, float scale,
-           cudaStream_t stream)
+}  // namespace
+
+int launch_ws(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale, cudaStream_t stream)
 {
     if (!(scale > 0.f)) return CLEAR_ERR_UNSUPPORTED;
     const long long total = (long long)p.sch.pair_items.size() * p.shape.B * p.shape.H;
@@ -1097,24 +1067,10 @@ int launch(const clear_plan &p, const void *q, const void *k, const void *v, voi
     prm.q = static_cast<const __nv_bfloat16 *>(q);
     prm.k = static_cast<const __nv_bfloat16 *>(k);
     prm.out = static_cast<__nv_bfloat16 *>(out);
-    prm.d_out = static_cast<const __nv_bfloat16 *>(d_out);
-    prm.stats = static_cast<float2 *>(stats);
     prm.status = p.d_status;
     if (p.shape.head_dim == 128) return launch_variant<128>(p, maps, prm, stream);
     if (p.shape.head_dim == 64) return launch_variant<64>(p, maps, prm, stream);
     return CLEAR_ERR_UNSUPPORTED;
-}
-
-}  // namespace
-
-int launch_ws(const clear_plan &p, const void *q, const void *k, const void *v, void *out, float scale, cudaStream_t stream)
-{
-    return launch(p, q, k, v, out, nullptr, nullptr, scale, stream);
-}
-int launch_ws_stats(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *stats, float scale,
-                    cudaStream_t stream)
-{
-    return launch(p, q, k, v, nullptr, d_out, stats, scale, stream);
 }
 
 }  // namespace clear

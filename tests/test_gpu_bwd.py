@@ -175,6 +175,8 @@ def test_tensor_core_backward_at_workload_sizes(name, heads):
     (24, 16, 64, 30.0, 128, None),   # four: one half more than the ring of the query role has stages
     (21, 33, 129, 9.0, 128, "0"),    # no mask table: every masked patch from the half widths
     (21, 33, 129, 9.0, 64, "2"),     # a table that runs out
+    (64, 72, 130, 2.0, 128, None),   # few heads: statistics in a launch of their own, 38 key tiles of a text tile in 3 parts
+    (48, 50, 300, 3.0, 64, None),    # three text tiles of 22 key tiles in 2 parts
 ])
 def test_tensor_core_backward_edges(gh, gw, T, r, d, cap, monkeypatch):
     """Ring lengths, halves outside the grid and table-free masks; the outputs start 16 but not 32 bytes off an aligned
@@ -198,6 +200,29 @@ def test_tensor_core_backward_edges(gh, gw, T, r, d, cap, monkeypatch):
         err = np.abs(got.cpu().double().numpy() - ref)
         assert err.max() <= _tc_bound(ref), f"{name}: max {err.max():.3e}"
         assert (buf[:pad] == 7.0).all() and (buf[pad + n:] == 7.0).all(), f"{name}: guard band"
+    clear.clear_cache_clear()
+
+
+@pytest.mark.parametrize("gh,gw,T,r,d", [(24, 40, 130, 8.0, 128), (13, 19, 7, 4.0, 64)])
+def test_tensor_core_backward_keeps_the_centred_gradients(gh, gw, T, r, d):
+    """Values with a large common part: every dP of a row has that part, and dP - delta takes it away, so delta has to be
+    as good as fp32 sums make it.  What rounds then are dS and the stored gradient, each to 8 bits (2^-8 / sqrt(3) of a
+    value at the start of a binade, 0.72 of that on average): 1.6e-3 twice, 2.3e-3 of the 2-norm together, and the bound
+    is 2^-8.  A delta that carries the rounding of P to bf16 leaves 1.0e-2 to 1.4e-2."""
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, dtype="bf16", seed=gh + gw)
+    v = (v.float() * 0.25 + 16.0).to(torch.bfloat16)
+    g = torch.Generator(device="cpu").manual_seed(gh * gw)
+    d_out = torch.randn(q.shape, generator=g, dtype=torch.float32).to(torch.bfloat16)
+    scale = 1 / math.sqrt(d)
+    want = oracle_bwd.attn_bwd(q, k, v, d_out, gh, gw, T, r, scale)
+    dev = torch.device("cuda:0")
+    outs = [torch.full_like(q, float("nan"), device=dev) for _ in range(3)]
+    clear.clear_attn_bwd_bf16_tc(*(t.to(dev) for t in (q, k, v, d_out)), *outs, gh, gw, T, r, scale)
+    torch.cuda.synchronize()
+    clear.clear_cache_check()
+    for name, got, ref in zip(("dq", "dk", "dv"), outs, want):
+        err = np.linalg.norm(got.cpu().double().numpy() - ref) / np.linalg.norm(ref)
+        assert err <= 2.0 ** -8, f"{name}: {err:.3e}"
     clear.clear_cache_clear()
 
 
