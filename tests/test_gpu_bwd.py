@@ -226,6 +226,37 @@ def test_tensor_core_backward_keeps_the_centred_gradients(gh, gw, T, r, d):
     clear.clear_cache_clear()
 
 
+@pytest.mark.parametrize("gh,gw,T,r,d", [(24, 40, 130, 8.0, 128), (64, 72, 130, 2.0, 64)], ids=["sweeps", "launches"])
+def test_a_backward_call_that_finds_the_status_word_raised_writes_nothing(gh, gw, T, r, d, monkeypatch):
+    """The word is preset when the plan is made (no wait is made to expire): every block of every role leaves, the gradients
+    stay untouched, the check reports it, and the call after the check runs."""
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, dtype="bf16", seed=3)
+    g = torch.Generator(device="cpu").manual_seed(4)
+    d_out = torch.randn(q.shape, generator=g, dtype=torch.float32).to(torch.bfloat16)
+    scale = 1 / math.sqrt(d)
+    dev = torch.device("cuda:0")
+    args = [t.to(dev) for t in (q, k, v, d_out)]
+    outs = [torch.full_like(args[0], 7.0) for _ in range(3)]
+    clear.clear_cache_clear()
+    monkeypatch.setenv("CLEAR_TEST_PRESET_STATUS", "77")
+    clear.clear_attn_bwd_bf16_tc(*args, *outs, gh, gw, T, r, scale)
+    monkeypatch.delenv("CLEAR_TEST_PRESET_STATUS")
+    torch.cuda.synchronize()
+    for name, got in zip(("dq", "dk", "dv"), outs):
+        assert (got == 7.0).all(), f"{name} was written"
+    with pytest.raises(clear.ClearError) as e:
+        clear.clear_cache_check()
+    assert e.value.status == clear.ERR_DEVICE_TIMEOUT and clear.last_device_status() == 77
+    clear.clear_attn_bwd_bf16_tc(*args, *outs, gh, gw, T, r, scale)
+    torch.cuda.synchronize()
+    clear.clear_cache_check()
+    want = oracle_bwd.attn_bwd(q, k, v, d_out, gh, gw, T, r, scale)
+    for name, got, ref in zip(("dq", "dk", "dv"), outs, want):
+        err = np.abs(got.cpu().double().numpy() - ref)
+        assert err.max() <= _tc_bound(ref), f"{name}: max {err.max():.3e}"
+    clear.clear_cache_clear()
+
+
 def test_tensor_core_backward_argument_errors():
     dev = torch.device("cuda:0")
     x = torch.zeros(1, 1, 272, 64, device=dev, dtype=torch.bfloat16)
