@@ -39,7 +39,12 @@ constexpr uint32_t kWaitHintNs = 20000;            // one sleep inside try_wait
 constexpr uint32_t kWaitLimitUs = 2000000;         // a wait that lasts 2 s has failed
 constexpr float kRescaleThreshold = 8.f;  // log2 units: a reference is moved only when a row's maximum exceeds it by more
 constexpr float kBumpSum = 256.f;         // a row sum of P above this raises the row's reference for the next tile
-constexpr float kMaxTileSum = 0x1p64f;    // a row sum above this (or none at all, a NaN) has its tile taken again
+constexpr float kMaxTileSum = 0x1p64f;    // a row sum above this has its tile taken again (a NaN comes from NaN inputs only, and stays)
+constexpr uint32_t kFirst = 1, kCareful = 2;   // why a step has a maximum pass
+// Scores of a row's first tile that lie this far apart (log2 units) give the item maximum passes from the start: with less,
+// normal ones would have to lie seven standard deviations above the maximum of 128 to be 64 above it.  (The least of 16 of
+// them is enough to tell; the least of all 128 cost 1 to 3 % of a call.)
+constexpr float kWideStep = 40.f;
 constexpr int kSchedDepth = 2;
 // arrivals that free a queue slot: one lane of each of the 2 MMA warps and the 8 softmax warps
 constexpr uint32_t kSchedReaders = 10;
@@ -237,7 +242,7 @@ __device__ __forceinline__ float sum4(const uint64_t (&lsum)[2])
 }
 
 struct RowState {
-    float ref, l, tile_sum;
+    float ref, l, tile_sum;   // tile_sum < 0: less that, and the row's maximum lies more than kWideStep above the least of 16 scores
 };
 // A step with a maximum pass: the maximum over the allowed keys, the row's reference, then P.  The scores are read from
 // tensor memory both times, 32 keys at a time (P of 32 keys takes 16 columns, so it never reaches scores still to be read).
@@ -245,7 +250,7 @@ template <int D>
 __device__ __noinline__ RowState exact_step(uint32_t tmem_s, uint32_t tmem_o, uint4 mask, float c, float ref, float l, bool first)
 {
     auto bits_of = [&](int w) { return w == 0 ? mask.x : w == 1 ? mask.y : w == 2 ? mask.z : mask.w; };
-    float mx = -INFINITY;
+    float mx = -INFINITY, mn = INFINITY;
 #pragma unroll 1
     for (int w = 0, n = opaque(4); w < n; ++w) {
         uint32_t sv[32];
@@ -258,6 +263,9 @@ __device__ __noinline__ RowState exact_step(uint32_t tmem_s, uint32_t tmem_o, ui
             mx2[(j >> 1) & 1] = ptx::max3(mx2[(j >> 1) & 1], ((bits >> j) & 1u) ? __uint_as_float(sv[j]) : -INFINITY,
                                           ((bits >> (j + 1)) & 1u) ? __uint_as_float(sv[j + 1]) : -INFINITY);
         mx = fmaxf(mx2[0], mx2[1]);
+#pragma unroll
+        for (int j = 0; j < 32; j += 8)
+            if ((bits >> j) & 1u) mn = fminf(mn, __uint_as_float(sv[j]));
     }
     const float m_new = fmaxf(ref, mx * c);
     if (first) {
@@ -282,61 +290,135 @@ __device__ __noinline__ RowState exact_step(uint32_t tmem_s, uint32_t tmem_o, ui
         exp_chunk<true>(sv, bits_of(w), c2, nmc2, lsum, pk);
         ptx::tmem_st16(tmem_s + 16 * w, pk);
     }
-    return RowState{ref, l, sum4(lsum)};
+    const float sum = sum4(lsum);
+    return RowState{ref, l, (mx - mn) * c > kWideStep ? -sum : sum};
 }
 
-// A step whose scores lie far above the row's reference: each row's scores once more, by its own thread from global memory
-// (those in tensor memory are gone), twice over -- for their maximum, and for P against it.  Slow, and as good as never run.
+// A step whose scores lie far above the row's reference: the warp's 32 x 128 scores once more from global memory (those in
+// tensor memory are gone), with warp-level MMAs and twice over -- for the rows' maxima, and for P against them.  The rows of
+// an MMA lie in the lanes of a quad; reference, mask and results of row r belong to lane r, and move by shuffles.  Scores of
+// one key at a time by scalar products took about a millisecond a step; the rest of the item has maximum passes, so that it
+// happens once an item and warp at most, and not at all where the first tile's scores are far apart already.  24 heads at
+// 1024 px, r = 8, Q times 20, 60 or 400: 157 us a call (2.7, 94 and 203 ms with scalar products and no memory of it; 100 us
+// with ordinary scores).
 template <int D>
 __device__ __noinline__ RowState rescue_step(const WsParams &prm, uint32_t tmem_p, uint32_t tmem_o, uint4 mask, float c, float ref, float l,
                                              long long row0, long long q_tok, int2 org, bool linear)
 {
     ptx::tmem_wait_st();
-    auto allowed = [&](int key) { return (((key < 32 ? mask.x : key < 64 ? mask.y : key < 96 ? mask.z : mask.w) >> (key & 31)) & 1u) != 0u; };
-    auto score = [&](int key) {
-        const int ky = org.y + (key >> 4), kx = org.x + (key & 15);
+    const int lane = threadIdx.x & 31, quad = lane >> 2, sub = lane & 3;
+    auto word = [&](int w) { return w == 0 ? mask.x : w == 1 ? mask.y : w == 2 ? mask.z : mask.w; };
+    // Contraction channels come in an order of their own, the same for both operands: of 32 channels a lane loads the 8 from
+    // 8 sub on as 16 bytes, and they serve as its four pairs of two MMAs.
+    // 16 rows at a time: in the quad's lanes the rows 16 m + quad and 8 further on
+    uint32_t a[D / 16][4];
+    auto load_rows = [&](int m) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int tok = __shfl_sync(0xffffffffu, (int)q_tok, 16 * m + 8 * h + quad);
+            const uint4 *row = reinterpret_cast<const uint4 *>(prm.q + (row0 + max(tok, 0)) * D) + sub;
+#pragma unroll
+            for (int kk = 0; kk < D / 32; ++kk) {
+                const uint4 x = tok >= 0 ? __ldg(row + 4 * kk) : make_uint4(0u, 0u, 0u, 0u);
+                a[2 * kk][h] = x.x;
+                a[2 * kk][2 + h] = x.y;
+                a[2 * kk + 1][h] = x.z;
+                a[2 * kk + 1][2 + h] = x.w;
+            }
+        }
+    };
+    // their scores with the keys 8 n .. 8 n + 7: the lane holds the keys 8 n + 2 sub, + 1
+    auto scores = [&](int n, float (&s)[4]) {
+        const int key = 8 * n + quad, ky = org.y + (key >> 4), kx = org.x + (key & 15);
         const bool on = linear ? org.x + key < prm.n_tokens : ky >= 0 && ky < prm.grid_h && kx >= 0 && kx < prm.grid_w;
         const long long tok = linear ? org.x + key : prm.n_text + (long long)ky * prm.grid_w + kx;
-        float dot = 0.f;
-        if (on && q_tok >= 0) {
-            const __nv_bfloat16 *q_row = prm.q + (row0 + q_tok) * D, *k_row = prm.k + (row0 + tok) * D;
-#pragma unroll 1
-            for (int e = 0; e < D; ++e) dot = fmaf(__bfloat162float(q_row[e]), __bfloat162float(k_row[e]), dot);
+        const uint4 *row = reinterpret_cast<const uint4 *>(prm.k + (row0 + (on ? tok : 0)) * D) + sub;
+        uint4 b[D / 32];
+#pragma unroll
+        for (int kk = 0; kk < D / 32; ++kk) b[kk] = on ? __ldg(row + 4 * kk) : make_uint4(0u, 0u, 0u, 0u);
+        s[0] = s[1] = s[2] = s[3] = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < D / 32; ++kk) {
+            const uint32_t b0[2] = {b[kk].x, b[kk].y}, b1[2] = {b[kk].z, b[kk].w};
+            ptx::mma_16816_bf16(s, a[2 * kk], b0);
+            ptx::mma_16816_bf16(s, a[2 * kk + 1], b1);
         }
-        return dot;
     };
+    // of the values for the two rows in the quad's lanes, the one of the lane's own row (if it is one of the 16)
+    auto to_owner = [&](float v0, float v1, int src_sub) {
+        const float x0 = __shfl_sync(0xffffffffu, v0, (lane & 7) * 4 + src_sub), x1 = __shfl_sync(0xffffffffu, v1, (lane & 7) * 4 + src_sub);
+        return lane & 8 ? x1 : x0;
+    };
+
     float mx = -INFINITY;
 #pragma unroll 1
-    for (int key = 0; key < 128; ++key)
-        if (allowed(key)) mx = fmaxf(mx, score(key));
+    for (int m = 0; m < 2; ++m) {
+        load_rows(m);
+        float top[2] = {-INFINITY, -INFINITY};
+#pragma unroll 1
+        for (int w = 0; w < 4; ++w) {
+            const uint32_t bits[2] = {__shfl_sync(0xffffffffu, word(w), 16 * m + quad), __shfl_sync(0xffffffffu, word(w), 16 * m + 8 + quad)};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float s[4];
+                scores(4 * w + j, s);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if ((bits[u >> 1] >> (8 * j + 2 * sub + (u & 1))) & 1u) top[u >> 1] = fmaxf(top[u >> 1], s[u]);
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            top[0] = fmaxf(top[0], __shfl_xor_sync(0xffffffffu, top[0], o));
+            top[1] = fmaxf(top[1], __shfl_xor_sync(0xffffffffu, top[1], o));
+        }
+        const float own = to_owner(top[0], top[1], 0);
+        if ((lane >> 4) == m) mx = own;
+    }
     const float m_new = fmaxf(ref, mx * c);
     const bool need = m_new - ref > kRescaleThreshold;
     const float alpha = need ? ptx::ex2(ref - m_new) : 1.f;
     if (need) ref = m_new;
     l *= alpha;
-    __syncwarp();
     rescale_rows<D>(tmem_o, alpha);
+
     const float mc = (ref == -INFINITY) ? 0.f : ref;
     float sum = 0.f;
 #pragma unroll 1
     for (int w = 0; w < 4; ++w) {
         uint32_t pk[16];
 #pragma unroll 1
-        for (int j = 0; j < 16; ++j) {
-            float p[2];
-#pragma unroll 1
-            for (int u = 0; u < 2; ++u) {
-                const int key = 32 * w + 2 * j + u;
-                const float x = allowed(key) ? ptx::ex2(fmaf(score(key), c, -mc)) : 0.f;
-                sum += x;
-                if (u == 0) p[0] = x;
-                else p[1] = x;
+        for (int m = 0; m < 2; ++m) {
+            load_rows(m);
+            const uint32_t bits[2] = {__shfl_sync(0xffffffffu, word(w), 16 * m + quad), __shfl_sync(0xffffffffu, word(w), 16 * m + 8 + quad)};
+            const float mc2[2] = {__shfl_sync(0xffffffffu, mc, 16 * m + quad), __shfl_sync(0xffffffffu, mc, 16 * m + 8 + quad)};
+            const bool mine = (lane >> 4) == m;
+            float part[2] = {0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float s[4], p[4];
+                scores(4 * w + j, s);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool on = ((bits[u >> 1] >> (8 * j + 2 * sub + (u & 1))) & 1u) != 0u;
+                    p[u] = on ? ptx::ex2(fmaf(s[u], c, -mc2[u >> 1])) : 0.f;
+                    part[u >> 1] += p[u];
+                }
+                const float pair[2] = {__uint_as_float(ptx::pack_bf16(p[0], p[1])), __uint_as_float(ptx::pack_bf16(p[2], p[3]))};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t x = __float_as_uint(to_owner(pair[0], pair[1], e));
+                    pk[4 * j + e] = mine ? x : m == 0 ? 0u : pk[4 * j + e];
+                }
             }
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (i == j) pk[i] = ptx::pack_bf16(p[0], p[1]);
+            for (int o = 1; o < 4; o <<= 1) {
+                part[0] += __shfl_xor_sync(0xffffffffu, part[0], o);
+                part[1] += __shfl_xor_sync(0xffffffffu, part[1], o);
+            }
+            const float own = to_owner(part[0], part[1], 0);
+            if (mine) sum += own;
         }
-        __syncwarp();
         ptx::tmem_st16(tmem_p + 16 * w, pk);
     }
     return RowState{ref, l, sum};
@@ -766,7 +848,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             const bool q_valid = is_text ? r < (t ? item.n_rows1 : item.n_rows0) : (q_y < prm.grid_h && q_x < prm.grid_w);
             float ref = -INFINITY, l = 0.f;  // reference of the row's exponents (log2 units) and row sum
             int bump = 0;                    // powers of two the reference is to be raised by before the next tile
-            bool first = true;
+            uint32_t exact_from = kFirst;    // kFirst: no step yet; kCareful: a step had to be taken again, maximum passes from here on
 
             // The flags and the key count (or mask entry) of 32 steps at a time, one step per lane, the 32 after them
             // fetched meanwhile; taken out of the lanes two steps ahead, and this row's precomputed mask words fetched one
@@ -850,7 +932,8 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                 // reference is raised before the next tile, by a whole power of two and without a look at the maximum.
                 // No maximum pass, then, on any tile but the first, and the scores die as their P is formed.  A row sum
                 // beyond 2^64 means scores 64 powers of two above everything seen before; the warp then computes its
-                // scores again, from global memory, before anybody has used P.
+                // scores again, from global memory, before anybody has used P, and takes the rest of the item's steps with
+                // maximum passes.
                 const bool raise = __any_sync(0xffffffffu, bump != 0);
                 float alpha = 1.f;
                 if (raise) {
@@ -859,7 +942,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                     l *= alpha;
                     bump = 0;
                 }
-                const bool exact = __any_sync(0xffffffffu, first || (ref == -INFINITY && q_valid));
+                const bool exact = __any_sync(0xffffffffu, exact_from != 0u || (ref == -INFINITY && q_valid));
                 float tile_sum = 0.f;
                 // warp-uniform outcome of the waits: the tcgen05.ld / st below need the whole warp.  Once the first half of
                 // S_t is complete, so is P_t V of the step before (same thread, same pipe, issued earlier).
@@ -908,7 +991,8 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                     }
                     tile_sum = sum4(lsum);
                     if (raise) rescale_rows<D>(tmem_O + lane_off, alpha);
-                    if (__builtin_expect(__any_sync(0xffffffffu, !(tile_sum <= kMaxTileSum)), 0)) {
+                    if (__builtin_expect(__any_sync(0xffffffffu, tile_sum > kMaxTileSum), 0)) {
+                        exact_from = kCareful;
                         const int2 org = load_side_origin(steps + s, t);
                         const long long q_tok = is_text ? (long long)item.qx + t * 128 + r : prm.n_text + (long long)q_y * prm.grid_w + q_x;
                         const RowState rs = rescue_step<D>(prm, tmem_S + lane_off, tmem_O + lane_off, make_uint4(mw[0], mw[1], mw[2], mw[3]), c, ref,
@@ -925,15 +1009,16 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                     }
                     ptx::tc_fence_after();
                     if (raise) rescale_rows<D>(tmem_O + lane_off, alpha);
-                    const RowState rs = exact_step<D>(tmem_S + lane_off, tmem_O + lane_off, make_uint4(mw[0], mw[1], mw[2], mw[3]), c, ref, l, first);
+                    const RowState rs = exact_step<D>(tmem_S + lane_off, tmem_O + lane_off, make_uint4(mw[0], mw[1], mw[2], mw[3]), c, ref, l, exact_from == kFirst);
                     ref = rs.ref;
                     l = rs.l;
-                    tile_sum = rs.tile_sum;
+                    tile_sum = fabsf(rs.tile_sum);
+                    if (__any_sync(0xffffffffu, rs.tile_sum < 0.f)) exact_from = kCareful;
                     ptx::tc_fence_before();
                     warp_arrive(ptx::smem_u32(&ctrl->sb_read[t]), lane);
                 }
                 ++n_s;
-                first = false;
+                exact_from &= kCareful;
                 l += tile_sum;
                 if (tile_sum > kBumpSum) bump = (int)((__float_as_uint(tile_sum) >> 23) & 0xffu) - 127;
                 // P_t (and a rescaled O_t) must be in tensor memory before the MMA thread is told

@@ -652,6 +652,68 @@ def test_ws_kernel_scores_far_above_a_rows_reference(gh, gw, T, r, d):
     assert_close_bf16(run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS), want, "far scores")
 
 
+@pytest.mark.parametrize("gh,gw,T,r,d,length", [(24, 40, 130, 8.0, 128, 60.0), (19, 23, 0, 4.0, 64, 400.0), (29, 35, 300, 6.5, 64, 60.0),
+                                                (45, 21, 37, 5.0, 128, 400.0)])
+def test_ws_kernel_with_long_queries(gh, gw, T, r, d, length):
+    """Logits of tens to hundreds everywhere, so that steps of any kind are taken again: ragged and whole text tiles, patches
+    over the border, query rows that do not exist.  A softmax this sharp takes whole values, so the rounding of P and of the
+    output to bf16 shows in full, 2^-8 of max |v| and of the output; logits of size L are good to a few 2^-24 L in fp32, and
+    P with them."""
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, seed=int(length) + gh)
+    q = (q.float() * length).to(torch.bfloat16)
+    scale = 1 / math.sqrt(d)
+    want = oracle.attn(q, k, v, gh, gw, T, r, scale)
+    got = run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS).double().numpy()
+    v_max = float(v.float().abs().max())
+    logit = scale * float(q.float().norm(dim=-1).max() * k.float().norm(dim=-1).max())
+    bound = 2.0 ** -8 * (np.abs(want) + v_max) + 2.0 ** -21 * logit * v_max
+    assert (np.abs(got - want) <= bound).all(), float(np.abs(got - want).max())
+
+
+def test_ws_kernel_nan_key_reaches_the_queries_that_see_it():
+    """A NaN in a key outside the first tile: the text queries and the image queries within its reach, no others."""
+    gh, gw, T, r, d = 24, 40, 20, 3.0, 64
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, seed=8)
+    y, x = 12, 20
+    k[0, 0, T + y * gw + x, 3] = float("nan")
+    got = run_plan(q, k, v, gh, gw, T, r, 1 / math.sqrt(d), clear.KERNEL_TCGEN05_WS)
+    ys, xs = np.arange(gh)[:, None], np.arange(gw)[None]
+    sees = np.concatenate([np.ones(T, bool), ((ys - y) ** 2 + (xs - x) ** 2 < r * r).ravel()])
+    assert (np.isnan(got[0, 0].float().numpy()).any(-1) == sees).all()
+    assert np.isfinite(got[0, 1].float().numpy()).all()
+
+
+@pytest.mark.parametrize("what", ["long queries", "nan keys"])
+def test_ws_kernel_cost_does_not_hang_on_the_values(what):
+    """Times of one shape with ordinary inputs and with others.  Maximum passes on every step cost half as much again, and a
+    step that is taken again is rare; the bound is five times the ordinary call, which leaves room for a busy device (scalar
+    products for every such step: 27 to 2000 times)."""
+    gh, gw, T, r, d, H = 64, 64, 512, 8.0, 128, 8
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    q, k, v = (torch.randn(1, H, T + gh * gw, d, generator=gen, device="cuda") for _ in range(3))
+    odd = [q, k]
+    if what == "long queries":
+        odd[0] = q * 40
+    else:
+        odd[1] = k.masked_fill(torch.rand(k.shape[:3], generator=gen, device="cuda")[..., None] < 0.01, float("nan"))
+    out = torch.empty_like(v, dtype=torch.bfloat16)
+
+    def median_ms(q, k):
+        args = [t.to(torch.bfloat16) for t in (q, k, v)]
+        times = []
+        for _ in range(7):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            clear.clear_attn_fwd(*args, out, gh, gw, T, r, 1 / math.sqrt(d))
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times)[3]
+
+    assert median_ms(*odd) <= 5 * median_ms(q, k)
+    clear.clear_cache_clear()
+
+
 @pytest.mark.parametrize("kernel", TC_KERNELS, ids=TC_IDS)
 @pytest.mark.parametrize("gh,gw,T,r,d", [(45, 70, 17, 12.5, 64), (40, 67, 3, 4.5, 128), (31, 33, 0, 7.5, 64)])
 def test_tc_kernels_with_key_patches_off_the_query_lattice(gh, gw, T, r, d, kernel):
