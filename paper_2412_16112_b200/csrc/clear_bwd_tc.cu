@@ -386,7 +386,8 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
             }
         } else if (warp == 2 && KEY_ROLE) {
             // ================= statistics of the streamed tiles' columns, ahead of the row warps =====================
-            // (a column that does not exist is masked; its address stays inside the buffer, which is padded by one tile)
+            // (zeros for a column that is none of the list's: P is 0 there, but P (dP - delta) is not if delta is another
+            // token's NaN, of the next head or of the next grid row)
             const float2 *stats = prm.stats + (long long)bh * prm.n_tokens;
             bool ok = true;
             if (prm.key_waits) {
@@ -401,21 +402,22 @@ clear_bwd_tc_kernel(const __grid_constant__ BwdMaps maps, const __grid_constant_
                 const uint32_t st = (uint32_t)i % kColStages, use = (uint32_t)i / kColStages;
                 const clear_kv_tile_t t = tiles[i];
                 float2 v[4];
+                bool here[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int c = 32 * j + lane;
-                    const long long tok = (t.flags & CLEAR_TILE_LINEAR)
-                                              ? (long long)t.x + c
-                                              : prm.n_text + (long long)min(t.y + (c >> 4), prm.grid_h - 1) * prm.grid_w + t.x + (c & 15);
-                    v[j] = __ldcg(stats + tok);
+                    const int c = 32 * j + lane, y = t.y + (c >> 4), x = t.x + (c & 15);
+                    const bool linear = (t.flags & CLEAR_TILE_LINEAR) != 0;
+                    const long long tok = linear ? (long long)t.x + c : prm.n_text + (long long)y * prm.grid_w + x;
+                    here[j] = linear ? c < t.n_valid : y < prm.grid_h && x < prm.grid_w;
+                    v[j] = __ldcg(stats + (here[j] ? tok : 0));
                 }
                 ok = __all_sync(0xffffffffu, bwd_wait(ptx::smem_u32(&ctrl->col_empty[st]), (use & 1u) ^ 1u, abort_flag, prm.status, 5));
                 if (!ok) break;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     float *dst = reinterpret_cast<float *>(&ctrl->col[st][16 * j + (lane >> 1)]) + (lane & 1);
-                    dst[0] = -v[j].x;
-                    dst[2] = -v[j].y;
+                    dst[0] = here[j] ? -v[j].x : 0.f;
+                    dst[2] = here[j] ? -v[j].y : 0.f;
                 }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&ctrl->col_full[st]));
@@ -770,11 +772,11 @@ int count_first(const std::vector<clear_work_item_t> &items)
     return n < items.size() ? (int)n : 0;
 }
 
-// Statistics of every row, and one tile of padding (those of columns past the end are read, and masked), to 256 bytes.
+// Statistics of every row, to 256 bytes.
 size_t row_stats_bytes(const clear_plan &p)
 {
     const Shape &s = p.shape;
-    const size_t rows = (size_t)s.B * s.H * ((size_t)s.n_text + (size_t)s.grid_h * s.grid_w) + kTileTokens;
+    const size_t rows = (size_t)s.B * s.H * ((size_t)s.n_text + (size_t)s.grid_h * s.grid_w);
     return (rows * sizeof(float2) + 255) / 256 * 256;
 }
 

@@ -257,6 +257,28 @@ def test_a_backward_call_that_finds_the_status_word_raised_writes_nothing(gh, gw
     clear.clear_cache_clear()
 
 
+@pytest.mark.parametrize("B,H,gh,gw,T,r,d", [(1, 2, 13, 19, 7, 2.5, 64), (2, 1, 20, 50, 130, 4.0, 128), (1, 2, 64, 70, 131, 2.0, 64)])
+def test_tensor_core_backward_keeps_heads_apart(B, H, gh, gw, T, r, d):
+    """NaN all over the second (batch, head), the first one's last tiles ragged: the first one's gradients are the ones it has
+    beside any other neighbour, bit for bit."""
+    q, k, v = workloads.make_custom(B, H, gh, gw, T, d, dtype="bf16", seed=gh + gw)
+    g = torch.Generator(device="cpu").manual_seed(gh * gw)
+    args = [q, k, v, torch.randn(q.shape, generator=g, dtype=torch.float32).to(torch.bfloat16)]
+    args = [t.to("cuda:0") for t in args]
+    grads = []
+    for rep in range(2):
+        outs = [torch.zeros_like(args[0]) for _ in range(3)]
+        clear.clear_attn_bwd_bf16_tc(*args, *outs, gh, gw, T, r, 1 / math.sqrt(d))
+        grads.append([o.view(B * H, -1)[0].clone() for o in outs])
+        for t in args:
+            t.view(B * H, -1)[1] = float("nan")
+    torch.cuda.synchronize()
+    clear.clear_cache_check()
+    for name, want, got in zip(("dq", "dk", "dv"), *grads):
+        assert torch.isfinite(want).all() and torch.equal(want, got), name
+    clear.clear_cache_clear()
+
+
 def test_tensor_core_backward_argument_errors():
     dev = torch.device("cuda:0")
     x = torch.zeros(1, 1, 272, 64, device=dev, dtype=torch.bfloat16)
