@@ -41,6 +41,7 @@ template <int DP> struct BwdSmem {
     KeyTile keys[3];
     int tokens[kRows];
     int red[8];
+    int bad[kRows];                                            // rows that came out non-finite
 };
 
 // One streamed step after another: in step s the second row set (B2: V, or dO) of tile s is used first, then the first
@@ -91,7 +92,7 @@ template <typename T, int DP> struct Stream {
 // Rows of an accumulator to global memory, summed over the cluster first when the list is cut.
 template <typename T, int DP>
 __device__ __forceinline__ void store_acc(const uint64_t (&acc)[4][DP / 64][2], float *scratch, T *out, const F32BwdParams &p,
-                                          const TileRef &tile, int part, int ty, int tx)
+                                          const TileRef &tile, int part, int ty, int tx, int *bad)
 {
     if (p.n_split == 1) {
 #pragma unroll
@@ -101,7 +102,9 @@ __device__ __forceinline__ void store_acc(const uint64_t (&acc)[4][DP / 64][2], 
 #pragma unroll
             for (int c = 0; c < DP / 64; ++c) {
                 const int ch = 64 * c + 4 * tx;
-                if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, acc_float4(acc[i][c], 1.f));
+                const float4 v = acc_float4(acc[i][c], 1.f);
+                if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, v);
+                if (!finite4(v)) bad[ty + 16 * i] = 1;
             }
         }
         return;
@@ -123,12 +126,42 @@ __device__ __forceinline__ void store_acc(const uint64_t (&acc)[4][DP / 64][2], 
             a.w += v.w;
         }
         if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, a);
+        if (!finite4(a)) bad[r] = 1;
     }
     cluster.sync();   // nobody leaves, or reuses the rows, while they are being read
 }
 
+// Row r of the block's tile by itself (one warp): the sums of the kernel below over the tokens that the row sees.
 template <typename T, int DP, bool KEY_ROLE>
-__global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kernel(const F32BwdParams p)
+__device__ __forceinline__ void redo_row(const F32BwdParams &p, int r)
+{
+    const TileRef tile = tile_of((int)(blockIdx.x / (unsigned)p.n_split), p.g);
+    const KeyRuns runs = runs_of(tile, p.g);
+    int y, x;
+    const int tok = tile_token(tile, r, p.g, y, x), d = p.g.d;
+    if (tok < 0) return;
+    const long long base = (long long)tile.bh * runs.n_tokens * d;
+    const T *b1 = static_cast<const T *>(KEY_ROLE ? p.q : p.k) + base, *b2 = static_cast<const T *>(KEY_ROLE ? p.d_out : p.v) + base;
+    const float *stats = p.stats + (long long)tile.bh * runs.n_tokens * 3;
+    LaneRow<DP> a1, a2, r1, r2, o1, o2;
+    a1.load(static_cast<const T *>(KEY_ROLE ? p.k : p.q) + base + (long long)tok * d, d);
+    a2.load(static_cast<const T *>(KEY_ROLE ? p.v : p.d_out) + base + (long long)tok * d, d);
+    o1.zero();
+    o2.zero();
+    for_each_seen(runs, y, x, [&](int t) {
+        r1.load(b1 + (long long)t * d, d);
+        r2.load(b2 + (long long)t * d, d);
+        const float *st = stats + 3ll * (KEY_ROLE ? t : tok);
+        const float pr = expf(a1.dot(r1) * p.scale - __ldcg(st)) * __ldcg(st + 1);
+        o1.add(pr * (a2.dot(r2) - __ldcg(st + 2)) * p.scale, r1);
+        if (KEY_ROLE) o2.add(pr, r2);
+    });
+    o1.store(static_cast<T *>(p.out1) + base + (long long)tok * d, d, 1.f);
+    if (KEY_ROLE) o2.store(static_cast<T *>(p.out2) + base + (long long)tok * d, d, 1.f);
+}
+
+template <typename T, int DP, bool KEY_ROLE>
+__global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kernel(const __grid_constant__ F32BwdParams p)
 {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     BwdSmem<DP> &sm = *reinterpret_cast<BwdSmem<DP> *>(smem_raw);
@@ -148,6 +181,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kern
     if (tid < kRows) {
         int y, x;
         sm.tokens[tid] = tile_token(tile, tid, p.g, y, x);
+        sm.bad[tid] = 0;
     }
     st.fill(0);
     st.fill(1);
@@ -206,7 +240,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kern
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            l[i] = l[i] > 0.f ? 1.f / l[i] : 0.f;   // l >= 1 for every row that exists (it sees itself or the text)
+            l[i] = l[i] == 0.f ? 0.f : 1.f / l[i];   // l >= 1 for every row that exists (it sees itself or the text); NaN stays
             dl[i] *= l[i];
             if (m[i] == -CUDART_INF_F) m[i] = 0.f;
             const long long tok = sm.tokens[ty + 16 * i];
@@ -247,6 +281,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kern
                     const int c = tx + 16 * j;
                     const bool on = kt.token[c] >= 0 && sees(runs, r_y[i], r_x[i], kt.ky[c], kt.kx[c]);
                     s[i][j] = on ? s[i][j] * p.scale : -CUDART_INF_F;
+                    g[i][j] = on ? g[i][j] : 0.f;   // (its weight is 0, but it may be no number)
                     mx = fmaxf(mx, s[i][j]);
                 }
                 const float m_new = fmaxf(m[i], row_max16(mx)), m_ref = m_new == -CUDART_INF_F ? 0.f : m_new;
@@ -276,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kern
                             de = KEY_ROLE ? sm.col[it % 3][2][c] : dl[i];
                 const float pr = on ? expf(s[i][j] * p.scale - mm) * il : 0.f;
                 s[i][j] = pr;
-                g[i][j] = pr * (g[i][j] - de) * p.scale;
+                g[i][j] = on ? pr * (g[i][j] - de) * p.scale : 0.f;
             }
         if (KEY_ROLE) {
             // dV += P^T dO; a row of weights is written and read by one warp
@@ -300,8 +335,12 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) clear_f32_bwd_kern
     }
     cp_async_wait<0>();
     __syncthreads();
-    store_acc<T, DP>(acc1, sm.ring[0], static_cast<T *>(p.out1) + base, p, tile, part, ty, tx);
-    if (KEY_ROLE) store_acc<T, DP>(acc2, sm.ring[1], static_cast<T *>(p.out2) + base, p, tile, part, ty, tx);
+    store_acc<T, DP>(acc1, sm.ring[0], static_cast<T *>(p.out1) + base, p, tile, part, ty, tx, sm.bad);
+    if (KEY_ROLE) store_acc<T, DP>(acc2, sm.ring[1], static_cast<T *>(p.out2) + base, p, tile, part, ty, tx, sm.bad);
+    __syncthreads();
+#pragma unroll 1
+    for (int r = tid >> 5; r < kRows; r += kThreads / 32)
+        if (sm.bad[r] != 0) redo_row<T, DP, KEY_ROLE>(p, r);
 }
 
 template <typename T, int DP>

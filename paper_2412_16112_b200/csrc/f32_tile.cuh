@@ -17,6 +17,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <math_constants.h>
 
 #include <cstdint>
 
@@ -338,6 +339,73 @@ __device__ __forceinline__ void fill_key_tile(KeyTile &t, KeyCursor &cur, const 
         t.ky[threadIdx.x] = ky;
         t.kx[threadIdx.x] = kx;
         cur.advance(k, kRows);
+    }
+}
+
+// ---- rows taken by themselves --------------------------------------------------------------------------------------
+// A weight of 0 hides a streamed row from a query that does not see it, unless the row holds a NaN or an infinity.  So the
+// rows of a tile that come out non-finite are taken again, a warp a row over the tokens that the row sees and no others:
+// non-finite values reach the rows that see them, and nobody pays for the rest.
+__device__ __forceinline__ bool finite4(float4 v)
+{
+    return fabsf(v.x) <= CUDART_MAX_NORMAL_F && fabsf(v.y) <= CUDART_MAX_NORMAL_F && fabsf(v.z) <= CUDART_MAX_NORMAL_F &&
+           fabsf(v.w) <= CUDART_MAX_NORMAL_F;
+}
+__device__ __forceinline__ float as_float(float x) { return x; }
+__device__ __forceinline__ float as_float(__nv_bfloat16 x) { return __bfloat162float(x); }
+__device__ __forceinline__ void put(float *p, float x) { *p = x; }
+__device__ __forceinline__ void put(__nv_bfloat16 *p, float x) { *p = __float2bfloat16_rn(x); }
+
+// A lane's channels of a row: lane, lane + 32, ...
+template <int DP> struct LaneRow {
+    float c[DP / 32];
+    template <typename T> __device__ __forceinline__ void load(const T *row, int d)
+    {
+#pragma unroll
+        for (int t = 0; t < DP / 32; ++t) {
+            const int e = (int)(threadIdx.x & 31) + 32 * t;
+            c[t] = e < d ? as_float(row[e]) : 0.f;
+        }
+    }
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int t = 0; t < DP / 32; ++t) c[t] = 0.f;
+    }
+    __device__ __forceinline__ void add(float f, const LaneRow &o)
+    {
+#pragma unroll
+        for (int t = 0; t < DP / 32; ++t) c[t] = fmaf(f, o.c[t], c[t]);
+    }
+    __device__ __forceinline__ float dot(const LaneRow &o) const
+    {
+        float x = 0.f;
+#pragma unroll
+        for (int t = 0; t < DP / 32; ++t) x = fmaf(c[t], o.c[t], x);
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) x += __shfl_xor_sync(0xffffffffu, x, s);
+        return x;
+    }
+    template <typename T> __device__ __forceinline__ void store(T *row, int d, float f) const
+    {
+#pragma unroll
+        for (int t = 0; t < DP / 32; ++t) {
+            const int e = (int)(threadIdx.x & 31) + 32 * t;
+            if (e < d) put(row + e, c[t] * f);
+        }
+    }
+};
+// body(token) for every token that the query at (qy, qx) sees, in order.
+template <typename Body> __device__ __forceinline__ void for_each_seen(const KeyRuns &k, int qy, int qx, Body &&body)
+{
+#pragma unroll 1
+    for (int t = 0; t < k.head_length(); ++t) body(t);
+    if (k.text) return;
+#pragma unroll 1
+    for (int y = max(0, qy - (k.n_half_width - 1)); y < min(k.grid_h, qy + k.n_half_width); ++y) {
+        const int w = __ldg(k.half_width + abs(y - qy));
+#pragma unroll 1
+        for (int x = max(qx - w, 0); x <= min(qx + w, k.grid_w - 1); ++x) body(k.n_text + y * k.grid_w + x);
     }
 }
 

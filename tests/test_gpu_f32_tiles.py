@@ -56,3 +56,64 @@ def test_backward_tiles(bh, gh, gw, T, r, d):
         # fp32 sums of a few hundred terms of order one (the bound of the small-shape tests)
         assert err.max() <= 1e-4, f"{name}: max {err.max():.3e}"
     clear.clear_cache_clear()
+
+
+def _mask(gh, gw, T, r):
+    ys, xs = np.repeat(np.arange(gh), gw), np.tile(np.arange(gw), gh)
+    M = np.ones((T + gh * gw,) * 2, dtype=bool)
+    M[T:, T:] = (ys[:, None] - ys) ** 2 + (xs[:, None] - xs) ** 2 < r * r
+    return M
+
+
+# B * H, grid, text tokens, radius, head size: lists cut over a cluster; whole ones; the two wider padded head sizes
+_ISOLATION = [(2, 24, 40, 20, 3.0, 64), (40, 24, 40, 0, 3.0, 8), (2, 13, 19, 7, 2.5, 128), (1, 9, 33, 5, 2.0, 256)]
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("which", ["q", "k", "v"])
+@pytest.mark.parametrize("H,gh,gw,T,r,d", _ISOLATION)
+def test_forward_tiles_keep_non_finite_values_to_the_rows_that_see_them(H, gh, gw, T, r, d, which, bad):
+    """One non-finite element: the rows that see its token are non-finite, all others are what they are without it (same
+    terms in fp32; the rows of its tile are summed in another order)."""
+    ts = dict(zip("qkv", workloads.make_custom(1, H, gh, gw, T, d, dtype="f32", qk_norm=False, seed=gh)))
+    scale, token = 1 / math.sqrt(d), T + (gh // 2) * gw + gw // 2
+    want = oracle.attn(ts["q"], ts["k"], ts["v"], gh, gw, T, r, scale)
+    ts[which][0, 0, token, 3] = bad
+    out = torch.full_like(ts["q"], 7.0, device="cuda:0")
+    clear.clear_attn_fwd_f32(*(t.to("cuda:0") for t in ts.values()), out, gh, gw, T, r, scale)
+    got = out.cpu().double().numpy()
+    M = _mask(gh, gw, T, r)
+    hit = np.zeros((H, M.shape[0]), dtype=bool)
+    hit[0] = np.arange(M.shape[0]) == token if which == "q" else M[:, token]
+    # (an infinite score of the right sign is a softmax on that key alone, or none: not every row has to be non-finite)
+    finite = np.isfinite(got[0]).all(-1)
+    assert finite[~hit].all()
+    if bad != bad or which == "v":
+        assert not finite[hit].any()
+    assert np.abs(got[0] - want[0])[~hit].max() <= 1e-5
+    clear.clear_cache_clear()
+
+
+@pytest.mark.parametrize("which", ["q", "k", "v", "g"])
+@pytest.mark.parametrize("H,gh,gw,T,r,d", _ISOLATION[:3])
+def test_backward_tiles_keep_non_finite_values_to_the_rows_that_see_them(H, gh, gw, T, r, d, which):
+    """The same for the gradients.  A NaN in q or dO makes row t of P, or of dS, NaN; one in k or v does so for every query
+    that sees it (the row's sum, or delta), v leaving P alone."""
+    ts = dict(zip("qkv", workloads.make_custom(1, H, gh, gw, T, d, dtype="f32", qk_norm=False, seed=gh)))
+    gen = torch.Generator(device="cpu").manual_seed(gh + gw)
+    ts["g"] = torch.randn(ts["q"].shape, generator=gen, dtype=torch.float32)
+    scale, token = 1 / math.sqrt(d), T + (gh // 2) * gw + gw // 2
+    want = oracle_bwd.attn_bwd(*ts.values(), gh, gw, T, r, scale)
+    ts[which][0, 0, token, 3] = float("nan")
+    outs = [torch.full_like(ts["q"], 7.0, device="cuda:0") for _ in range(3)]
+    clear.clear_attn_bwd_f32(*(t.to("cuda:0") for t in ts.values()), *outs, gh, gw, T, r, scale)
+    M = _mask(gh, gw, T, r)
+    rows = np.arange(M.shape[0]) == token if which in "qg" else M[:, token]
+    keys = M[rows].any(0)
+    hit = {"dq": rows, "dk": keys, "dv": np.zeros_like(keys) if which == "v" else keys}
+    for (name, bad_rows), got, ref in zip(hit.items(), outs, want):
+        x = got.cpu().double().numpy()[0]
+        finite = np.isfinite(x).all(-1)
+        assert (finite[0] == ~bad_rows).all() and finite[1:].all(), name
+        assert np.abs(x - ref[0])[finite].max() <= 1e-4, name
+    clear.clear_cache_clear()
