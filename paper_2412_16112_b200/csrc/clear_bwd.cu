@@ -3,8 +3,9 @@
 // through which the distillation losses of Sec. 3.3 (Eq. 4-6) reach the attention parameters.
 //
 // Two kernels, one warp per token, lanes split the head dimension, tokens walked as clear_simt.cu
-// does (the text tokens, then per grid row within reach the clipped run of columns).  Head sizes above 128 only: up to
-// there the tiled kernels of clear_f32_bwd.cu are 6 to 8 times faster, above their row sets do not fit shared memory.
+// does (the text tokens, then per grid row within reach the clipped run of columns).  Head sizes above 128, whose row sets do
+// not fit the tiled kernels of clear_f32_bwd.cu, and windows of a few keys without text; for the rest those are 6 to 8 times
+// faster.
 //   query kernel: sweep 1 over the query's keys: online softmax -> row maximum m, row sum l, the un-normalised
 //       output, hence delta = dO . O; the three row statistics are kept for the second kernel;
 //       sweep 2: p = exp(s - m) / l, dP = dO . v, dS = p (dP - delta), dQ += scale dS k;
@@ -228,6 +229,10 @@ int launch_bwd_typed(const clear_plan &p, const void *q, const void *k, const vo
                                                                p.d_half_width, n_hw, scale);                            \
         break;
     switch (epl) {
+        CLEAR_BWD_CASE(1)
+        CLEAR_BWD_CASE(2)
+        CLEAR_BWD_CASE(3)
+        CLEAR_BWD_CASE(4)
         CLEAR_BWD_CASE(5)
         CLEAR_BWD_CASE(6)
         CLEAR_BWD_CASE(7)
@@ -261,7 +266,14 @@ int ensure_bwd_stats(const clear_plan &p)
 int launch_bwd(const clear_plan &p, const void *q, const void *k, const void *v, const void *d_out, void *dq, void *dk,
                void *dv, float scale, cudaStream_t stream)
 {
-    if (p.shape.head_dim <= 128) return launch_f32_bwd(p, q, k, v, d_out, dq, dk, dv, scale, stream);
+    // Keys of an interior query.  The tiles work on the union of 64 windows, a warp on one token's own: with few keys and no
+    // text (whose rows see everything) the warps win.  24 heads at 32 x 32, tiles and warps in us, 64 channels: 1 key 88 and
+    // 28, 9 keys 150 and 84, 25 keys 192 and 184, 45 keys 246 and 307; 128 channels: 163 and 35, 278 and 106, 322 and 236,
+    // 397 and 401.
+    int64_t window = 0;
+    for (size_t dy = 0; dy < p.sch.half_width.size(); ++dy) window += (dy == 0 ? 1 : 2) * (2 * (int64_t)p.sch.half_width[dy] + 1);
+    const bool few = p.shape.n_text == 0 && window <= 25;
+    if (p.shape.head_dim <= 128 && !few) return launch_f32_bwd(p, q, k, v, d_out, dq, dk, dv, scale, stream);
     const int rc = ensure_bwd_stats(p);
     if (rc != CLEAR_OK) return rc;
     if (p.shape.dtype == CLEAR_F32) return launch_bwd_typed<float>(p, q, k, v, d_out, dq, dk, dv, scale, stream);

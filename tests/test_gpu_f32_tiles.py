@@ -58,6 +58,21 @@ def test_backward_tiles(bh, gh, gw, T, r, d):
     clear.clear_cache_clear()
 
 
+@pytest.mark.parametrize("d", [8, 40, 96, 128])
+@pytest.mark.parametrize("gh,gw,r", [(9, 13, 1.0), (24, 21, 3.0), (24, 21, 3.2), (1, 70, 12.9)])
+def test_backward_with_few_keys_and_no_text(gh, gw, r, d):
+    """Both sides of the line between the kernel with a warp per token (1 and 25 keys, and 25 in a row) and the tiles (37)."""
+    q, k, v, g = _inputs(2, gh, gw, 0, d, 4, 13)
+    scale = 1 / math.sqrt(d)
+    want = oracle_bwd.attn_bwd(q, k, v, g, gh, gw, 0, r, scale)
+    outs = [torch.full_like(q, float("nan"), device="cuda:0") for _ in range(3)]
+    clear.clear_attn_bwd_f32(*(t.cuda() for t in (q, k, v, g)), *outs, gh, gw, 0, r, scale)
+    for name, got, ref in zip(("dq", "dk", "dv"), outs, want):
+        err = np.abs(got.cpu().double().numpy() - ref)
+        assert err.max() <= 1e-4, f"{name}: max {err.max():.3e}"
+    clear.clear_cache_clear()
+
+
 def _mask(gh, gw, T, r):
     ys, xs = np.repeat(np.arange(gh), gw), np.tile(np.arange(gw), gh)
     M = np.ones((T + gh * gw,) * 2, dtype=bool)
