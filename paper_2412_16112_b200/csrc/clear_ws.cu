@@ -88,6 +88,7 @@ struct Ctrl {
     int32_t sched_item[kSchedDepth];            // queue position, >= total: no more work
     int32_t sched_bh[kSchedDepth];
     clear_pair_item_t sched_rec[kSchedDepth];   // the item's record, read once from global memory
+    uint32_t copies[3];   // issued by the loader: Q tiles of tile 0 and 1, K/V stages
     uint32_t tmem_base;
     int abort_flag;
     int skip;
@@ -639,15 +640,9 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                 }
                 if (!ok) break;
             }
-            if (*abort_flag) {
-                // leave no copy in flight: whatever was issued must land before the block exits
-                for (int t = 0; t < 2; ++t)
-                    if (n_q[t] > 0) drain_bar(ptx::smem_u32(&ctrl->q_full[t]), (n_q[t] - 1) & 1u);
-                for (uint32_t j = 0; j < kRing && j < n_loads; ++j) {
-                    const uint32_t idx = n_loads - 1 - j;
-                    drain_bar(ptx::smem_u32(&ctrl->kv_full[idx % kRing]), (idx / kRing) & 1u);
-                }
-            }
+            ctrl->copies[0] = n_q[0];
+            ctrl->copies[1] = n_q[1];
+            ctrl->copies[2] = n_loads;
         } else if ((warp == 1 || warp == 2) && ptx::elect_one()) {
             // ================= MMA issue: S_t = Q_t K^T, O_t += P_t V, one warp per query tile t ==============
             // S_t of a step comes in two halves of 64 keys.  The softmax warps take the second half first; P_t of the whole
@@ -1045,6 +1040,14 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
         ptx::tmem_dealloc(tmem, kTmemCols);
     }
     if (tid == 0) {
+        if (*abort_flag) {
+            // leave no copy in flight: whatever was issued must land before the block exits (looked at only now: the block
+            // may give up after the loader has issued its last copy)
+            for (int t = 0; t < 2; ++t)
+                if (ctrl->copies[t] > 0) drain_bar(ptx::smem_u32(&ctrl->q_full[t]), (ctrl->copies[t] - 1) & 1u);
+            for (uint32_t j = 0, n = ctrl->copies[2]; j < kRing && j < n; ++j)
+                drain_bar(ptx::smem_u32(&ctrl->kv_full[(n - 1 - j) % kRing]), ((n - 1 - j) / kRing) & 1u);
+        }
         // the last block to finish puts the queue back to zero for the next launch
         const int done = atomicAdd(prm.status + 2, 1);
         if (done == (int)gridDim.x - 1) close_launch(prm.status);
