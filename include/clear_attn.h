@@ -127,8 +127,9 @@ typedef struct clear_pair_step {
     int32_t load_base;  /* where this step's tiles sit among the tiles the item stages, counted for every step in
                            turn, its K tiles and then its V tiles.  Low 16 bits: position of the step's first K
                            tile; high 16 bits: position of its first V tile (a step with two distinct key tiles
-                           takes two consecutive positions each time, tile 0's first).  An item whose positions
-                           outgrow 16 bits is not built. */
+                           takes two consecutive positions each time, tile 0's first).  For readers of the
+                           table, like CLEAR_STEP_CLIP* and n_loads: the kernel counts for itself.  An item whose
+                           positions outgrow 16 bits is not built. */
 } clear_pair_step_t;
 
 /* One unit of work of the TCGEN05_WS kernel: two 128-query tiles walking one step list. */
@@ -343,6 +344,11 @@ int clear_plan_create_mask(clear_plan_t **plan, int B, int H, int grid_h, int gr
  * (forward calls return PLAN_MISMATCH).  Errors: INVALID_ARG, UNSUPPORTED, NO_MEMORY. */
 int clear_plan_create_host(clear_plan_t **plan, int B, int H, int grid_h, int grid_w, int n_text,
                            int head_dim, float radius, int dtype, int kernel);
+
+/* The same with the schedule of clear_attn_bwd_bf16_tc (head_dim 64 or 128), whose masked patches name mask-table entries in
+ * n_valid: read it with clear_plan_tables and clear_plan_mask_table. */
+int clear_plan_create_backward_host(clear_plan_t **plan, int B, int H, int grid_h, int grid_w, int n_text, int head_dim,
+                                    float radius);
 
 /* Borrow the host copies of the schedule tables (valid until the plan is destroyed).  Any output
  * pointer may be NULL.  `half_width[dy]`, dy in [0, n_half_width), is the largest |dx| allowed at

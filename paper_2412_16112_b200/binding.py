@@ -26,7 +26,7 @@ STEP_USE0, STEP_USE1, STEP_SHARED, STEP_LINEAR, STEP_MASKED0, STEP_MASKED1 = 1, 
 STEP_CLIP0, STEP_CLIP1 = 64, 128
 
 EXPORTS = [
-    "clear_attn_fwd", "clear_attn_fwd_f32", "clear_plan_create", "clear_plan_create_host",
+    "clear_attn_fwd", "clear_attn_fwd_f32", "clear_plan_create", "clear_plan_create_host", "clear_plan_create_backward_host",
     "clear_plan_tables", "clear_attn_fwd_planned", "clear_attn_fwd_host", "clear_plan_info",
     "clear_plan_check", "clear_plan_destroy", "clear_cache_clear", "clear_status_string",
     "clear_last_cuda_error", "clear_attn_fwd_static", "clear_plan_pair_tables",
@@ -113,6 +113,7 @@ def load() -> ctypes.CDLL:
         plan_args = [ctypes.POINTER(vp), i32, i32, i32, i32, i32, i32, f32, i32, i32]
         lib.clear_plan_create.argtypes = plan_args
         lib.clear_plan_create_host.argtypes = plan_args
+        lib.clear_plan_create_backward_host.argtypes = plan_args[:8]
         lib.clear_plan_create_ex.argtypes = plan_args + [i32, i32]
         lib.clear_plan_tables.argtypes = [vp, ctypes.POINTER(ctypes.POINTER(WorkItem)), ctypes.POINTER(ctypes.c_int32),
                                           ctypes.POINTER(ctypes.POINTER(KvTile)), ctypes.POINTER(ctypes.c_int32),
@@ -278,11 +279,17 @@ class Plan:
     """Owner of a ``clear_plan_t``."""
 
     def __init__(self, B, H, grid_h, grid_w, n_text, head_dim, radius, dtype=BF16, kernel=KERNEL_AUTO,
-                 host_only=False, mask_kind=MASK_DISC, mask_param=0):
+                 host_only=False, mask_kind=MASK_DISC, mask_param=0, backward=False):
         """``radius``: r of the disc / square window, the window size of ``MASK_WINDOWS``, the stride of
-        ``MASK_STRIDED``; ``mask_param``: the shift of the window grid / the layer index of the strided mask."""
+        ``MASK_STRIDED``; ``mask_param``: the shift of the window grid / the layer index of the strided mask;
+        ``backward`` (with ``host_only``): the schedule of the tensor-core backward pass."""
         self._h = ctypes.c_void_p()
-        if mask_kind in (MASK_WINDOWS, MASK_STRIDED) or mask_param != 0:
+        if backward:
+            if not host_only or dtype != BF16 or kernel not in (KERNEL_AUTO, KERNEL_TCGEN05) or mask_kind != MASK_DISC:
+                raise ClearError(ERR_UNSUPPORTED, "clear_plan_create_backward_host")
+            _check(load().clear_plan_create_backward_host(ctypes.byref(self._h), B, H, grid_h, grid_w, n_text, head_dim,
+                                                          float(radius)), "clear_plan_create_backward_host")
+        elif mask_kind in (MASK_WINDOWS, MASK_STRIDED) or mask_param != 0:
             if kernel not in (KERNEL_AUTO, KERNEL_SIMT):
                 raise ClearError(ERR_UNSUPPORTED, "clear_plan_create_mask")
             _check(load().clear_plan_create_mask(ctypes.byref(self._h), B, H, grid_h, grid_w, n_text, head_dim, dtype,

@@ -96,10 +96,9 @@ int create_plan(clear_plan_t **out, const Shape &shape_in, bool host_only)
     try {
         if (kernel == CLEAR_KERNEL_TCGEN05_WS) {
             build_pair_schedule(s, p->sch);
-            // An item whose key-tile list outgrows the 16-bit ring positions of the step records (radii of
-            // about a thousand tokens on grids of millions) cannot run on this kernel, and tile lists of
-            // that length would take gigabytes: the CUDA-core kernel, which walks Eq. 3 without any list,
-            // takes over when the choice was left to the library.
+            // Lists that outgrow the 16-bit positions of the step records (radii of about a thousand tokens on grids
+            // of millions) are not built.  The kernel itself could walk them, but they would take gigabytes: the
+            // CUDA-core kernel, which needs no list, takes over when the choice was left to the library.
             if (p->sch.pair_overflow) {
                 if (s.kernel != CLEAR_KERNEL_AUTO) return CLEAR_ERR_UNSUPPORTED;
                 kernel = CLEAR_KERNEL_SIMT;
@@ -466,6 +465,14 @@ int clear_plan_create_host(clear_plan_t **plan, int B, int H, int grid_h, int gr
                            float radius, int dtype, int kernel)
 {
     Shape s{B, H, grid_h, grid_w, n_text, head_dim, radius, dtype, kernel};
+    return create_plan(plan, s, true);
+}
+
+int clear_plan_create_backward_host(clear_plan_t **plan, int B, int H, int grid_h, int grid_w, int n_text, int head_dim,
+                                    float radius)
+{
+    Shape s{B, H, grid_h, grid_w, n_text, head_dim, radius, CLEAR_BF16, CLEAR_KERNEL_TCGEN05};
+    s.backward = 1;
     return create_plan(plan, s, true);
 }
 

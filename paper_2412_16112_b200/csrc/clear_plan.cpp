@@ -530,8 +530,8 @@ static void build_pairs(const Shape &s, Schedule &sch, MaskTable &masks)
             }
             for (; own < n_own; ++own) own_step(own);
             finish_item(it);
-            // a list too long for the step records' 16-bit ring positions: this kernel cannot run the
-            // shape, and the remaining lists (gigabytes at such radii) are not worth building
+            // a list beyond the 16-bit positions of the step records: the remaining ones (gigabytes at such radii) are
+            // not worth building
             if (sch.pair_overflow) return;
         }
     }

@@ -111,8 +111,8 @@ def test_geometry_matches_the_oracle_mask(gh, gw, T, r):
 
 
 @pytest.mark.parametrize("gh,gw,T,r", SHAPES)
-def test_tile_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r):
-    p = clear.Plan(1, 1, gh, gw, T, 128, r, kernel=clear.KERNEL_TCGEN05, host_only=True)
+def test_tile_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r, backward=False):
+    p = clear.Plan(1, 1, gh, gw, T, 128, r, kernel=clear.KERNEL_TCGEN05, host_only=True, backward=backward)
     info = p.info()
     items, tiles, _ = p.tables()
     N = T + gh * gw
@@ -183,9 +183,23 @@ def test_tile_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r):
     assert np.all(seen_queries[T:] == 1)
     for q0 in range(0, T, 128):
         assert sorted(text_cover[q0]) == list(range(N))
+    if backward:
+        assert info.n_text_splits <= 1
+        table = p.mask_table()
+        for it in items:
+            for t in tiles[it.tile_begin: it.tile_begin + it.tile_count]:
+                if it.kind == 0 and t.flags & clear.TILE_MASKED and not t.flags & clear.TILE_LINEAR:
+                    check_mask_entry(table, t.n_valid, t.x, t.y, it.qx, it.qy, gh, gw, T, r, th, tw)
     if info.n_text_splits > 1:
         assert len(slots) == math.ceil(T / 128) * info.n_text_splits
         assert info.workspace_bytes == len(slots) * 128 * (128 + 2) * 4
+
+
+@pytest.mark.parametrize("gh,gw,T,r", SHAPES + [(45, 70, 17, 12.5), (40, 67, 3, 4.5)])
+def test_backward_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r):
+    """The same schedule but for its text tiles, which are not split, and its masked patches, which name their mask-table
+    entries."""
+    test_tile_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r, backward=True)
 
 
 def key_tokens(x, y, linear, n_valid, gh, gw, T, th, tw):
@@ -197,9 +211,25 @@ def key_tokens(x, y, linear, n_valid, gh, gw, T, th, tw):
     return (T + ys * gw + xs)[ok], bool(ok.all())
 
 
+def check_mask_entry(table, e, x, y, qx, qy, gh, gw, T, r, th, tw):
+    """The table entry of the key patch at (y, x) for the queries at (qy, qx) is the oracle's mask, and 0 for keys off the
+    grid: their rows arrive as zeros, and the kernels rely on the table to leave them out."""
+    assert 0 <= e < len(table), "masked 2-D tile without a mask-table entry"
+    ys, xs = np.meshgrid(np.arange(y, y + th), np.arange(x, x + tw), indexing="ij")
+    on_grid = ((ys >= 0) & (ys < gh) & (xs >= 0) & (xs < gw)).reshape(-1)
+    bits = ((table[e][:, :, None] >> np.arange(32, dtype=np.uint32)) & 1).reshape(128, 128).astype(bool)
+    toks = (T + ys * gw + xs).reshape(-1)
+    assert not bits[:, ~on_grid].any(), "a key off the grid is allowed"
+    for rr in range(128):
+        q_y, q_x = qy + rr // tw, qx + rr % tw
+        if q_y < gh and q_x < gw:
+            row = oracle.mask_row(T + q_y * gw + q_x, gh, gw, T, r).astype(bool)
+            assert np.array_equal(bits[rr][on_grid], row[toks[on_grid]])
+
+
 def check_mask_table(p, items, steps, gh, gw, T, r, th, tw):
-    """Every masked 2-D tile's table entry, restricted to the keys on the grid, is the oracle's mask;
-    the clip flag is set exactly when part of the key patch is off the grid."""
+    """Every masked 2-D tile's table entry (see above); the clip flag is set exactly when part of the key patch is off
+    the grid."""
     table = p.mask_table()
     for it in items:
         if it.kind != 0:
@@ -218,15 +248,7 @@ def check_mask_table(p, items, steps, gh, gw, T, r, th, tw):
                 assert clip == (not on_grid.all())
                 if not st.flags & (clear.STEP_MASKED1 if side else clear.STEP_MASKED0):
                     continue
-                assert 0 <= e < len(table), "masked 2-D tile without a mask-table entry"
-                bits = ((table[e][:, :, None] >> np.arange(32, dtype=np.uint32)) & 1).reshape(128, 128).astype(bool)
-                toks = (T + ys * gw + xs).reshape(-1)
-                for rr in range(128):
-                    q_y, q_x = qy + rr // tw, it.qx + rr % tw
-                    if q_y >= gh or q_x >= gw:
-                        continue
-                    row = oracle.mask_row(T + q_y * gw + q_x, gh, gw, T, r).astype(bool)
-                    assert np.array_equal(bits[rr][on_grid], row[toks[on_grid]])
+                check_mask_entry(table, e, x, y, it.qx, qy, gh, gw, T, r, th, tw)
 
 
 @pytest.mark.parametrize("gh,gw,T,r", SHAPES + [(40, 40, 300, 9.0), (17, 16, 129, 4.0)])
