@@ -7,7 +7,7 @@
 // What bounds it: the fp32 multiply-add units (2 x 64 x 64 x DP multiply-adds a step, DP = the head size rounded up
 // to 64, 128 or 256).  The keys are those of the union of the tile's windows and no others: rows are gathered run by
 // run, 64 at a time, so a step is only ever short at the end of the list.  An 8 x 8 patch is the split that wastes
-// least at the paper's radii with a 4 x 4 register tile: at r = 8 a patch walks 464 + n_text keys for windows of 193.
+// least at the paper's radii with a 4 x 4 register tile: at r = 8 a patch walks 452 + n_text keys for windows of 193.
 // Two blocks share an SM (DP <= 128): one computes while the other waits for its rows.
 // A problem too small to give every SM a tile cuts the lists over a cluster of up to 8 blocks, which merge their
 // partial softmax through distributed shared memory in a fixed order: no workspace, no second launch.
@@ -295,7 +295,7 @@ Extent extent_of(const clear_plan &p, const Geometry &g)
 
 // The fewest blocks with which the longest list is no longer than an even share of all steps over the resident
 // blocks, each with a step of its own: 1 where there are plenty of tiles; 8 for the tiny configuration (10 tiles of at
-// most 5 steps) and for a 1024px problem of two heads, whose text tiles walk 72 steps and its patches 15.
+// most 5 steps) and for a 1024px problem of two heads, whose text tiles walk 72 steps and its patches 16.
 int split_of(const Extent &e, int n_bh, int slots)
 {
     int n = 1;

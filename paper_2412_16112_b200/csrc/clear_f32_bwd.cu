@@ -8,7 +8,8 @@
 //   key kernel: stationary K_j, V_j, streamed Q_i, dO_i with their statistics (the mask is symmetric, so the queries
 //       that see a key are the tokens that key's own query sees).  dV += P^T dO, dK += dS^T Q.
 // Bound by the fp32 multiply-add units: nine products of 64 x 64 x DP per pair of tiles.  The streamed rows go through
-// a ring of three buffers, so a row set travels while the two before it are worked on and a step has two barriers.
+// a ring of three buffers, so a row set travels while the two before it are worked on; a step has two barriers in the query kernel
+// and three in the key kernel.
 // Every output element has one writer and a fixed order of summation (a list cut over a cluster is summed in the order
 // of the ranks): results repeat bit for bit.
 #include <cuda_bf16.h>

@@ -662,7 +662,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             // tiles: 560 us; a third one for the second halves: their MMAs get in the way of the critical ones, 552).
             // One elected lane walks the whole loop.  With the warp walking in step and a lane elected for each group, a vote
             // and two warp barriers stood between a wait's end and the first MMA (1024px: 106 us against 98.5, 2048px: 517
-            // against 499, 8K: 8.40 ms against 8.24).
+            // against 499, 8K: 8.40 ms against 8.24, in short runs at full clock, as the figures above).
             const int t = warp - 1;
             const int use_bit = t ? CLEAR_STEP_USE1 : CLEAR_STEP_USE0;
             constexpr uint32_t kDescHiK = ptx::smem_desc_hi_sw128(1024);  // 8-row groups are 1024 bytes apart
