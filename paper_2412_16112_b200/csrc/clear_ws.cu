@@ -761,18 +761,14 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                     const uint32_t v_st = take_own(pend);
                     // the epilogue must have read the previous item's O_t out of tensor memory
                     if (pv && !acc) wait_lane(ptx::smem_u32(&ctrl->o_empty[t]), (n_it & 1u) ^ 1u, 8);
-                    // Which wait comes first was decided by the clock: P's at 64 channels (67 x 120: 231 us, the turn first
-                    // 236), the turn at 128 (2048px: 506 us, P first 511; 1024px: no difference).
-                    auto wait_p = [&]() {
-                        if (pv) {
-                            wait_lane(b_p, p_par, 7);
-                            p_par ^= 1u;
-                        }
-                    };
-                    if constexpr (D == 64) wait_p();
+                    // P's wait first, then the turn's: the other way round 67 x 120 of 64 channels took 236 us instead of 231;
+                    // at 128 channels there is no difference (2048px 588 and 590 us, runs of one side 0.4 % apart).
+                    if (pv) {
+                        wait_lane(b_p, p_par, 7);
+                        p_par ^= 1u;
+                    }
                     wait_lane(b_turn, turn_par, 11);
                     turn_par ^= 1u;
-                    if constexpr (D != 64) wait_p();
                     if (!ok) break;
                     ptx::tc_fence_after();
                     if (pv) {
