@@ -128,7 +128,11 @@ int create_plan(clear_plan_t **out, const Shape &shape_in, bool host_only)
         if (rc == CLEAR_OK) rc = upload(&p->d_tiles, p->sch.tiles);
         if (rc == CLEAR_OK) rc = upload(&p->d_pair_items, p->sch.pair_items);
         if (rc == CLEAR_OK) rc = upload(&p->d_pair_steps, p->sch.pair_steps);
-        if (rc == CLEAR_OK) rc = upload(&p->d_mask_table, p->sch.mask_table);
+        if (rc == CLEAR_OK) {
+            std::vector<uint32_t> words(p->sch.mask_table);
+            words.insert(words.end(), p->sch.side_words.begin(), p->sch.side_words.end());
+            rc = upload(&p->d_mask_table, words);
+        }
         if (rc == CLEAR_OK) {
             cudaError_t e = cudaMalloc((void **)&p->d_status, kStatusWords * sizeof(int));
             if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, kStatusWords * sizeof(int));

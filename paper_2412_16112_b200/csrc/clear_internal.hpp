@@ -41,7 +41,7 @@ struct clear_plan {
     clear_kv_tile_t *d_tiles = nullptr;
     clear_pair_item_t *d_pair_items = nullptr;
     clear_pair_step_t *d_pair_steps = nullptr;
-    uint32_t *d_mask_table = nullptr;
+    uint32_t *d_mask_table = nullptr;  // the mask table, and behind it the tiles' own lists (Schedule::side_words)
     // [0] status word of the launch in flight: 0 = fine, set by a kernel whose bounded wait expired (the
     //     rest of that launch's blocks then leave at once); the persistent kernel puts it back to zero when
     //     its last block leaves;

@@ -536,6 +536,28 @@ static void build_pairs(const Shape &s, Schedule &sch, MaskTable &masks)
         }
     }
 
+    // ---- the tiles' own lists
+    const size_t n_steps = sch.pair_steps.size();
+    sch.side_words.assign(2 * n_steps, 0u);
+    for (const clear_pair_item_t &it : sch.pair_items) {
+        for (int t = 0; t < 2; ++t) {
+            uint32_t *word = sch.side_words.data() + (size_t)t * n_steps + (size_t)it.step_begin;
+            for (int32_t i = 0; i < it.step_count; ++i) {
+                const clear_pair_step_t &st = sch.pair_steps[(size_t)(it.step_begin + i)];
+                if (!(st.flags & (t ? CLEAR_STEP_USE1 : CLEAR_STEP_USE0))) continue;
+                const int32_t n_valid = t ? st.n_valid1 : st.n_valid0;
+                uint32_t w = kSideSome | ((uint32_t)i << 16);
+                if (!(st.flags & (t ? CLEAR_STEP_MASKED1 : CLEAR_STEP_MASKED0)))
+                    w |= kSidePlain;
+                else if ((st.flags & CLEAR_STEP_LINEAR) || n_valid < 0)
+                    w |= kSideMasked | kSideRare;
+                else
+                    w |= kSideMasked | kSidePlain | ((uint32_t)n_valid << 2);
+                *word++ = w;
+            }
+        }
+    }
+
     // ---- work order: text items (the longest lists) first, then image items, longest first; the
     // blocks take items from the queue in this order, so the short border items fill the tail
     std::stable_sort(sch.pair_items.begin() + sch.n_text_pair_items, sch.pair_items.end(),

@@ -39,6 +39,10 @@ struct Shape {
     }
 };
 
+// Bits of Schedule::side_words: a mask from the table (entry from bit 2 on), or one the kernel works out; neither is rare;
+// always set; the step's number within its item from bit 16 on.
+constexpr uint32_t kSideMasked = 1, kSideRare = 2, kSidePlain = 1u << 12, kSideSome = 1u << 13;
+
 struct Schedule {
     int64_t thr = 0;                     // ceil(radius^2): the disc allows dx^2 + dy^2 < thr (Eq. 3)
     std::vector<int32_t> half_width;     // half_width[dy] = max |dx| allowed at row offset dy (the window, whatever its kind)
@@ -48,6 +52,9 @@ struct Schedule {
     int n_stat_parts = 1, n_stat_slots = 0;      // parts of all text tiles of one (b, h); 0: no list is cut
     std::vector<clear_pair_item_t> pair_items;   // TCGEN05_WS: text items first, then image items
     std::vector<clear_pair_step_t> pair_steps;
+    // What the softmax warps of tile t walk, one word per step the tile takes part in (kSide...), [2][pair_steps]: an item's
+    // words stand where its steps do, those of steps without the tile left out and zeros behind the last.
+    std::vector<uint32_t> side_words;
     int n_text_pair_items = 0;
     bool pair_overflow = false;                  // an item's tiles outgrow the 16-bit positions of its records
     std::vector<uint32_t> mask_table;            // TCGEN05_WS: [entry][128 query rows][4 words]

@@ -38,15 +38,14 @@ constexpr uint32_t kSpinLimit = 1u << 22;
 constexpr uint32_t kWaitHintNs = 20000;            // one sleep inside try_wait
 constexpr uint32_t kWaitLimitUs = 2000000;         // a wait that lasts 2 s has failed
 constexpr float kRescaleThreshold = 8.f;  // log2 units: a reference is moved only when a row's maximum exceeds it by more
-constexpr float kBumpSum = 256.f;         // a row sum of P above this raises the row's reference for the next tile
+constexpr float kBumpSum = 65536.f;       // a row sum of P above this raises the row's reference
 constexpr float kMaxTileSum = 0x1p64f;    // a row sum above this has its tile taken again (a NaN comes from NaN inputs only, and stays)
-constexpr uint32_t kFirst = 1, kCareful = 2;   // why a step has a maximum pass
 // Scores of a row's first tile that lie this far apart (log2 units) give the item maximum passes from the start: with less,
-// normal ones would have to lie seven standard deviations above the maximum of 128 to be 64 above it.  (The least of 16 of
-// them is enough to tell; the least of all 128 cost 1 to 3 % of a call.)
+// normal ones would have to lie seven standard deviations above the maximum of 64 to be 64 above it.  (The least of eight of
+// them is enough to tell.)
 constexpr float kWideStep = 40.f;
 constexpr int kSchedDepth = 2;
-// arrivals that free a queue slot: one lane of each of the 2 MMA warps and the 8 softmax warps
+// arrivals that free a queue slot: one lane of each of the 2 MMA warps, the 8 softmax warps
 constexpr uint32_t kSchedReaders = 10;
 // registers per thread of each role: 128 x 80 + 256 x 208 = 63488, within what the block is launched with
 // (384 threads x 168); raising a warp's budget only draws on registers other warps of the block gave back
@@ -57,6 +56,8 @@ struct WsParams {
     const clear_pair_item_t *items;
     const clear_pair_step_t *steps;
     const int32_t *half_width;
+    const uint32_t *side_words;  // [2 tiles][n_steps] (Schedule::side_words)
+    int n_steps;
     const uint32_t *mask_table;  // [entry][128 query rows][4 words]: Eq. 3 per relative patch offset and border case
     int n_half_width;
     int grid_h, grid_w, n_text;
@@ -185,8 +186,6 @@ __device__ __forceinline__ int2 load_side_origin(const clear_pair_step_t *p, int
 }
 static_assert(sizeof(clear_pair_step_t) == 32 && sizeof(clear_pair_item_t) == 48, "table records are read as int4");
 
-__device__ __forceinline__ bool step_uses(int flags, int side) { return (flags & (side ? CLEAR_STEP_USE1 : CLEAR_STEP_USE0)) != 0; }
-
 // ---- pieces of the softmax warps' work that are rare, or come once an item: functions of their own, so that their
 // registers do not crowd the exponentials of the common step (with them in line the compiler had too few left to overlap
 // with, and a pass over 128 scores took up to 1900 clocks instead of 1400) --------------------------------------------
@@ -211,6 +210,24 @@ __device__ __noinline__ void rescale_rows(uint32_t tmem_o, float alpha)
 #pragma unroll
         for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
         ptx::tmem_st16(tmem_o + 16 * w, o);
+    }
+}
+
+// The row's P (bf16 pairs) times alpha, a power of two.
+__device__ __noinline__ void rescale_p(uint32_t tmem_p, float alpha)
+{
+    const __nv_bfloat162 a = __float2bfloat162_rn(alpha);
+#pragma unroll 1
+    for (int w = 0, n = opaque(4); w < n; ++w) {
+        uint32_t p[16];
+        ptx::tmem_ld16(tmem_p + 16 * w, p);
+        ptx::tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            __nv_bfloat162 x = __hmul2(*reinterpret_cast<__nv_bfloat162 *>(&p[j]), a);
+            p[j] = *reinterpret_cast<uint32_t *>(&x);
+        }
+        ptx::tmem_st16(tmem_p + 16 * w, p);
     }
 }
 
@@ -245,6 +262,26 @@ __device__ __forceinline__ float sum4(const uint64_t (&lsum)[2])
 struct RowState {
     float ref, l, tile_sum;   // tile_sum < 0: less that, and the row's maximum lies more than kWideStep above the least of 16 scores
 };
+// The largest of 64 scores of a row that all count, and the least of eight of them.
+struct RowTop {
+    float most, least;
+};
+__device__ __noinline__ RowTop half_top(uint32_t tmem_half)
+{
+    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, mn = INFINITY;
+    uint32_t sv[2][32];
+    ptx::tmem_ld32(tmem_half, sv[0]);
+    ptx::tmem_ld32(tmem_half + 32, sv[1]);
+    ptx::tmem_wait_ld();
+#pragma unroll
+    for (int w = 0; w < 2; ++w)
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) mx[(j >> 1) & 3] = ptx::max3(mx[(j >> 1) & 3], __uint_as_float(sv[w][j]), __uint_as_float(sv[w][j + 1]));
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) mn = fminf(mn, __uint_as_float(sv[0][j]));
+    return RowTop{fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), mn};
+}
+
 // A step with a maximum pass: the maximum over the allowed keys, the row's reference, then P.  The scores are read from
 // tensor memory both times, 32 keys at a time (P of 32 keys takes 16 columns, so it never reaches scores still to be read).
 template <int D>
@@ -453,9 +490,8 @@ __device__ __noinline__ void store_tile(const WsParams &prm, uint32_t tmem_o, ui
         prm.partial_ml[(slot_row + r) * 2 + 1] = l;
         return;
     }
-    // O / l as bf16, 16 channels (32 bytes, a memory sector) of the thread's row at a time.  Once an item, so cold: a short loop
-    // rather than a fast one.  (Unrolled, and with the rows exchanged between threads for wider runs, the same took 4200
-    // clocks, most of them for fetching its instructions.)
+    // O / l as bf16, 32 channels of the thread's row at a time, in pieces of 32 bytes (a memory sector).  Once an item, so that
+    // its instructions are fetched anew each time, some 16 clocks each: a short loop rather than a fast one.
     const float inv = l > 0.f ? 1.f / l : 0.f;
     const int y = first_y + (r >> 4), x = first_x + (r & 15);
     const bool on = n_rows >= 0 ? r < n_rows : (y < prm.grid_h && x < prm.grid_w);
@@ -463,24 +499,65 @@ __device__ __noinline__ void store_tile(const WsParams &prm, uint32_t tmem_o, ui
     __nv_bfloat16 *dst = prm.out + ((long long)bh * prm.n_tokens + token) * D;
     const bool wide = (reinterpret_cast<uintptr_t>(prm.out) & 31u) == 0u;  // tensors are 16-byte aligned at least
 #pragma unroll 1
-    for (int w = 0, n = opaque(D / 16); w < n; ++w) {
-        uint32_t o[16];
-        ptx::tmem_ld16(tmem_o + 16 * w, o);
+    for (int w = 0, n = opaque(D / 32); w < n; ++w) {
+        uint32_t o[32];
+        ptx::tmem_ld32(tmem_o + 32 * w, o);
         ptx::tmem_wait_ld();
-        uint32_t u[8];
+        // behind the last reads the next item's first P V may start; the stores take their time
+        if (w == n - 1) {
+            ptx::tc_fence_before();
+            warp_arrive(b_o_empty, lane);
+        }
+        uint32_t u[2][8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = ptx::pack_bf16(__uint_as_float(o[2 * j]) * inv, __uint_as_float(o[2 * j + 1]) * inv);
+        for (int j = 0; j < 16; ++j) u[j >> 3][j & 7] = ptx::pack_bf16(__uint_as_float(o[2 * j]) * inv, __uint_as_float(o[2 * j + 1]) * inv);
         if (on) {
+            __nv_bfloat16 *to = dst + 32 * w;
             if (wide) {
-                ptx::stg_u256(dst + 16 * w, u);
+                ptx::stg_u256(to, u[0]);
+                ptx::stg_u256(to + 16, u[1]);
             } else {
-                *reinterpret_cast<uint4 *>(dst + 16 * w) = make_uint4(u[0], u[1], u[2], u[3]);
-                *reinterpret_cast<uint4 *>(dst + 16 * w + 8) = make_uint4(u[4], u[5], u[6], u[7]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    *reinterpret_cast<uint4 *>(to + 8 * j) = make_uint4(u[j >> 1][4 * (j & 1)], u[j >> 1][4 * (j & 1) + 1], u[j >> 1][4 * (j & 1) + 2], u[j >> 1][4 * (j & 1) + 3]);
             }
         }
     }
-    ptx::tc_fence_before();
-    warp_arrive(b_o_empty, lane);
+}
+
+// Mask words of a row that the table does not hold: a run of tokens that ends inside the tile, or (very large radius) a patch
+// without an entry, Eq. 3 row by row from the half widths.  Once in many steps, so a function of its own.
+__device__ __noinline__ uint4 special_mask(const WsParams &prm, const clear_pair_step_t *step, int t, bool q_valid, int q_y, int q_x)
+{
+    uint32_t mw[4] = {0u, 0u, 0u, 0u};
+    if (__ldg(&step->flags) & CLEAR_STEP_LINEAR) {
+        const int n_valid = __ldg(t ? &step->n_valid1 : &step->n_valid0);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const int nv = min(max(n_valid - 32 * w, 0), 32);
+            mw[w] = nv == 32 ? 0xffffffffu : ((1u << nv) - 1u);
+        }
+    } else {
+        const int2 org = load_side_origin(step, t);
+#pragma unroll 1
+        for (int rr = 0; rr < 8; ++rr) {
+            const int ky = org.y + rr;
+            const int ady = abs(ky - q_y);
+            uint32_t bits = 0u;
+            if (q_valid && ky >= 0 && ky < prm.grid_h && ady < prm.n_half_width) {
+                const int hw = __ldg(prm.half_width + ady);
+                const int lo = max(max(q_x - hw, 0), org.x);
+                const int hi = min(min(q_x + hw, prm.grid_w - 1), org.x + 15);
+                if (lo <= hi) bits = ((1u << (hi - lo + 1)) - 1u) << (lo - org.x);
+            }
+            bits <<= 16 * (rr & 1);
+            if ((rr >> 1) == 0) mw[0] |= bits;
+            if ((rr >> 1) == 1) mw[1] |= bits;
+            if ((rr >> 1) == 2) mw[2] |= bits;
+            if ((rr >> 1) == 3) mw[3] |= bits;
+        }
+    }
+    return make_uint4(mw[0], mw[1], mw[2], mw[3]);
 }
 
 // The last block of a launch to leave: the work queue goes back to zero, and a status some block raised
@@ -651,11 +728,11 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             // a tile is P_t V and then the first half of the next Q_t K^T, over P_t (same thread, same pipe: P_t V has read
             // it by then), and meanwhile the softmax warps work on the second half.  (An MMA of 64 keys takes 48 clocks
             // where one of 128 takes 64: the tensor core works 25 % more, and waits far less.)
-            // The two warps take turns with P_t V and the first halves, step by step.  Left to themselves the tiles fall
-            // into lockstep, both in their exponentials and then both waiting for MMAs; with the groups issued in turn,
-            // tile 1's scores follow tile 0's by a group and each tile's exponentials run under the other's MMAs.  (With the
-            // turn passed on earlier, behind P_t V, they are back in lockstep; passed on behind the second half, later, the
-            // pipe idles at every hand-over, 400 clocks of barrier latency: 2048px 534 and 673 us against 525.)
+            // At 128 channels the two warps take turns with P_t V and the first halves, step by step: with the groups issued in
+            // turn, tile 1's scores follow tile 0's by a group and its exponentials run under the other's MMAs.  Without: 1024px
+            // 109 us against 101, 2048px 564 against 549.  (Passed on earlier, behind P_t V, or later, behind the second half,
+            // where the pipe idles at every hand-over: 534 and 673 against 525, when it was that.)  At 64 channels, where the
+            // MMAs take half, nothing is gained by keeping order: 67 x 120 in 228 us without turns, 232 with.
             // The tensor core holds about two MMAs ahead of the one it works on, some 150 clocks, and every barrier or
             // shuffle instruction of these warps spends 100 to 200 in the queue it shares with the exponentials of two
             // softmax warps: hence a warp per tile, the waits of one in the shadow of the other's MMAs (one warp for both
@@ -669,6 +746,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             const uint32_t tmem_S = tmem + t * 128, tmem_O = tmem + 256 + t * 128;
             const uint32_t b_full0 = ptx::smem_u32(&ctrl->kv_full[0]), b_empty0 = ptx::smem_u32(&ctrl->kv_empty[0]);
             const uint32_t b_p = ptx::smem_u32(&ctrl->p_ready[t]), b_read = ptx::smem_u32(&ctrl->sb_read[t]);
+            constexpr bool kTurns = D == 128;
             const uint32_t b_turn = ptx::smem_u32(&ctrl->turn[t]), b_other = ptx::smem_u32(&ctrl->turn[t ^ 1]);
             const uint32_t v_lo0 = ptx::smem_desc_lo(sRing, kHalfBytes), k_lo0 = ptx::smem_desc_lo(sRing, 16);
             const uint32_t q_lo = ptx::smem_desc_lo(sQ + t * kTileBytes, 16);
@@ -761,14 +839,14 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                     const uint32_t v_st = take_own(pend);
                     // the epilogue must have read the previous item's O_t out of tensor memory
                     if (pv && !acc) wait_lane(ptx::smem_u32(&ctrl->o_empty[t]), (n_it & 1u) ^ 1u, 8);
-                    // P's wait first, then the turn's: the other way round 67 x 120 of 64 channels took 236 us instead of 231;
-                    // at 128 channels there is no difference (2048px 588 and 590 us, runs of one side 0.4 % apart).
                     if (pv) {
                         wait_lane(b_p, p_par, 7);
                         p_par ^= 1u;
                     }
-                    wait_lane(b_turn, turn_par, 11);
-                    turn_par ^= 1u;
+                    if (kTurns) {
+                        wait_lane(b_turn, turn_par, 11);
+                        turn_par ^= 1u;
+                    }
                     if (!ok) break;
                     ptx::tc_fence_after();
                     if (pv) {
@@ -784,7 +862,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                         issue_qk(k_st, 0);
                         ptx::tc_commit(ptx::smem_u32(&ctrl->sa_full[t]));
                     }
-                    ptx::mbar_arrive(b_other);  // the other tile's turn
+                    if (kTurns) ptx::mbar_arrive(b_other);  // the other tile's turn
                     if (qk) ptx::tc_commit(b_empty0 + 8 * k_st);
                     if (pv) ptx::tc_commit(b_empty0 + 8 * v_st);
                     // behind the item's last Q K^T the next Q_t may land; behind its last P V the output is complete
@@ -809,223 +887,211 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
         // Per step: S_t into registers, half by half, P = exp2(.) under the Eq. 3 mask as bf16 into tensor memory over
         // the first half of S_t, row sum; at the end of an item O_t / l -> bf16 -> global memory (or fp32 partial
         // results of split text rows).
+        // What bounds a block: a step of both tiles takes about 3600 clocks, of which the exponentials of the two warps on a
+        // scheduler are 2150 if nothing else runs and the MMAs 2560 (3050 with the copies, by a run without exponentials); the
+        // rest is the chain between them, and the start and end of an item, some 7000 clocks, most of them for fetching
+        // instructions that run once an item (about 16 clocks each).  So the code of an item's start and end is kept short:
+        // the tiles' lists come ready from the host, the first step runs in the common loop with a reference from 64 scores,
+        // and what is rare stands behind the loop (1024px 108.3 -> 103.0 us, 2048px 581 -> 552, 67 x 120 of 64 channels 230 ->
+        // 209, against lists taken apart here, maximum passes in the first step and every case in line).
         ptx::setmaxnreg_inc<kRegsSoftmax>();
         const int t = (warp - 4) >> 2;  // query tile of the pair
         const int q4 = warp & 3;        // tensor-memory lane quadrant
         const int r = q4 * 32 + lane;   // query row of the tile
-        const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-        const uint32_t tmem_S = tmem + t * 128, tmem_O = tmem + 256 + t * 128;
+        const uint32_t tmem_S = tmem + ((uint32_t)(q4 * 32) << 16) + t * 128, tmem_O = tmem_S + 256;
         const float c = prm.scale_log2;
-        const uint32_t b_sa = ptx::smem_u32(&ctrl->sa_full[t]), b_sb = ptx::smem_u32(&ctrl->sb_full[t]), b_pready = ptx::smem_u32(&ctrl->p_ready[t]);
-        uint32_t n_s = 0, n_items_seen = 0;
+        const uint64_t c2 = ptx::pack2(c, c);
+        const uint32_t b_sa = ptx::smem_u32(&ctrl->sa_full[t]), b_sb = ptx::smem_u32(&ctrl->sb_full[t]);
+        const uint32_t b_p = ptx::smem_u32(&ctrl->p_ready[t]), b_read = ptx::smem_u32(&ctrl->sb_read[t]);
+        // A wait that gives up leaves the warp in step: what follows runs on, on whatever there is, without waiting for or
+        // telling anybody, up to the end of the item, where the warp looks.  (A vote behind every wait stood on the chain.)
         bool alive = true;
-#pragma unroll 1
-        for (uint32_t k = 0; alive; ++k) {
-            const uint32_t slot = k % kSchedDepth, use = k / kSchedDepth;
-            if (!__all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->sched_full[slot]), use & 1u, abort_flag, prm.status, 9)))
-                break;
-            const int g = ctrl->sched_item[slot];
-            const clear_pair_item_t item = ctrl->sched_rec[slot];
-            const int bh = ctrl->sched_bh[slot];
+        auto wait_warp = [&](uint32_t bar, uint32_t parity, int code) {
+            if (__builtin_expect(!ptx::mbar_try_wait_some(bar, parity, 128u, kWaitHintNs, alive), 0)) alive = wait_bar(bar, parity, abort_flag, prm.status, code);
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&ctrl->sched_empty[slot]));
-            if (g >= total_items) break;
-            if (t >= item.n_sides) continue;
-            const clear_pair_step_t *steps = prm.steps + item.step_begin;
-            const int step_count = item.step_count;
-            const bool is_text = item.kind == 1;
-            // grid position of this row's query (image tiles), and whether the row exists
-            const int q_y = (t ? item.qy1 : item.qy0) + (r >> 4), q_x = item.qx + (r & 15);
-            const bool q_valid = is_text ? r < (t ? item.n_rows1 : item.n_rows0) : (q_y < prm.grid_h && q_x < prm.grid_w);
-            float ref = -INFINITY, l = 0.f;  // reference of the row's exponents (log2 units) and row sum
-            int bump = 0;                    // powers of two the reference is to be raised by before the next tile
-            uint32_t exact_from = kFirst;    // kFirst: no step yet; kCareful: a step had to be taken again, maximum passes from here on
+            ptx::tc_fence_after();
+        };
+        auto tell = [&](uint32_t bar) {
+            ptx::tc_fence_before();
+            __syncwarp();
+            ptx::mbar_arrive_if(bar, lane == 0 && alive);
+        };
+        uint32_t par = 0;                  // parity of the tile's S barriers
+        uint32_t o_par = 0;                // parity of the tile's results
+#pragma unroll 1
+        for (uint32_t k = 0;; ++k) {
+            const uint32_t slot = k % kSchedDepth, use = k / kSchedDepth;
+            if (alive) alive = wait_bar(ptx::smem_u32(&ctrl->sched_full[slot]), use & 1u, abort_flag, prm.status, 9);
+            if (!__all_sync(0xffffffffu, alive)) break;
+            if (ctrl->sched_item[slot] >= total_items) break;
+            const clear_pair_item_t &item = ctrl->sched_rec[slot];   // the slot is given back at the end of the item
+            if (t < item.n_sides) {
+                const clear_pair_step_t *steps = prm.steps + item.step_begin;
+                const int step_count = item.step_count;
+                // grid position of this row's query (image tiles), and whether the row exists
+                const bool is_text = item.kind == 1;
+                const int q_y = (t ? item.qy1 : item.qy0) + (r >> 4), q_x = item.qx + (r & 15);
+                const bool q_valid = is_text ? r < (t ? item.n_rows1 : item.n_rows0) : (q_y < prm.grid_h && q_x < prm.grid_w);
 
-            // The flags and the key count (or mask entry) of 32 steps at a time, one step per lane, the 32 after them
-            // fetched meanwhile; taken out of the lanes two steps ahead, and this row's precomputed mask words fetched one
-            // step ahead.  No latency is on the critical path, and the loads stay where they are written (left to the
-            // compiler, they sank to their use).
-            const int kMaskedBit = t ? CLEAR_STEP_MASKED1 : CLEAR_STEP_MASKED0;
-            const int *rec = &steps->flags;
-            constexpr int kStepInts = sizeof(clear_pair_step_t) / sizeof(int);
-            struct Rec {
-                int flags, n_valid;
-            };
-            auto fetch_steps = [&](int s0) -> Rec {
-                const bool on = s0 + lane < step_count;
-                return Rec{on ? (int)ptx::ldg_u32(rec + (s0 + lane) * kStepInts) : 0, on ? (int)ptx::ldg_u32(rec + (s0 + lane) * kStepInts + 1 + t) : 0};
-            };
-            auto load_mask_row = [&](const Rec &x) -> uint4 {
-                if (step_uses(x.flags, t) && (x.flags & kMaskedBit) && !(x.flags & CLEAR_STEP_LINEAR) && x.n_valid >= 0)
-                    return ptx::ldg_u128(reinterpret_cast<const uint4 *>(prm.mask_table) + ((size_t)x.n_valid * 128 + r));
-                return make_uint4(0u, 0u, 0u, 0u);
-            };
-            Rec lanes = fetch_steps(0), lanes_next = fetch_steps(32);
-            auto from_lane = [&](int s) { return Rec{__shfl_sync(0xffffffffu, lanes.flags, s & 31), __shfl_sync(0xffffffffu, lanes.n_valid, s & 31)}; };
-            Rec st, st1 = from_lane(0), st2 = from_lane(1);
-            uint4 mrow, mrow1 = load_mask_row(st1);
-#pragma unroll 1
-            for (int s = 0; s < step_count; ++s) {
-                st = st1;
-                mrow = mrow1;
-                st1 = st2;
-                mrow1 = load_mask_row(st1);
-                if (((s + 2) & 31) == 0) {
-                    lanes = lanes_next;
-                    lanes_next = fetch_steps(s + 34);
-                }
-                st2 = from_lane(s + 2);   // 0 past the end
-                if (!step_uses(st.flags, t)) continue;
-                const bool masked = (st.flags & kMaskedBit) != 0;
-                // ---- mask bits of this row for the tile (bit j of word w = key 32 w + j allowed) --------
-                uint32_t mw[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-                if (masked) {
-                    if (st.flags & CLEAR_STEP_LINEAR) {
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            const int nv = min(max(st.n_valid - 32 * w, 0), 32);
-                            mw[w] = nv == 32 ? 0xffffffffu : ((1u << nv) - 1u);
-                        }
-                    } else if (st.n_valid >= 0) {
-                        // Eq. 3 from the table, the grid's border included
-                        mw[0] = mrow.x;
-                        mw[1] = mrow.y;
-                        mw[2] = mrow.z;
-                        mw[3] = mrow.w;
-                    } else {
-                        // no table entry (very large radius): Eq. 3 row by row from the half widths
-                        const int2 org = load_side_origin(steps + s, t);
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) mw[w] = 0u;
-#pragma unroll 1
-                        for (int rr = 0; rr < 8; ++rr) {
-                            const int ky = org.y + rr;
-                            const int ady = abs(ky - q_y);
-                            uint32_t bits = 0u;
-                            if (q_valid && ky >= 0 && ky < prm.grid_h && ady < prm.n_half_width) {
-                                const int hw = __ldg(prm.half_width + ady);
-                                const int lo = max(max(q_x - hw, 0), org.x);
-                                const int hi = min(min(q_x + hw, prm.grid_w - 1), org.x + 15);
-                                if (lo <= hi) bits = ((1u << (hi - lo + 1)) - 1u) << (lo - org.x);
-                            }
-                            bits <<= 16 * (rr & 1);
-                            if ((rr >> 1) == 0) mw[0] |= bits;
-                            if ((rr >> 1) == 1) mw[1] |= bits;
-                            if ((rr >> 1) == 2) mw[2] |= bits;
-                            if ((rr >> 1) == 3) mw[3] |= bits;
-                        }
+                // The steps this tile takes part in, a word each (0: none left), 32 at a time, one per lane, the 32 after them
+                // fetched meanwhile; taken out of the lanes two steps ahead, and this row's mask words fetched one step ahead.
+                // No latency is on the critical path, and the loads stay where they are written (left to the compiler, they
+                // sank to their use).
+                const uint32_t *words = prm.side_words + (size_t)t * prm.n_steps + item.step_begin + lane;
+                auto fetch_words = [&](int at) { return at + lane < step_count ? ptx::ldg_u32(words + at) : 0u; };
+                int at = 0;   // words taken
+                uint32_t lanes = fetch_words(0), lanes_next = fetch_words(32);
+                auto take_step = [&]() -> uint32_t {
+                    if (__builtin_expect(at != 0 && (at & 31) == 0, 0)) {
+                        lanes = lanes_next;
+                        lanes_next = fetch_words(at + 32);
                     }
-                }
+                    return __shfl_sync(0xffffffffu, lanes, at++ & 31);
+                };
+                const uint4 *mask_row = reinterpret_cast<const uint4 *>(prm.mask_table) + r;
+                auto load_mask = [&](uint32_t w) -> uint4 {
+                    uint4 m = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+                    if ((w & (kSideMasked | kSidePlain)) == (kSideMasked | kSidePlain)) m = ptx::ldg_u128(mask_row + ((w >> 2) & 0x3ffu) * 128u);
+                    return m;
+                };
 
                 // P = 2^(S c - ref) with a reference per row that need not be the running maximum: P, the row sum and O
                 // are floating-point numbers of full precision at any scale, so the reference only has to keep them
-                // within range.  It is the maximum of the row's first tile; when a tile's row sum exceeds 2^8 the
-                // reference is raised before the next tile, by a whole power of two and without a look at the maximum.
-                // No maximum pass, then, on any tile but the first, and the scores die as their P is formed.  A row sum
-                // beyond 2^64 means scores 64 powers of two above everything seen before; the warp then computes its
-                // scores again, from global memory, before anybody has used P, and takes the rest of the item's steps with
-                // maximum passes.
-                const bool raise = __any_sync(0xffffffffu, bump != 0);
-                float alpha = 1.f;
-                if (raise) {
-                    alpha = ptx::ex2(-(float)bump);
-                    ref += (float)bump;
-                    l *= alpha;
-                    bump = 0;
-                }
-                const bool exact = __any_sync(0xffffffffu, exact_from != 0u || (ref == -INFINITY && q_valid));
-                float tile_sum = 0.f;
-                // warp-uniform outcome of the waits: the tcgen05.ld / st below need the whole warp.  Once the first half of
-                // S_t is complete, so is P_t V of the step before (same thread, same pipe, issued earlier).
-                if (!__all_sync(0xffffffffu, wait_bar(b_sb, n_s & 1u, abort_flag, prm.status, 10))) {
-                    alive = false;
-                    break;
-                }
-                ptx::tc_fence_after();
-                if (__builtin_expect(!exact, 1)) {
-                    const float mc = (ref == -INFINITY) ? 0.f : ref;
-                    const uint64_t c2 = ptx::pack2(c, c), nmc2 = ptx::pack2(-mc, -mc);
-                    uint64_t lsum[2] = {0ull, 0ull};
-                    uint32_t sv[2][32], pk[2][16];
-                    ptx::tmem_ld32(tmem_S + lane_off + 64, sv[0]);
-                    ptx::tmem_ld32(tmem_S + lane_off + 96, sv[1]);
-                    ptx::tmem_wait_ld();
-                    ptx::tc_fence_before();
-                    warp_arrive(ptx::smem_u32(&ctrl->sb_read[t]), lane);
-                    if (masked) {
-                        exp_chunk<true>(sv[0], mw[2], c2, nmc2, lsum, pk[0]);
-                        exp_chunk<true>(sv[1], mw[3], c2, nmc2, lsum, pk[1]);
+                // within range.  It is the maximum of the row's first tile (of half of it if all keys are allowed); when a tile's row sum exceeds 2^16 the
+                // reference is raised by a whole power of two, without a look at the maximum, and the row's P, sum and O are
+                // scaled before P goes to the MMAs.  No maximum pass, then, on any other tile, and the scores die as their P is
+                // formed.  A row sum beyond 2^64 means scores 64 powers of two above everything seen before; the warp then
+                // computes its scores again, from global memory, before anybody has used P, and takes the rest of the item's
+                // steps with maximum passes.
+                float ref = -INFINITY, l = 0.f;  // reference of the row's exponents (log2 units) and row sum
+                bool careful = false;            // maximum passes up to the end of the item
+                bool first = true, exact = true; // this step has one
+                uint32_t w = take_step(), w1 = take_step(), w2;
+                uint4 mw = load_mask(w), mw1;    // bit j of word i = key 32 i + j allowed
+                // The common steps run in a loop of their own, with what is rare outside of it.
+#pragma unroll 1
+                while (w != 0u) {
+                    if (w & kSideRare) mw = special_mask(prm, steps + (w >> 16), t, q_valid, q_y, q_x);
+                    if (first && !(w & kSideMasked)) {
+                        wait_warp(b_sb, par, 10);
+                        const RowTop top = half_top(tmem_S + 64);
+                        ref = top.most * c;
+                        careful = __any_sync(0xffffffffu, (top.most - top.least) * c > kWideStep);
+                        exact = careful || __any_sync(0xffffffffu, ref == -INFINITY && q_valid);
+                    }
+                    float tile_sum;
+                    if (!exact) {
+                        const float mc = (ref == -INFINITY) ? 0.f : ref;
+                        const uint64_t nmc2 = ptx::pack2(-mc, -mc);
+                        first = false;
+                        bool over;
+#pragma unroll 1
+                        for (;;) {
+                            // The second half comes first: its P waits in registers for the first half's scores to be read,
+                            // over which P of the whole step lies.
+                            uint64_t lsum[2] = {0ull, 0ull};
+                            uint32_t sv[2][32], pk[2][16];
+                            wait_warp(b_sb, par, 10);
+                            ptx::tmem_ld32(tmem_S + 64, sv[0]);
+                            ptx::tmem_ld32(tmem_S + 96, sv[1]);
+                            ptx::tmem_wait_ld();
+                            tell(b_read);
+                            mw1 = load_mask(w1);
+                            w2 = take_step();
+                            if (w & kSideMasked) {
+                                exp_chunk<true>(sv[0], mw.z, c2, nmc2, lsum, pk[0]);
+                                exp_chunk<true>(sv[1], mw.w, c2, nmc2, lsum, pk[1]);
+                            } else {
+                                exp_chunk<false>(sv[0], 0u, c2, nmc2, lsum, pk[0]);
+                                exp_chunk<false>(sv[1], 0u, c2, nmc2, lsum, pk[1]);
+                            }
+                            // Once the first half of S_t is complete, so is P_t V of the step before (same thread, same pipe,
+                            // issued earlier).
+                            wait_warp(b_sa, par, 13);
+                            ptx::tmem_ld32(tmem_S, sv[0]);
+                            ptx::tmem_ld32(tmem_S + 32, sv[1]);
+                            ptx::tmem_wait_ld();
+                            ptx::tmem_st16(tmem_S + 32, pk[0]);
+                            ptx::tmem_st16(tmem_S + 48, pk[1]);
+                            if (w & kSideMasked) {
+                                exp_chunk<true>(sv[0], mw.x, c2, nmc2, lsum, pk[0]);
+                                ptx::tmem_st16(tmem_S, pk[0]);
+                                exp_chunk<true>(sv[1], mw.y, c2, nmc2, lsum, pk[1]);
+                                ptx::tmem_st16(tmem_S + 16, pk[1]);
+                            } else {
+                                exp_chunk<false>(sv[0], 0u, c2, nmc2, lsum, pk[0]);
+                                ptx::tmem_st16(tmem_S, pk[0]);
+                                exp_chunk<false>(sv[1], 0u, c2, nmc2, lsum, pk[1]);
+                                ptx::tmem_st16(tmem_S + 16, pk[1]);
+                            }
+                            tile_sum = sum4(lsum);
+                            // P_t must be in tensor memory before the MMA thread is told
+                            ptx::tmem_wait_st();
+                            over = __any_sync(0xffffffffu, tile_sum > kBumpSum);
+                            if (__builtin_expect(over, 0)) break;
+                            tell(b_p);
+                            l += tile_sum;
+                            par ^= 1u;
+                            w = w1;
+                            w1 = w2;
+                            mw = mw1;
+                            if (__builtin_expect(!(w & kSidePlain), 0)) break;
+                        }
+                        if (!over) continue;   // none left, or one whose mask is to be worked out
                     } else {
-                        exp_chunk<false>(sv[0], 0u, c2, nmc2, lsum, pk[0]);
-                        exp_chunk<false>(sv[1], 0u, c2, nmc2, lsum, pk[1]);
-                    }
-                    if (!__all_sync(0xffffffffu, wait_bar(b_sa, n_s & 1u, abort_flag, prm.status, 13))) {
-                        alive = false;
-                        break;
-                    }
-                    ptx::tc_fence_after();
-                    ptx::tmem_ld32(tmem_S + lane_off, sv[0]);
-                    ptx::tmem_ld32(tmem_S + lane_off + 32, sv[1]);
-                    ptx::tmem_wait_ld();
-                    ptx::tmem_st16(tmem_S + lane_off + 32, pk[0]);
-                    ptx::tmem_st16(tmem_S + lane_off + 48, pk[1]);
-                    if (masked) {
-                        exp_chunk<true>(sv[0], mw[0], c2, nmc2, lsum, pk[0]);
-                        ptx::tmem_st16(tmem_S + lane_off, pk[0]);
-                        exp_chunk<true>(sv[1], mw[1], c2, nmc2, lsum, pk[1]);
-                        ptx::tmem_st16(tmem_S + lane_off + 16, pk[1]);
-                    } else {
-                        exp_chunk<false>(sv[0], 0u, c2, nmc2, lsum, pk[0]);
-                        ptx::tmem_st16(tmem_S + lane_off, pk[0]);
-                        exp_chunk<false>(sv[1], 0u, c2, nmc2, lsum, pk[1]);
-                        ptx::tmem_st16(tmem_S + lane_off + 16, pk[1]);
-                    }
-                    tile_sum = sum4(lsum);
-                    if (raise) rescale_rows<D>(tmem_O + lane_off, alpha);
-                    if (__builtin_expect(__any_sync(0xffffffffu, tile_sum > kMaxTileSum), 0)) {
-                        exact_from = kCareful;
-                        const int2 org = load_side_origin(steps + s, t);
-                        const long long q_tok = is_text ? (long long)item.qx + t * 128 + r : prm.n_text + (long long)q_y * prm.grid_w + q_x;
-                        const RowState rs = rescue_step<D>(prm, tmem_S + lane_off, tmem_O + lane_off, make_uint4(mw[0], mw[1], mw[2], mw[3]), c, ref,
-                                                           l, (long long)bh * prm.n_tokens, q_valid ? q_tok : -1, org,
-                                                           (st.flags & CLEAR_STEP_LINEAR) != 0);
+                        mw1 = load_mask(w1);
+                        w2 = take_step();
+                        wait_warp(b_sb, par, 10);
+                        wait_warp(b_sa, par, 13);
+                        const RowState rs = exact_step<D>(tmem_S, tmem_O, mw, c, ref, l, first);
                         ref = rs.ref;
                         l = rs.l;
-                        tile_sum = rs.tile_sum;
+                        tile_sum = fabsf(rs.tile_sum);
+                        careful = careful || __any_sync(0xffffffffu, rs.tile_sum < 0.f);
+                        exact = careful || __any_sync(0xffffffffu, ref == -INFINITY && q_valid);
+                        first = false;
+                        tell(b_read);
                     }
-                } else {
-                    if (!__all_sync(0xffffffffu, wait_bar(b_sa, n_s & 1u, abort_flag, prm.status, 13))) {
-                        alive = false;
-                        break;
+                    if (!careful && __any_sync(0xffffffffu, tile_sum > kBumpSum)) {
+                        if (__any_sync(0xffffffffu, tile_sum > kMaxTileSum)) {
+                            careful = exact = true;
+                            const int2 org = load_side_origin(steps + (w >> 16), t);
+                            const long long q_tok = is_text ? (long long)item.qx + t * 128 + r : prm.n_text + (long long)q_y * prm.grid_w + q_x;
+                            const RowState rs = rescue_step<D>(prm, tmem_S, tmem_O, mw, c, ref, l, (long long)ctrl->sched_bh[slot] * prm.n_tokens,
+                                                               q_valid ? q_tok : -1, org, (__ldg(&steps[w >> 16].flags) & CLEAR_STEP_LINEAR) != 0);
+                            ref = rs.ref;
+                            l = rs.l;
+                            tile_sum = rs.tile_sum;
+                        } else {
+                            const float bump = tile_sum > kBumpSum ? (float)((int)((__float_as_uint(tile_sum) >> 23) & 0xffu) - 127) : 0.f;
+                            const float alpha = ptx::ex2(-bump);
+                            rescale_rows<D>(tmem_O, alpha);   // at rest; in an item's first step nobody looks at it
+                            rescale_p(tmem_S, alpha);
+                            ref += bump;
+                            l *= alpha;
+                            tile_sum *= alpha;
+                        }
                     }
-                    ptx::tc_fence_after();
-                    if (raise) rescale_rows<D>(tmem_O + lane_off, alpha);
-                    const RowState rs = exact_step<D>(tmem_S + lane_off, tmem_O + lane_off, make_uint4(mw[0], mw[1], mw[2], mw[3]), c, ref, l, exact_from == kFirst);
-                    ref = rs.ref;
-                    l = rs.l;
-                    tile_sum = fabsf(rs.tile_sum);
-                    if (__any_sync(0xffffffffu, rs.tile_sum < 0.f)) exact_from = kCareful;
-                    ptx::tc_fence_before();
-                    warp_arrive(ptx::smem_u32(&ctrl->sb_read[t]), lane);
+                    l += tile_sum;
+                    ptx::tmem_wait_st();
+                    tell(b_p);
+                    par ^= 1u;
+                    w = w1;
+                    w1 = w2;
+                    mw = mw1;
                 }
-                ++n_s;
-                exact_from &= kCareful;
-                l += tile_sum;
-                if (tile_sum > kBumpSum) bump = (int)((__float_as_uint(tile_sum) >> 23) & 0xffu) - 127;
-                // P_t (and a rescaled O_t) must be in tensor memory before the MMA thread is told
-                ptx::tmem_wait_st();
-                ptx::tc_fence_before();
-                warp_arrive(b_pready, lane);
-            }
-            if (!alive) break;
 
-            // ---- epilogue: the last P_t V has retired once o_full completes; O_t / l -> global memory -----
-            if (!__all_sync(0xffffffffu, wait_bar(ptx::smem_u32(&ctrl->o_full[t]), n_items_seen & 1u, abort_flag, prm.status, 14)))
-                break;
-            ++n_items_seen;
-            ptx::tc_fence_after();
-            store_tile<D>(prm, tmem_O, ptx::smem_u32(&ctrl->o_empty[t]), item.qx + (is_text ? t * 128 : 0), t ? item.qy1 : item.qy0,
-                          is_text ? (t ? item.n_rows1 : item.n_rows0) : -1, t ? item.partial_slot1 : item.partial_slot0, bh, ref, l);
+                // ---- epilogue: the last P_t V has retired once o_full completes; O_t / l -> global memory -----
+                if (alive) alive = wait_bar(ptx::smem_u32(&ctrl->o_full[t]), o_par, abort_flag, prm.status, 14);
+                if (!__all_sync(0xffffffffu, alive)) break;
+                o_par ^= 1u;
+                ptx::tc_fence_after();
+                store_tile<D>(prm, tmem + 256 + t * 128, ptx::smem_u32(&ctrl->o_empty[t]), item.qx + (is_text ? t * 128 : 0), t ? item.qy1 : item.qy0,
+                              is_text ? (t ? item.n_rows1 : item.n_rows0) : -1, t ? item.partial_slot1 : item.partial_slot0,
+                              ctrl->sched_bh[slot], ref, l);
+            }
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&ctrl->sched_empty[slot]));
         }
     }
 
@@ -1136,6 +1202,8 @@ int launch_ws(const clear_plan &p, const void *q, const void *k, const void *v, 
     prm.steps = p.d_pair_steps;
     prm.half_width = p.d_half_width;
     prm.mask_table = p.d_mask_table;
+    prm.side_words = p.d_mask_table + p.sch.mask_table.size();
+    prm.n_steps = (int)p.sch.pair_steps.size();
     prm.n_half_width = (int)p.sch.half_width.size();
     prm.grid_h = p.shape.grid_h;
     prm.grid_w = p.shape.grid_w;

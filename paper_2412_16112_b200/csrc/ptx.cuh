@@ -58,6 +58,33 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
         : "memory");
     return ok != 0;
 }
+// Up to `tries` of them in one piece, which a completed phase passes in straight line; true at once if not `on`.
+__device__ __forceinline__ bool mbar_try_wait_some(uint32_t bar, uint32_t parity, uint32_t tries, uint32_t ns, bool on)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
+        "setp.eq.u32 p, %5, 0;\n\t"
+        "mov.u32 n, %3;\n\t"
+        "@p bra DONE;\n\t"
+        "AGAIN:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %4;\n\t"
+        "@p bra DONE;\n\t"
+        "sub.u32 n, n, 1;\n\t"
+        "setp.ne.u32 q, n, 0;\n\t"
+        "@q bra AGAIN;\n\t"
+        "DONE:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(tries), "r"(ns), "r"((uint32_t)on)
+        : "memory");
+    return ok != 0;
+}
+// One arrival if `on`, without a branch.
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool on)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}\n" ::"r"(bar), "r"((uint32_t)on) : "memory");
+}
 __device__ __forceinline__ uint64_t globaltimer_ns()
 {
     uint64_t t;

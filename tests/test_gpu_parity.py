@@ -670,6 +670,25 @@ def test_ws_kernel_with_long_queries(gh, gw, T, r, d, length):
     assert (np.abs(got - want) <= bound).all(), float(np.abs(got - want).max())
 
 
+@pytest.mark.parametrize("rise", [10, 20, 55, 70])
+@pytest.mark.parametrize("gh,gw,T,r,d", [(24, 40, 300, 8.0, 128), (19, 23, 0, 6.0, 64), (40, 72, 20, 40.0, 64)])
+def test_ws_kernel_raises_references_step_by_step(gh, gw, T, r, d, rise):
+    """Scores that climb by `rise` powers of two every 64 text tokens and every eight rows of the grid: sums of a tile below the
+    bound of 2^16 that raises a row's reference, above it (P, sum and O scaled in place, by the first half of a tile or by the
+    second), and above 2^64 (taken again); lists of up to 40 steps, more than a window of 32.  Bound as for long queries."""
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, seed=rise + gh)
+    climb = torch.cat([torch.arange(T) // 64, T // 64 + torch.arange(gh).repeat_interleave(gw) // 8]).float() * rise
+    q[..., 0], k[..., 0] = 8.0, (climb / 8.0).to(torch.bfloat16)
+    scale = math.log(2.0)
+    q[..., 1:] *= 0.25
+    want = oracle.attn(q, k, v, gh, gw, T, r, scale)
+    got = run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS).double().numpy()
+    v_max = float(v.float().abs().max())
+    logit = scale * float(q.float().norm(dim=-1).max() * k.float().norm(dim=-1).max())
+    bound = 2.0 ** -8 * (np.abs(want) + v_max) + 2.0 ** -21 * logit * v_max
+    assert (np.abs(got - want) <= bound).all(), float((np.abs(got - want) - bound).max())
+
+
 def test_ws_kernel_nan_key_reaches_the_queries_that_see_it():
     """A NaN in a key outside the first tile: the text queries and the image queries within its reach, no others."""
     gh, gw, T, r, d = 24, 40, 20, 3.0, 64
