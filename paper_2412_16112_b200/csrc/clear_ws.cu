@@ -41,7 +41,7 @@ constexpr float kRescaleThreshold = 8.f;  // log2 units: a reference is moved on
 constexpr float kBumpSum = 65536.f;       // a row sum of P above this raises the row's reference
 constexpr float kMaxTileSum = 0x1p64f;    // a row sum above this has its tile taken again (a NaN comes from NaN inputs only, and stays)
 // Scores of a row's first tile that lie this far apart (log2 units) give the item maximum passes from the start: with less,
-// normal ones would have to lie seven standard deviations above the maximum of 64 to be 64 above it.  (The least of eight of
+// normal ones would have to lie seven standard deviations above the maximum of 128 to be 64 above it.  (The least of 16 of
 // them is enough to tell.)
 constexpr float kWideStep = 40.f;
 constexpr int kSchedDepth = 2;
@@ -262,23 +262,27 @@ __device__ __forceinline__ float sum4(const uint64_t (&lsum)[2])
 struct RowState {
     float ref, l, tile_sum;   // tile_sum < 0: less that, and the row's maximum lies more than kWideStep above the least of 16 scores
 };
-// The largest of 64 scores of a row that all count, and the least of eight of them.
+// The largest of the 128 scores of a row that all count, and the least of 16 of them.  (Of 64 only: 0.5 % more rounding error of P
+// at 512 text tokens, where the row's largest weight is then more often not a whole 1.)
 struct RowTop {
     float most, least;
 };
-__device__ __noinline__ RowTop half_top(uint32_t tmem_half)
+__device__ __noinline__ RowTop first_top(uint32_t tmem_s)
 {
     float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, mn = INFINITY;
-    uint32_t sv[2][32];
-    ptx::tmem_ld32(tmem_half, sv[0]);
-    ptx::tmem_ld32(tmem_half + 32, sv[1]);
-    ptx::tmem_wait_ld();
+#pragma unroll 1
+    for (int h = 0, n = opaque(2); h < n; ++h) {
+        uint32_t sv[2][32];
+        ptx::tmem_ld32(tmem_s + 64 * h, sv[0]);
+        ptx::tmem_ld32(tmem_s + 64 * h + 32, sv[1]);
+        ptx::tmem_wait_ld();
 #pragma unroll
-    for (int w = 0; w < 2; ++w)
+        for (int w = 0; w < 2; ++w)
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) mx[(j >> 1) & 3] = ptx::max3(mx[(j >> 1) & 3], __uint_as_float(sv[w][j]), __uint_as_float(sv[w][j + 1]));
+            for (int j = 0; j < 32; j += 2) mx[(j >> 1) & 3] = ptx::max3(mx[(j >> 1) & 3], __uint_as_float(sv[w][j]), __uint_as_float(sv[w][j + 1]));
 #pragma unroll
-    for (int j = 0; j < 32; j += 4) mn = fminf(mn, __uint_as_float(sv[0][j]));
+        for (int j = 0; j < 32; j += 4) mn = fminf(mn, __uint_as_float(sv[0][j]));
+    }
     return RowTop{fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), mn};
 }
 
@@ -891,7 +895,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
         // scheduler are 2150 if nothing else runs and the MMAs 2560 (3050 with the copies, by a run without exponentials); the
         // rest is the chain between them, and the start and end of an item, some 7000 clocks, most of them for fetching
         // instructions that run once an item (about 16 clocks each).  So the code of an item's start and end is kept short:
-        // the tiles' lists come ready from the host, the first step runs in the common loop with a reference from 64 scores,
+        // the tiles' lists come ready from the host, the first step runs in the common loop with a reference taken beforehand,
         // and what is rare stands behind the loop (1024px 108.3 -> 103.0 us, 2048px 581 -> 552, 67 x 120 of 64 channels 230 ->
         // 209, against lists taken apart here, maximum passes in the first step and every case in line).
         ptx::setmaxnreg_inc<kRegsSoftmax>();
@@ -957,7 +961,7 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
 
                 // P = 2^(S c - ref) with a reference per row that need not be the running maximum: P, the row sum and O
                 // are floating-point numbers of full precision at any scale, so the reference only has to keep them
-                // within range.  It is the maximum of the row's first tile (of half of it if all keys are allowed); when a tile's row sum exceeds 2^16 the
+                // within range.  It is the maximum of the row's first tile; when a tile's row sum exceeds 2^16 the
                 // reference is raised by a whole power of two, without a look at the maximum, and the row's P, sum and O are
                 // scaled before P goes to the MMAs.  No maximum pass, then, on any other tile, and the scores die as their P is
                 // formed.  A row sum beyond 2^64 means scores 64 powers of two above everything seen before; the warp then
@@ -974,7 +978,8 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                     if (w & kSideRare) mw = special_mask(prm, steps + (w >> 16), t, q_valid, q_y, q_x);
                     if (first && !(w & kSideMasked)) {
                         wait_warp(b_sb, par, 10);
-                        const RowTop top = half_top(tmem_S + 64);
+                        wait_warp(b_sa, par, 13);
+                        const RowTop top = first_top(tmem_S);
                         ref = top.most * c;
                         careful = __any_sync(0xffffffffu, (top.most - top.least) * c > kWideStep);
                         exact = careful || __any_sync(0xffffffffu, ref == -INFINITY && q_valid);
