@@ -4,10 +4,16 @@
 // Serves fp32 tensors (where tensor-core input rounding would break a 1e-5 agreement), bf16 tensors of head sizes the
 // tensor-core kernels do not take, and non-positive scales, under the windows around the query (disc, square).
 //
+// Up to 128 channels (padded to 64 or 128) a block is four warps with 16 whole rows each (clear_f32_rows_kernel); above, the
+// accumulators of 16 rows would not fit a warp's registers, and 256 threads take 4 x 4 results each (clear_f32_tile_kernel).
 // What bounds it: the fp32 multiply-add units (2 x 64 x 64 x DP multiply-adds a step, DP = the head size rounded up
-// to 64, 128 or 256).  The keys are those of the union of the tile's windows and no others: rows are gathered run by
+// to 64, 128 or 256), and in the scores the reads from shared memory beside them.  1024 px, radius 8, 24 heads of 128: 2034 us
+// with 4 x 4 results a thread (shared memory at 77 % of its peak, multiply-adds at 64 %), 1734 us with whole rows (62 % and
+// 70 %): about 780 for the scores and 550 for the weights times V, each of which is 525 of multiply-adds, 130 for the copies
+// and 100 for the softmax, by runs without the one or the other.
+// The keys are those of the union of the tile's windows and no others: rows are gathered run by
 // run, 64 at a time, so a step is only ever short at the end of the list.  An 8 x 8 patch is the split that wastes
-// least at the paper's radii with a 4 x 4 register tile: at r = 8 a patch walks 452 + n_text keys for windows of 193.
+// least at the paper's radii: at r = 8 a patch walks 452 + n_text keys for windows of 193.
 // Two blocks share an SM (DP <= 128): one computes while the other waits for its rows.
 // A problem too small to give every SM a tile cuts the lists over a cluster of up to 8 blocks, which merge their
 // partial softmax through distributed shared memory in a fixed order: no workspace, no second launch.
@@ -71,7 +77,7 @@ __device__ __forceinline__ void redo_row(const F32Params &p, int r)
 }
 
 template <typename T, int DP>
-__global__ void __launch_bounds__(kThreads, DP <= 128 ? 2 : 1)
+__global__ void __launch_bounds__(kThreads, 1)
 clear_f32_tile_kernel(const F32Params p)
 {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -244,13 +250,223 @@ clear_f32_tile_kernel(const F32Params p)
     cluster.sync();   // nobody leaves while its rows are being read
 }
 
+// The same with a warp to 16 whole rows, for up to 128 channels.
+constexpr float kMaxExponent = 16.f;   // a score this far above its row's reference moves it
+
+// Shared memory: Q, V, then the keys, whose place the weights take once the scores are in registers (with 64 channels they are
+// longer than the keys), the key lists, row values.
+template <int DP> constexpr size_t kRowsLists =
+    (2 * kRows * kStride<DP> + (kStride<DP> > 4 * kPairStride ? kStride<DP> : 4 * kPairStride) * kRows) * sizeof(float);
+template <int DP> constexpr size_t kRowsSmem = kRowsLists<DP> + 2 * sizeof(KeyTile) + 2 * kRows * sizeof(float) + 64 * sizeof(int);
+
+template <typename T, int DP>
+__global__ void __launch_bounds__(kRowThreads, 2)
+clear_f32_rows_kernel(const F32Params p)
+{
+    constexpr int C = DP / 32;
+    extern __shared__ __align__(16) uint8_t smem[];
+    float *sQ = reinterpret_cast<float *>(smem), *sV = sQ + kRows * kStride<DP>, *sK = sV + kRows * kStride<DP>;
+    KeyTile *keys = reinterpret_cast<KeyTile *>(smem + kRowsLists<DP>);
+    float *sM = reinterpret_cast<float *>(keys + 2), *sL = sM + kRows;
+    int *red = reinterpret_cast<int *>(sL + kRows);
+
+    const int tid = threadIdx.x, lane = tid & 31, row0 = (tid >> 5) * kWarpRows;
+    float *sP = sK + (tid >> 5) * kRows * kPairStride;   // the warp's weights
+    const int part = (int)(blockIdx.x % (unsigned)p.n_split);   // rank in the cluster
+    const TileRef tile = tile_of((int)(blockIdx.x / (unsigned)p.n_split), p.g);
+    const KeyRuns runs = runs_of(tile, p.g);
+    const long long base = (long long)tile.bh * runs.n_tokens * p.g.d;
+    const T *q = static_cast<const T *>(p.q) + base, *k = static_cast<const T *>(p.k) + base,
+            *v = static_cast<const T *>(p.v) + base;
+
+    // this block's share of the list: whole steps of 64 keys
+    const int n_steps_all = (list_length<kRowThreads>(runs, red) + kRows - 1) / kRows;
+    const int per = (n_steps_all + p.n_split - 1) / p.n_split;
+    const int step0 = min(part * per, n_steps_all), n_steps = min(per, n_steps_all - step0);
+    KeyCursor cur;
+    if (tid < kRows) {
+        cur.start(runs);
+        cur.advance(runs, step0 * kRows + tid);
+        int qy, qx;
+        keys[1].token[tid] = tile_token(tile, tid, p.g, qy, qx);
+    }
+    fill_key_tile(keys[0], cur, runs, n_steps > 0);
+    __syncthreads();
+    load_rows<T, DP, kRowThreads>(sQ, q, keys[1].token, p.g.d);
+
+    uint64_t o[kWarpRows / 2][C];
+    float m[kWarpRows], l[kWarpRows];   // per row its reference; of its sum the lane's share
+#pragma unroll
+    for (int i = 0; i < kWarpRows / 2; ++i)
+#pragma unroll
+        for (int c = 0; c < C; ++c) o[i][c] = 0ull;
+#pragma unroll
+    for (int i = 0; i < kWarpRows; ++i) {
+        m[i] = -CUDART_INF_F;
+        l[i] = 0.f;
+    }
+
+    for (int s = 0; s < n_steps; ++s) {
+        const KeyTile &kt = keys[s & 1];
+        load_rows<T, DP, kRowThreads>(sK, k, kt.token, p.g.d);
+        load_rows<T, DP, kRowThreads>(sV, v, kt.token, p.g.d);
+        uint32_t on[2];   // rows that see the lane's keys
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int c = lane + 32 * j;
+            on[j] = kt.token[c] >= 0 ? seen_by(runs, tile, p.g, row0, kt.ky[c], kt.kx[c]) : 0u;
+        }
+        cp_async_wait<1>();   // Q and K are here
+        __syncthreads();
+        if (s + 1 < n_steps) fill_key_tile(keys[(s + 1) & 1], cur, runs, true);
+
+        float w[kWarpRows][2];
+        warp_dot<DP>(sQ + row0 * kStride<DP>, sK, lane, w);
+        __syncthreads();      // every warp is done with the keys: the weights may land on them
+
+        // Softmax against a reference per row that is moved only when a score lies far above it (and by the first scores that
+        // a row has): no maximum over the lanes and no scaling in the common step.
+        float far = -CUDART_INF_F;
+#pragma unroll
+        for (int i = 0; i < kWarpRows; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                w[i][j] = ((on[j] >> i) & 1u) ? w[i][j] * p.scale : -CUDART_INF_F;
+                far = fmaxf(far, w[i][j] - m[i]);   // (-inf minus -inf is a NaN, which fmaxf passes over)
+            }
+        if (__any_sync(0xffffffffu, far > kMaxExponent)) {
+#pragma unroll
+            for (int i = 0; i < kWarpRows; i += 2) {
+                float alpha[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    float mx = fmaxf(w[i + u][0], w[i + u][1]);
+#pragma unroll
+                    for (int x = 16; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+                    const float m_new = fmaxf(m[i + u], mx);
+                    alpha[u] = expf(m[i + u] - (m_new == -CUDART_INF_F ? 0.f : m_new));   // m = -inf: 0
+                    m[i + u] = m_new;
+                    l[i + u] *= alpha[u];
+                }
+                const uint64_t a2 = ptx::pack2(alpha[0], alpha[1]);
+#pragma unroll
+                for (int c = 0; c < C; ++c) o[i >> 1][c] = ptx::mul2(o[i >> 1][c], a2);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int i = 0; i < kWarpRows; i += 4) {
+                float e[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    e[u] = expf(w[i + u][j] - (m[i + u] == -CUDART_INF_F ? 0.f : m[i + u]));
+                    l[i + u] += e[u];
+                }
+                *reinterpret_cast<float4 *>(sP + (lane + 32 * j) * kPairStride + i) = make_float4(e[0], e[1], e[2], e[3]);
+            }
+        cp_async_wait<0>();
+        __syncthreads();      // V has landed for everybody, and the weights are written
+        warp_accumulate<DP>(sP, sV, lane, o);
+        __syncthreads();      // before the next rows overwrite K, V
+    }
+#pragma unroll
+    for (int i = 0; i < kWarpRows; ++i)
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
+
+    // rows that came out non-finite are taken again, each by a warp; `bad` lies over the list lengths, which are done with
+    int *bad = red;
+    auto redo_bad = [&]() {
+#pragma unroll 1
+        for (int r = tid >> 5; r < kRows; r += kRowThreads / 32)
+            if (bad[r] != 0) redo_row<T, DP>(p, r);
+    };
+    if (tid < kRows) bad[tid] = 0;
+    __syncthreads();
+
+    T *out = static_cast<T *>(p.out) + base;
+    const int ch = C * lane;
+    bool all_finite = true;
+    if (p.n_split == 1) {
+#pragma unroll
+        for (int i = 0; i < kWarpRows; ++i) {
+            // a query sees itself or the text keys: l > 0 for every row that exists
+            const float inv = l[i] > 0.f ? 1.f / l[i] : 0.f;
+            int qy, qx;
+            const long long tok = tile_token(tile, row0 + i, p.g, qy, qx);
+            float x[C];
+            acc_row(o, i, x);
+            bool fine = true;
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                x[c] *= inv;
+                fine = fine && fabsf(x[c]) <= CUDART_MAX_NORMAL_F;
+            }
+            if (tok >= 0 && ch < p.g.d) store_channels(out + tok * p.g.d + ch, x);
+            if (!fine) {
+                bad[row0 + i] = 1;
+                all_finite = false;
+            }
+        }
+        if (__syncthreads_or(!all_finite)) redo_bad();
+        return;
+    }
+
+    // merge over the cluster: every block leaves its un-normalised rows, references and sums in its own shared memory and
+    // finishes 64 / n_split rows from everybody's, in the order of the ranks
+    cg::cluster_group cluster = cg::this_cluster();
+    cp_async_wait<0>();
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kWarpRows; ++i) {
+        float x[C];
+        acc_row(o, i, x);
+        store_channels(sV + (row0 + i) * kStride<DP> + ch, x);
+        if (lane == 0) {
+            sM[row0 + i] = m[i];
+            sL[row0 + i] = l[i];
+        }
+    }
+    cluster.sync();
+    const int rows = kRows / p.n_split;
+    for (int e = tid; e < rows * (DP / 4); e += kRowThreads) {
+        const int r = part * rows + e / (DP / 4), c4 = e % (DP / 4) * 4;
+        int qy, qx;
+        const long long tok = tile_token(tile, r, p.g, qy, qx);
+        float mx = -CUDART_INF_F;
+        for (int c = 0; c < p.n_split; ++c) mx = fmaxf(mx, cluster.map_shared_rank(sM, c)[r]);
+        if (mx == -CUDART_INF_F) mx = 0.f;
+        float sum = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < p.n_split; ++c) {
+            const float f = expf(cluster.map_shared_rank(sM, c)[r] - mx);
+            sum = fmaf(f, cluster.map_shared_rank(sL, c)[r], sum);
+            const float4 x = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(sV, c) + r * kStride<DP> + c4);
+            acc.x = fmaf(f, x.x, acc.x);
+            acc.y = fmaf(f, x.y, acc.y);
+            acc.z = fmaf(f, x.z, acc.z);
+            acc.w = fmaf(f, x.w, acc.w);
+        }
+        const float inv = sum > 0.f ? 1.f / sum : 0.f;
+        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+        if (tok >= 0 && c4 < p.g.d) store4(out + tok * p.g.d + c4, acc);
+        if (!finite4(acc)) {
+            bad[r] = 1;
+            all_finite = false;
+        }
+    }
+    if (__syncthreads_or(!all_finite)) redo_bad();
+    cluster.sync();   // nobody leaves while its rows are being read
+}
+
 constexpr int blocks_per_sm(int d) { return d <= 128 ? 2 : 1; }
 
 template <typename T>
 int launch_typed(const F32Params &p, long long tiles, cudaStream_t stream)
 {
-    if (p.g.d <= 64) return launch_tiles(clear_f32_tile_kernel<T, 64>, p, tiles, p.n_split, forward_smem<64>(), stream);
-    if (p.g.d <= 128) return launch_tiles(clear_f32_tile_kernel<T, 128>, p, tiles, p.n_split, forward_smem<128>(), stream);
+    if (p.g.d <= 64) return launch_tiles(clear_f32_rows_kernel<T, 64>, p, tiles, p.n_split, kRowsSmem<64>, stream, kRowThreads);
+    if (p.g.d <= 128) return launch_tiles(clear_f32_rows_kernel<T, 128>, p, tiles, p.n_split, kRowsSmem<128>, stream, kRowThreads);
     return launch_tiles(clear_f32_tile_kernel<T, 256>, p, tiles, p.n_split, forward_smem<256>(), stream);
 }
 

@@ -1,9 +1,9 @@
-// Building blocks of the fp32 tile kernels (forward and backward pass on the CUDA cores): a block of 256 threads
-// works on a tile of 64 tokens (an 8 x 8 patch of the grid,
+// Building blocks of the fp32 tile kernels (forward and backward pass on the CUDA cores): a block of 256 threads, or of 128
+// with whole rows to a warp (warp_dot), works on a tile of 64 tokens (an 8 x 8 patch of the grid,
 // longer and flatter on grids narrower than 8, or 64 consecutive text tokens) against the tokens its
 // queries can see, 64 at a time.
 //
-// Thread (ty, tx), 16 x 16, owns the rows ty + 16 i (i < 4) of the tile; one warp holds two values of ty with all
+// Of 256, thread (ty, tx), 16 x 16, owns the rows ty + 16 i (i < 4) of the tile; one warp holds two values of ty with all
 // their tx, so everything that is exchanged along a row stays inside a warp.
 //   product of two row sets (tile_dot):    4 x 4 results a thread, both operands as float4 along the channels, even
 //       and odd channels summed apart in the two halves of a packed fp32 pair (fma.rn.f32x2): no operand is ever
@@ -30,6 +30,7 @@ namespace f32tile {
 constexpr int kThreads = 256;
 constexpr int kRows = 64;        // tokens of a tile, and of a streamed tile
 constexpr int kPStride = 68;     // floats between rows of the 64 x 64 weight matrix
+constexpr int kWarpRows = 16, kRowThreads = 128;   // kernels with a warp to 16 whole rows
 
 template <int DP> constexpr int kStride = DP + 4;   // floats between rows of 64 x DP
 
@@ -89,18 +90,19 @@ struct KeyCursor {
     }
 };
 
-// Number of tokens in the list (every thread of the block gets it; `red` is 8 ints of shared memory).
+// Number of tokens in the list (every one of the block's NT threads gets it; `red` is 8 ints of shared memory).
+template <int NT = kThreads>
 __device__ __forceinline__ int list_length(const KeyRuns &k, int *red)
 {
     int n = 0, xf;
-    for (int y = k.first_row() + (int)threadIdx.x; y < k.end_row(); y += kThreads) n += k.run(y, xf);
+    for (int y = k.first_row() + (int)threadIdx.x; y < k.end_row(); y += NT) n += k.run(y, xf);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = n;
     __syncthreads();
     int sum = k.head_length();
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) sum += red[w];
+    for (int w = 0; w < NT / 32; ++w) sum += red[w];
     return sum;
 }
 
@@ -114,11 +116,11 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 
 // 64 rows of d channels into shared memory as fp32 (row stride DP + 4), zeros for absent rows (token < 0) and for the
 // channels d .. DP - 1.  fp32 rows travel asynchronously (one commit group), bf16 rows through registers.
-template <typename T, int DP>
+template <typename T, int DP, int NT = kThreads>
 __device__ __forceinline__ void load_rows(float *dst, const T *__restrict__ base, const int *tokens, int d)
 {
-    constexpr int kChunks = DP / 4;                    // float4 of a row
-    constexpr int kRowsPerPass = kThreads / kChunks;   // DP = 64, 128, 256: 16, 8, 4
+    constexpr int kChunks = DP / 4;              // float4 of a row
+    constexpr int kRowsPerPass = NT / kChunks;   // of 256 threads: DP = 64, 128, 256: 16, 8, 4
     const int chunk = threadIdx.x % kChunks, r0 = threadIdx.x / kChunks;
 #pragma unroll
     for (int i = 0; i < kRows / kRowsPerPass; ++i) {
@@ -242,6 +244,95 @@ __device__ __forceinline__ float row_sum16(float x)
     return x;
 }
 
+// ---- a warp to 16 whole rows (blocks of 128 threads, DP <= 128) -----------------------------------------------------
+// Shared memory serves 16-byte reads eight lanes at a time, and lanes in different eights share nothing unless all 32 read one
+// address: so a warp's own rows are read by all its lanes at once (1 wavefront a read) and the streamed rows by a lane each (4).
+// 16 own rows x 2 streamed ones a lane take 24 wavefronts a 64 packed multiply-adds; 4 x 4 results a thread, with 2 x 16
+// threads a warp, took 24 a 32, and shared memory was the bound (77 % of its peak, the multiply-add pipe at 64 %).
+constexpr int kPairStride = 20;   // floats between the streamed rows of a warp's weights [64][16]: 16-byte stores, no conflicts
+
+// s[i][j] = sum over channels of A[i] . B[lane + 32 j], even and odd channels apart as in tile_dot
+template <int DP>
+__device__ __forceinline__ void warp_dot(const float *A, const float *B, int lane, float (&s)[kWarpRows][2])
+{
+    uint64_t acc[kWarpRows][2];
+#pragma unroll
+    for (int i = 0; i < kWarpRows; ++i) acc[i][0] = acc[i][1] = 0ull;
+    const float *b0 = B + lane * kStride<DP>;
+#pragma unroll 2
+    for (int c = 0; c < DP; c += 4) {
+        const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(b0 + c), y = *reinterpret_cast<const ulonglong2 *>(b0 + 32 * kStride<DP> + c);
+#pragma unroll
+        for (int i0 = 0; i0 < kWarpRows; i0 += 4) {   // four rows at a time: eight chains side by side
+            ulonglong2 a[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2 *>(A + (i0 + i) * kStride<DP> + c);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                acc[i0 + i][0] = ptx::fma2(a[i].x, x.x, acc[i0 + i][0]);
+                acc[i0 + i][1] = ptx::fma2(a[i].x, y.x, acc[i0 + i][1]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                acc[i0 + i][0] = ptx::fma2(a[i].y, x.y, acc[i0 + i][0]);
+                acc[i0 + i][1] = ptx::fma2(a[i].y, y.y, acc[i0 + i][1]);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kWarpRows; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float lo, hi;
+            ptx::unpack2(acc[i][j], lo, hi);
+            s[i][j] = lo + hi;
+        }
+}
+
+// acc[k][c]: rows 2 k, 2 k + 1 of the warp (a packed pair) of channel DP / 32 lane + c; += sum over the 64 streamed rows j of
+// W[j][rows] * B[j][channels]
+template <int DP>
+__device__ __forceinline__ void warp_accumulate(const float *W, const float *B, int lane, uint64_t (&acc)[kWarpRows / 2][DP / 32])
+{
+    constexpr int C = DP / 32;
+    const float *b0 = B + lane * C;
+#pragma unroll 8
+    for (int j = 0; j < kRows; ++j) {
+        float b[C];
+        if constexpr (C == 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(b0 + j * kStride<DP>);
+            b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+        } else {
+            const float2 v = *reinterpret_cast<const float2 *>(b0 + j * kStride<DP>);
+            b[0] = v.x; b[1] = v.y;
+        }
+        uint64_t b2[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) b2[c] = ptx::pack2(b[c], b[c]);
+#pragma unroll
+        for (int k = 0; k < kWarpRows / 2; k += 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(W + j * kPairStride + 2 * k);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                acc[k][c] = ptx::fma2(w.x, b2[c], acc[k][c]);
+                acc[k + 1][c] = ptx::fma2(w.y, b2[c], acc[k + 1][c]);
+            }
+        }
+    }
+}
+
+// Row i of the warp's accumulators, the lane's channels.
+template <int C>
+__device__ __forceinline__ void acc_row(const uint64_t (&acc)[kWarpRows / 2][C], int i, float (&x)[C])
+{
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        float lo, hi;
+        ptx::unpack2(acc[i >> 1][c], lo, hi);
+        x[c] = (i & 1) ? hi : lo;
+    }
+}
+
 __device__ __forceinline__ void store4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
 __device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v)
 {
@@ -250,6 +341,10 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v)
     u.y = ptx::pack_bf16(v.z, v.w);
     *reinterpret_cast<uint2 *>(p) = u;
 }
+__device__ __forceinline__ void store_channels(float *p, const float (&x)[4]) { store4(p, make_float4(x[0], x[1], x[2], x[3])); }
+__device__ __forceinline__ void store_channels(__nv_bfloat16 *p, const float (&x)[4]) { store4(p, make_float4(x[0], x[1], x[2], x[3])); }
+__device__ __forceinline__ void store_channels(float *p, const float (&x)[2]) { *reinterpret_cast<float2 *>(p) = make_float2(x[0], x[1]); }
+__device__ __forceinline__ void store_channels(__nv_bfloat16 *p, const float (&x)[2]) { *reinterpret_cast<uint32_t *>(p) = ptx::pack_bf16(x[0], x[1]); }
 __device__ __forceinline__ float4 acc_float4(const uint64_t (&a)[2], float f)
 {
     float4 v;
@@ -324,6 +419,24 @@ __device__ __forceinline__ bool sees(const KeyRuns &k, int qy, int qx, int ky, i
     if (k.text || ky < 0) return true;
     const int dy = abs(ky - qy);
     return dy < k.n_half_width && abs(kx - qx) <= __ldg(k.half_width + dy);
+}
+
+// Which of the 16 rows of the tile from `row0` on see the token at (ky, kx), one bit each.
+__device__ __forceinline__ uint32_t seen_by(const KeyRuns &k, const TileRef &t, const Geometry &g, int row0, int ky, int kx)
+{
+    if (k.text || ky < 0) return 0xffffu;
+    const int w_log = min(g.patch_w_log, 4), width = 1 << w_log;   // of the 16 rows, so many lie in one row of the patch
+    const int x0 = t.x + (row0 & (g.patch_w() - 1));
+    int dy = ky - (t.y + (row0 >> g.patch_w_log));
+    uint32_t bits = 0u;
+#pragma unroll 2
+    for (int b = 0; b < kWarpRows; b += width, --dy) {
+        const int dist = abs(dy);
+        if (dist >= k.n_half_width) continue;
+        const int w = __ldg(k.half_width + dist), lo = max(kx - w - x0, 0), hi = min(kx + w - x0, width - 1);
+        if (lo <= hi) bits |= ((2u << hi) - (1u << lo)) << b;
+    }
+    return bits;
 }
 
 // The list of one streamed tile in shared memory, filled by the first 64 threads a tile ahead.
@@ -420,14 +533,14 @@ Extent extent_of(const clear_plan &p, const Geometry &g);
 int split_of(const Extent &e, int n_bh, int slots);
 
 template <typename Kernel, typename Params>
-int launch_tiles(Kernel kernel, const Params &prm, long long tiles, int n_split, size_t smem, cudaStream_t stream)
+int launch_tiles(Kernel kernel, const Params &prm, long long tiles, int n_split, size_t smem, cudaStream_t stream, int threads = kThreads)
 {
     if (tiles * n_split > INT32_MAX) return CLEAR_ERR_UNSUPPORTED;
     // set again on every call: a table lookup in the runtime, per device, without a lock of our own
     CLEAR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(tiles * n_split));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];

@@ -43,6 +43,22 @@ def test_forward_tiles(bh, gh, gw, T, r, d):
     clear.clear_cache_clear()
 
 
+@pytest.mark.parametrize("rise", [10, 17, 90, -17])
+@pytest.mark.parametrize("bh,gh,gw,T,r,d", [(1, 24, 40, 130, 8.0, 64), (40, 19, 23, 0, 6.0, 128), (2, 3, 90, 70, 9.0, 40)])
+def test_forward_tiles_with_scores_that_climb(bh, gh, gw, T, r, d, rise):
+    """Scores that climb (or fall) by `rise` every 32 text tokens and every four rows or 16 columns of the grid: rows whose reference stays, and
+    rows whose reference moves, at every step.  Scores of size L are good to a few 2^-24 L, and so are the weights."""
+    q, k, v = _inputs(bh, gh, gw, T, d, 3, 14)
+    ys, xs = torch.arange(gh).repeat_interleave(gw), torch.arange(gw).repeat(gh)
+    q[..., 0], k[..., 0] = 1.0, rise * torch.cat([torch.arange(T) // 32, T // 32 + ys // 4 + xs // 16]).float()
+    want = oracle.attn(q, k, v, gh, gw, T, r, 1.0)
+    out = torch.full_like(q, float("nan"), device="cuda:0")
+    clear.clear_attn_fwd_f32(*(t.cuda() for t in (q, k, v)), out, gh, gw, T, r, 1.0)
+    logit = float(q.norm(dim=-1).max() * k.norm(dim=-1).max())
+    assert np.abs(out.cpu().double().numpy() - want).max() <= 1e-5 + 2.0 ** -21 * logit * float(v.abs().max())
+    clear.clear_cache_clear()
+
+
 @pytest.mark.parametrize("bh,gh,gw,T,r,d", SHAPES)
 def test_backward_tiles(bh, gh, gw, T, r, d):
     q, k, v, g = _inputs(bh, gh, gw, T, d, 4, 12)
