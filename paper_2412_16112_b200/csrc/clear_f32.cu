@@ -252,11 +252,12 @@ clear_f32_tile_kernel(const F32Params p)
 
 // The same with a warp to 16 whole rows, for up to 128 channels.
 constexpr float kMaxExponent = 16.f;   // a score this far above its row's reference moves it
+constexpr int kWarpRows = 16, kRowThreads = 32 * kRows / kWarpRows;
 
 // Shared memory: Q, V, then the keys, whose place the weights take once the scores are in registers (with 64 channels they are
 // longer than the keys), the key lists, row values.
 template <int DP> constexpr size_t kRowsLists =
-    (2 * kRows * kStride<DP> + (kStride<DP> > 4 * kPairStride ? kStride<DP> : 4 * kPairStride) * kRows) * sizeof(float);
+    (2 * kRows * kStride<DP> + (kStride<DP> > 4 * kPairStride<kWarpRows> ? kStride<DP> : 4 * kPairStride<kWarpRows>) * kRows) * sizeof(float);
 template <int DP> constexpr size_t kRowsSmem = kRowsLists<DP> + 2 * sizeof(KeyTile) + 2 * kRows * sizeof(float) + 64 * sizeof(int);
 
 template <typename T, int DP>
@@ -271,7 +272,7 @@ clear_f32_rows_kernel(const F32Params p)
     int *red = reinterpret_cast<int *>(sL + kRows);
 
     const int tid = threadIdx.x, lane = tid & 31, row0 = (tid >> 5) * kWarpRows;
-    float *sP = sK + (tid >> 5) * kRows * kPairStride;   // the warp's weights
+    float *sP = sK + (tid >> 5) * kRows * kPairStride<kWarpRows>;   // the warp's weights
     const int part = (int)(blockIdx.x % (unsigned)p.n_split);   // rank in the cluster
     const TileRef tile = tile_of((int)(blockIdx.x / (unsigned)p.n_split), p.g);
     const KeyRuns runs = runs_of(tile, p.g);
@@ -314,7 +315,7 @@ clear_f32_rows_kernel(const F32Params p)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int c = lane + 32 * j;
-            on[j] = kt.token[c] >= 0 ? seen_by(runs, tile, p.g, row0, kt.ky[c], kt.kx[c]) : 0u;
+            on[j] = kt.token[c] >= 0 ? seen_by<kWarpRows>(runs, tile, p.g, row0, kt.ky[c], kt.kx[c]) : 0u;
         }
         cp_async_wait<1>();   // Q and K are here
         __syncthreads();
@@ -363,11 +364,11 @@ clear_f32_rows_kernel(const F32Params p)
                     e[u] = expf(w[i + u][j] - (m[i + u] == -CUDART_INF_F ? 0.f : m[i + u]));
                     l[i + u] += e[u];
                 }
-                *reinterpret_cast<float4 *>(sP + (lane + 32 * j) * kPairStride + i) = make_float4(e[0], e[1], e[2], e[3]);
+                *reinterpret_cast<float4 *>(sP + (lane + 32 * j) * kPairStride<kWarpRows> + i) = make_float4(e[0], e[1], e[2], e[3]);
             }
         cp_async_wait<0>();
         __syncthreads();      // V has landed for everybody, and the weights are written
-        warp_accumulate<DP>(sP, sV, lane, o);
+        warp_accumulate<DP, kWarpRows>(sP, sV, lane, o);
         __syncthreads();      // before the next rows overwrite K, V
     }
 #pragma unroll

@@ -30,7 +30,6 @@ namespace f32tile {
 constexpr int kThreads = 256;
 constexpr int kRows = 64;        // tokens of a tile, and of a streamed tile
 constexpr int kPStride = 68;     // floats between rows of the 64 x 64 weight matrix
-constexpr int kWarpRows = 16, kRowThreads = 128;   // kernels with a warp to 16 whole rows
 
 template <int DP> constexpr int kStride = DP + 4;   // floats between rows of 64 x DP
 
@@ -244,26 +243,27 @@ __device__ __forceinline__ float row_sum16(float x)
     return x;
 }
 
-// ---- a warp to 16 whole rows (blocks of 128 threads, DP <= 128) -----------------------------------------------------
+// ---- a warp to R whole rows (DP <= 128) --------------------------------------------------------------------------------
 // Shared memory serves 16-byte reads eight lanes at a time, and lanes in different eights share nothing unless all 32 read one
 // address: so a warp's own rows are read by all its lanes at once (1 wavefront a read) and the streamed rows by a lane each (4).
-// 16 own rows x 2 streamed ones a lane take 24 wavefronts a 64 packed multiply-adds; 4 x 4 results a thread, with 2 x 16
-// threads a warp, took 24 a 32, and shared memory was the bound (77 % of its peak, the multiply-add pipe at 64 %).
-constexpr int kPairStride = 20;   // floats between the streamed rows of a warp's weights [64][16]: 16-byte stores, no conflicts
+// 16 own rows x 2 streamed ones a lane take 24 wavefronts a 64 packed multiply-adds, 8 own rows 16 a 32; 4 x 4 results a
+// thread, with 2 x 16 threads a warp, take 24 a 32.
+template <int R> constexpr int kPairStride = R + 4;   // floats between the streamed rows of a warp's weights [64][R]: no conflicts
 
 // s[i][j] = sum over channels of A[i] . B[lane + 32 j], even and odd channels apart as in tile_dot
-template <int DP>
-__device__ __forceinline__ void warp_dot(const float *A, const float *B, int lane, float (&s)[kWarpRows][2])
+template <int DP, int R>
+__device__ __forceinline__ void warp_dot(const float *A, const float *B, int lane, float (&s)[R][2])
 {
-    uint64_t acc[kWarpRows][2];
+    uint64_t acc[R][2];
 #pragma unroll
-    for (int i = 0; i < kWarpRows; ++i) acc[i][0] = acc[i][1] = 0ull;
+    for (int i = 0; i < R; ++i) acc[i][0] = acc[i][1] = 0ull;
     const float *b0 = B + lane * kStride<DP>;
-#pragma unroll 2
+    constexpr int kUnroll = R == 16 ? 2 : 4;   // what the registers hold
+#pragma unroll kUnroll
     for (int c = 0; c < DP; c += 4) {
         const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(b0 + c), y = *reinterpret_cast<const ulonglong2 *>(b0 + 32 * kStride<DP> + c);
 #pragma unroll
-        for (int i0 = 0; i0 < kWarpRows; i0 += 4) {   // four rows at a time: eight chains side by side
+        for (int i0 = 0; i0 < R; i0 += 4) {   // four rows at a time: eight chains side by side
             ulonglong2 a[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2 *>(A + (i0 + i) * kStride<DP> + c);
@@ -280,7 +280,7 @@ __device__ __forceinline__ void warp_dot(const float *A, const float *B, int lan
         }
     }
 #pragma unroll
-    for (int i = 0; i < kWarpRows; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             float lo, hi;
@@ -291,8 +291,8 @@ __device__ __forceinline__ void warp_dot(const float *A, const float *B, int lan
 
 // acc[k][c]: rows 2 k, 2 k + 1 of the warp (a packed pair) of channel DP / 32 lane + c; += sum over the 64 streamed rows j of
 // W[j][rows] * B[j][channels]
-template <int DP>
-__device__ __forceinline__ void warp_accumulate(const float *W, const float *B, int lane, uint64_t (&acc)[kWarpRows / 2][DP / 32])
+template <int DP, int R>
+__device__ __forceinline__ void warp_accumulate(const float *W, const float *B, int lane, uint64_t (&acc)[R / 2][DP / 32])
 {
     constexpr int C = DP / 32;
     const float *b0 = B + lane * C;
@@ -310,8 +310,8 @@ __device__ __forceinline__ void warp_accumulate(const float *W, const float *B, 
 #pragma unroll
         for (int c = 0; c < C; ++c) b2[c] = ptx::pack2(b[c], b[c]);
 #pragma unroll
-        for (int k = 0; k < kWarpRows / 2; k += 2) {
-            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(W + j * kPairStride + 2 * k);
+        for (int k = 0; k < R / 2; k += 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(W + j * kPairStride<R> + 2 * k);
 #pragma unroll
             for (int c = 0; c < C; ++c) {
                 acc[k][c] = ptx::fma2(w.x, b2[c], acc[k][c]);
@@ -322,8 +322,8 @@ __device__ __forceinline__ void warp_accumulate(const float *W, const float *B, 
 }
 
 // Row i of the warp's accumulators, the lane's channels.
-template <int C>
-__device__ __forceinline__ void acc_row(const uint64_t (&acc)[kWarpRows / 2][C], int i, float (&x)[C])
+template <int R2, int C>
+__device__ __forceinline__ void acc_row(const uint64_t (&acc)[R2][C], int i, float (&x)[C])
 {
 #pragma unroll
     for (int c = 0; c < C; ++c) {
@@ -421,16 +421,17 @@ __device__ __forceinline__ bool sees(const KeyRuns &k, int qy, int qx, int ky, i
     return dy < k.n_half_width && abs(kx - qx) <= __ldg(k.half_width + dy);
 }
 
-// Which of the 16 rows of the tile from `row0` on see the token at (ky, kx), one bit each.
+// Which of the R (8 or 16) rows of the tile from `row0` on see the token at (ky, kx), one bit each.
+template <int R>
 __device__ __forceinline__ uint32_t seen_by(const KeyRuns &k, const TileRef &t, const Geometry &g, int row0, int ky, int kx)
 {
-    if (k.text || ky < 0) return 0xffffu;
-    const int w_log = min(g.patch_w_log, 4), width = 1 << w_log;   // of the 16 rows, so many lie in one row of the patch
+    if (k.text || ky < 0) return (1u << R) - 1u;
+    const int w_log = min(g.patch_w_log, R == 16 ? 4 : 3), width = 1 << w_log;   // of the R rows, so many lie in one row of the patch
     const int x0 = t.x + (row0 & (g.patch_w() - 1));
     int dy = ky - (t.y + (row0 >> g.patch_w_log));
     uint32_t bits = 0u;
 #pragma unroll 2
-    for (int b = 0; b < kWarpRows; b += width, --dy) {
+    for (int b = 0; b < R; b += width, --dy) {
         const int dist = abs(dy);
         if (dist >= k.n_half_width) continue;
         const int w = __ldg(k.half_width + dist), lo = max(kx - w - x0, 0), hi = min(kx + w - x0, width - 1);
