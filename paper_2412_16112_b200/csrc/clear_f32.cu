@@ -4,7 +4,8 @@
 // Serves fp32 tensors (where tensor-core input rounding would break a 1e-5 agreement), bf16 tensors of head sizes the
 // tensor-core kernels do not take, and non-positive scales, under the windows around the query (disc, square).
 //
-// Up to 128 channels (padded to 64 or 128) a block is four warps with 16 whole rows each (clear_f32_rows_kernel); above, the
+// Up to 128 channels (padded to 64 or 128) a block is four warps with 16 whole rows each, or eight with 8
+// (clear_f32_rows_kernel); above, the
 // accumulators of 16 rows would not fit a warp's registers, and 256 threads take 4 x 4 results each (clear_f32_tile_kernel).
 // What bounds it: the fp32 multiply-add units (2 x 64 x 64 x DP multiply-adds a step, DP = the head size rounded up
 // to 64, 128 or 256), and in the scores the reads from shared memory beside them.  1024 px, radius 8, 24 heads of 128: 2034 us
@@ -250,29 +251,29 @@ clear_f32_tile_kernel(const F32Params p)
     cluster.sync();   // nobody leaves while its rows are being read
 }
 
-// The same with a warp to 16 whole rows, for up to 128 channels.
+// The same with a warp to R whole rows, for up to 128 channels: 16, or 8 where every block has an SM to itself (launch_rows).
 constexpr float kMaxExponent = 16.f;   // a score this far above its row's reference moves it
-constexpr int kWarpRows = 16, kRowThreads = 32 * kRows / kWarpRows;
+template <int R> constexpr int kRowThreads = 32 * kRows / R;
 
 // Shared memory: Q, V, then the keys, whose place the weights take once the scores are in registers (with 64 channels they are
 // longer than the keys), the key lists, row values.
-template <int DP> constexpr size_t kRowsLists =
-    (2 * kRows * kStride<DP> + (kStride<DP> > 4 * kPairStride<kWarpRows> ? kStride<DP> : 4 * kPairStride<kWarpRows>) * kRows) * sizeof(float);
-template <int DP> constexpr size_t kRowsSmem = kRowsLists<DP> + 2 * sizeof(KeyTile) + 2 * kRows * sizeof(float) + 64 * sizeof(int);
+template <int DP, int R> constexpr size_t kRowsLists =
+    (2 * kRows * kStride<DP> + std::max(kStride<DP>, kRows / R * kPairStride<R>) * kRows) * sizeof(float);
+template <int DP, int R> constexpr size_t kRowsSmem = kRowsLists<DP, R> + 2 * sizeof(KeyTile) + 2 * kRows * sizeof(float) + 64 * sizeof(int);
 
-template <typename T, int DP>
-__global__ void __launch_bounds__(kRowThreads, 2)
+template <typename T, int DP, int R>
+__global__ void __launch_bounds__(kRowThreads<R>, R == 16 ? 2 : 1)
 clear_f32_rows_kernel(const F32Params p)
 {
     constexpr int C = DP / 32;
     extern __shared__ __align__(16) uint8_t smem[];
     float *sQ = reinterpret_cast<float *>(smem), *sV = sQ + kRows * kStride<DP>, *sK = sV + kRows * kStride<DP>;
-    KeyTile *keys = reinterpret_cast<KeyTile *>(smem + kRowsLists<DP>);
+    KeyTile *keys = reinterpret_cast<KeyTile *>(smem + kRowsLists<DP, R>);
     float *sM = reinterpret_cast<float *>(keys + 2), *sL = sM + kRows;
     int *red = reinterpret_cast<int *>(sL + kRows);
 
-    const int tid = threadIdx.x, lane = tid & 31, row0 = (tid >> 5) * kWarpRows;
-    float *sP = sK + (tid >> 5) * kRows * kPairStride<kWarpRows>;   // the warp's weights
+    const int tid = threadIdx.x, lane = tid & 31, row0 = (tid >> 5) * R;
+    float *sP = sK + (tid >> 5) * kRows * kPairStride<R>;   // the warp's weights
     const int part = (int)(blockIdx.x % (unsigned)p.n_split);   // rank in the cluster
     const TileRef tile = tile_of((int)(blockIdx.x / (unsigned)p.n_split), p.g);
     const KeyRuns runs = runs_of(tile, p.g);
@@ -281,7 +282,7 @@ clear_f32_rows_kernel(const F32Params p)
             *v = static_cast<const T *>(p.v) + base;
 
     // this block's share of the list: whole steps of 64 keys
-    const int n_steps_all = (list_length<kRowThreads>(runs, red) + kRows - 1) / kRows;
+    const int n_steps_all = (list_length<kRowThreads<R>>(runs, red) + kRows - 1) / kRows;
     const int per = (n_steps_all + p.n_split - 1) / p.n_split;
     const int step0 = min(part * per, n_steps_all), n_steps = min(per, n_steps_all - step0);
     KeyCursor cur;
@@ -293,35 +294,35 @@ clear_f32_rows_kernel(const F32Params p)
     }
     fill_key_tile(keys[0], cur, runs, n_steps > 0);
     __syncthreads();
-    load_rows<T, DP, kRowThreads>(sQ, q, keys[1].token, p.g.d);
+    load_rows<T, DP, kRowThreads<R>>(sQ, q, keys[1].token, p.g.d);
 
-    uint64_t o[kWarpRows / 2][C];
-    float m[kWarpRows], l[kWarpRows];   // per row its reference; of its sum the lane's share
+    uint64_t o[R / 2][C];
+    float m[R], l[R];   // per row its reference; of its sum the lane's share
 #pragma unroll
-    for (int i = 0; i < kWarpRows / 2; ++i)
+    for (int i = 0; i < R / 2; ++i)
 #pragma unroll
         for (int c = 0; c < C; ++c) o[i][c] = 0ull;
 #pragma unroll
-    for (int i = 0; i < kWarpRows; ++i) {
+    for (int i = 0; i < R; ++i) {
         m[i] = -CUDART_INF_F;
         l[i] = 0.f;
     }
 
     for (int s = 0; s < n_steps; ++s) {
         const KeyTile &kt = keys[s & 1];
-        load_rows<T, DP, kRowThreads>(sK, k, kt.token, p.g.d);
-        load_rows<T, DP, kRowThreads>(sV, v, kt.token, p.g.d);
+        load_rows<T, DP, kRowThreads<R>>(sK, k, kt.token, p.g.d);
+        load_rows<T, DP, kRowThreads<R>>(sV, v, kt.token, p.g.d);
         uint32_t on[2];   // rows that see the lane's keys
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int c = lane + 32 * j;
-            on[j] = kt.token[c] >= 0 ? seen_by<kWarpRows>(runs, tile, p.g, row0, kt.ky[c], kt.kx[c]) : 0u;
+            on[j] = kt.token[c] >= 0 ? seen_by<R>(runs, tile, p.g, row0, kt.ky[c], kt.kx[c]) : 0u;
         }
         cp_async_wait<1>();   // Q and K are here
         __syncthreads();
         if (s + 1 < n_steps) fill_key_tile(keys[(s + 1) & 1], cur, runs, true);
 
-        float w[kWarpRows][2];
+        float w[R][2];
         warp_dot<DP>(sQ + row0 * kStride<DP>, sK, lane, w);
         __syncthreads();      // every warp is done with the keys: the weights may land on them
 
@@ -329,7 +330,7 @@ clear_f32_rows_kernel(const F32Params p)
         // a row has): no maximum over the lanes and no scaling in the common step.
         float far = -CUDART_INF_F;
 #pragma unroll
-        for (int i = 0; i < kWarpRows; ++i)
+        for (int i = 0; i < R; ++i)
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 w[i][j] = ((on[j] >> i) & 1u) ? w[i][j] * p.scale : -CUDART_INF_F;
@@ -337,7 +338,7 @@ clear_f32_rows_kernel(const F32Params p)
             }
         if (__any_sync(0xffffffffu, far > kMaxExponent)) {
 #pragma unroll
-            for (int i = 0; i < kWarpRows; i += 2) {
+            for (int i = 0; i < R; i += 2) {
                 float alpha[2];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
@@ -357,22 +358,22 @@ clear_f32_rows_kernel(const F32Params p)
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int i = 0; i < kWarpRows; i += 4) {
+            for (int i = 0; i < R; i += 4) {
                 float e[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     e[u] = expf(w[i + u][j] - (m[i + u] == -CUDART_INF_F ? 0.f : m[i + u]));
                     l[i + u] += e[u];
                 }
-                *reinterpret_cast<float4 *>(sP + (lane + 32 * j) * kPairStride<kWarpRows> + i) = make_float4(e[0], e[1], e[2], e[3]);
+                *reinterpret_cast<float4 *>(sP + (lane + 32 * j) * kPairStride<R> + i) = make_float4(e[0], e[1], e[2], e[3]);
             }
         cp_async_wait<0>();
         __syncthreads();      // V has landed for everybody, and the weights are written
-        warp_accumulate<DP, kWarpRows>(sP, sV, lane, o);
+        warp_accumulate<DP, R>(sP, sV, lane, o);
         __syncthreads();      // before the next rows overwrite K, V
     }
 #pragma unroll
-    for (int i = 0; i < kWarpRows; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int x = 16; x > 0; x >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
 
@@ -380,7 +381,7 @@ clear_f32_rows_kernel(const F32Params p)
     int *bad = red;
     auto redo_bad = [&]() {
 #pragma unroll 1
-        for (int r = tid >> 5; r < kRows; r += kRowThreads / 32)
+        for (int r = tid >> 5; r < kRows; r += kRowThreads<R> / 32)
             if (bad[r] != 0) redo_row<T, DP>(p, r);
     };
     if (tid < kRows) bad[tid] = 0;
@@ -391,7 +392,7 @@ clear_f32_rows_kernel(const F32Params p)
     bool all_finite = true;
     if (p.n_split == 1) {
 #pragma unroll
-        for (int i = 0; i < kWarpRows; ++i) {
+        for (int i = 0; i < R; ++i) {
             // a query sees itself or the text keys: l > 0 for every row that exists
             const float inv = l[i] > 0.f ? 1.f / l[i] : 0.f;
             int qy, qx;
@@ -420,7 +421,7 @@ clear_f32_rows_kernel(const F32Params p)
     cp_async_wait<0>();
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kWarpRows; ++i) {
+    for (int i = 0; i < R; ++i) {
         float x[C];
         acc_row(o, i, x);
         store_channels(sV + (row0 + i) * kStride<DP> + ch, x);
@@ -431,7 +432,7 @@ clear_f32_rows_kernel(const F32Params p)
     }
     cluster.sync();
     const int rows = kRows / p.n_split;
-    for (int e = tid; e < rows * (DP / 4); e += kRowThreads) {
+    for (int e = tid; e < rows * (DP / 4); e += kRowThreads<R>) {
         const int r = part * rows + e / (DP / 4), c4 = e % (DP / 4) * 4;
         int qy, qx;
         const long long tok = tile_token(tile, r, p.g, qy, qx);
@@ -463,11 +464,22 @@ clear_f32_rows_kernel(const F32Params p)
 
 constexpr int blocks_per_sm(int d) { return d <= 128 ? 2 : 1; }
 
-template <typename T>
-int launch_typed(const F32Params &p, long long tiles, cudaStream_t stream)
+// 16 rows to a warp read least; but a block alone on its SM, which is what the tiny configurations come to, is the chain of one
+// warp, and 8 rows to each of twice as many make that shorter: 16 x 16 + 16, two heads of 64, 13.0 us against 14.3; of 128, 18.2
+// against 18.5.  With more blocks than SMs: two heads at 24 x 40 + 130 36.9 against 28.7, 24 of them 180 against 148.
+template <typename T, int DP>
+int launch_rows(const F32Params &p, long long tiles, int n_sm, cudaStream_t stream)
 {
-    if (p.g.d <= 64) return launch_tiles(clear_f32_rows_kernel<T, 64>, p, tiles, p.n_split, kRowsSmem<64>, stream, kRowThreads);
-    if (p.g.d <= 128) return launch_tiles(clear_f32_rows_kernel<T, 128>, p, tiles, p.n_split, kRowsSmem<128>, stream, kRowThreads);
+    if (tiles * p.n_split <= n_sm)
+        return launch_tiles(clear_f32_rows_kernel<T, DP, 8>, p, tiles, p.n_split, kRowsSmem<DP, 8>, stream, kRowThreads<8>);
+    return launch_tiles(clear_f32_rows_kernel<T, DP, 16>, p, tiles, p.n_split, kRowsSmem<DP, 16>, stream, kRowThreads<16>);
+}
+
+template <typename T>
+int launch_typed(const F32Params &p, long long tiles, int n_sm, cudaStream_t stream)
+{
+    if (p.g.d <= 64) return launch_rows<T, 64>(p, tiles, n_sm, stream);
+    if (p.g.d <= 128) return launch_rows<T, 128>(p, tiles, n_sm, stream);
     return launch_tiles(clear_f32_tile_kernel<T, 256>, p, tiles, p.n_split, forward_smem<256>(), stream);
 }
 
@@ -534,8 +546,8 @@ int launch_f32(const clear_plan &p, const void *q, const void *k, const void *v,
     const Extent e = extent_of(p, prm.g);
     prm.n_split = split_of(e, prm.g.n_bh, p.n_sm * blocks_per_sm(prm.g.d));
     const long long tiles = e.tiles * prm.g.n_bh;
-    if (p.shape.dtype == CLEAR_F32) return launch_typed<float>(prm, tiles, stream);
-    return launch_typed<__nv_bfloat16>(prm, tiles, stream);
+    if (p.shape.dtype == CLEAR_F32) return launch_typed<float>(prm, tiles, p.n_sm, stream);
+    return launch_typed<__nv_bfloat16>(prm, tiles, p.n_sm, stream);
 }
 
 }  // namespace clear
