@@ -269,6 +269,16 @@ __global__ void __launch_bounds__(kThreads, 2) clear_f32_bwd_kernel(const __grid
     for (int it = 0; it < st.n_iters; ++it) {
         const bool sweep1 = !KEY_ROLE && it < n_steps;
         const KeyTile &kt = sm.keys[it % 3];
+        // which of the thread's streamed tokens its rows see, while the rows are on their way: bit 4 i + j
+        uint32_t on = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = tx + 16 * j, ky = kt.ky[c], kx = kt.kx[c];
+            const bool here = kt.token[c] >= 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (here && sees(runs, r_y[i], r_x[i], ky, kx)) on |= 1u << (4 * i + j);
+        }
         cp_async_wait<1>();   // the stationary rows and B2 of this step are here
         __syncthreads();      // ... for everybody, and B1 of the step before is free
         st.load_b2(it + 1);
@@ -291,10 +301,9 @@ __global__ void __launch_bounds__(kThreads, 2) clear_f32_bwd_kernel(const __grid
                 float mx = -CUDART_INF_F;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int c = tx + 16 * j;
-                    const bool on = kt.token[c] >= 0 && sees(runs, r_y[i], r_x[i], kt.ky[c], kt.kx[c]);
-                    s[i][j] = on ? s[i][j] * p.scale : -CUDART_INF_F;
-                    g[i][j] = on ? g[i][j] : 0.f;   // (its weight is 0, but it may be no number)
+                    const bool here = (on >> (4 * i + j)) & 1u;
+                    s[i][j] = here ? s[i][j] * p.scale : -CUDART_INF_F;
+                    g[i][j] = here ? g[i][j] : 0.f;   // (its weight is 0, but it may be no number)
                     mx = fmaxf(mx, s[i][j]);
                 }
                 const float m_new = fmaxf(m[i], row_max16(mx)), m_ref = m_new == -CUDART_INF_F ? 0.f : m_new;
@@ -319,12 +328,12 @@ __global__ void __launch_bounds__(kThreads, 2) clear_f32_bwd_kernel(const __grid
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int c = tx + 16 * j;
-                const bool on = kt.token[c] >= 0 && sees(runs, r_y[i], r_x[i], kt.ky[c], kt.kx[c]);
+                const bool here = (on >> (4 * i + j)) & 1u;
                 const float mm = KEY_ROLE ? sm.col[it % 3][0][c] : m[i], il = KEY_ROLE ? sm.col[it % 3][1][c] : l[i],
                             de = KEY_ROLE ? sm.col[it % 3][2][c] : dl[i];
-                const float pr = on ? expf(s[i][j] * p.scale - mm) * il : 0.f;
+                const float pr = here ? expf(s[i][j] * p.scale - mm) * il : 0.f;
                 s[i][j] = pr;
-                g[i][j] = on ? pr * (g[i][j] - de) * p.scale : 0.f;
+                g[i][j] = here ? pr * (g[i][j] - de) * p.scale : 0.f;
             }
         if (KEY_ROLE) {
             // dV += P^T dO; a row of weights is written and read by one warp
