@@ -489,6 +489,17 @@ static void build_pairs(const Shape &s, Schedule &sch, MaskTable &masks)
             }
             for (const PatchTile &t : b)
                 if (!find(a, t)) only_b.push_back(t);
+            // Without text the nearest patches come first: a row's softmax has its reference from the first keys it is allowed,
+            // and until every row of a warp has one, its steps have maximum passes.
+            if (T == 0) {
+                auto far = [&](const PatchTile &t) {
+                    const int64_t dx = 2 * ((int64_t)t.x - it.qx), dy = 2 * (int64_t)t.y - it.qy0 - (it.n_sides == 2 ? it.qy1 : it.qy0);
+                    return dx * dx + dy * dy;
+                };
+                std::stable_sort(both.begin(), both.end(), [&](const std::pair<PatchTile, PatchTile> &u, const std::pair<PatchTile, PatchTile> &w) {
+                    return far(u.first) < far(w.first);
+                });
+            }
             // Key patches only one tile needs are taken two at a time, one per tile, so that both tiles stay busy; what
             // is left over runs one-sided.  Such a step stages twice the tiles of a shared one, so these steps are
             // spread evenly between the shared ones: in a row, they would outrun the copies behind the staging ring.
