@@ -734,9 +734,9 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
             // where one of 128 takes 64: the tensor core works 25 % more, and waits far less.)
             // At 128 channels the two warps take turns with P_t V and the first halves, step by step: with the groups issued in
             // turn, tile 1's scores follow tile 0's by a group and its exponentials run under the other's MMAs.  Without: 1024px
-            // 109 us against 101, 2048px 564 against 549.  (Passed on earlier, behind P_t V, or later, behind the second half,
+            // 103 us against 99, 2048px 551 against 530.  (Passed on earlier, behind P_t V, or later, behind the second half,
             // where the pipe idles at every hand-over: 534 and 673 against 525, when it was that.)  At 64 channels, where the
-            // MMAs take half, nothing is gained by keeping order: 67 x 120 in 228 us without turns, 232 with.
+            // MMAs take half, nothing is gained by keeping order: 67 x 120 in 208 us without turns, 215 with.
             // The tensor core holds about two MMAs ahead of the one it works on, some 150 clocks, and every barrier or
             // shuffle instruction of these warps spends 100 to 200 in the queue it shares with the exponentials of two
             // softmax warps: hence a warp per tile, the waits of one in the shadow of the other's MMAs (one warp for both
