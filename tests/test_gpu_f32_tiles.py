@@ -59,6 +59,34 @@ def test_forward_tiles_with_scores_that_climb(bh, gh, gw, T, r, d, rise):
     clear.clear_cache_clear()
 
 
+def _climb_by_twelve(bh, d, n_low, seed):
+    """An 8 x 8 grid at r = 1 behind n_low + 2 text tokens: the first n_low keys of every query score -12, the next two q0 k0, below 1 and
+    with all of fp32's bits, and the image keys -112.  A row's softmax is that of the two."""
+    T, gen = n_low + 2, torch.Generator(device="cpu").manual_seed(seed)
+    q, k, v = (torch.zeros(1, bh, T + 64, d) for _ in range(3))
+    q[..., 0], q[..., 1] = torch.rand(q.shape[:-1], generator=gen), 1.0
+    k[..., n_low, 0], k[..., n_low + 1, 0] = 0.7, -0.3
+    k[..., :n_low, 1], k[..., T:, 1] = -12.0, -112.0
+    v[..., n_low, :], v[..., n_low + 1, :] = 1.0, -1.0
+    return T, q, k, v
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("bh,n_low", [(100, 64), (1, 1024)])   # whole lists; lists cut eight ways, a block to an SM
+def test_forward_weights_of_rows_whose_first_keys_score_low(bh, n_low, d):
+    """out = tanh((s1 - s2) / 2), nearly.  A weight expf(s - m) is good to the rounding of s and of s - m and to expf's last bit: for s - m
+    within [-1, 2] at most 2^-25 + 2^-24 + 2^-23 of it, two of which a row has at half weight: 2.1e-7 and the output's 3e-8 at the most; a
+    third of that, for errors spread evenly, over all rows.  Against the -12 of the first tiles s - m is rounded at 2^-21: 1.9e-7 over all
+    rows."""
+    T, q, k, v = _climb_by_twelve(bh, d, n_low, 21)
+    want = oracle.attn(q, k, v, 8, 8, T, 1.0, 1.0)
+    out = torch.full_like(q, float("nan"), device="cuda:0")
+    clear.clear_attn_fwd_f32(*(t.cuda() for t in (q, k, v)), out, 8, 8, T, 1.0, 1.0)
+    err = np.abs(out.cpu().double().numpy() - want)
+    assert err.max() <= 2.4e-7 and np.sqrt((err ** 2).mean()) <= 0.8e-7, (err.max(), np.sqrt((err ** 2).mean()))
+    clear.clear_cache_clear()
+
+
 @pytest.mark.parametrize("bh,gh,gw,T,r,d", SHAPES)
 def test_backward_tiles(bh, gh, gw, T, r, d):
     q, k, v, g = _inputs(bh, gh, gw, T, d, 4, 12)
