@@ -366,11 +366,12 @@ __global__ void __launch_bounds__(kThreads, 2) clear_f32_bwd_kernel(const __grid
 }
 
 // The same with a warp to 8 whole rows (warp_dot), for 65 to 128 channels: less shared memory is read for the products, and in the
-// first sweep a row's reference moves only when a score lies far above it, so lanes exchange nothing.  24 heads of 128 at
-// 24 x 40 + 130, radius 8: 1194 us, 1351 with 4 x 4 results a thread.  At 64 channels, where the products are half as long and
+// first sweep lanes exchange nothing in a step without a new maximum.  24 heads of 128 at
+// 24 x 40 + 130, radius 8: 1211 us, 1357 with 4 x 4 results a thread.  At 64 channels, where the products are half as long and
 // two blocks share an SM, 801 against 672 (and 704 with 16 rows to a warp of 128 threads, at 128 channels 1681).
+// A row's reference is its running maximum: against one that may lie 16 below (1201 us) weights were rounded at 2^-21, 14 % more error
+// of the gradients where keys climb, and delta's sum of weights times dP left fp32's range where dP was 10^7 times smaller.
 constexpr int kWarpRows = 8, kRowThreads = 32 * kRows / kWarpRows;
-constexpr float kMaxExponent = 16.f;   // a score this far above its row's reference moves it
 
 template <int DP> using RowsSmem = BwdSmem<DP, kRows / kWarpRows * kRows * kPairStride<kWarpRows>>;
 
@@ -505,8 +506,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) clear_f32_bwd_rows_kernel(cons
         warp_dot<DP>(sm.a1 + row0 * kStride<DP>, st.b1_rows(it), lane, s);
 
         if (sweep1) {
-            // against a reference per row that is moved only when a score lies far above it
-            float far = -CUDART_INF_F;
+            bool higher = false;   // than the row's reference
 #pragma unroll
             for (int i = 0; i < kWarpRows; ++i)
 #pragma unroll
@@ -514,9 +514,9 @@ __global__ void __launch_bounds__(kRowThreads, 1) clear_f32_bwd_rows_kernel(cons
                     const bool here = (on[j] >> i) & 1u;
                     s[i][j] = here ? s[i][j] * p.scale : -CUDART_INF_F;
                     g[i][j] = here ? g[i][j] : 0.f;   // (its weight is 0, but it may be no number)
-                    far = fmaxf(far, s[i][j] - m[i]);
+                    higher = higher || s[i][j] > m[i];
                 }
-            if (__any_sync(0xffffffffu, far > kMaxExponent)) {
+            if (__any_sync(0xffffffffu, higher)) {
 #pragma unroll
                 for (int i = 0; i < kWarpRows; ++i) {
                     float mx = fmaxf(s[i][0], s[i][1]);

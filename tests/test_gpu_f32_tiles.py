@@ -59,14 +59,14 @@ def test_forward_tiles_with_scores_that_climb(bh, gh, gw, T, r, d, rise):
     clear.clear_cache_clear()
 
 
-def _climb_by_twelve(bh, d, n_low, seed):
-    """An 8 x 8 grid at r = 1 behind n_low + 2 text tokens: the first n_low keys of every query score -12, the next two q0 k0, below 1 and
-    with all of fp32's bits, and the image keys -112.  A row's softmax is that of the two."""
+def _low_keys_first(bh, d, n_low, seed, low=-12.0):
+    """An 8 x 8 grid at r = 1 behind n_low + 2 text tokens: the first n_low keys of every query score `low`, the next two q0 k0, below 1
+    and with all of fp32's bits, and the image keys -112.  A row's softmax is that of the two."""
     T, gen = n_low + 2, torch.Generator(device="cpu").manual_seed(seed)
     q, k, v = (torch.zeros(1, bh, T + 64, d) for _ in range(3))
     q[..., 0], q[..., 1] = torch.rand(q.shape[:-1], generator=gen), 1.0
     k[..., n_low, 0], k[..., n_low + 1, 0] = 0.7, -0.3
-    k[..., :n_low, 1], k[..., T:, 1] = -12.0, -112.0
+    k[..., :n_low, 1], k[..., T:, 1] = low, -112.0
     v[..., n_low, :], v[..., n_low + 1, :] = 1.0, -1.0
     return T, q, k, v
 
@@ -78,7 +78,7 @@ def test_forward_weights_of_rows_whose_first_keys_score_low(bh, n_low, d):
     within [-1, 2] at most 2^-25 + 2^-24 + 2^-23 of it, two of which a row has at half weight: 2.1e-7 and the output's 3e-8 at the most; a
     third of that, for errors spread evenly, over all rows.  Against the -12 of the first tiles s - m is rounded at 2^-21: 1.9e-7 over all
     rows."""
-    T, q, k, v = _climb_by_twelve(bh, d, n_low, 21)
+    T, q, k, v = _low_keys_first(bh, d, n_low, 21)
     want = oracle.attn(q, k, v, 8, 8, T, 1.0, 1.0)
     out = torch.full_like(q, float("nan"), device="cuda:0")
     clear.clear_attn_fwd_f32(*(t.cuda() for t in (q, k, v)), out, 8, 8, T, 1.0, 1.0)
@@ -99,6 +99,40 @@ def test_backward_tiles(bh, gh, gw, T, r, d):
         err = np.abs(got.cpu().double().numpy() - ref)
         # fp32 sums of a few hundred terms of order one (the bound of the small-shape tests)
         assert err.max() <= 1e-4, f"{name}: max {err.max():.3e}"
+    clear.clear_cache_clear()
+
+
+@pytest.mark.parametrize("d", [96, 128])
+@pytest.mark.parametrize("bh,n_low", [(100, 64), (1, 1024)])   # whole lists; lists cut eight ways
+def test_backward_weights_of_rows_whose_first_keys_score_low(bh, n_low, d):
+    """dO = 1 in channel c of row c alone: dV of a key is its weight p in the first d rows.  p = e1 / (e1 + e2) at about a half is good to
+    half of e1's and the sum's errors (2^-25 for s, 2^-25 for s - m, 2^-23 for expf, twice) and two roundings of 2^-24: 2.4e-7 at the
+    most, and a quarter of that, for errors spread evenly, over all rows.  Against the -12 of the first tiles: 1.0e-7 over all rows."""
+    T, q, k, v = _low_keys_first(bh, d, n_low, 22)
+    g = torch.zeros_like(q)
+    g[..., torch.arange(d), torch.arange(d)] = 1.0
+    want = oracle_bwd.attn_bwd(q, k, v, g, 8, 8, T, 1.0, 1.0)[2]
+    outs = [torch.full_like(q, float("nan"), device="cuda:0") for _ in range(3)]
+    clear.clear_attn_bwd_f32(*(t.cuda() for t in (q, k, v, g)), *outs, 8, 8, T, 1.0, 1.0)
+    err = np.abs(outs[2].cpu().double().numpy() - want)[..., n_low:n_low + 2, :]
+    assert err.max() <= 2.4e-7 and np.sqrt((err ** 2).mean()) <= 0.6e-7, (err.max(), np.sqrt((err ** 2).mean()))
+    clear.clear_cache_clear()
+
+
+@pytest.mark.parametrize("d", [64, 96, 128])
+@pytest.mark.parametrize("bh,n_low", [(100, 64), (1, 1024)])
+def test_backward_sums_stay_in_range_where_first_keys_score_low(bh, n_low, d):
+    """dP of 1e34: times a weight, which no maximum keeps at one, it would leave fp32's range.  Bound: 1e-5 of the largest gradient, for
+    fp32 sums of up to a thousand terms."""
+    T, q, k, v = _low_keys_first(bh, d, n_low, 23, low=-15.0)
+    v, g = v * 0.0, torch.zeros_like(q)
+    v[..., n_low, 3], v[..., n_low + 1, 3], g[..., 3] = 1e17, -1e17, 1e17
+    want = oracle_bwd.attn_bwd(q, k, v, g, 8, 8, T, 1.0, 1.0)
+    outs = [torch.full_like(q, float("nan"), device="cuda:0") for _ in range(3)]
+    clear.clear_attn_bwd_f32(*(t.cuda() for t in (q, k, v, g)), *outs, 8, 8, T, 1.0, 1.0)
+    for name, got, ref in zip(("dq", "dk", "dv"), outs, want):
+        err = np.abs(got.cpu().double().numpy() - ref)
+        assert err.max() <= 1e-5 * np.abs(ref).max(), f"{name}: max {err.max():.3e} of {np.abs(ref).max():.3e}"
     clear.clear_cache_clear()
 
 
