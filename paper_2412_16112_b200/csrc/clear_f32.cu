@@ -5,8 +5,8 @@
 // tensor-core kernels do not take, and non-positive scales, under the windows around the query (disc, square).
 //
 // Up to 128 channels (padded to 64 or 128) a block is four warps with 16 whole rows each, or eight with 8
-// (clear_f32_rows_kernel); above, the
-// accumulators of 16 rows would not fit a warp's registers, and 256 threads take 4 x 4 results each (clear_f32_tile_kernel).
+// (clear_f32_rows_kernel).  256 threads with 4 x 4 results each (clear_f32_tile_kernel) remain above, where the accumulators
+// of 16 rows would not fit a warp's registers, and for bf16 tensors where blocks share an SM (launch_rows).
 // What bounds it: the fp32 multiply-add units (2 x 64 x 64 x DP multiply-adds a step, DP = the head size rounded up
 // to 64, 128 or 256), and in the scores the reads from shared memory beside them.  1024 px, radius 8, 24 heads of 128: 2034 us
 // with 4 x 4 results a thread (shared memory at 77 % of its peak, multiply-adds at 64 %), 1734 us with whole rows (62 % and
@@ -78,7 +78,7 @@ __device__ __forceinline__ void redo_row(const F32Params &p, int r)
 }
 
 template <typename T, int DP>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, DP <= 128 ? 2 : 1)
 clear_f32_tile_kernel(const F32Params p)
 {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -471,12 +471,18 @@ constexpr int blocks_per_sm(int d) { return d <= 128 ? 2 : 1; }
 // 16 rows to a warp read least; but a block alone on its SM, which is what the tiny configurations come to, is the chain of one
 // warp, and 8 rows to each of twice as many make that shorter: 16 x 16 + 16, two heads of 64, 13.0 us against 14.3; of 128, 18.2
 // against 18.5.  With more blocks than SMs: two heads at 24 x 40 + 130 36.9 against 28.7, 24 of them 180 against 148.
+// bf16 rows pass through registers on their way to shared memory, with nothing else to do for the warps meanwhile: there 256 threads
+// hide more of it than 128.  24 heads of 128 at 40 x 40, radius 4, 165 us with 4 x 4 results a thread, 194 with 16 rows a warp;
+// at 24 x 40 + 130 344 and 371, at 1024 px, radius 8, 2400 and 2570; of 40 channels 102 and 116, 205 and 211, 1399 and 1398.
 template <typename T, int DP>
 int launch_rows(const F32Params &p, long long tiles, int n_sm, cudaStream_t stream)
 {
     if (tiles * p.n_split <= n_sm)
         return launch_tiles(clear_f32_rows_kernel<T, DP, 8>, p, tiles, p.n_split, kRowsSmem<DP, 8>, stream, kRowThreads<8>);
-    return launch_tiles(clear_f32_rows_kernel<T, DP, 16>, p, tiles, p.n_split, kRowsSmem<DP, 16>, stream, kRowThreads<16>);
+    if constexpr (sizeof(T) == 2)
+        return launch_tiles(clear_f32_tile_kernel<T, DP>, p, tiles, p.n_split, forward_smem<DP>(), stream);
+    else
+        return launch_tiles(clear_f32_rows_kernel<T, DP, 16>, p, tiles, p.n_split, kRowsSmem<DP, 16>, stream, kRowThreads<16>);
 }
 
 template <typename T>

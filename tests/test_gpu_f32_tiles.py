@@ -43,6 +43,26 @@ def test_forward_tiles(bh, gh, gw, T, r, d):
     clear.clear_cache_clear()
 
 
+@pytest.mark.parametrize("negative", [False, True])
+@pytest.mark.parametrize("bh,gh,gw,T,r,d", [
+    (1, 8, 8, 1, 20.0, 72),      # one block with two steps: 8 rows a warp
+    (40, 17, 23, 20, 4.0, 72),   # more blocks than SMs: 4 x 4 results a thread
+    (40, 13, 19, 0, 4.0, 8),
+    (3, 24, 40, 130, 8.0, 40),   # cut lists, more blocks than SMs
+    (2, 9, 21, 33, 3.0, 136),
+])
+def test_forward_tiles_of_bf16_tensors(bh, gh, gw, T, r, d, negative):
+    """Head sizes that the tensor-core kernels do not take, and a scale that they do not: fp32 arithmetic (1e-5, as above), the output
+    rounded to 8 bits."""
+    q, k, v = (x.to(torch.bfloat16) for x in _inputs(bh, gh, gw, T, d, 3, 15))
+    scale = (-1 if negative else 1) / math.sqrt(d)
+    want = oracle.attn(q, k, v, gh, gw, T, r, scale)
+    out = torch.full_like(q, float("nan"), device="cuda:0")
+    clear.clear_attn_fwd(*(t.cuda() for t in (q, k, v)), out, gh, gw, T, r, scale)
+    assert (np.abs(out.cpu().double().numpy() - want) <= 1e-5 + 2.0 ** -8 * np.abs(want)).all()
+    clear.clear_cache_clear()
+
+
 @pytest.mark.parametrize("rise", [10, 17, 90, -17])
 @pytest.mark.parametrize("bh,gh,gw,T,r,d", [(1, 24, 40, 130, 8.0, 64), (40, 19, 23, 0, 6.0, 128), (2, 3, 90, 70, 9.0, 40)])
 def test_forward_tiles_with_scores_that_climb(bh, gh, gw, T, r, d, rise):
