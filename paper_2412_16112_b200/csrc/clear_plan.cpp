@@ -489,16 +489,21 @@ static void build_pairs(const Shape &s, Schedule &sch, MaskTable &masks)
             }
             for (const PatchTile &t : b)
                 if (!find(a, t)) only_b.push_back(t);
-            // Without text the nearest patches come first: a row's softmax has its reference from the first keys it is allowed,
-            // and until every row of a warp has one, its steps have maximum passes.
+            // Without text the nearest patches come first, those of one tile as well as the shared ones: a row's softmax has its
+            // reference from the first keys it is allowed, and until every row of a warp has one, its steps have maximum passes.
+            // 24 heads of 64 at 128 x 128, radius 2, four steps an item: 188 us in raster order, 145 so; with the shared ones
+            // alone in this order 211, as the lower tile's last rows then saw their first key in its last step.
             if (T == 0) {
-                auto far = [&](const PatchTile &t) {
-                    const int64_t dx = 2 * ((int64_t)t.x - it.qx), dy = 2 * (int64_t)t.y - it.qy0 - (it.n_sides == 2 ? it.qy1 : it.qy0);
+                auto far = [&](const PatchTile &t, int64_t qy) {
+                    const int64_t dx = (int64_t)t.x - it.qx, dy = t.y - qy;
                     return dx * dx + dy * dy;
                 };
+                const int64_t y0 = it.qy0, y1 = it.n_sides == 2 ? it.qy1 : it.qy0;
                 std::stable_sort(both.begin(), both.end(), [&](const std::pair<PatchTile, PatchTile> &u, const std::pair<PatchTile, PatchTile> &w) {
-                    return far(u.first) < far(w.first);
+                    return far(u.first, y0) + far(u.first, y1) < far(w.first, y0) + far(w.first, y1);
                 });
+                std::stable_sort(only_a.begin(), only_a.end(), [&](const PatchTile &u, const PatchTile &w) { return far(u, y0) < far(w, y0); });
+                std::stable_sort(only_b.begin(), only_b.end(), [&](const PatchTile &u, const PatchTile &w) { return far(u, y1) < far(w, y1); });
             }
             // Key patches only one tile needs are taken two at a time, one per tile, so that both tiles stay busy; what
             // is left over runs one-sided.  Such a step stages twice the tiles of a shared one, so these steps are

@@ -359,6 +359,60 @@ def test_pair_schedule_covers_each_allowed_pair_exactly_once(gh, gw, T, r):
         assert info.workspace_bytes == len(slots) * 128 * (128 + 2) * 4
 
 
+def _patches_of_sides(p):
+    """Per image item (its tile origins), per side: [(x, y, shared, mask entry or -1)] in the order of its steps, patches only."""
+    items, steps = p.pair_tables()
+    out = {}
+    for it in items:
+        if it.kind == 1:
+            continue
+        sides = []
+        for t in range(it.n_sides):
+            use, masked = (clear.STEP_USE1, clear.STEP_MASKED1) if t else (clear.STEP_USE0, clear.STEP_MASKED0)
+            sides.append([(st.x1 if t else st.x0, st.y1 if t else st.y0, bool(st.flags & clear.STEP_SHARED),
+                           (st.n_valid1 if t else st.n_valid0) if st.flags & masked else -1)
+                          for st in steps[it.step_begin:it.step_begin + it.step_count]
+                          if st.flags & use and not st.flags & clear.STEP_LINEAR])
+        out[it.qx, it.qy0] = (it, sides)
+    return out
+
+
+@pytest.mark.parametrize("gh,gw,r", [(64, 80, 2.0), (64, 80, 4.0), (40, 67, 5.5), (45, 70, 12.5), (33, 48, 20.0), (9, 33, 5.5), (1, 70, 3.0)])
+def test_order_of_the_key_patches_with_and_without_text(gh, gw, r):
+    """Raster order behind text; without text the nearest first, the shared patches by their distance from both tiles and the others by
+    that from their own.  The patches are the same."""
+    plans = [clear.Plan(1, 1, gh, gw, T, 64, r, kernel=clear.KERNEL_TCGEN05_WS, host_only=True) for T in (0, 128)]
+    plain, text = (_patches_of_sides(p) for p in plans)
+    assert plain.keys() == text.keys()
+    for key, (it, sides) in plain.items():
+        far = lambda t, x, y: (x - it.qx) ** 2 + (y - (it.qy1 if t else it.qy0)) ** 2
+        for t, patches in enumerate(sides):
+            behind_text = text[key][1][t]
+            assert sorted(p[:3] for p in patches) == sorted(p[:3] for p in behind_text)
+            assert len({p[:2] for p in patches}) == len(patches)
+            for shared in (False, True):
+                mine = [(x, y) for x, y, s, _ in patches if s == shared]
+                dist = [far(0, x, y) + far(1, x, y) if shared else far(t, x, y) for x, y in mine]
+                assert dist == sorted(dist)
+                raster = [(y, x) for x, y, s, _ in behind_text if s == shared]
+                assert raster == sorted(raster)
+
+
+@pytest.mark.parametrize("gh,gw,r", [(128, 128, 1.5), (128, 128, 2.0), (128, 128, 3.0), (128, 128, 4.0), (67, 120, 3.0), (100, 100, 6.0)])
+def test_without_text_a_row_sees_a_key_in_its_tiles_first_two_patches(gh, gw, r):
+    """So that the steps behind them need no maximum passes.  (Tiles whose rows all exist.)"""
+    p = clear.Plan(1, 1, gh, gw, 0, 64, r, kernel=clear.KERNEL_TCGEN05_WS, host_only=True)
+    table = p.mask_table()
+    for (qx, qy), (it, sides) in _patches_of_sides(p).items():
+        for t, patches in enumerate(sides):
+            if qx + 16 > gw or (it.qy1 if t else it.qy0) + 8 > gh:
+                continue
+            seen = np.zeros(128, dtype=bool)
+            for _, _, _, entry in patches[:2]:
+                seen |= table[entry].any(1) if entry >= 0 else True
+            assert seen.all(), (qx, qy, t, patches)
+
+
 def test_mask_table_cap_sends_patches_to_the_table_free_path(monkeypatch):
     monkeypatch.setenv("CLEAR_MAX_MASK_ENTRIES", "3")
     p = clear.Plan(1, 1, 40, 40, 0, 128, 9.0, kernel=clear.KERNEL_TCGEN05_WS, host_only=True)
