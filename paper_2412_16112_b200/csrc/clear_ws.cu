@@ -970,6 +970,12 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                 float ref = -INFINITY, l = 0.f;  // reference of the row's exponents (log2 units) and row sum
                 bool careful = false;            // maximum passes up to the end of the item
                 bool first = true, exact = true; // this step has one
+                // At 128 channels the first tile is looked at once: its own step runs against the maxima just found, and where
+                // the steps behind it want maximum passes it is alone in the common loop.  1024px, Q times 20: 169 us with a
+                // second look, 165 without.  At 64 channels that costs the common loop more than it saves (67 x 120: 218 us
+                // with a second look, 222 without; Q times 20 355 and 351).
+                constexpr bool kLookOnce = D == 128;
+                uint32_t go_on = kSidePlain;     // bits that a step has to have to follow in the common loop
                 uint32_t w = take_step(), w1 = take_step(), w2;
                 uint4 mw = load_mask(w), mw1;    // bit j of word i = key 32 i + j allowed
                 // The common steps run in a loop of their own, with what is rare outside of it.
@@ -983,6 +989,10 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                         ref = top.most * c;
                         careful = __any_sync(0xffffffffu, (top.most - top.least) * c > kWideStep);
                         exact = careful || __any_sync(0xffffffffu, ref == -INFINITY && q_valid);
+                        if (kLookOnce && exact) {
+                            exact = false;
+                            go_on = 0u;
+                        }
                     }
                     float tile_sum;
                     if (!exact) {
@@ -1040,9 +1050,13 @@ clear_ws_kernel(const __grid_constant__ WsMaps maps, const __grid_constant__ WsP
                             w = w1;
                             w1 = w2;
                             mw = mw1;
-                            if (__builtin_expect(!(w & kSidePlain), 0)) break;
+                            if (__builtin_expect(!(w & go_on), 0)) break;
                         }
-                        if (!over) continue;   // none left, or one whose mask is to be worked out
+                        if (!over) {   // none left, one with a maximum pass, or one whose mask is to be worked out
+                            exact = go_on == 0u;
+                            go_on = kSidePlain;
+                            continue;
+                        }
                     } else {
                         mw1 = load_mask(w1);
                         w2 = take_step();

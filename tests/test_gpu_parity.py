@@ -670,6 +670,31 @@ def test_ws_kernel_with_long_queries(gh, gw, T, r, d, length):
     assert (np.abs(got - want) <= bound).all(), float(np.abs(got - want).max())
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("gh,gw,T,r,length,dead", [
+    (8, 16, 128, 1.0, 60.0, False),    # a whole first tile, then one patch
+    (8, 16, 130, 2.0, 20.0, False),    # ... a run of two tokens, then one patch
+    (24, 40, 300, 8.0, 60.0, False),
+    (24, 40, 300, 8.0, 1.0, True),     # minus infinity for all scores of the first tile
+    (8, 16, 130, 2.0, 1.0, True),
+])
+def test_ws_kernel_whose_first_tile_sends_the_next_steps_to_maximum_passes(gh, gw, T, r, d, length, dead):
+    """Scores of a whole first tile that lie far apart, or are no reference at all: its own step has its maxima from the first look, the
+    steps behind it look for theirs.  Bound as for long queries."""
+    q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, seed=gh + T)
+    q = (q.float() * length).to(torch.bfloat16)
+    q[..., 0], k[..., 0] = 1.0, 0.0
+    scale = 1 / math.sqrt(d)
+    logit = scale * float(q.float().norm(dim=-1).max() * k.float().norm(dim=-1).max())
+    if dead:
+        k[:, :, :128, 0] = float("-inf")
+    want = oracle.attn(q, k, v, gh, gw, T, r, scale)
+    got = run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS).double().numpy()
+    v_max = float(v.float().abs().max())
+    bound = 2.0 ** -8 * (np.abs(want) + v_max) + 2.0 ** -21 * logit * v_max
+    assert (np.abs(got - want) <= bound).all(), float(np.abs(got - want).max())
+
+
 @pytest.mark.parametrize("rise", [10, 20, 55, 70])
 @pytest.mark.parametrize("gh,gw,T,r,d", [(24, 40, 300, 8.0, 128), (19, 23, 0, 6.0, 64), (40, 72, 20, 40.0, 64)])
 def test_ws_kernel_raises_references_step_by_step(gh, gw, T, r, d, rise):
