@@ -368,6 +368,12 @@ int clear_plan_pair_tables(const clear_plan_t *plan, const clear_pair_item_t **i
  * patch (row-major) exists and lies within the radius of that query.  Errors: INVALID_ARG. */
 int clear_plan_mask_table(const clear_plan_t *plan, const uint32_t **words, int32_t *n_entries);
 
+/* What the softmax warps of a TCGEN05_WS plan walk: a word per step that a query tile takes part in, 2 * n_steps words.  Those of
+ * side t of an item begin at t * n_steps + step_begin, without gaps, zeros behind them up to step_count.  Bit 0: a masked tile;
+ * bit 1: its mask is not in the table; bits 2..11: its entry there; bit 12: bit 1 is clear; bit 13: set; bits 16..31: the step's
+ * number within the item.  Empty for other plans.  Errors: INVALID_ARG. */
+int clear_plan_side_words(const clear_plan_t *plan, const uint32_t **words, int32_t *n_steps);
+
 /* Forward pass with an explicit plan.  Tensor dtype is the plan's.  Calls on one plan share its
  * workspace and work queue; the library orders them on the device as described at clear_attn_fwd, so
  * they may be made on any streams (two plans of one shape run side by side).

@@ -33,7 +33,7 @@ EXPORTS = [
     "clear_last_device_status", "clear_plan_mask_table", "clear_cache_check", "clear_plan_trim", "clear_attn_bwd_f32", "clear_plan_create_ex",
     "clear_qk_norm_rope", "clear_log_scale_factor",
     "clear_band_geometry", "clear_plan_create_band", "clear_attn_text_partial", "clear_text_merge",
-    "clear_plan_create_mask", "clear_attn_bwd_bf16", "clear_attn_bwd_bf16_tc",
+    "clear_plan_create_mask", "clear_attn_bwd_bf16", "clear_attn_bwd_bf16_tc", "clear_plan_side_words",
 ]
 
 
@@ -124,6 +124,8 @@ def load() -> ctypes.CDLL:
                                                ctypes.POINTER(ctypes.POINTER(PairStep)),
                                                ctypes.POINTER(ctypes.c_int32)]
         lib.clear_plan_mask_table.argtypes = [vp, ctypes.POINTER(ctypes.POINTER(ctypes.c_uint32)),
+                                              ctypes.POINTER(ctypes.c_int32)]
+        lib.clear_plan_side_words.argtypes = [vp, ctypes.POINTER(ctypes.POINTER(ctypes.c_uint32)),
                                               ctypes.POINTER(ctypes.c_int32)]
         lib.clear_attn_fwd_planned.argtypes = [vp, vp, vp, vp, vp, f32, vp]
         lib.clear_attn_fwd_host.argtypes = [vp, vp, vp, vp, vp, f32, vp]
@@ -339,6 +341,15 @@ class Plan:
         if n.value == 0:
             return np.zeros((0, 128, 4), dtype=np.uint32)
         return np.ctypeslib.as_array(words, shape=(n.value, 128, 4)).copy()
+
+    def side_words(self):
+        """Step words of a TCGEN05_WS plan's two query tiles as a numpy array [2, n_steps] of uint32 (a copy)."""
+        import numpy as np
+        words, n = ctypes.POINTER(ctypes.c_uint32)(), ctypes.c_int32()
+        _check(load().clear_plan_side_words(self._h, ctypes.byref(words), ctypes.byref(n)), "clear_plan_side_words")
+        if n.value == 0:
+            return np.zeros((2, 0), dtype=np.uint32)
+        return np.ctypeslib.as_array(words, shape=(2, n.value)).copy()
 
     def forward(self, q, k, v, out, scale, stream=None):
         ptrs = _tensor_args(q, k, v, out, self.dtype)

@@ -513,6 +513,14 @@ int clear_plan_mask_table(const clear_plan_t *plan, const uint32_t **words, int3
     return CLEAR_OK;
 }
 
+int clear_plan_side_words(const clear_plan_t *plan, const uint32_t **words, int32_t *n_steps)
+{
+    if (!plan) return CLEAR_ERR_INVALID_ARG;
+    if (words) *words = plan->sch.side_words.data();
+    if (n_steps) *n_steps = (int32_t)(plan->sch.side_words.size() / 2);
+    return CLEAR_OK;
+}
+
 int clear_attn_fwd_planned(const clear_plan_t *plan, const void *q, const void *k, const void *v, void *out,
                            float scale, void *stream)
 {

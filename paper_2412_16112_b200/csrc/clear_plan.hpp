@@ -42,6 +42,8 @@ struct Shape {
 // Bits of Schedule::side_words: a mask from the table (entry from bit 2 on), or one the kernel works out; neither is rare;
 // always set; the step's number within its item from bit 16 on.
 constexpr uint32_t kSideMasked = 1, kSideRare = 2, kSidePlain = 1u << 12, kSideSome = 1u << 13;
+static_assert(kMaxMaskEntries <= 1024, "entries have the ten bits below kSidePlain");
+// (Step numbers stay below 2^15: a step has at least two of the 2^16 positions that pair_overflow allows an item.)
 
 struct Schedule {
     int64_t thr = 0;                     // ceil(radius^2): the disc allows dx^2 + dy^2 < thr (Eq. 3)

@@ -377,6 +377,60 @@ def _patches_of_sides(p):
     return out
 
 
+def check_side_words(p):
+    """Side t of an item has one word for each of its steps that the tile takes part in, in their order, and zeros behind them.
+    Returns the longest list."""
+    items, steps = p.pair_tables()
+    words = p.side_words()
+    assert words.shape == (2, len(steps))
+    n_entries, longest, rest = len(p.mask_table()), 0, words.copy()
+    for it in items:
+        for t in range(2):
+            use, masked = (clear.STEP_USE1, clear.STEP_MASKED1) if t else (clear.STEP_USE0, clear.STEP_MASKED0)
+            want = []
+            for i, st in enumerate(steps[it.step_begin:it.step_begin + it.step_count]):
+                if not st.flags & use:
+                    continue
+                entry = st.n_valid1 if t else st.n_valid0
+                if not st.flags & masked:
+                    kind = 1 << 12
+                elif st.flags & clear.STEP_LINEAR or entry < 0:   # the kernel works the mask out
+                    kind = 1 | 2
+                else:
+                    assert entry < n_entries
+                    kind = 1 | entry << 2 | 1 << 12
+                want.append(kind | 1 << 13 | i << 16)
+            mine = slice(it.step_begin, it.step_begin + it.step_count)
+            assert words[t, mine].tolist() == want + [0] * (it.step_count - len(want))
+            assert len(want) > 0 if t < it.n_sides else not want
+            rest[t, mine] = 0
+            longest = max(longest, len(want))
+    assert not rest.any()
+    return longest
+
+
+@pytest.mark.parametrize("gh,gw,T,r,cap,at_least", [
+    (16, 16, 16, 4.0, None, 1), (13, 19, 7, 2.5, None, 1),    # an odd row of patches: one-sided items
+    (24, 40, 130, 8.0, None, 1), (9, 33, 0, 5.5, None, 1),
+    (24, 40, 130, 8.0, "0", 1), (33, 48, 0, 20.0, "3", 1),    # no mask table, one that runs out
+    (64, 64, 512, 16.0, None, 33), (96, 96, 512, 64.0, None, 65),   # lists over one and over two windows of 32 steps
+    (40, 40, 300, 9.0, None, 1),
+])
+def test_side_words_are_the_steps_of_each_tile(gh, gw, T, r, cap, at_least, monkeypatch):
+    if cap is not None:
+        monkeypatch.setenv("CLEAR_MAX_MASK_ENTRIES", cap)
+    p = clear.Plan(1, 1, gh, gw, T, 128, r, kernel=clear.KERNEL_TCGEN05_WS, host_only=True)
+    assert check_side_words(p) >= at_least
+
+
+def test_side_words_of_band_plans_and_of_other_kernels():
+    for part, text_keys in ((clear.PART_BAND_IMAGE, True), (clear.PART_BAND_TEXT, True), (clear.PART_BAND_TEXT, False)):
+        for T in (0, 130) if part == clear.PART_BAND_IMAGE else (130,):
+            assert check_side_words(clear.BandPlan(1, 2, 64, 40, T, 64, 9.0, part, 16, 48, text_keys=text_keys, host_only=True)) > 0
+    assert clear.Plan(1, 1, 16, 16, 16, 64, 4.0, kernel=clear.KERNEL_TCGEN05, host_only=True).side_words().shape == (2, 0)
+    assert clear.load().clear_plan_side_words(None, None, None) == clear.ERR_INVALID_ARG
+
+
 @pytest.mark.parametrize("gh,gw,r", [(64, 80, 2.0), (64, 80, 4.0), (40, 67, 5.5), (45, 70, 12.5), (33, 48, 20.0), (9, 33, 5.5), (1, 70, 3.0)])
 def test_order_of_the_key_patches_with_and_without_text(gh, gw, r):
     """Raster order behind text; without text the nearest first, the shared patches by their distance from both tiles and the others by
