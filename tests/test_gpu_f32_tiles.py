@@ -107,7 +107,11 @@ def test_forward_weights_of_rows_whose_first_keys_score_low(bh, n_low, d):
     clear.clear_cache_clear()
 
 
-@pytest.mark.parametrize("bh,gh,gw,T,r,d", SHAPES)
+# more tiles than SMs above 64 channels: lists not cut, results stored without a merge
+_WHOLE_LISTS = [(40, 19, 23, 0, 6.0, 68), (40, 19, 23, 0, 6.0, 96), (40, 19, 23, 0, 6.0, 128)]
+
+
+@pytest.mark.parametrize("bh,gh,gw,T,r,d", SHAPES + _WHOLE_LISTS)
 def test_backward_tiles(bh, gh, gw, T, r, d):
     q, k, v, g = _inputs(bh, gh, gw, T, d, 4, 12)
     scale = 1 / math.sqrt(d)
@@ -119,6 +123,29 @@ def test_backward_tiles(bh, gh, gw, T, r, d):
         err = np.abs(got.cpu().double().numpy() - ref)
         # fp32 sums of a few hundred terms of order one (the bound of the small-shape tests)
         assert err.max() <= 1e-4, f"{name}: max {err.max():.3e}"
+    clear.clear_cache_clear()
+
+
+@pytest.mark.parametrize("rise", [10, 17, 90, -17])
+@pytest.mark.parametrize("bh,gh,gw,T,r,d", [(40, 19, 23, 0, 6.0, 128), (1, 24, 40, 130, 8.0, 96), (2, 3, 90, 70, 9.0, 40), (40, 19, 23, 0, 6.0, 64)])
+def test_backward_tiles_with_scores_that_climb(bh, gh, gw, T, r, d, rise):
+    """As in the forward test: references, and the sums against them, that move at every step, and that differ between the blocks of a
+    cut list.  Weights are good to eps, a few 2^-24 of the largest score and the rounding of fp32 sums, and each gradient to eps times
+    its sum with every term taken positive."""
+    q, k, v, g = _inputs(bh, gh, gw, T, d, 4, 16)
+    ys, xs = torch.arange(gh).repeat_interleave(gw), torch.arange(gw).repeat(gh)
+    q[..., 0], k[..., 0] = 1.0, rise * torch.cat([torch.arange(T) // 32, T // 32 + ys // 4 + xs // 16]).float()
+    want = oracle_bwd.attn_bwd(q, k, v, g, gh, gw, T, r, 1.0)
+    outs = [torch.full_like(q, float("nan"), device="cuda:0") for _ in range(3)]
+    clear.clear_attn_bwd_f32(*(t.cuda() for t in (q, k, v, g)), *outs, gh, gw, T, r, 1.0)
+    eps = 2.0 ** -21 * float(q.norm(dim=-1).max() * k.norm(dim=-1).max()) + 4e-6
+    q, k, v, g = (t.double() for t in (q, k, v, g))
+    P = (q @ k.mT).masked_fill(~torch.from_numpy(_mask(gh, gw, T, r)), -math.inf).softmax(-1)
+    dP = (g @ v.mT).abs()
+    dS = P * (dP + (P * dP).sum(-1, keepdim=True))
+    for name, got, ref, size in zip(("dq", "dk", "dv"), outs, want, (dS @ k.abs(), dS.mT @ q.abs(), P.mT @ g.abs())):
+        err = np.abs(got.cpu().double().numpy() - ref)
+        assert (err <= eps * size.numpy() + 1e-6).all(), f"{name}: {np.max(err - eps * size.numpy()):.3e}"
     clear.clear_cache_clear()
 
 
@@ -208,7 +235,7 @@ def test_forward_tiles_keep_non_finite_values_to_the_rows_that_see_them(H, gh, g
 
 
 @pytest.mark.parametrize("which", ["q", "k", "v", "g"])
-@pytest.mark.parametrize("H,gh,gw,T,r,d", _ISOLATION[:3])
+@pytest.mark.parametrize("H,gh,gw,T,r,d", _ISOLATION[:3] + _WHOLE_LISTS[2:])
 def test_backward_tiles_keep_non_finite_values_to_the_rows_that_see_them(H, gh, gw, T, r, d, which):
     """The same for the gradients.  A NaN in q or dO makes row t of P, or of dS, NaN; one in k or v does so for every query
     that sees it (the row's sum, or delta), v leaving P alone."""

@@ -700,12 +700,29 @@ def test_ws_kernel_whose_first_tile_sends_the_next_steps_to_maximum_passes(gh, g
 def test_ws_kernel_raises_references_step_by_step(gh, gw, T, r, d, rise):
     """Scores that climb by `rise` powers of two every 64 text tokens and every eight rows of the grid: sums of a tile below the
     bound of 2^16 that raises a row's reference, above it (P, sum and O scaled in place, by the first half of a tile or by the
-    second), and above 2^64 (taken again); lists of up to 40 steps, more than a window of 32.  Bound as for long queries."""
+    second), and above 2^64 (taken again); lists of up to 26 steps.  Bound as for long queries."""
     q, k, v = workloads.make_custom(1, 2, gh, gw, T, d, seed=rise + gh)
     climb = torch.cat([torch.arange(T) // 64, T // 64 + torch.arange(gh).repeat_interleave(gw) // 8]).float() * rise
     q[..., 0], k[..., 0] = 8.0, (climb / 8.0).to(torch.bfloat16)
     scale = math.log(2.0)
     q[..., 1:] *= 0.25
+    want = oracle.attn(q, k, v, gh, gw, T, r, scale)
+    got = run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS).double().numpy()
+    v_max = float(v.float().abs().max())
+    logit = scale * float(q.float().norm(dim=-1).max() * k.float().norm(dim=-1).max())
+    bound = 2.0 ** -8 * (np.abs(want) + v_max) + 2.0 ** -21 * logit * v_max
+    assert (np.abs(got - want) <= bound).all(), float((np.abs(got - want) - bound).max())
+
+
+@pytest.mark.parametrize("rise", [20, 70])
+def test_ws_kernel_raises_references_across_windows_of_steps(rise):
+    """The same over lists of up to 76 steps, whose words come to the warps 32 at a time: three windows."""
+    gh, gw, T, r, d = 96, 96, 512, 64.0, 64
+    q, k, v = workloads.make_custom(1, 1, gh, gw, T, d, seed=rise)
+    climb = torch.cat([torch.arange(T) // 64, T // 64 + torch.arange(gh).repeat_interleave(gw) // 8]).float() * rise
+    q[..., 0], k[..., 0] = 8.0, (climb / 8.0).to(torch.bfloat16)
+    q[..., 1:] *= 0.25
+    scale = math.log(2.0)
     want = oracle.attn(q, k, v, gh, gw, T, r, scale)
     got = run_plan(q, k, v, gh, gw, T, r, scale, clear.KERNEL_TCGEN05_WS).double().numpy()
     v_max = float(v.float().abs().max())
