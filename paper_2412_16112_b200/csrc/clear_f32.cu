@@ -77,6 +77,54 @@ __device__ __forceinline__ void redo_row(const F32Params &p, int r)
     o.store(static_cast<T *>(p.out) + base + (long long)tok * p.g.d, p.g.d, l == 0.f ? 0.f : 1.f / l);
 }
 
+// Rows of the block's tile that came out non-finite, each by a warp of its NT threads.
+template <typename T, int DP, int NT>
+__device__ __forceinline__ void redo_bad(const F32Params &p, const int *bad)
+{
+#pragma unroll 1
+    for (int r = (int)threadIdx.x >> 5; r < kRows; r += NT / 32)
+        if (bad[r] != 0) redo_row<T, DP>(p, r);
+}
+
+// The merge over a cluster: every block has left its un-normalised rows, references and sums in its own shared memory, and
+// finishes 64 / n_split rows from everybody's, in the order of the ranks.  Marks rows that are not finite; false if there is one.
+// The block stays until the cluster has met again.
+template <typename T, int DP, int NT>
+__device__ __forceinline__ bool merge_rows(const F32Params &p, const TileRef &tile, int part, float *sM, float *sL, float *sO, T *out, int *bad)
+{
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    bool all_finite = true;
+    const int rows = kRows / p.n_split;
+    for (int e = threadIdx.x; e < rows * (DP / 4); e += NT) {
+        const int r = part * rows + e / (DP / 4), ch = e % (DP / 4) * 4;
+        int qy, qx;
+        const long long tok = tile_token(tile, r, p.g, qy, qx);
+        float mx = -CUDART_INF_F;
+        for (int c = 0; c < p.n_split; ++c) mx = fmaxf(mx, cluster.map_shared_rank(sM, c)[r]);
+        if (mx == -CUDART_INF_F) mx = 0.f;
+        float sum = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < p.n_split; ++c) {
+            const float f = expf(cluster.map_shared_rank(sM, c)[r] - mx);
+            sum = fmaf(f, cluster.map_shared_rank(sL, c)[r], sum);
+            const float4 x = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(sO, c) + r * kStride<DP> + ch);
+            acc.x = fmaf(f, x.x, acc.x);
+            acc.y = fmaf(f, x.y, acc.y);
+            acc.z = fmaf(f, x.z, acc.z);
+            acc.w = fmaf(f, x.w, acc.w);
+        }
+        const float inv = sum > 0.f ? 1.f / sum : 0.f;
+        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+        if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, acc);
+        if (!finite4(acc)) {
+            bad[r] = 1;
+            all_finite = false;
+        }
+    }
+    return all_finite;
+}
+
 template <typename T, int DP>
 __global__ void __launch_bounds__(kThreads, DP <= 128 ? 2 : 1)
 clear_f32_tile_kernel(const F32Params p)
@@ -176,11 +224,6 @@ clear_f32_tile_kernel(const F32Params p)
 
     // rows that came out non-finite are taken again, each by a warp; `bad` lies over the list lengths, which are done with
     int *bad = red;
-    auto redo_bad = [&]() {
-#pragma unroll 1
-        for (int r = tid >> 5; r < kRows; r += kThreads / 32)
-            if (bad[r] != 0) redo_row<T, DP>(p, r);
-    };
     if (tid < kRows) bad[tid] = 0;
     __syncthreads();
 
@@ -202,12 +245,10 @@ clear_f32_tile_kernel(const F32Params p)
                 }
             }
         }
-        if (__syncthreads_or(!all_finite)) redo_bad();
+        if (__syncthreads_or(!all_finite)) redo_bad<T, DP, kThreads>(p, bad);
         return;
     }
 
-    // merge over the cluster: every block leaves its un-normalised rows, maxima and sums in its own shared memory and
-    // finishes 64 / n_split rows from everybody's, in the order of the ranks
     cg::cluster_group cluster = cg::this_cluster();
     cp_async_wait<0>();
     __syncthreads();
@@ -219,35 +260,8 @@ clear_f32_tile_kernel(const F32Params p)
             sL[ty + 16 * i] = l[i];
         }
     }
-    cluster.sync();
-    const int rows = kRows / p.n_split;
-    for (int e = tid; e < rows * (DP / 4); e += kThreads) {
-        const int r = part * rows + e / (DP / 4), ch = e % (DP / 4) * 4;
-        int qy, qx;
-        const long long tok = tile_token(tile, r, p.g, qy, qx);
-        float mx = -CUDART_INF_F;
-        for (int c = 0; c < p.n_split; ++c) mx = fmaxf(mx, cluster.map_shared_rank(sM, c)[r]);
-        if (mx == -CUDART_INF_F) mx = 0.f;
-        float sum = 0.f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int c = 0; c < p.n_split; ++c) {
-            const float f = expf(cluster.map_shared_rank(sM, c)[r] - mx);
-            sum = fmaf(f, cluster.map_shared_rank(sL, c)[r], sum);
-            const float4 x = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(sV, c) + r * kStride<DP> + ch);
-            acc.x = fmaf(f, x.x, acc.x);
-            acc.y = fmaf(f, x.y, acc.y);
-            acc.z = fmaf(f, x.z, acc.z);
-            acc.w = fmaf(f, x.w, acc.w);
-        }
-        const float inv = sum > 0.f ? 1.f / sum : 0.f;
-        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
-        if (tok >= 0 && ch < p.g.d) store4(out + tok * p.g.d + ch, acc);
-        if (!finite4(acc)) {
-            bad[r] = 1;
-            all_finite = false;
-        }
-    }
-    if (__syncthreads_or(!all_finite)) redo_bad();
+    all_finite = merge_rows<T, DP, kThreads>(p, tile, part, sM, sL, sV, out, bad);
+    if (__syncthreads_or(!all_finite)) redo_bad<T, DP, kThreads>(p, bad);
     cluster.sync();   // nobody leaves while its rows are being read
 }
 
@@ -383,11 +397,6 @@ clear_f32_rows_kernel(const F32Params p)
 
     // rows that came out non-finite are taken again, each by a warp; `bad` lies over the list lengths, which are done with
     int *bad = red;
-    auto redo_bad = [&]() {
-#pragma unroll 1
-        for (int r = tid >> 5; r < kRows; r += kRowThreads<R> / 32)
-            if (bad[r] != 0) redo_row<T, DP>(p, r);
-    };
     if (tid < kRows) bad[tid] = 0;
     __syncthreads();
 
@@ -415,12 +424,10 @@ clear_f32_rows_kernel(const F32Params p)
                 all_finite = false;
             }
         }
-        if (__syncthreads_or(!all_finite)) redo_bad();
+        if (__syncthreads_or(!all_finite)) redo_bad<T, DP, kRowThreads<R>>(p, bad);
         return;
     }
 
-    // merge over the cluster: every block leaves its un-normalised rows, references and sums in its own shared memory and
-    // finishes 64 / n_split rows from everybody's, in the order of the ranks
     cg::cluster_group cluster = cg::this_cluster();
     cp_async_wait<0>();
     __syncthreads();
@@ -434,35 +441,8 @@ clear_f32_rows_kernel(const F32Params p)
             sL[row0 + i] = l[i];
         }
     }
-    cluster.sync();
-    const int rows = kRows / p.n_split;
-    for (int e = tid; e < rows * (DP / 4); e += kRowThreads<R>) {
-        const int r = part * rows + e / (DP / 4), c4 = e % (DP / 4) * 4;
-        int qy, qx;
-        const long long tok = tile_token(tile, r, p.g, qy, qx);
-        float mx = -CUDART_INF_F;
-        for (int c = 0; c < p.n_split; ++c) mx = fmaxf(mx, cluster.map_shared_rank(sM, c)[r]);
-        if (mx == -CUDART_INF_F) mx = 0.f;
-        float sum = 0.f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int c = 0; c < p.n_split; ++c) {
-            const float f = expf(cluster.map_shared_rank(sM, c)[r] - mx);
-            sum = fmaf(f, cluster.map_shared_rank(sL, c)[r], sum);
-            const float4 x = *reinterpret_cast<const float4 *>(cluster.map_shared_rank(sV, c) + r * kStride<DP> + c4);
-            acc.x = fmaf(f, x.x, acc.x);
-            acc.y = fmaf(f, x.y, acc.y);
-            acc.z = fmaf(f, x.z, acc.z);
-            acc.w = fmaf(f, x.w, acc.w);
-        }
-        const float inv = sum > 0.f ? 1.f / sum : 0.f;
-        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
-        if (tok >= 0 && c4 < p.g.d) store4(out + tok * p.g.d + c4, acc);
-        if (!finite4(acc)) {
-            bad[r] = 1;
-            all_finite = false;
-        }
-    }
-    if (__syncthreads_or(!all_finite)) redo_bad();
+    all_finite = merge_rows<T, DP, kRowThreads<R>>(p, tile, part, sM, sL, sV, out, bad);
+    if (__syncthreads_or(!all_finite)) redo_bad<T, DP, kRowThreads<R>>(p, bad);
     cluster.sync();   // nobody leaves while its rows are being read
 }
 
