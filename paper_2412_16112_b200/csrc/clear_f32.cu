@@ -15,7 +15,7 @@
 // The keys are those of the union of the tile's windows and no others: rows are gathered run by
 // run, 64 at a time, so a step is only ever short at the end of the list.  An 8 x 8 patch is the split that wastes
 // least at the paper's radii: at r = 8 a patch walks 452 + n_text keys for windows of 193.
-// Two blocks share an SM (DP <= 128): one computes while the other waits for its rows.
+// Two blocks share an SM (DP <= 128, except with 8 rows to a warp): one computes while the other waits for its rows.
 // A problem too small to give every SM a tile cuts the lists over a cluster of up to 8 blocks, which merge their
 // partial softmax through distributed shared memory in a fixed order: no workspace, no second launch.
 #include <cuda_bf16.h>
@@ -46,8 +46,8 @@ template <int DP> constexpr size_t forward_smem()
     return 3 * (size_t)kRows * kStride<DP> * sizeof(float) + 2 * sizeof(KeyTile) + 2 * kRows * sizeof(float) + 64 * sizeof(int);
 }
 
-// Row r of the block's tile by itself (one warp).  (The code alone costs the kernel 1.6 % at 1024 px, 2.00 -> 2.03 ms; as a
-// function that is not inlined, or with addresses of its own, it costs as much.)
+// Row r of the block's tile by itself (one warp).  (The code alone cost the kernel with 4 x 4 results a thread 1.6 % at 1024 px, 2.00 ->
+// 2.03 ms; as a function that is not inlined, or with addresses of its own, it cost as much.)
 template <typename T, int DP>
 __device__ __forceinline__ void redo_row(const F32Params &p, int r)
 {

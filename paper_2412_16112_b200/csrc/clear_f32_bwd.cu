@@ -7,8 +7,9 @@
 //       p = exp(S - m) / l, dS = p (dP - delta) scale, dQ += dS K.
 //   key kernel: stationary K_j, V_j, streamed Q_i, dO_i with their statistics (the mask is symmetric, so the queries
 //       that see a key are the tokens that key's own query sees).  dV += P^T dO, dK += dS^T Q.
-// Two forms of both: 4 x 4 results a thread up to 64 channels (clear_f32_bwd_kernel), whole rows to a warp above
-// (clear_f32_bwd_rows_kernel).
+// Two forms of both: 4 x 4 results a thread up to 64 channels (clear_f32_bwd_kernel; two blocks an SM leave 128 registers, too few
+// with the mask bits of a step: the query kernel spills 48 bytes, and is 1.4 % faster all the same than with the windows asked for
+// where they are used, and 4 bytes), whole rows to a warp above (clear_f32_bwd_rows_kernel, no spills).
 // Bound by the fp32 multiply-add units: nine products of 64 x 64 x DP per pair of tiles.  The streamed rows go through
 // a ring of three buffers, so a row set travels while the two before it are worked on; a step has two barriers in the query kernel
 // and three in the key kernel.

@@ -341,8 +341,8 @@ __device__ __noinline__ RowState exact_step(uint32_t tmem_s, uint32_t tmem_o, ui
 // an MMA lie in the lanes of a quad; reference, mask and results of row r belong to lane r, and move by shuffles.  Scores of
 // one key at a time by scalar products took about a millisecond a step; the rest of the item has maximum passes, so that it
 // happens once an item and warp at most, and not at all where the first tile's scores are far apart already.  24 heads at
-// 1024 px, r = 8, Q times 20, 60 or 400: 157 us a call (2.7, 94 and 203 ms with scalar products and no memory of it; 100 us
-// with ordinary scores).
+// 1024 px, r = 8, Q times 20 or 60: 165 us a call (2.7 and 94 ms with scalar products and no memory of it; 105 us with ordinary
+// scores).  The slowest measured is Q times 5, 171 us: warps of one tile with maximum passes, and others without.
 template <int D>
 __device__ __noinline__ RowState rescue_step(const WsParams &prm, uint32_t tmem_p, uint32_t tmem_o, uint4 mask, float c, float ref, float l,
                                              long long row0, long long q_tok, int2 org, bool linear)

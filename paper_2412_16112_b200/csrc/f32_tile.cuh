@@ -1,15 +1,15 @@
-// Building blocks of the fp32 tile kernels (forward and backward pass on the CUDA cores): a block of 256 threads, or of 128
-// with whole rows to a warp (warp_dot), works on a tile of 64 tokens (an 8 x 8 patch of the grid,
-// longer and flatter on grids narrower than 8, or 64 consecutive text tokens) against the tokens its
-// queries can see, 64 at a time.
+// Building blocks of the fp32 tile kernels (forward and backward pass on the CUDA cores): a block works on a tile of 64 tokens
+// (an 8 x 8 patch of the grid, longer and flatter on grids narrower than 8, or 64 consecutive text tokens) against the tokens
+// its queries can see, 64 at a time.  Two ways to share the work: 4 x 4 results a thread, of 256, or whole rows to a warp
+// (warp_dot below), 8 of 256 threads or 16 of 128.
 //
-// Of 256, thread (ty, tx), 16 x 16, owns the rows ty + 16 i (i < 4) of the tile; one warp holds two values of ty with all
+// 4 x 4 results: thread (ty, tx), 16 x 16, owns the rows ty + 16 i (i < 4) of the tile; one warp holds two values of ty with all
 // their tx, so everything that is exchanged along a row stays inside a warp.
 //   product of two row sets (tile_dot):    4 x 4 results a thread, both operands as float4 along the channels, even
 //       and odd channels summed apart in the two halves of a packed fp32 pair (fma.rn.f32x2): no operand is ever
 //       repacked.  Rows are padded to DP + 4 floats, so the 16 rows a warp reads at one channel lie 16 bytes apart
-//       modulo 128: 2 shared-memory wavefronts per float4 of the streamed rows, 1 per float4 of the thread's own,
-//       12 per 16 clocks of multiply-adds.
+//       modulo 128: 4 shared-memory wavefronts per float4 of the streamed rows, 2 per float4 of the thread's own,
+//       24 per 16 clocks of multiply-adds.
 //   accumulation (tile_accumulate): row weights (64 x 64, in shared memory) times the streamed rows; a thread owns
 //       4 rows x DP / 16 channels, pairs of channels in packed arithmetic.
 #pragma once
@@ -246,8 +246,8 @@ __device__ __forceinline__ float row_sum16(float x)
 // ---- a warp to R whole rows (DP <= 128) --------------------------------------------------------------------------------
 // Shared memory serves 16-byte reads eight lanes at a time, and lanes in different eights share nothing unless all 32 read one
 // address: so a warp's own rows are read by all its lanes at once (1 wavefront a read) and the streamed rows by a lane each (4).
-// 16 own rows x 2 streamed ones a lane take 24 wavefronts a 64 packed multiply-adds, 8 own rows 16 a 32; 4 x 4 results a
-// thread, with 2 x 16 threads a warp, take 24 a 32.
+// 16 own rows x 2 streamed ones a lane take 24 wavefronts per 64 packed multiply-adds a lane (32 clocks), 8 own rows 16 per 32;
+// 4 x 4 results a thread, with 2 x 16 threads a warp, take 24 per 32.
 template <int R> constexpr int kPairStride = R + 4;   // floats between the streamed rows of a warp's weights [64][R]: no conflicts
 
 // s[i][j] = sum over channels of A[i] . B[lane + 32 j], even and odd channels apart as in tile_dot
