@@ -9,7 +9,7 @@
 // of 16 rows would not fit a warp's registers, and for bf16 tensors where blocks share an SM (launch_rows).
 // What bounds it: the fp32 multiply-add units (2 x 64 x 64 x DP multiply-adds a step, DP = the head size rounded up
 // to 64, 128 or 256), and in the scores the reads from shared memory beside them.  1024 px, radius 8, 24 heads of 128: 2034 us
-// with 4 x 4 results a thread (shared memory at 77 % of its peak, multiply-adds at 64 %), 1734 us with whole rows (62 % and
+// with 4 x 4 results a thread (shared memory at 77 % of its peak, multiply-adds at 64 %), 1734 us with whole rows (64 % and
 // 70 %): about 780 for the scores and 550 for the weights times V, each of which is 525 of multiply-adds, 130 for the copies
 // and 100 for the softmax, by runs without the one or the other.
 // The keys are those of the union of the tile's windows and no others: rows are gathered run by
